@@ -327,17 +327,9 @@ const char *firp_kernel_class_name(int32_t c);
  * entries ordered by (value descending, token id ascending) -- the same selection firp_step makes
  * for its rows -- and writes d_ids [rows][b] and d_vals [rows][b] (DEVICE, caller-owned).
  *
- * The intermediate candidates of the two-pass selection live in a 256 KiB array that is part of
- * the library image on every GPU that loads it; nothing is allocated or freed, by this call or by
- * anything it uses.  The array limits the problem size: rows * ceil(vocab / 2048) must not exceed
- * FIRP_TOPB_STATIC_MAX_SLOTS, otherwise FIRP_ERR_CAPACITY is returned (and a line on stderr says
- * which limit was hit); 1 <= b <= 8.
- *
- * The first call on a device looks up the array's device address (once per device, under a lock):
- * make that first call outside any stream capture.  All calls on a device share the one array and it
- * keeps whatever the previous call left; every entry a call reads it has written itself, so no clearing
- * is needed, but two calls whose kernels can overlap on the GPU (different streams, no ordering between
- * them) race on it and must be serialised by the caller.
+ * One kernel; nothing is allocated or freed, and it keeps no state: calls on different streams may overlap.
+ * Limits: rows * ceil(vocab / 2048) must not exceed FIRP_TOPB_STATIC_MAX_SLOTS, otherwise FIRP_ERR_CAPACITY is
+ * returned (and a line on stderr says which limit was hit); 1 <= b <= 8.
  * Work is enqueued on `stream`; nothing synchronises.  Returns FIRP_OK or a negative firp_status.
  */
 #define FIRP_TOPB_STATIC_MAX_SLOTS 4096

@@ -299,9 +299,8 @@ def firp_profile_read(ctx, stream: int = 0) -> dict:
 
 
 def firp_topb_static(d_logits_ptr: int, rows: int, vocab: int, b: int, d_ids_ptr: int, d_vals_ptr: int, stream: int = 0):
-    """Top-b of `rows` rows of device logits into caller-owned device arrays; allocates nothing (the
-    candidate scratch is a fixed array inside the library).  Raises FirpError on a bad argument or when
-    rows * ceil(vocab / 2048) exceeds the built-in scratch."""
+    """Top-b of `rows` rows of device logits into caller-owned device arrays; allocates nothing.
+    Raises FirpError on a bad argument or when rows * ceil(vocab / 2048) exceeds the limit of the ABI."""
     rc = load_library().firp_topb_static(d_logits_ptr, rows, vocab, b, d_ids_ptr, d_vals_ptr, stream)
     if rc != 0:
         raise FirpError(rc, "firp_topb_static rejected the call (see stderr)")

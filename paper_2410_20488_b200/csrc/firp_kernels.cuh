@@ -110,12 +110,9 @@ cudaError_t launch_rmsnorm(const Rows &rw, int v0, int v1, float *h, const Parti
 // source row's RMS (GemmArgs::ss of the EPI_PSEUDO finisher)
 void launch_root_split(const Rows &rw, const float *h, const bf16 *g, int d, bf16 *xp, size_t xp_lo_off, bool pdl, cudaStream_t st);
 
-// top-B of every row of logits by (value desc, id asc)
-// Two passes: per 2048-logit segment candidates (scratch cand_*: [R][topb_segments(V)][B]), then the row's top-B.
-constexpr int kTopSeg = 2048;
-int topb_segments(int V);
-void launch_topb(const float *logits, int R, int V, int B, int32_t *cand_ids, float *cand_vals, int32_t *ids, float *vals,
-                 bool pdl, cudaStream_t st);
+// top-B (B <= kMaxTopB) of every row of logits by (value desc, id asc) into ids, vals [R][B]; a row with fewer than B
+// numbers is padded with (-inf, INT_MAX)
+void launch_topb(const float *logits, int R, int V, int B, int32_t *ids, float *vals, bool pdl, cudaStream_t st);
 
 struct AcceptArgs {
   const int32_t *tokens;        // [n_seq][T]

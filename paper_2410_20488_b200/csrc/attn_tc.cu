@@ -140,6 +140,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   // mbarriers: K landed [2], V landed [2], S^T complete [2], P written [2], O^T complete [2], Q written
   __shared__ __align__(8) uint64_t s_bar[11];
   __shared__ uint32_t s_tmem;
+  __shared__ int s_sn[2];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   TC_STAMP(0);
@@ -176,8 +177,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int split = blockIdx.x, nsplits = gridDim.x;
   const int qrows_total = a.rows_active * G, q0 = qb * qper;
   const int ncols = min(qper, qrows_total - q0);
-  const int slot = a.seq_ids[s];
-  const int n = a.pos[s * a.rw.Ms];                 // position of the root row = committed length
   // queries of this block (all softmax threads share the work): column j = query row q0 + j -> (tree row
   // (q0 + j) / G, head kvh G + (q0 + j) % G).  Their loads go out before the context length above is first used.
   constexpr int QIT = (NQ * 16 + kTcSoft - 1) / kTcSoft;
@@ -194,6 +193,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
     }
   }
+  // one warp loads the slot and the committed length (position of the root row): thousands of warps asking L2 for the
+  // same two words at once took microseconds
+  if (warp == 18 && lane < 2) s_sn[lane] = lane == 0 ? __ldcg(a.seq_ids + s) : __ldcg(a.pos + s * a.rw.Ms);
+  __syncthreads();
+  const int slot = s_sn[0], n = s_sn[1];
   const int kv_len = min(n + a.rows_active, a.max_ctx);
   const int tiles_total = (kv_len + kTcTile - 1) / kTcTile;
   const int t0 = (split * tiles_total + nsplits - 1) / nsplits, t1 = ((split + 1) * tiles_total + nsplits - 1) / nsplits;

@@ -1,4 +1,4 @@
-// Device bodies of the finishers of the stream-K GEMMs: each sums the partial tiles a GEMM left in scratch
+// Device bodies of the finishers of the persistent kernel's stream-K GEMMs: each sums the partial tiles a GEMM left in scratch
 // (fixed order: ascending CTA index) and applies the elementwise step that follows the contraction:
 //   qkv     rotary embedding at the row's tree position (Section 3.4: a tree token keeps its
 //           positional index), queries as (hi, lo) bf16 planes, keys / values into the bf16 cache
@@ -74,6 +74,42 @@ __device__ __forceinline__ void split4(const float v[4], uint2 &hi, uint2 &lo) {
 __device__ __forceinline__ uint2 round4(const float v[4]) {
   const __nv_bfloat162 h01 = __floats2bfloat162_rn(v[0], v[1]), h23 = __floats2bfloat162_rn(v[2], v[3]);
   return make_uint2(*reinterpret_cast<const uint32_t *>(&h01), *reinterpret_cast<const uint32_t *>(&h23));
+}
+
+__device__ __forceinline__ float4 load_bf16x4(const bf16 *p) {
+  const uint2 v = *reinterpret_cast<const uint2 *>(p);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// A row of the residual stream has its new value: store it, and what the next GEMM reads of it -- x = h * g as bf16 planes
+// (not yet divided by the row's RMS: the consumer's epilogue does that), the sum of squares of these 128 columns and, for
+// the rows Eq. 3 reads at the next layer, their own planes.  One warp, 4 neighbouring columns per lane.
+template <typename Args>   // LinArgs or PrepArgs
+__device__ __forceinline__ void store_residual(const Args &a, int row, int xp_row, int col, float4 v, float4 g, int lane) {
+  *reinterpret_cast<float4 *>(a.h + (size_t)row * a.d + col) = v;
+  if (a.x == nullptr) return;
+  float sq = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if (lane == 0) a.ss_out[(size_t)row * kNormMaxWarps + (col >> 7)] = sq;
+  const float y[4] = {v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w};
+  uint2 hi, lo;
+  split4(y, hi, lo);
+  bf16 *dst = a.x + (size_t)row * a.d + col;
+  *reinterpret_cast<uint2 *>(dst) = hi;
+  *reinterpret_cast<uint2 *>(dst + a.x_plane) = lo;
+  if (a.x_planes == 3) {     // what hi + lo still miss
+    const float4 fh = load_bf16x4(reinterpret_cast<const bf16 *>(&hi)), fl = load_bf16x4(reinterpret_cast<const bf16 *>(&lo));
+    const float t[4] = {y[0] - fh.x - fl.x, y[1] - fh.y - fl.y, y[2] - fh.z - fl.z, y[3] - fh.w - fl.w};
+    *reinterpret_cast<uint2 *>(dst + 2 * a.x_plane) = round4(t);
+  }
+  if (xp_row >= 0) {
+    if (!a.xp_normed) { const float raw[4] = {v.x, v.y, v.z, v.w}; split4(raw, hi, lo); }
+    bf16 *dp = a.xp + (size_t)xp_row * a.d + col;
+    *reinterpret_cast<uint2 *>(dp) = hi;
+    *reinterpret_cast<uint2 *>(dp + a.xp_plane) = lo;
+  }
 }
 
 // ---- q, k, v: rotary embedding, query planes, cache rows --------------------------------------

@@ -84,7 +84,7 @@ struct firp_ctx {
   int pseudo_masked = 0;     // Section 4.3 "Masked": pseudo rows do not see one another
   int pred_prenorm = 0;      // Eq. 3 reads the anchor through the insertion layer's input RMSNorm
   int planes[5] = {2, 2, 2, 2, 2};
-  int attn_tc = -1;                  // head dimension 128: 1 the tcgen05 attention kernel, 0 the mma.sync one, -1 by the step's shape
+  int attn_tc = -1;                  // head dimension 128: 1, -1 the tcgen05 attention kernel, 0 the mma.sync one
   int attn_planes[2] = {2, 2};       // of the queries and of the probabilities in the attention   // bf16 planes of the activations per GEMM class: qkv, o, gate/up, down, lm-head
 
   // cache layout [layer][K|V][row][kv_head][head_dim]; row = slot * max_ctx + position, or through the page table
@@ -225,20 +225,22 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
   const firp_step_out *out = ra.out;
   int &nl = c->launches;
   const bool pdl = c->use_pdl;
-  // L2 lookahead per GEMM class (32 KB units beyond the ring): qkv, o, gate/up, down, lm-head.  Measured at the
-  // 7B shape: it pays before the GEMMs whose predecessor is short or cannot share the SM (o, gate/up) and
-  // costs before the down projection, whose finisher it slows by more than it saves.
-  static const int ahead[5] = {0, 48, 48, 0, 48};
-
-  const int mw_out = (rw.Ms + 31) / 32;
-  { FIRP_TIMED(KC_TREE_PREP);
-    launch_tree_prep(rw, c->parents, ra.parents_stride, c->seq_ids, c->ctx_len, dh, cfg.rope_theta, c->meta, out ? out->depth : nullptr,
-                     out ? out->mask : nullptr, mw_out, c->grid_bar, pdl, st); ++nl; }
-  { FIRP_TIMED(KC_EMBED);
-    launch_embed(rw, ra.d_tokens, (const bf16 *)c->w.embed, d, cfg.vocab, c->h, pdl, st); ++nl; }
-
   const FusedShape fshape{cfg.n_layers, d, H, Hkv, dh, F, cfg.vocab, cfg.max_ctx, cfg.rms_eps};
   const bool fused = c->use_fused && fused_eligible(fshape, rw);
+  const int per_step = rw.chains ? rw.T : 1;                   // pseudo rows one prediction step adds per sequence
+  const int x_planes = c->planes[0] == 3 ? 3 : 2;              // of the QKV projection's operand
+  { FIRP_TIMED(KC_TREE_PREP);
+    PrepArgs a{};
+    a.rw = rw; a.parents = c->parents; a.parents_stride = ra.parents_stride; a.seq_ids = c->seq_ids; a.ctx_len = c->ctx_len;
+    a.dh = dh; a.theta = cfg.rope_theta; a.meta = c->meta; a.zero_word = c->grid_bar;
+    if (out) { a.out_depth = out->depth; a.out_mask = out->mask; a.out_mask_words = (rw.Ms + 31) / 32; }
+    a.tokens = ra.d_tokens; a.embed = (const bf16 *)c->w.embed; a.d = d; a.vocab = cfg.vocab; a.h = c->h;
+    if (!fused) {
+      a.g = (const bf16 *)c->g_attn[0]; a.x = c->x; a.x_plane = Rp * d; a.x_planes = x_planes; a.ss_out = c->ss;
+      if (rw.kc > 0 && ra.tl[0] == 0) { a.xp = c->xp; a.xp_plane = Rp * d; a.xp_normed = c->pred_prenorm; }
+    }
+    launch_prep(a, pdl, st); ++nl; }
+
   if (fused) {      // all decoder layers (and the lm-head) as one persistent kernel
     FusedStep fs{};
     fs.shape = fshape; fs.rw = rw; memcpy(fs.tl, ra.tl, sizeof(fs.tl)); fs.want_head = ra.want_head; fs.prenorm = c->pred_prenorm != 0; fs.Rp = (int)Rp;
@@ -259,71 +261,43 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
     FIRP_CUDA(c, launch_fused_layers(plan, fs, pdl, st, &nl));
   }
 
-  auto gemm_base = [&](const bf16 *X, size_t lo_off, const void *W, int N, int K, int act) {
-    GemmArgs g{};
-    g.X = X; g.x_lo_off = lo_off; g.plane_rows = (int)Rp; g.err = c->dev_status; g.wait_ns = c->wait_ns;
-    g.W = (const bf16 *)W; g.R = rw.R; g.N = N; g.K = K; g.rw = rw; g.rows_active = act; g.planes = 2;
-    g.ws = c->gemm_ws; g.l2_ahead = 48;
-    if (X == c->x) { g.ss = c->ss; g.eps = cfg.rms_eps; }   // x = h * g: the finisher divides by the row's RMS
-    return g;
+  enum { G_QKV = 0, G_O, G_GATE_UP, G_DOWN, G_LM_HEAD };     // index of c->planes
+  auto launch = [&](GemmEpilogue epi, const void *W, int N, int K, int planes, int R, LinArgs &l) -> cudaError_t {
+    l.W = (const bf16 *)W; l.N = N; l.K = K; l.R = R; l.F = F; l.dh = dh; l.planes = planes; l.plane_rows = (int)Rp;
+    l.rw = rw; l.err = c->dev_status; l.wait_ns = c->wait_ns; l.eps = cfg.rms_eps;
+    ++nl;
+    return launch_gemm(epi, l, pdl, st);
   };
-  // partial tiles a residual GEMM left behind: the next RMSNorm adds them into the residual stream
-  Partials pending{};
-  pending.ws = c->gemm_ws; pending.ws_rows = (int)Rp;
-  const Partials none{};
-  // every GEMM names its successor, whose first units it prefetches into L2 at its own tail
-  // (32 KB units per CTA, by the GEMM that issues the prefetch: qkv, o, gate/up, down; 3 and 8 measured worse)
-  static const int next_units[4] = {5, 5, 5, 5};
-  auto set_next = [&](GemmArgs &g, int cls, GemmEpilogue epi, const void *W, int N, int K) {
-    g.next_W = (const bf16 *)W; g.next_epi = epi; g.next_N = N; g.next_K = K; g.next_F = F; g.next_heads = H + 2 * Hkv;
-    g.next_dh = dh; g.next_units = next_units[cls];
+  // what a residual GEMM leaves for the GEMM that reads the stream next: g * h as planes and the sums of squares
+  auto residual_out = [&](LinArgs &l, const void *g, int planes) {
+    l.h = c->h; l.d = d; l.g = (const bf16 *)g; l.x = c->x; l.x_plane = Rp * d; l.x_planes = planes; l.ss_out = c->ss;
   };
   int alive = 0;   // prediction steps appended below this layer
-  const int per_step = rw.chains ? rw.T : 1;                   // pseudo rows one prediction step adds per sequence
   for (int j = 0; j < cfg.n_layers && !fused; ++j) {
     int ins = 0;     // prediction steps whose layer this is
     while (alive + ins < rw.kc && ra.tl[alive + ins] == j) ++ins;
-    const bool insert = ins > 0;
-    // the rows that took part in the last residual GEMM get its pending sums; new pseudo rows have none
-    const int carried = rw.T + alive * per_step;
-    const int act = carried + ins * per_step;                  // rows alive in this layer
-    { FIRP_TIMED(KC_RMSNORM);
-      FIRP_CUDA(c, launch_rmsnorm(rw, 0, carried, c->h, pending, (const bf16 *)c->g_attn[j], d, c->x, Rp * d, c->planes[0] == 3 ? 3 : 2, c->ss, pdl, st)); ++nl; }
-    pending.sk.U = 0;
-    if (insert) {   // Eq. 3 on the raw (now complete) residual row of the root, then the norm of the new rows
-      { FIRP_TIMED(KC_PSEUDO_PROJ);      // this layer's maps as one [ins d][d] GEMM on the source rows (the anchor of
-                                         // each sequence, or every tree row when each node carries a chain)
-        launch_root_split(rw, c->h, c->pred_prenorm ? (const bf16 *)c->g_attn[j] : nullptr, d, c->xp, Rp * d, pdl, st); ++nl;
-        GemmArgs g{};
-        g.X = c->xp; g.x_lo_off = Rp * d; g.plane_rows = (int)Rp; g.planes = 2; g.err = c->dev_status; g.wait_ns = c->wait_ns;
-        g.W = (const bf16 *)c->w.pred_w + (size_t)alive * d * d; g.R = rw.n_seq * per_step; g.N = ins * d; g.K = d; g.rw = rw;
-        g.rows_active = act;
-        g.ws = c->gemm_ws; g.l2_ahead = 48;
-        g.h_rows = c->h; g.pseudo0 = alive;      // map i of this GEMM is prediction step alive + i
-        if (c->pred_prenorm) { g.ss = c->ss; g.eps = cfg.rms_eps; }   // the finisher divides by the source row's RMS
-        g.pred_b = c->w.pred_b ? (const bf16 *)c->w.pred_b + (size_t)alive * d : nullptr;
-        Partials p = pending;
-        FIRP_CUDA(c, launch_gemm_tc(EPI_PSEUDO, g, pdl, st, &p.sk)); ++nl;
-        p.ws_rows = (int)Rp;
-        FIRP_CUDA(c, launch_gemm_finish(EPI_PSEUDO, p, g, pdl, st)); ++nl; }
-      FIRP_TIMED(KC_RMSNORM);
-      FIRP_CUDA(c, launch_rmsnorm(rw, carried, act, c->h, none, (const bf16 *)c->g_attn[j], d, c->x, Rp * d, c->planes[0] == 3 ? 3 : 2, c->ss, pdl, st)); ++nl;
+    int ins_next = 0;
+    while (alive + ins + ins_next < rw.kc && ra.tl[alive + ins + ins_next] == j + 1) ++ins_next;
+    const int act = rw.T + (alive + ins) * per_step;           // rows alive in this layer
+    if (ins > 0) {   // Eq. 3: this layer's maps as one [ins d][d] GEMM on the source rows (the anchor of each sequence, or every
+                     // tree row when each node carries a chain), on the raw residual or (pre-norm) on its normalised rows
+      FIRP_TIMED(KC_PSEUDO_PROJ);
+      LinArgs l{};
+      l.X = c->xp; l.rows_active = act; l.pseudo0 = alive;     // map i of this GEMM is prediction step alive + i
+      if (c->pred_prenorm) l.ss = c->ss;
+      l.pred_b = c->w.pred_b ? (const bf16 *)c->w.pred_b + (size_t)alive * d : nullptr;
+      residual_out(l, c->g_attn[j], x_planes);
+      FIRP_CUDA(c, launch(EPI_PSEUDO, (const bf16 *)c->w.pred_w + (size_t)alive * d * d, ins * d, d, 2, rw.n_seq * per_step, l));
       alive += ins;
     }
     bf16 *kplane = c->kv + (size_t)j * c->kv_layer();
     {
-      GemmArgs g = gemm_base(c->x, Rp * d, c->wqkv[j], (H + 2 * Hkv) * dh, d, act);
-      g.H = H; g.Hkv = Hkv; g.dh = dh;
-      g.l2_ahead = ahead[0];
-      set_next(g, 0, EPI_RESIDUAL, c->wo[j], d, nq);
-      g.planes = c->planes[0];
-      g.rope = c->meta.rope; g.seq_ids = c->seq_ids; g.ctx_len = c->ctx_len; g.pos = c->meta.pos;
-      g.q = c->q; g.q_lo_off = Rp * nq; g.kcache = kplane; g.seq_stride = c->kv_seq(); g.kv_stride = c->kv_plane(); g.max_ctx = cfg.max_ctx; g.pages = c->pages();
-      Partials p = pending;
-      { FIRP_TIMED(KC_GEMM_QKV);
-        FIRP_CUDA(c, launch_gemm_tc(EPI_QKV_ROPE, g, pdl, st, &p.sk)); ++nl; }
-      FIRP_TIMED(KC_QKV_FINISH);
-      FIRP_CUDA(c, launch_gemm_finish(EPI_QKV_ROPE, p, g, pdl, st)); ++nl;
+      FIRP_TIMED(KC_GEMM_QKV);
+      LinArgs l{};
+      l.X = c->x; l.ss = c->ss; l.rows_active = act;
+      l.H = H; l.Hkv = Hkv; l.rope = c->meta.rope; l.seq_ids = c->seq_ids; l.pos = c->meta.pos;
+      l.q = c->q; l.q_plane = Rp * nq; l.kcache = kplane; l.kv_stride = c->kv_plane(); l.max_ctx = cfg.max_ctx; l.pages = c->pages();
+      FIRP_CUDA(c, launch(EPI_QKV_ROPE, c->wqkv[j], (H + 2 * Hkv) * dh, d, c->planes[G_QKV], rw.R, l));
     }
     {
       AttnArgs a{};
@@ -335,79 +309,52 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       const int G = H / Hkv, qblocks = (act * G + 63) / 64;
       a.splits = attention_splits(rw.n_seq * Hkv * qblocks, tiles);
       a.o = c->o; a.o_lo_off = Rp * nq; a.err = c->dev_status; a.wait_ns = c->wait_ns;
-      // Early (programmatic) launch of the mma.sync attention pays only when the rotary finisher before it has well
-      // over one CTA per SM (5/4).  Measured at the 7B shape, ms per step with / without it: 35 rows 3.61 / 3.76 at
-      // 512 cached tokens and 5.25 / 5.44 at 8192; 67 and 131 rows likewise 0.1 ms better with it; but 27 rows (162
-      // CTAs on 148 SMs) 3.70 / 3.66 and 6.30 / 5.33, 19 rows 3.68 / 3.60 and 6.36 / 5.26, 1 row 3.52 / 3.43 and
-      // 6.27 / 5.11.  The tensor-core kernel (one CTA per SM, all of them resident and set up before the finisher
-      // ends) gains from it at every size: 1 row 3.27 / 3.14 at 512, 27 rows 3.60 / 3.49, 35 rows 3.69 / 3.60.
-      const int half_dh = dh / 2, qkv_st = (H + 2 * Hkv + 128 / half_dh - 1) / (128 / half_dh);
-      const bool attn_early = pdl && (qkv_st * rw.R * 32 + 255) / 256 >= c->sm_count * 5 / 4;
-      bool tc = false;
-      if (dh == 128 && c->attn_tc != 0) {
+      // Head dimension 128 runs on the tensor-core kernel unless told otherwise.  Measured at the 7B shape, us per step
+      // mma.sync / tcgen05: 1 row at 128 cached tokens 2850 / 2724; 35 rows at 512 3441 / 3242, at 8192 6208 / 4185; 131
+      // rows at 2047 6890 / 6810; 6 sequences x 18 rows at 128-1024 6170 / 5130.
+      const bool tc = dh == 128 && c->attn_tc != 0;
+      if (tc) {
         int qb_tc, qper_tc;
         attention_tc_blocks(act * G, &qb_tc, &qper_tc);
-        const int tiles_tc = (ra.n_hi_max + act + kAttnTcTile - 1) / kAttnTcTile;
-        // Left to itself the tensor-core kernel takes every step the other kernel would not be launched early for
-        // and every step of at most 16 query columns; otherwise those whose longest context spans at least three of
-        // its 128-position tiles (four when the query columns need more than one block, eight when several
-        // sequences are stepped together): its fixed cost is higher, its tile loop faster.  Measured at the 7B
-        // shape, ms per step mma.sync / tcgen05, one sequence: 1 column 3.23 / 3.06 at 64 cached tokens, 3.37 /
-        // 3.28 at 512, 5.04 / 4.06 at 8192; 35 columns 3.57 / 3.61 at 64, 3.64 / 3.65 at 128, 3.72 / 3.65 at 512,
-        // 5.23 / 4.48 at 8192; 131 columns (three blocks) 5.96 / 5.91 at 64, 6.09 / 6.07 at 256, 10.35 / 9.68 at
-        // 8192; 4 sequences x 35 columns 5.77 / 5.88 at 256, 6.78 / 6.36 at 1024, 9.13 / 7.75 at 4096; 16 sequences
-        // x 9 columns 6.77 / 6.56 at 256, 19.41 / 12.13 at 4096.
-        const int min_tiles = qper_tc <= 16 ? 1 : (rw.n_seq > 1 ? 8 : (qb_tc == 1 ? 3 : 4));
-        tc = c->attn_tc > 0 || !attn_early || tiles_tc >= min_tiles;
-        if (tc) a.splits = attention_tc_splits(rw.n_seq * Hkv * qb_tc, tiles_tc, c->sm_count);
+        a.splits = attention_tc_splits(rw.n_seq * Hkv * qb_tc, (ra.n_hi_max + act + kAttnTcTile - 1) / kAttnTcTile, c->sm_count);
       }
       FIRP_TIMED(KC_ATTENTION);
-      FIRP_CUDA(c, tc ? launch_attention_tc(a, pdl, st) : launch_attention(a, attn_early, st)); ++nl;
+      FIRP_CUDA(c, tc ? launch_attention_tc(a, pdl, st) : launch_attention(a, pdl, st)); ++nl;
     }
     {
-      GemmArgs g = gemm_base(c->o, Rp * nq, c->wo[j], d, nq, act);
-      g.planes = c->planes[1];
-      g.l2_ahead = ahead[1];
-      set_next(g, 1, EPI_SWIGLU, c->wgu[j], 2 * F, d);
       FIRP_TIMED(KC_GEMM_O);
-      FIRP_CUDA(c, launch_gemm_tc(EPI_RESIDUAL, g, pdl, st, &pending.sk)); ++nl;
-    }
-    { FIRP_TIMED(KC_RMSNORM);
-      FIRP_CUDA(c, launch_rmsnorm(rw, 0, act, c->h, pending, (const bf16 *)c->g_mlp[j], d, c->x, Rp * d, 2, c->ss, pdl, st)); ++nl; }
-    pending.sk.U = 0;
-    {
-      GemmArgs g = gemm_base(c->x, Rp * d, c->wgu[j], 2 * F, d, act);
-      g.planes = c->planes[2];
-      g.y = c->y; g.y_lo_off = Rp * F; g.F = F; g.l2_ahead = ahead[2];
-      set_next(g, 2, EPI_RESIDUAL, c->wd[j], d, F);
-      Partials p = pending;
-      { FIRP_TIMED(KC_GEMM_GATE_UP);
-        FIRP_CUDA(c, launch_gemm_tc(EPI_SWIGLU, g, pdl, st, &p.sk)); ++nl; }
-      FIRP_TIMED(KC_SWIGLU_FINISH);
-      FIRP_CUDA(c, launch_gemm_finish(EPI_SWIGLU, p, g, pdl, st)); ++nl;
+      LinArgs l{};
+      l.X = c->o; l.rows_active = act;
+      residual_out(l, c->g_mlp[j], 2);
+      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wo[j], d, nq, c->planes[G_O], rw.R, l));
     }
     {
-      GemmArgs g = gemm_base(c->y, Rp * F, c->wd[j], d, F, act);
-      g.planes = c->planes[3];
-      g.l2_ahead = ahead[3];
-      if (j + 1 < cfg.n_layers) set_next(g, 3, EPI_QKV_ROPE, c->wqkv[j + 1], (H + 2 * Hkv) * dh, d);
-      else if (ra.want_head) set_next(g, 3, EPI_LOGITS, c->w.lm_head, cfg.vocab, d);
+      FIRP_TIMED(KC_GEMM_GATE_UP);
+      LinArgs l{};
+      l.X = c->x; l.ss = c->ss; l.rows_active = act; l.y = c->y; l.y_plane = Rp * F;
+      FIRP_CUDA(c, launch(EPI_SWIGLU, c->wgu[j], 2 * F, d, c->planes[G_GATE_UP], rw.R, l));
+    }
+    {
       FIRP_TIMED(KC_GEMM_DOWN);
-      FIRP_CUDA(c, launch_gemm_tc(EPI_RESIDUAL, g, pdl, st, &pending.sk)); ++nl;
+      LinArgs l{};
+      l.X = c->y; l.rows_active = act;
+      if (j + 1 < cfg.n_layers) {
+        residual_out(l, c->g_attn[j + 1], x_planes);
+        if (ins_next > 0) { l.xp = c->xp; l.xp_plane = Rp * d; l.xp_normed = c->pred_prenorm; }
+      } else if (ra.want_head) {
+        residual_out(l, c->w.g_final, 2);
+      } else {
+        l.h = c->h; l.d = d;     // nothing reads the stream after the last layer of a prompt's inner chunk
+      }
+      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wd[j], d, F, c->planes[G_DOWN], rw.R, l));
     }
   }
   if (ra.want_head) {
     if (!fused) {
-      { FIRP_TIMED(KC_RMSNORM);
-        FIRP_CUDA(c, launch_rmsnorm(rw, 0, rw.Ms, c->h, pending, (const bf16 *)c->w.g_final, d, c->x, Rp * d, 2, c->ss, pdl, st)); ++nl; }
-      GemmArgs g = gemm_base(c->x, Rp * d, c->w.lm_head, cfg.vocab, d, rw.Ms);
-      g.planes = c->planes[4];
-      g.logits = ra.logits_dst; g.l2_ahead = ahead[4];
-      Partials p = pending;
-      { FIRP_TIMED(KC_GEMM_LM_HEAD);
-        FIRP_CUDA(c, launch_gemm_tc(EPI_LOGITS, g, pdl, st, &p.sk)); ++nl; }
-      FIRP_TIMED(KC_LOGITS_FINISH);
-      FIRP_CUDA(c, launch_gemm_finish(EPI_LOGITS, p, g, pdl, st)); ++nl;
+      FIRP_TIMED(KC_GEMM_LM_HEAD);
+      LinArgs l{};
+      l.X = c->x; l.ss = c->ss; l.rows_active = rw.Ms; l.logits = ra.logits_dst;
+      FIRP_CUDA(c, launch(EPI_LOGITS, c->w.lm_head, cfg.vocab, d, c->planes[G_LM_HEAD], rw.R, l));
     }
     { FIRP_TIMED(KC_TOPB);
       launch_topb(ra.logits_dst, rw.R, cfg.vocab, cfg.top_b, c->top_ids, c->top_vals, pdl, st); ++nl; }

@@ -73,15 +73,23 @@ struct TreeMeta {
   uint32_t *mask;      // [R][kMaskWords] bit u: row v attends to new row u of its sequence
   float2 *rope;        // [R][dh/2] (cos, sin) of pos * theta^(-2c/dh)
 };
-// d_parents: [T] shared by the sequences (parents_stride 0) or [n_seq][T] (parents_stride T).
-// zero_word (may be NULL): a device word the kernel clears (the arrival counter of the fused decoder kernel)
-void launch_tree_prep(const Rows &rw, const int32_t *d_parents, int parents_stride, const int32_t *d_seq_ids, const int32_t *d_ctx_len,
-                      int dh, float theta, TreeMeta meta, int32_t *out_depth, uint32_t *out_mask, int out_mask_words,
-                      unsigned *zero_word, bool pdl, cudaStream_t st);
-
-// h[r] = embed[token] for tree rows, 0 for pseudo rows
-void launch_embed(const Rows &rw, const int32_t *d_tokens, const bf16 *embed, int d, int vocab, float *h, bool pdl,
-                  cudaStream_t st);
+struct PrepArgs {
+  Rows rw;
+  const int32_t *parents; int parents_stride;     // [T] shared by the sequences (stride 0) or [n_seq][T] (stride T)
+  const int32_t *seq_ids, *ctx_len;
+  int dh; float theta;
+  TreeMeta meta;
+  int32_t *out_depth; uint32_t *out_mask; int out_mask_words;     // caller's copies or NULL
+  unsigned *zero_word;                            // a device word to clear (the arrival counter of the persistent kernel)
+  const int32_t *tokens; const bf16 *embed; int d, vocab;
+  float *h;
+  // operand of the first layer's QKV projection: x = h * g as bf16 planes and the sums of squares (x == NULL: not wanted),
+  // and, if that layer inserts pseudo rows, the rows Eq. 3 reads (xp, as in LinArgs)
+  const bf16 *g; bf16 *x; size_t x_plane; int x_planes; float *ss_out;
+  bf16 *xp; size_t xp_plane; int xp_normed;
+};
+// The step's bookkeeping (Section 3.4 "Tree attention") and h[r] = embed[token] of the tree rows.
+void launch_prep(const PrepArgs &a, bool pdl, cudaStream_t st);
 
 // Activations that feed a GEMM or the attention are stored as two bf16 planes (hi, lo) with
 // hi + lo = the fp32 value to ~16 mantissa bits; the lo plane starts *_lo_off elements after hi.
@@ -93,22 +101,7 @@ struct Partials {
   const float *ws;   // its scratch slots
   int ws_rows;       // token rows per scratch tile
 };
-// For rows with v in [v0, v1): if `pending` has units, first h[r] += the partial tiles of a residual GEMM;
-// then x[r] = h[r] * g as `planes` bf16 planes (hi, lo or hi, mid, lo) and ss[r][w] = sum of squares of the
-// 128 columns of warp w.
-// The 1 / sqrt(mean(h^2) + eps) of RMSNorm is applied by the finisher of the GEMM that consumes x.
-constexpr int kNormMaxWarps = 64;   // d <= 8192
-cudaError_t launch_rmsnorm(const Rows &rw, int v0, int v1, float *h, const Partials &pending, const bf16 *g, int d,
-                           bf16 *x, size_t x_lo_off, int planes, float *ss, bool pdl, cudaStream_t st);
-
-// Eq. 3, h[s*Ms + T + i] = W_i h[s*Ms + anchor] + b_i, as a GEMM of the k maps stacked into one [k d][d] matrix:
-// launch_root_split writes the raw residual rows Eq. 3 reads (every sequence's anchor, or all its T tree rows when
-// every node carries a chain: row s * T + v) as (hi, lo) bf16 planes; one chain: into row s of
-// xp; the GEMM (EPI_PSEUDO) multiplies; launch_gemm_finish(EPI_PSEUDO) sums the partial tiles, adds the bias and
-// stores the k new residual rows (GemmArgs: h_rows = residual stream, pred_b = bias or NULL, R = n_seq).
-// g (may be NULL): gain vector of the pre-norm variant: the planes then hold h * g and the finisher divides by the
-// source row's RMS (GemmArgs::ss of the EPI_PSEUDO finisher)
-void launch_root_split(const Rows &rw, const float *h, const bf16 *g, int d, bf16 *xp, size_t xp_lo_off, bool pdl, cudaStream_t st);
+constexpr int kNormMaxWarps = 64;   // sums of squares per row, one for 128 columns (d <= 8192)
 
 // top-B (B <= kMaxTopB) of every row of logits by (value desc, id asc) into ids, vals [R][B]; a row with fewer than B
 // numbers is padded with (-inf, INT_MAX)
@@ -149,28 +142,57 @@ struct CommitArgs {
 void launch_commit(int n_seq, const CommitArgs &a, bool pdl, cudaStream_t st);
 void launch_advance_ctx(int n_seq, const int32_t *seq_ids, int32_t *ctx_len, int amount, bool pdl, cudaStream_t st);
 
-// ---- skinny weight-streaming GEMM ------------------------------------------
+// ---- weight-streaming GEMM ---------------------------------------------------
 enum GemmEpilogue { EPI_RESIDUAL = 0, EPI_QKV_ROPE = 1, EPI_SWIGLU = 2, EPI_LOGITS = 3, EPI_PSEUDO = 4 };
 
-struct GemmArgs {
-  const bf16 *X;    // [R][K] activations, first (hi) plane (row-major, K contiguous)
-  size_t x_lo_off;  // elements from one plane to the next ( = plane_rows * K )
-  int plane_rows;   // rows per plane of X
-  int planes;       // 2: hi + lo (~16 mantissa bits), 3: hi + mid + lo (~24 bits)
+// One GEMM of the kernel-per-operation mode: out[m][n] = sum_k X[m][k] W[n][k] and the elementwise step behind it.
+struct LinArgs {
+  const bf16 *X;    // [planes][plane_rows][K] activations as bf16 planes
+  int plane_rows, planes;
   const bf16 *W;    // [N][K] weights
-  int R;            // valid rows
+  int R, N, K;      // token rows (<= kMaxTreeRows)
+  Rows rw; int rows_active;      // rows with v < rows_active are written, the others skipped
   int *err;         // device status word (set to a non-zero code if a bounded wait gives up)
   unsigned long long wait_ns;   // bounded waits give up after this many nanoseconds (0: the default of 2 s)
-  int N, K;
+  // X holds h * g, not yet divided by the RMS: row m of the result is scaled by 1 / sqrt(sum_w ss[m][w] / K + eps)
+  // (ss == NULL: X is used as it is)
+  const float *ss; float eps;
+  // EPI_RESIDUAL, EPI_PSEUDO: rows of the residual stream h [R][d].  x (NULL: nothing reads it) gets h * g as x_planes
+  // bf16 planes, ss_out[row][c / 128] the sums of squares; xp (NULL: the next layer inserts no pseudo rows) the rows
+  // Eq. 3 reads there, raw or (xp_normed) as h * g: every sequence's anchor, or all its tree rows when every node
+  // carries a chain.
+  float *h; int d;
+  const bf16 *g; bf16 *x; size_t x_plane; int x_planes; float *ss_out;
+  bf16 *xp; size_t xp_plane; int xp_normed;
+  // EPI_PSEUDO (Eq. 3): output n = i * d + o of map pseudo0 + i (+ pred_b[n]).  One chain: token row m = sequence m, result
+  // to h row m * Ms + T + pseudo0 + i.  A chain per node: token row m = s * T + v, result to h row
+  // s * Ms + T + (pseudo0 + i) * T + v.
+  const bf16 *pred_b; int pseudo0;
+  // EPI_QKV_ROPE
+  int H, Hkv, dh;
+  const float2 *rope; const int32_t *seq_ids, *pos;   // pos[R]: row positions
+  bf16 *q; size_t q_plane;       // [R][H*dh] hi plane, lo plane
+  bf16 *kcache; size_t kv_stride; int max_ctx;        // kcache points at this layer's K plane (row 0)
+  KvPages pages;
+  // EPI_SWIGLU: y[R][F], N = 2F
+  bf16 *y; size_t y_plane; int F;
+  // EPI_LOGITS: logits[R][N]
+  float *logits;
+};
+// row of ss that belongs to token row m (Eq. 3 multiplies rows of the residual stream that lie elsewhere)
+template <int EPI> __device__ __forceinline__ int lin_src_row(const LinArgs &a, int m) {
+  if (EPI != EPI_PSEUDO) return m;
+  return a.rw.chains ? m / a.rw.T * a.rw.Ms + m % a.rw.T : m * a.rw.Ms + a.rw.anchor;
+}
+// pdl: launch with programmatic stream serialization (the kernel waits on its predecessor itself).
+cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream_t st);
+bool gemm_tc_available();         // the driver entry point for tensor-map encoding was found
+
+// What the finishers of the persistent kernel's GEMMs read (fused_step.cu).
+struct GemmArgs {
+  int R, N, K;      // token rows; output columns; contraction length
   Rows rw; int rows_active;      // rows with v < rows_active are written, the others skipped
-  // stream-K scratch: partial tiles [kGemmMaxCtas][kGemmSlots][2][plane_rows][128] fp32
-  float *ws;
-  int l2_ahead;     // 32 KB units each CTA prefetches into L2 beyond its shared-memory ring while it waits
-  // The GEMM that follows this one in the step (NULL: none).  Once a CTA has issued its own last load it
-  // prefetches the first next_units units of the same CTA's range of THAT GEMM into L2, so that HBM keeps
-  // streaming through this kernel's tail and the hand-over, and the next kernel's ring fills from L2.
-  const bf16 *next_W; int next_epi, next_N, next_K, next_F, next_heads, next_dh, next_units;
-  // finishers: X holds h * g, not yet divided by the RMS: row m of the result is scaled by
+  // X holds h * g, not yet divided by the RMS: row m of the result is scaled by
   // 1 / sqrt(sum_w ss[m][w] / K + eps) (ss == NULL: X is used as it is)
   const float *ss; float eps;
   // EPI_QKV_ROPE
@@ -188,12 +210,6 @@ struct GemmArgs {
   // h_rows[(s * Ms + T + (pseudo0 + i) * T + v) * K + o].
   float *h_rows; const bf16 *pred_b; int pseudo0;
 };
-// The GEMM leaves partial tiles in a.ws under the schedule *sk_out, to be finished by launch_gemm_finish
-// (or, for EPI_RESIDUAL, by launch_rmsnorm).  `epi` only selects how weight rows are grouped into supertiles.
-// pdl: launch with programmatic stream serialization (the kernel waits on its predecessor itself).
-cudaError_t launch_gemm_tc(GemmEpilogue epi, const GemmArgs &a, bool pdl, cudaStream_t st, StreamK *sk_out);
-cudaError_t launch_gemm_finish(GemmEpilogue epi, const Partials &p, const GemmArgs &a, bool pdl, cudaStream_t st);
-bool gemm_tc_available();         // the driver entry point for tensor-map encoding was found
 
 // ---- tree-masked split-KV attention ---------------------------------------
 constexpr int kAttnMaxSplits = 8;   // kv splits = CTAs per cluster (portable cluster size limit)

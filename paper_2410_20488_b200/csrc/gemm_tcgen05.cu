@@ -1,165 +1,178 @@
-// Skinny weight-streaming GEMM on the 5th-generation tensor cores (tcgen05 + TMEM), operands
-// staged by TMA.  out[m][n] = sum_k X[m][k] * W[n][k], M = T + k token rows, W read once.
+// Weight-streaming GEMM of the step on the 5th-generation tensor cores (tcgen05 + TMEM), operands staged by TMA, with
+// the elementwise step that follows the contraction in its epilogue.
+//   out[m][n] = sum_k X[m][k] * W[n][k], m = T + k token rows (at most 144), W read once.
 //
-// Roles are swapped: weight rows are the MMA M dimension (one TMEM lane each), token rows the
-// MMA N dimension (one TMEM column each).  A "supertile" is 2 x 128 weight rows that share one
-// activation tile per k block, chosen so that both operands of a fused epilogue meet in one
-// thread: lane i of the first 128 rows and lane i of the second are a rotary pair (c, c + dh/2),
-// a gate row and its up row, or simply rows n and n + 128.
+// Roles are swapped: weight rows are the MMA M dimension (one TMEM lane each), token rows the MMA N dimension (one
+// TMEM column each).  A tile is 128 weight rows that one thread block finishes by itself: 128 neighbouring rows, or 64
+// gate rows and the 64 up rows that go with them.  A job is up to TM tiles; the k blocks of a job are cut over the
+// `split` CTAs of a cluster, and grid = jobs x split, one wave wherever the matrix allows it.
 //
-// Persistent stream-K schedule: the (supertile, k block) units of the whole matrix, 32 KB of
-// weights each, are cut into one contiguous range per SM, so every SM streams the same number of
-// bytes whatever the matrix shape.  A range crosses supertile boundaries; each piece ("segment")
-// accumulates in TMEM and its fp32 partial tile is stored to the CTA's scratch slot.  The kernel
-// that consumes the GEMM (RMSNorm for the residual GEMMs, the rotary / SwiGLU / logits finishers
-// otherwise) sums the slots of a supertile in CTA order, so every sum has a fixed order and results
-// are identical from run to run; no CTA ever waits for another.  The finishers are small-footprint
-// kernels that stay resident beside the next GEMM's CTAs: under programmatic dependent launch the
-// next weight stream starts while they run.
+// Why whole tiles and not one equal share of the matrix per SM: HBM does not need every SM.  A TMA ring of 6 x 32 KB per
+// CTA streams 6.7 TB/s from 86 CTAs, 6.8 from 108, 6.9 from 128 (measured), so a schedule that leaves some SMs without
+// weights costs 1-3 % of the stream, while shares that end in mid-tile cost a pass over fp32 partial tiles in global
+// memory, a kernel of its own to sum them and a hand-over: 7 us after the QKV, gate/up and down projections and 14 us after
+// the O projection at 35 rows of the 7B shape, 37 of 102 us per layer.  Step at the 7B shape, 35 rows, 512 cached tokens:
+// 3534 -> 3121 us; one row 3062 -> 2696; 13B shape, 67 rows 8958 -> 6734; 34B shape, 140 rows 6631 -> 6230.
 //
-// Per CTA (one per SM):
-//   warp 0   : weight producer (one thread, TMA, 128-byte swizzle, deep ring).  Weights never
-//              depend on the previous kernel, so under programmatic dependent launch this stream
-//              starts while the predecessor drains.
-//   warp 6   : activation producer: the (hi, lo) bf16 planes of the matching k block (L2
-//              resident, own shorter ring), after waiting for the previous kernel.
-//   warp 1   : MMA issuer: tcgen05.mma kind::f16, M = 128, K = 16; the bf16 planes of the
-//              activations (hi, lo, or hi, mid, lo) sit one after the other in shared memory and are
-//              multiplied as ONE operand of N = planes x NPAD token columns (the sums over each
-//              plane land in neighbouring TMEM columns and are added in the epilogue);
-//              tcgen05.commit releases ring slots.
-//   warps 2-5: epilogue: tcgen05.ld (lane = weight row, column = token), hi + lo, store of the
-//              partial tile; overlapped with the next segment's main loop through a second
-//              accumulator buffer.
-// Every mbarrier wait is bounded (~2 s): on expiry the status word is set and the kernel runs to
-// its end; TMEM is always released.
+// Bound now, per layer of 98 us: the weight stream (QKV 15.1, gate/up 27.8, down 13.1 us at 6.7-6.9 TB/s; the O projection
+// 5.5), the epilogues (4 + 2.5 + 2 + 2), five hand-overs of 2 us and the attention's 12.
+//
+// Per CTA (one per SM at the large shapes):
+//   warp 0     : weight producer (one thread, TMA, 128-byte swizzle, deep ring).  Weights never depend on the previous
+//                kernel, so under programmatic dependent launch this stream starts while the predecessor drains.  Its
+//                own loads issued, it brings the head of the next GEMM's weights into L2.
+//   warp 2     : activation producer: the bf16 planes of the k block, after waiting for the previous kernel.
+//   warp 1     : MMA issuer: tcgen05.mma kind::f16, M = 128, K = 16.  The planes of the activations (hi, lo) either sit
+//                side by side as ONE operand of N = planes x npad columns (added in the epilogue) or are accumulated
+//                one after the other into npad columns.  The whole warp runs the loop and an elected lane issues, which
+//                keeps the descriptors in uniform registers (M = 128, N = 80: 59 cycles per MMA; one lane alone: 86).
+//   warps 4-11 : epilogue.  TMEM -> shared memory of the CTA of the cluster that finishes the token row (the ring's
+//                memory, no longer needed), cluster barrier, sum over the k slices in rank order, then the fused step:
+//                residual + RMSNorm operand, rotary + cache, SwiGLU, logits, or Eq. 3.
+// Every mbarrier wait is bounded (~2 s): on expiry the status word is set and the kernel runs to its end; TMEM is
+// always released.
+#include <cooperative_groups.h>
 #include <cuda.h>
 
-#include <cstdlib>
+#include <algorithm>
 #include <map>
+#include <mutex>
 #include <tuple>
 
+#include "finish_device.cuh"
 #include "firp_kernels.cuh"
 #include "launch_util.cuh"
 #include "tc_device.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace firp {
 
 namespace {
 
 constexpr int BM = 128;            // weight rows per MMA tile
-constexpr int TM = 2;              // MMA tiles per supertile
 constexpr int BK = kGemmBK;        // 64 bf16 = 128 bytes = one swizzle row
-constexpr int kThreads = 224;      // 7 warps
+constexpr int kThreads = 384;      // 12 warps
+constexpr int kEpiWarps = 8;
 constexpr int W_TILE = BM * 128;   // bytes of one 128-row weight tile of a k block
-constexpr int W_STAGE = TM * W_TILE;
+constexpr int kSmemMax = 227 * 1024;
+constexpr int kTailBytes = 1536;   // row scales, row indices, slots and lengths, barriers, TMEM address (behind the rings)
+constexpr int kMaxRows = kMaxTreeRows;
+constexpr int kMaxStages = 12;       // of either ring
 
-constexpr int pow2_cols(int c) { return c <= 32 ? 32 : c <= 64 ? 64 : c <= 128 ? 128 : c <= 256 ? 256 : 512; }
-
-// NPAD = token rows padded to a multiple of 8; P = bf16 planes of the activations (2: hi + lo,
-// 3: hi + mid + lo).  The planes of a stage sit one after the other in shared memory; when P * NPAD is
-// a legal MMA N (a multiple of 16, <= 256) they are multiplied as one operand, otherwise plane by plane.
-template <int NPAD, int P> struct TcCfg {
-  static constexpr int X_PLANE = NPAD * 128;                   // bytes of one activation plane per stage
-  static constexpr int X_STAGE = P * X_PLANE;
-  // two planes are merged only while two accumulator buffers still fit the 512 TMEM columns (measured: the
-  // second buffer -- epilogue of one segment under the main loop of the next -- is worth more than one MMA
-  // instead of two); three planes are always merged when legal (measured the other way round)
-  static constexpr bool MERGE = (P * NPAD <= 256) && ((P * NPAD) % 16 == 0) && (2 * TM * P * NPAD <= 512 || NPAD % 16 != 0 || P > 2);
-  static constexpr int ACC_COLS = MERGE ? P * NPAD : NPAD;     // accumulator columns per weight tile
-  static constexpr int NBUF = (2 * TM * ACC_COLS <= 512) ? 2 : 1;   // accumulator buffers
-  static constexpr int TMEM_COLS = pow2_cols(NBUF * TM * ACC_COLS);
-  // ring depths: as many 32 KB weight stages as fit beside two to four activation stages
-  // (an activation stage of the 144-row variant is 36 KB and comes from L2 in ~2 us: with two stages that
-  // latency, not the weight stream or the MMAs, set the pace of a unit; three stages beside three weight stages)
-  static constexpr int SX = X_STAGE <= 8 * 1024 ? 4 : (X_STAGE <= 40 * 1024 ? 3 : 2);
-  static constexpr int SW = (227 * 1024 - 1280 - SX * X_STAGE) / W_STAGE > 6 ? 6 : (227 * 1024 - 1280 - SX * X_STAGE) / W_STAGE;
-  static constexpr int RING_BYTES = SW * W_STAGE + SX * X_STAGE;
-  static constexpr int SMEM = RING_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
-  static_assert(!MERGE || NPAD % 8 == 0, "planes must start on a swizzle atom");
-  static_assert(MERGE || NPAD % 16 == 0, "MMA N must be a multiple of 16");
-  static_assert(SW >= 3 && SMEM <= 227 * 1024, "shared memory budget");
-  static_assert((2 * SW + 2 * SX + 2 * NBUF) * 8 + 8 <= 256, "barrier area");
-};
-
-// How the 2 x 128 rows of supertile `st` map to weight rows.
-//   ROWS_LINEAR   rows st*256 .. +255 (two boxes of 128 rows)
-//   ROWS_GATE_UP  gate rows st*128 .. +127, then the matching up rows F + st*128 ..
-//   ROWS_ROTARY   first halves (c < dh/2) of 128/(dh/2) heads, then their second halves, fetched
-//                 through a 4-D view [head][half][c][k] of the weight so that each is one box
+// How the rows of the weight are dealt to tiles of 128, each one TMA box per k block.
+//   ROWS_LINEAR   128 neighbouring rows
+//   ROWS_GATE_UP  even tiles: 128 gate rows, odd tiles: the up rows that go with them (a job is one such pair)
+//   ROWS_ROTARY   128 / dh heads; the rows of a head in groups of 32: 16 columns of its first half, then their partners in
+//                 the second half, so that a rotary pair is 16 lanes apart in one warp
 enum RowMode { ROWS_LINEAR = 0, ROWS_GATE_UP = 1, ROWS_ROTARY = 2 };
-struct Sched {
-  StreamK sk;      // units, k blocks per supertile, CTAs
-  int mode;        // RowMode
-  int F;           // ROWS_GATE_UP: rows of the gate matrix
-  int half;        // ROWS_ROTARY: dh / 2
-  int n_st;        // supertiles
-  int pdl;         // launched with programmatic stream serialization
-  int ws_rows;     // token rows per scratch tile
-  int l2_ahead;    // units each CTA prefetches into L2 beyond its shared-memory ring
+// Which tiles and k blocks a CTA multiplies.
+struct TileSched {
+  int mode, heads;   // heads: of a tile (ROWS_ROTARY)
+  int n_tiles, KB;   // tiles; 64-wide k blocks
+  int jobs, split;   // job j = tiles [n_tiles j / jobs, n_tiles (j + 1) / jobs), its k blocks cut over `split` CTAs
+};
+// A CTA starts its k range at a place of its own and wraps around: CTAs that march through k together would ask the same
+// L2 slices for the same activation rows, and HBM for weight rows whose addresses differ only above bit 12.
+struct CtaWork { int t0, nt, kb0, kb1, off; };
+__device__ __forceinline__ CtaWork cta_work(const TileSched &s, int cta) {
+  const int j = cta / s.split, r = cta - j * s.split;
+  CtaWork w;
+  w.t0 = s.n_tiles * j / s.jobs;
+  w.nt = s.n_tiles * (j + 1) / s.jobs - w.t0;
+  w.kb0 = s.KB * r / s.split;
+  w.kb1 = s.KB * (r + 1) / s.split;
+  w.off = (cta * 10) % (w.kb1 - w.kb0) & ~1;      // even: pairs of k blocks share 256-byte lines
+  return w;
+}
+// k block of unit u
+__device__ __forceinline__ int unit_kb(const CtaWork &w, int u) { const int k = w.kb0 + w.off + u; return k < w.kb1 ? k : k - (w.kb1 - w.kb0); }
+
+// Shared memory and operand shape of a launch.
+struct TileCfg {
+  int planes, npad;     // activation planes; token rows padded to the MMA's N
+  int acc;              // accumulator columns per tile
+  int issuers, by_tile; // MMA issuing warps: they take the units in turn, each with accumulators of its own, or the tiles
+  int sets, acc_set;    // accumulator sets (summed in the epilogue), columns per set
+  int sw, sx;           // ring depths: weight tiles, activation stages
+  int planes_side;      // planes that sit side by side in the accumulator's columns
+  int tpo, inv_tpo;     // token rows finished per CTA of a cluster; ceil(65536 / tpo)
+  int tp;               // tiles per epilogue pass (what the ring's memory holds)
+  int tail;             // bytes from the rings' start to what lies behind them
+  int red_off;          // where the sums over the k slices go: behind the rings, or 0: over them
+  int rope_off, rope_bytes;      // the step's rotary table, if it is brought into shared memory
+  int pdl;
+  uint32_t idesc, tmem_cols;
 };
 
-// L2 prefetch of the two weight tiles of unit (supertile st, k block kb) under schedule sc
-__device__ __forceinline__ void prefetch_unit(const CUtensorMap *tm, const Sched &sc, int st, int kb, uint64_t pol) {
-  if (sc.mode == ROWS_ROTARY) {
-    const int hp = BM / sc.half;
-    tma_prefetch_4d(tm, kb * BK, 0, 0, st * hp, pol);
-    tma_prefetch_4d(tm, kb * BK, 0, 1, st * hp, pol);
-  } else if (sc.mode == ROWS_GATE_UP) {
-    tma_prefetch_2d(tm, kb * BK, st * BM, pol);
-    tma_prefetch_2d(tm, kb * BK, sc.F + st * BM, pol);
-  } else {
-    tma_prefetch_2d(tm, kb * BK, st * (TM * BM), pol);
-    tma_prefetch_2d(tm, kb * BK, st * (TM * BM) + BM, pol);
-  }
+// one k block of one tile: 16 KB
+__device__ __forceinline__ void load_tile(uint32_t dst, const CUtensorMap *tm, const TileSched &s, int tile, int kb, uint32_t bar, uint64_t pol) {
+  if (s.mode == ROWS_ROTARY) tma_load_5d(dst, tm, kb * BK, tile * s.heads, bar, pol);
+  else if (s.mode == ROWS_GATE_UP) tma_load_3d(dst, tm, kb * BK, (tile >> 1) * BM, tile & 1, bar, pol);
+  else tma_load_2d(dst, tm, kb * BK, tile * BM, bar, pol);
 }
 
-template <int NPAD, int P>
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+// every thread of the cluster has got as far as cluster_arrive
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ float4 mul4(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
+// MERGED: the activation planes sit side by side in one operand (or there is only one); else one after the other.
+// The epilogue's code runs once per launch from a cold instruction cache, in the shadow of nothing: one kernel per epilogue
+// and rolled loops keep it short (all five in one kernel, four items unrolled: 5-7 us instead of 1-2).
+template <int TM, bool MERGED, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-               const __grid_constant__ CUtensorMap tmNext, GemmArgs a, Sched sc, Sched nx) {
-  using Cfg = TcCfg<NPAD, P>;
-  constexpr int SW = Cfg::SW, SX = Cfg::SX, X_STAGE = Cfg::X_STAGE, X_PLANE = Cfg::X_PLANE, NBUF = Cfg::NBUF;
-  constexpr int ACC = Cfg::ACC_COLS;
-  constexpr bool MERGE = Cfg::MERGE;
+gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ LinArgs a,
+            const __grid_constant__ TileSched sc, const __grid_constant__ TileCfg cf) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;      // swizzled tiles need 1024-byte alignment
   uint8_t *data = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t w_ring = base, x_ring = base + SW * W_STAGE;
-  const uint32_t bars = base + Cfg::RING_BYTES;                     // 8-byte barriers
-  const uint32_t full_w = bars, empty_w = full_w + 8 * SW, full_x = empty_w + 8 * SW, empty_x = full_x + 8 * SX,
-                 acc_full = empty_x + 8 * SX, acc_empty = acc_full + 8 * NBUF, tmem_slot = acc_empty + 8 * NBUF;
-  volatile uint32_t *tmem_slot_ptr =
-      reinterpret_cast<volatile uint32_t *>(data + Cfg::RING_BYTES + 16 * SW + 16 * SX + 16 * NBUF);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cta = blockIdx.x;
-  const StreamK sk = sc.sk;
-  const int KB = sk.KB;
-  const int u0 = sk_begin(sk, cta), u1 = sk_begin(sk, cta + 1);
-  const int n_units = u1 - u0;
+  const int sx_n = cf.sx;
+  const uint32_t x_plane = (uint32_t)cf.npad * 128u, x_stage = x_plane * cf.planes;
+  const uint32_t w_ring = base, x_ring = base + cf.sw * W_TILE;
+  float *s_rs = reinterpret_cast<float *>(data + cf.tail);          // 1 / RMS of every token row
+  int *s_slot = reinterpret_cast<int *>(s_rs + kMaxRows), *s_pos = s_slot + kMaxSeq;      // of every sequence
+  uint16_t *s_row = reinterpret_cast<uint16_t *>(s_pos + kMaxSeq);                        // sequence << 8 | row of every token row
+  const uint32_t bars = base + cf.tail + kMaxRows * 6 + 2 * kMaxSeq * 4;
+  const uint32_t full_w = bars, empty_w = full_w + 8 * kMaxStages, full_x = empty_w + 8 * kMaxStages, empty_x = full_x + 8 * kMaxStages,
+                 acc_full = empty_x + 8 * kMaxStages, rope_full = acc_full + 8, tmem_slot = rope_full + 8;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const CtaWork wk = cta_work(sc, blockIdx.x);
+  const int n_units = wk.kb1 - wk.kb0;
+  // The weight ring holds single tiles (16 KB slots: a slot is free again after four MMAs).  Its depth is a multiple of the
+  // job's tiles, so that a slot always holds the same tile and is read by the same issuer: one that skipped a phase of a
+  // slot's barrier would take the phase before it for its own (parity tells neighbouring phases apart, no more).
+  const int sw_n = cf.by_tile ? cf.sw / wk.nt * wk.nt : cf.sw;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < SW; ++i) { mbar_init(full_w + 8 * i, 1); mbar_init(empty_w + 8 * i, 1); }
-    for (int i = 0; i < SX; ++i) { mbar_init(full_x + 8 * i, 1); mbar_init(empty_x + 8 * i, 1); }
-    for (int i = 0; i < NBUF; ++i) { mbar_init(acc_full + 8 * i, 1); mbar_init(acc_empty + 8 * i, 4); }
+    const int readers = cf.by_tile ? cf.issuers : 1;
+    for (int i = 0; i < sw_n; ++i) { mbar_init(full_w + 8 * i, 1); mbar_init(empty_w + 8 * i, 1); }
+    for (int i = 0; i < sx_n; ++i) { mbar_init(full_x + 8 * i, 1); mbar_init(empty_x + 8 * i, readers); }
+    mbar_init(acc_full, cf.issuers);
+    mbar_init(rope_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();                 // barriers are initialised
-  if (sc.pdl) griddep_launch();    // the next kernel may start its own weight stream as SMs free up
-  // The two producers start at once; the warps that touch TMEM (MMA issuer and epilogue) meet on their own
-  // barrier once warp 1 has allocated (and later frees) the accumulator columns.
-  uint32_t tmem_base = 0;
-  if (warp >= 1 && warp <= 5) {
-    if (warp == 1) {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(Cfg::TMEM_COLS) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    asm volatile("bar.sync 2, 160;" ::: "memory");
-    tc_fence_after();
-    tmem_base = *tmem_slot_ptr;
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(cf.tmem_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(data + (tmem_slot - base));
+  // Dependents may start as SMs free up.  Not before TMEM is allocated: a dependent on the same SM then only ever waits
+  // for columns of a kernel that does not wait for it.
+  if (cf.pdl) griddep_launch();
+  if (sc.split > 1 && cf.red_off) cluster_arrive();
 
   bool dead = false;
   const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kDefaultWaitNs;
@@ -167,148 +180,406 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     if (lane == 0) {             // ---- weight producer: does not wait for the previous kernel
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
-      // While the ring is full (typically: the activations are not there yet because the previous kernel is
-      // still running) the stream goes on into L2: units up to l2_ahead beyond the ring are prefetched, so
-      // HBM stays busy during the small kernels between two GEMMs and the ring later refills from L2.
-      int pf = SW;
+      int sl = 0;
+      uint32_t par = 1;
       for (int it = 0; it < n_units; ++it) {
-        for (const int upto = min(n_units, it + SW + sc.l2_ahead); pf < upto; ++pf) {
-          const int up = u0 + pf;
-          prefetch_unit(&tmW, sc, up / KB, up % KB, pol);
+        const int kb = unit_kb(wk, it);
+        for (int t = 0; t < wk.nt; ++t) {
+          mbar_wait(empty_w + 8 * sl, par, a.err, dead, wait_ns);
+          mbar_expect_tx(full_w + 8 * sl, W_TILE);
+          load_tile(w_ring + sl * W_TILE, &tmW, sc, wk.t0 + t, kb, full_w + 8 * sl, pol);
+          if (++sl == sw_n) { sl = 0; par ^= 1; }
         }
-        const int u = u0 + it;
-        const int st = u / KB, kb = u - st * KB;
-        const int sl = it % SW;
-        mbar_wait(empty_w + 8 * sl, ((it / SW) & 1) ^ 1, a.err, dead, wait_ns);
-        mbar_expect_tx(full_w + 8 * sl, W_STAGE);
-        const uint32_t dst = w_ring + sl * W_STAGE, bar = full_w + 8 * sl;
-        if (sc.mode == ROWS_ROTARY) {
-          const int hp = BM / sc.half;               // heads per supertile
-          tma_load_4d(dst, &tmW, kb * BK, 0, 0, st * hp, bar, pol);
-          tma_load_4d(dst + W_TILE, &tmW, kb * BK, 0, 1, st * hp, bar, pol);
-        } else if (sc.mode == ROWS_GATE_UP) {
-          tma_load_2d(dst, &tmW, kb * BK, st * BM, bar, pol);
-          tma_load_2d(dst + W_TILE, &tmW, kb * BK, sc.F + st * BM, bar, pol);
-        } else {
-          tma_load_2d(dst, &tmW, kb * BK, st * (TM * BM), bar, pol);
-          tma_load_2d(dst + W_TILE, &tmW, kb * BK, st * (TM * BM) + BM, bar, pol);
-        }
-      }
-      // all own loads are out: bring the head of the next GEMM's range of this CTA into L2
-      if (nx.l2_ahead > 0 && cta < nx.sk.G) {
-        const int v0 = sk_begin(nx.sk, cta), v1 = min(sk_begin(nx.sk, cta + 1), v0 + nx.l2_ahead);
-        for (int v = v0; v < v1; ++v) prefetch_unit(&tmNext, nx, v / nx.sk.KB, v % nx.sk.KB, pol);
       }
     }
-  } else if (warp == 6) {
+  } else if (warp == 2) {
     if (lane == 0) {             // ---- activation producer
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-      if (sc.pdl) griddep_wait();
-      const int xrows = min((a.R + 7) & ~7, NPAD);
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
+      if (cf.pdl) griddep_wait();
+      if (EPI == EPI_QKV_ROPE && cf.rope_bytes) {
+        const int r0 = (int)(blockIdx.x % sc.split) * cf.tpo, bytes = max(0, min(cf.tpo, a.R - r0)) * (a.dh >> 1) * 8;   // of the rows finished here
+        mbar_expect_tx(rope_full, bytes);
+        if (bytes) bulk_load(base + cf.rope_off, a.rope + (size_t)r0 * (a.dh >> 1), bytes, rope_full);
+      }
+      int sl = 0;
+      uint32_t par = 1;
       for (int it = 0; it < n_units; ++it) {
-        const int kb = (int)((u0 + it) % KB);
-        const int sl = it % SX;
-        mbar_wait(empty_x + 8 * sl, ((it / SX) & 1) ^ 1, a.err, dead, wait_ns);
-        mbar_expect_tx(full_x + 8 * sl, P * xrows * 128);
-        const uint32_t dst = x_ring + sl * X_STAGE;
-#pragma unroll
-        for (int pl = 0; pl < P; ++pl)
-          tma_load_2d(dst + pl * X_PLANE, &tmX, kb * BK, pl * a.plane_rows, full_x + 8 * sl, pol);
+        mbar_wait(empty_x + 8 * sl, par, a.err, dead, wait_ns);
+        mbar_expect_tx(full_x + 8 * sl, x_stage);
+        tma_load_3d(x_ring + sl * x_stage, &tmX, unit_kb(wk, it) * BK, 0, 0, full_x + 8 * sl, pol);   // all planes
+        if (++sl == sx_n) { sl = 0; par ^= 1; }
       }
     }
-  } else if (warp == 1) {
-    if (lane == 0) {             // ---- MMA issuer
-      constexpr uint32_t idesc = instr_desc_m128(MERGE ? P * NPAD : NPAD);
-      int it = 0, seg = 0;
-      int u = u0;
-      while (u < u1) {
-        const int st = u / KB, kb0 = u - st * KB;
-        const int kb1 = min(KB, kb0 + (u1 - u));
-        const int buf = seg % NBUF;
-        mbar_wait(acc_empty + 8 * buf, ((seg / NBUF) & 1) ^ 1, a.err, dead, wait_ns);   // epilogue has drained this buffer
-        tc_fence_after();
-        const uint32_t acc = tmem_base + (uint32_t)(buf * TM * ACC);
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int sw = it % SW, sx = it % SX;
-          mbar_wait(full_w + 8 * sw, (it / SW) & 1, a.err, dead, wait_ns);
-          mbar_wait(full_x + 8 * sx, (it / SX) & 1, a.err, dead, wait_ns);
-          tc_fence_after();
-          const uint32_t wst = w_ring + sw * W_STAGE, xst = x_ring + sx * X_STAGE;
-          const uint64_t dx = smem_desc(xst);
+  } else if (warp == 1 || warp == 3) {        // ---- MMA issuers
+    const int iw = warp >> 1;
+    if (iw < cf.issuers) {
+      // by units: unit iw, iw + issuers, ... into accumulators of its own; by tiles: every unit, tiles iw, iw + issuers, ...
+      const int u0 = cf.by_tile ? 0 : iw, du = cf.by_tile ? 1 : cf.issuers;
+      const uint32_t tm0 = __shfl_sync(0xffffffffu, tmem, 0) + (cf.by_tile ? 0u : (uint32_t)(iw * cf.acc_set));
+      int sw = cf.by_tile ? iw : u0, sx = u0;            // slot of the unit's first tile of this issuer; X slot
+      uint32_t parw = 0, parx = 0;
+      if (sw >= sw_n) { sw -= sw_n; parw ^= 1; }
+      if (sx >= sx_n) { sx -= sx_n; parx ^= 1; }
+      for (int it = u0; it < n_units; it += du) {
+        const uint64_t dx = smem_desc(x_ring + sx * x_stage);
+        bool first = true;
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
+        for (int t = 0; t < TM; ++t) {
+          if (t < wk.nt && (!cf.by_tile || (t & 1) == iw)) {
+            const int sl = cf.by_tile ? sw + t - iw : sw;
+            mbar_wait(full_w + 8 * sl, parw, a.err, dead, wait_ns);
+            if (first) mbar_wait(full_x + 8 * sx, parx, a.err, dead, wait_ns);
+            first = false;
+            __syncwarp();                // lanes may leave a wait one by one; what follows is for a converged warp
+            tc_fence_after();
+            const uint64_t dw = smem_desc(w_ring + sl * W_TILE);
 #pragma unroll
-            for (int t = 0; t < TM; ++t) {
-              const uint64_t da = smem_desc(wst + t * W_TILE) + 2 * kk;
-              tc_mma(acc + t * ACC, da, dx + 2 * kk, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
-              if (!MERGE) {
+            for (int kk = 0; kk < BK / 16; ++kk) {
+              if (elect_one()) tc_mma(tm0 + t * cf.acc, dw + 2 * kk, dx + 2 * kk, cf.idesc, (it > u0 || kk > 0) ? 1u : 0u);
 #pragma unroll
-                for (int pl = 1; pl < P; ++pl) tc_mma(acc + t * ACC, da, dx + (pl * X_PLANE >> 4) + 2 * kk, idesc, 1u);
+              for (int pl = 1; pl < 3; ++pl)
+                if (!MERGED && pl < cf.planes && elect_one()) tc_mma(tm0 + t * cf.acc, dw + 2 * kk, dx + (uint64_t)(pl * (x_plane >> 4)) + 2 * kk, cf.idesc, 1u);
+            }
+            if (elect_one()) tc_commit(empty_w + 8 * sl);      // the slot is free once these MMAs have read it
+          }
+        }
+        if (first) mbar_wait(full_x + 8 * sx, parx, a.err, dead, wait_ns);      // an issuer without tiles only keeps count
+        __syncwarp();
+        if (elect_one()) tc_commit(empty_x + 8 * sx);
+        sw += cf.by_tile ? wk.nt : du;
+        if (sw >= sw_n) { sw -= sw_n; parw ^= 1; }
+        sx += du;
+        if (sx >= sx_n) { sx -= sx_n; parx ^= 1; }
+      }
+      if (elect_one()) tc_commit(acc_full);
+    }
+  }
+  __syncwarp();
+
+  // ---- epilogue: warps 4..11 work, the others only take part in the cluster's barriers
+  const bool epi = warp >= 4;
+  const int ew = warp - 4, quarter = warp & 3, half_w = ew >> 2;
+  const int split = sc.split;
+  const uint32_t rank = (uint32_t)(blockIdx.x % split);
+  const int own0 = (int)rank * cf.tpo, n_own = max(0, min(cf.tpo, a.R - own0));     // token rows this CTA finishes
+  const float *red = reinterpret_cast<const float *>(data + cf.red_off);         // [k slice][own row][tile of the pass][128]
+  constexpr bool kDirect = EPI == EPI_QKV_ROPE || EPI == EPI_SWIGLU || EPI == EPI_LOGITS;   // may leave from registers
+  const int half = EPI == EPI_QKV_ROPE ? a.dh >> 1 : 1;
+  const int pitch = EPI == EPI_SWIGLU ? 2 : 1;       // tiles per item
+  if (epi) {
+    if (cf.pdl) griddep_wait();
+    // one load per CTA (thousands of warps asking L2 for the same word at once take microseconds)
+    if (EPI == EPI_QKV_ROPE && warp == 4 && lane < a.rw.n_seq) {
+      s_slot[lane] = __ldcg(a.seq_ids + lane);
+      s_pos[lane] = __ldcg(a.pos + lane * a.rw.Ms);      // committed length (position of the root row)
+    }
+    // of every row this CTA finishes: its sequence and row (0xffff: none, or not to be written), and
+    // 1 / sqrt(mean(h^2) + eps) from the per-128-column sums of squares, added in a fixed order
+    const int nw = a.K >> 7, per = EPI == EPI_PSEUDO ? (a.rw.chains ? a.rw.T : 1) : a.rw.Ms;
+    const int m_end = min(kMaxRows, own0 + ((n_own + 15) & ~15));
+    for (int m0 = own0 + ew; m0 < m_end; m0 += 4 * kEpiWarps) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        v[u] = 0.f;
+        if (a.ss == nullptr) continue;
+        const float *p = a.ss + (size_t)lin_src_row<EPI>(a, min(m0 + u * kEpiWarps, a.R - 1)) * kNormMaxWarps;
+        v[u] = (lane < nw ? __ldcg(p + lane) : 0.f) + (lane + 32 < nw ? __ldcg(p + lane + 32) : 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[u] += __shfl_xor_sync(0xffffffffu, v[u], o);
+        const int m = m0 + u * kEpiWarps;
+        if (lane == 0 && m < m_end) {
+          s_rs[m] = a.ss ? rsqrtf(v[u] / (float)a.K + a.eps) : 1.f;
+          const int s = m / per, row = m - s * per;
+          s_row[m] = (uint16_t)(m < own0 + n_own && (EPI == EPI_PSEUDO || row < a.rows_active) ? s << 8 | row : 0xffff);
+        }
+      }
+    }
+  }
+  // columns [c0, c0 + 16) of tile t: the sums over the planes' columns and the issuers' accumulators (all loads in flight
+  // together)
+  const uint32_t tquarter = tmem + ((uint32_t)(quarter * 32) << 16);
+  auto load_acc = [&](int t, int c0, float *r) {
+    const uint32_t ta = tquarter + (uint32_t)(t * cf.acc + c0);
+    float l[3][16];
+    tc_ld16(ta, r);
+    if (cf.planes_side > 1) tc_ld16(ta + cf.npad, l[0]);
+    if (cf.sets > 1) {
+      tc_ld16(ta + cf.acc_set, l[1]);
+      if (cf.planes_side > 1) tc_ld16(ta + cf.acc_set + cf.npad, l[2]);
+    }
+    tc_ld_wait();
+    if (cf.planes_side > 1) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) r[j] += l[0][j];
+    }
+    if (cf.sets > 1) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) r[j] += l[1][j];
+      if (cf.planes_side > 1) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) r[j] += l[2][j];
+      }
+    }
+    if (cf.planes_side > 2) {                      // a third plane
+      tc_ld16(ta + 2 * cf.npad, l[0]);
+      if (cf.sets > 1) tc_ld16(ta + cf.acc_set + 2 * cf.npad, l[1]);
+      tc_ld_wait();
+#pragma unroll
+      for (int j = 0; j < 16; ++j) r[j] += cf.sets > 1 ? l[0][j] + l[1][j] : l[0][j];
+    }
+  };
+  auto wait_acc = [&]() {
+    // one warp polls, the others sleep at a block barrier: eight polling warps halve the rate of the producer's and the
+    // issuers' shared-memory operations
+    if (warp == 4) mbar_wait(acc_full, 0, a.err, dead, wait_ns);
+    if (EPI == EPI_QKV_ROPE && cf.rope_bytes) mbar_wait(rope_full, 0, a.err, dead, wait_ns);      // long complete
+    epi_sync();
+    tc_fence_after();
+  };
+  if (kDirect && split == 1) {
+    // ---- no other CTA contributes: a thread has one weight row of its tile in 8 token rows at a time, and what it is
+    // combined with in the same thread (gate and up) or 16 lanes away (rotary pair)
+    if (epi) {
+      const int rowi = quarter * 32 + lane;                     // row of the tile
+      const int c = EPI == EPI_QKV_ROPE ? (quarter * 16 + (lane & 15)) & (half - 1) : 0, hi_half = (lane >> 4) & 1;
+      // the rotary table of the step lies in shared memory, or, when it does not fit beside the rings, in L2
+      const float2 *rope = cf.rope_bytes ? reinterpret_cast<const float2 *>(data + cf.rope_off) : a.rope;
+      wait_acc();
+#pragma unroll 1
+      for (int t = 0; t < wk.nt; t += pitch) {
+        const int tile = wk.t0 + t;
+        const int unit = EPI == EPI_QKV_ROPE ? tile * sc.heads + (sc.heads == 2 ? quarter >> 1 : 0) : 0;    // query, key or value head
+#pragma unroll 1
+        for (int c0 = half_w * 16; c0 < a.R; c0 += 32) {
+          float r[16], r2[16], rs[16];
+          uint32_t row[8];                                      // two rows each
+          load_acc(t, c0, r);
+          if (EPI == EPI_SWIGLU) load_acc(t + 1, c0, r2);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) *reinterpret_cast<float4 *>(rs + 4 * q) = *reinterpret_cast<const float4 *>(s_rs + c0 + 4 * q);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) *reinterpret_cast<uint4 *>(row + 4 * q) = *reinterpret_cast<const uint4 *>(s_row + c0 + 8 * q);
+          auto row_of = [&](int j) { return (int)((row[j >> 1] >> (16 * (j & 1))) & 0xffffu); };       // 0xffff: not to be written
+          if (EPI == EPI_LOGITS) {
+            const int n = tile * BM + rowi;
+            float *dst = a.logits + (size_t)c0 * a.N + n;
+            if (n < a.N) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) if (row_of(j) != 0xffff) dst[(size_t)j * a.N] = r[j] * rs[j];
+            }
+          } else if (EPI == EPI_SWIGLU) {
+            const int n = (tile >> 1) * BM + rowi;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) { const float g = r[j] * rs[j]; r[j] = g / (1.f + __expf(-g)) * (r2[j] * rs[j]); }
+            bf16 *dst = a.y + (size_t)c0 * a.F + n;
+            if (n < a.F) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const bf16 h = __float2bfloat16_rn(r[j]);
+                if (row_of(j) != 0xffff) {
+                  dst[(size_t)j * a.F] = h;
+                  dst[(size_t)j * a.F + a.y_plane] = __float2bfloat16_rn(r[j] - __bfloat162float(h));
+                }
+              }
+            }
+          } else {
+            // queries and keys are rotated at the row's tree position (Section 3.4): y = x cos -+ (other half) sin
+#pragma unroll
+            for (int j = 0; j < 16; ++j) r[j] *= rs[j];
+            if (unit < a.H + a.Hkv) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const float2 cs = rope[min(c0 + j, a.R - 1) * half + c];
+                const float o = __shfl_xor_sync(0xffffffffu, r[j], 16);
+                r[j] = r[j] * cs.x + (hi_half ? o : -o) * cs.y;
+              }
+            }
+            const int col = c + hi_half * half;
+            if (unit < a.H) {
+              bf16 *dst = a.q + (size_t)c0 * a.H * a.dh + unit * a.dh + col;
+              const int stride = a.H * a.dh;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const bf16 h = __float2bfloat16_rn(r[j]);
+                if (row_of(j) != 0xffff) {
+                  dst[(size_t)j * stride] = h;
+                  dst[(size_t)j * stride + a.q_plane] = __float2bfloat16_rn(r[j] - __bfloat162float(h));
+                }
+              }
+            } else if (unit < a.H + 2 * a.Hkv) {                // the cache stores bf16: one rounding, on store
+              const int is_v = unit >= a.H + a.Hkv, kvh = unit - a.H - (is_v ? a.Hkv : 0);
+              bf16 *dst = a.kcache + (is_v ? a.kv_stride : 0) + kvh * a.dh + col;
+              const size_t stride = (size_t)a.Hkv * a.dh;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const int w = row_of(j);
+                if (w != 0xffff) {
+                  const int pos = s_pos[w >> 8] + (w & 255);
+                  if (pos < a.max_ctx) dst[kv_row(a.pages, s_slot[w >> 8], pos, a.max_ctx) * stride] = __float2bfloat16_rn(r[j]);
+                }
               }
             }
           }
-          tc_commit(empty_w + 8 * sw);   // the slots are free once these MMAs have read them
-          tc_commit(empty_x + 8 * sx);
         }
-        tc_commit(acc_full + 8 * buf);
-        u += kb1 - kb0;
-        ++seg;
       }
     }
-  } else {                       // ---- epilogue warps 2..5: TMEM lane quarter = warp % 4
-    if (sc.pdl) griddep_wait();
-    const int quarter = warp & 3;
-    const int i = quarter * 32 + lane;            // row within each 128-row tile = TMEM lane
-    const size_t plane_elems = (size_t)sc.ws_rows * BM, slot_elems = TM * plane_elems;
-    int seg = 0;
-    int u = u0;
-    while (u < u1) {
-      const int st = u / KB, kb0 = u - st * KB;
-      const int kb1 = min(KB, kb0 + (u1 - u));
-      const int buf = seg % NBUF;
-      mbar_wait(acc_full + 8 * buf, (seg / NBUF) & 1, a.err, dead, wait_ns);
-      tc_fence_after();
-      const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * TM * ACC);
-      float *my_ws = a.ws + (size_t)(cta * kGemmSlots + seg) * slot_elems + i;
-      for (int c0 = 0; c0 < a.R && seg < kGemmSlots; c0 += 16) {
-        float r0[16], r1[16];
-        tc_ld16(tacc + c0, r0);
-        tc_ld16(tacc + ACC + c0, r1);
-        tc_ld_wait();
-        if (MERGE) {             // columns pl * NPAD .. hold the sums over plane pl
+  } else {
+  for (int p0 = 0; p0 < wk.nt; p0 += cf.tp) {
+    const int tp = min(cf.tp, wk.nt - p0);
+    // the residual rows a warp adds to first are on their way before the contraction is complete
+    float4 g0, h1;
+    auto residual = [&](int loc, int tl) {
+      return __ldcg(reinterpret_cast<const float4 *>(a.h + (size_t)min(own0 + loc, a.R - 1) * a.d + (wk.t0 + p0 + tl) * BM + lane * 4));
+    };
+    if (epi) {
+      if (EPI == EPI_RESIDUAL) {
+        g0 = residual(ew, 0);
+        h1 = ew + kEpiWarps < n_own ? residual(ew + kEpiWarps, 0) : residual(ew, min(1, tp - 1));
+      }
+      if (p0 == 0) wait_acc();
+    }
+    if (split > 1) {
+      // No CTA of the cluster reads its ring, or the previous pass's sums, any more.  With room of their own for the sums
+      // the first pass only needs every CTA to have started.
+      if (p0 == 0 && cf.red_off) cluster_wait(); else cg::this_cluster().sync();
+    } else if (epi && p0 > 0) {
+      epi_sync();
+    }
+    if (epi) {
+      const uint32_t mine = base + cf.red_off + (uint32_t)((quarter * 32 + lane) * 4), step = (uint32_t)tp * 512u;
+#pragma unroll 1
+      for (int tl = 0; tl < tp; ++tl) {
+#pragma unroll 1
+        for (int c0 = half_w * 16; c0 < a.R; c0 += 32) {
+          float r[16];
+          load_acc(p0 + tl, c0, r);
 #pragma unroll
-          for (int pl = 1; pl < P; ++pl) {
-            float l0[16], l1[16];
-            tc_ld16(tacc + pl * NPAD + c0, l0);
-            tc_ld16(tacc + ACC + pl * NPAD + c0, l1);
-            tc_ld_wait();
+          for (int g = 0; g < 4; ++g) {            // four token rows go to one CTA (tpo is a multiple of four)
+            const int m = c0 + 4 * g;
+            if (m < a.R) {
+              const int o = (m * cf.inv_tpo) >> 16;
+              const uint32_t dst = map_rank(mine + (uint32_t)(((int)rank * cf.tpo + m - o * cf.tpo) * tp + tl) * 512u, (uint32_t)o);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) { r0[j] += l0[j]; r1[j] += l1[j]; }
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int m = c0 + j;
-          if (m < a.R) {
-            __stcg(my_ws + (size_t)m * BM, r0[j]);
-            __stcg(my_ws + plane_elems + (size_t)m * BM, r1[j]);
+              for (int j = 0; j < 4; ++j) st_cluster(dst + j * step, r[4 * g + j]);
+            }
           }
         }
       }
       tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty + 8 * buf);   // the MMA warp may reuse this accumulator
-      u += kb1 - kb0;
-      ++seg;
     }
+    if (split > 1) cg::this_cluster().sync();
+    else if (epi) epi_sync();
+    if (!epi) continue;
+    const int slice = cf.tpo * tp * BM;            // floats of one k slice's part
+    auto sums = [&](int idx) {                     // sum over the k slices, in rank order
+      float4 v = *reinterpret_cast<const float4 *>(red + idx);
+#pragma unroll 1
+      for (int s = 1; s < split; ++s) v = add4(v, *reinterpret_cast<const float4 *>(red + s * slice + idx));
+      return v;
+    };
+    // a warp per (token row, tile or pair of tiles): 4 neighbouring columns, or pairs, per lane; half a warp for rotary pairs
+    const int loc0 = EPI == EPI_QKV_ROPE ? 2 * ew + (lane >> 4) : ew, dloc = EPI == EPI_QKV_ROPE ? 2 * kEpiWarps : kEpiWarps;
+    int loc = loc0, tl = loc0 >= n_own ? tp : 0;
+#pragma unroll 1
+    while (tl < tp) {
+      int nloc = loc + dloc, ntl = tl;
+      if (nloc >= n_own) { nloc = loc0; ntl += pitch; }
+      const float4 c0 = g0;
+      if (EPI == EPI_RESIDUAL) {
+        g0 = h1;
+        int l2 = nloc + dloc, t2 = ntl;
+        if (l2 >= n_own) { l2 = loc0; ++t2; }
+        if (t2 < tp) h1 = residual(l2, t2);
+      }
+      const int m = own0 + loc, tile = wk.t0 + p0 + tl, row = s_row[m], s = row >> 8, v = row & 255;
+      const float rs = s_rs[m];
+      const int idx = (loc * tp + tl) * BM, rope_row = (cf.rope_bytes ? loc : m) * half;
+      loc = nloc; tl = ntl;
+      if (row == 0xffff) continue;
+      if (EPI == EPI_RESIDUAL || EPI == EPI_PSEUDO || EPI == EPI_LOGITS) {
+        const int n0 = tile * BM + lane * 4;
+        const float4 sum = mul4(sums(idx + lane * 4), rs);
+        if (EPI == EPI_RESIDUAL) {
+          int xp_row = -1;
+          if (a.xp != nullptr) {
+            if (a.rw.chains) xp_row = v < a.rw.T ? s * a.rw.T + v : -1;
+            else xp_row = v == a.rw.anchor ? s : -1;
+          }
+          store_residual(a, m, xp_row, n0, add4(c0, sum), a.x ? load_bf16x4(a.g + n0) : sum, lane);
+        } else if (EPI == EPI_PSEUDO) {            // output column = (map, column); d is a multiple of 128: one map per tile
+          const int i = n0 / a.d, o = n0 - i * a.d;
+          const float4 r = a.pred_b ? add4(sum, load_bf16x4(a.pred_b + n0)) : sum;
+          store_residual(a, s * a.rw.Ms + a.rw.T + (a.rw.chains ? (a.pseudo0 + i) * a.rw.T + v : a.pseudo0 + i), -1, o, r, load_bf16x4(a.g + o), lane);
+        } else if (n0 < a.N) {                     // EPI_LOGITS
+          float *dst = a.logits + (size_t)m * a.N + n0;
+          if ((a.N & 3) == 0) {
+            *reinterpret_cast<float4 *>(dst) = sum;
+          } else {
+            const float t[4] = {sum.x, sum.y, sum.z, sum.w};
+            for (int j = 0; j < 4 && n0 + j < a.N; ++j) dst[j] = t[j];
+          }
+        }
+      } else if (EPI == EPI_SWIGLU) {
+        const int j0 = (tile >> 1) * BM + lane * 4;
+        if (j0 >= a.F) continue;
+        const float4 va = mul4(sums(idx + lane * 4), rs), vb = mul4(sums(idx + BM + lane * 4), rs);
+        const float gg[4] = {va.x, va.y, va.z, va.w}, uu[4] = {vb.x, vb.y, vb.z, vb.w};
+        float y[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[j] = gg[j] / (1.f + __expf(-gg[j])) * uu[j];
+        uint2 hi, lo;
+        split4(y, hi, lo);
+        bf16 *dst = a.y + (size_t)m * a.F + j0;
+        *reinterpret_cast<uint2 *>(dst) = hi;
+        *reinterpret_cast<uint2 *>(dst + a.y_plane) = lo;
+      } else {
+        const int e = (lane & 15) * 4, hd = e / half, c = e - hd * half;
+        const int i1 = hd * a.dh + (c >> 4) * 32 + (c & 15);
+        const int unit = tile * sc.heads + hd;     // query, key or value head
+        if (unit >= a.H + 2 * a.Hkv) continue;
+        const float4 va = mul4(sums(idx + i1), rs), vb = mul4(sums(idx + i1 + 16), rs);
+        const float2 *rope = (cf.rope_bytes ? reinterpret_cast<const float2 *>(data + cf.rope_off) : a.rope) + rope_row + c;
+        const float4 c0 = *reinterpret_cast<const float4 *>(rope), c1 = *reinterpret_cast<const float4 *>(rope + 2);
+        float x1[4] = {va.x, va.y, va.z, va.w}, x2[4] = {vb.x, vb.y, vb.z, vb.w};
+        if (unit < a.H + a.Hkv) {        // queries and keys are rotated at the row's tree position (Section 3.4)
+          const float co[4] = {c0.x, c0.z, c1.x, c1.z}, si[4] = {c0.y, c0.w, c1.y, c1.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float y1 = x1[j] * co[j] - x2[j] * si[j], y2 = x2[j] * co[j] + x1[j] * si[j];
+            x1[j] = y1; x2[j] = y2;
+          }
+        }
+        if (unit < a.H) {
+          uint2 h1, l1, h2, l2;
+          split4(x1, h1, l1); split4(x2, h2, l2);
+          bf16 *dst = a.q + (size_t)m * a.H * a.dh + unit * a.dh + c;
+          *reinterpret_cast<uint2 *>(dst) = h1;
+          *reinterpret_cast<uint2 *>(dst + half) = h2;
+          *reinterpret_cast<uint2 *>(dst + a.q_plane) = l1;
+          *reinterpret_cast<uint2 *>(dst + a.q_plane + half) = l2;
+        } else {                         // the cache stores bf16: one rounding, on store
+          const int is_v = unit >= a.H + a.Hkv, kvh = unit - a.H - (is_v ? a.Hkv : 0), pos = s_pos[s] + v;
+          if (pos < a.max_ctx) {
+            bf16 *dst = a.kcache + (is_v ? a.kv_stride : 0) + (kv_row(a.pages, s_slot[s], pos, a.max_ctx) * a.Hkv + kvh) * a.dh + c;
+            *reinterpret_cast<uint2 *>(dst) = round4(x1);
+            *reinterpret_cast<uint2 *>(dst + half) = round4(x2);
+          }
+        }
+      }
+    }
+  }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(Cfg::TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cf.tmem_cols) : "memory");
   }
 }
 
@@ -331,149 +602,234 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// bf16 tensor maps with 64-element (128-byte) inner boxes, 128-byte swizzle, zero fill out of bounds.
-//   half == 0: 2-D [rows][K], box [box_rows][64]
-//   half  > 0: 4-D view [rows / (2 half)][2][half][K] of a QKV weight, box [128 / half][1][half][64]:
-//              the same half of 128 / half neighbouring heads
-// Encoded maps are cached: the same few (pointer, shape) pairs recur every step.
-bool make_map(CUtensorMap *m, const void *ptr, uint64_t rows, uint64_t K, uint32_t box_rows, uint32_t half) {
-  typedef std::tuple<const void *, uint64_t, uint64_t, uint32_t, uint32_t> Key;
+// Tensor maps of bf16 matrices with 64-element (128-byte) inner boxes, 128-byte swizzle, zero fill out of bounds; `rank`
+// dimensions from the second on in dims / strides (bytes) / box.  Encoded maps are cached: the same few (pointer, shape)
+// pairs recur every step.
+struct MapDims { int rank; cuuint64_t dim[5], stride[4]; cuuint32_t box[5]; };
+bool make_map(CUtensorMap *m, const void *ptr, const MapDims &d) {
+  typedef std::tuple<const void *, cuuint64_t, cuuint64_t, cuuint64_t, cuuint64_t, cuuint64_t, cuuint64_t, cuuint32_t, cuuint32_t> Key;
   static std::map<Key, CUtensorMap> cache;
-  const Key key(ptr, rows, K, box_rows, half);
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  const Key key(ptr, d.dim[0], d.dim[1], d.dim[2], d.dim[3], d.dim[4], d.stride[1], d.box[1], d.box[2] * 8u + (cuuint32_t)d.rank);
   auto it = cache.find(key);
   if (it != cache.end()) { *m = it->second; return true; }
-  CUresult rc;
-  if (half == 0) {
-    const cuuint64_t dims[2] = {K, rows};
-    const cuuint64_t strides[1] = {K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    rc = encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else {
-    const cuuint64_t dims[4] = {K, half, 2, rows / (2 * half)};
-    const cuuint64_t strides[3] = {K * 2, (cuuint64_t)half * K * 2, (cuuint64_t)2 * half * K * 2};
-    const cuuint32_t box[4] = {(cuuint32_t)BK, half, 1, (cuuint32_t)BM / half};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    rc = encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(ptr), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  }
-  if (rc != CUDA_SUCCESS) return false;
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  if (encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)d.rank, const_cast<void *>(ptr), d.dim, d.stride, d.box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return false;
   if (cache.size() > 4096) cache.clear();
   cache[key] = *m;
   return true;
 }
-
-int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-  }
-  return n;
-}
-
-Sched make_sched(GemmEpilogue epi, const GemmArgs &a, bool pdl);
-
-template <int NPAD, int P>
-cudaError_t launch_np(const GemmArgs &a, const Sched &sc, cudaStream_t st) {
-  using Cfg = TcCfg<NPAD, P>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<NPAD, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  const int xrows = std::min((a.R + 7) & ~7, NPAD);
-  CUtensorMap tmW, tmX;
-  if (!make_map(&tmW, a.W, (uint64_t)a.N, (uint64_t)a.K, BM, sc.mode == ROWS_ROTARY ? (uint32_t)sc.half : 0u))
-    return cudaErrorInvalidValue;
-  if (!make_map(&tmX, a.X, (uint64_t)(P - 1) * a.plane_rows + a.R, (uint64_t)a.K, (uint32_t)xrows, 0)) return cudaErrorInvalidValue;
-  // the GEMM that follows (if any): its weight map and schedule, for the tail prefetch
-  CUtensorMap tmNext = tmW;
-  Sched nx{};
-  if (a.next_W && a.next_units > 0) {
-    GemmArgs b{};
-    b.W = a.next_W; b.N = a.next_N; b.K = a.next_K; b.F = a.next_F; b.dh = a.next_dh; b.plane_rows = a.plane_rows;
-    b.H = a.next_heads; b.Hkv = 0;
-    nx = make_sched((GemmEpilogue)a.next_epi, b, false);
-    nx.l2_ahead = a.next_units;
-    if (!make_map(&tmNext, b.W, (uint64_t)b.N, (uint64_t)b.K, BM, nx.mode == ROWS_ROTARY ? (uint32_t)nx.half : 0u))
-      return cudaErrorInvalidValue;
-  }
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)sc.sk.G);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg::SMEM;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = sc.pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<NPAD, P>, tmW, tmX, tmNext, a, sc, nx);
-}
-
-cudaError_t launch_rows(const GemmArgs &a, const Sched &sc, cudaStream_t st) {
-  if (a.planes == 3) {   // N = 3 NPAD must be a multiple of 16
-    if (a.R <= 16) return launch_np<16, 3>(a, sc, st);
-    if (a.R <= 48) return launch_np<48, 3>(a, sc, st);
-    if (a.R <= 80) return launch_np<80, 3>(a, sc, st);
-    return launch_np<144, 3>(a, sc, st);
-  }
-  if (a.planes == 1) {   // plain bf16 activations (the hi plane alone)
-    if (a.R <= 16) return launch_np<16, 1>(a, sc, st);
-    if (a.R <= 48) return launch_np<48, 1>(a, sc, st);
-    if (a.R <= 80) return launch_np<80, 1>(a, sc, st);
-    return launch_np<144, 1>(a, sc, st);
-  }
-  if (a.R <= 16) return launch_np<16, 2>(a, sc, st);
-  if (a.R <= 40) return launch_np<40, 2>(a, sc, st);
-  if (a.R <= 48) return launch_np<48, 2>(a, sc, st);
-  if (a.R <= 80) return launch_np<80, 2>(a, sc, st);
-  return launch_np<144, 2>(a, sc, st);
-}
-
-Sched make_sched(GemmEpilogue epi, const GemmArgs &a, bool pdl) {
-  Sched sc{};
-  sc.pdl = pdl ? 1 : 0;
-  sc.ws_rows = a.plane_rows;
-  sc.l2_ahead = a.l2_ahead < 0 ? 0 : a.l2_ahead;
-  sc.mode = ROWS_LINEAR; sc.n_st = (a.N + TM * BM - 1) / (TM * BM);
+// weights [N][K] in the tile order of the epilogue
+bool weight_map(CUtensorMap *m, int epi, const void *W, uint64_t N, uint64_t K, uint64_t F, uint64_t dh) {
+  MapDims d{};
+  d.dim[0] = K; d.box[0] = BK;
   if (epi == EPI_SWIGLU) {
-    sc.mode = ROWS_GATE_UP; sc.F = a.F; sc.n_st = (a.F + BM - 1) / BM;
+    d.rank = 3; d.dim[1] = F; d.dim[2] = 2; d.stride[0] = K * 2; d.stride[1] = F * K * 2; d.box[1] = BM; d.box[2] = 1;
   } else if (epi == EPI_QKV_ROPE) {
-    sc.mode = ROWS_ROTARY; sc.half = a.dh / 2;
-    const int hp = BM / sc.half;
-    sc.n_st = (a.H + 2 * a.Hkv + hp - 1) / hp;
+    const uint64_t half = dh / 2;
+    d.rank = 5; d.dim[1] = 16; d.dim[2] = 2; d.dim[3] = half / 16; d.dim[4] = N / dh;
+    d.stride[0] = K * 2; d.stride[1] = half * K * 2; d.stride[2] = 16 * K * 2; d.stride[3] = dh * K * 2;
+    d.box[1] = 16; d.box[2] = 2; d.box[3] = (cuuint32_t)(half / 16); d.box[4] = (cuuint32_t)(BM / dh);
+  } else {
+    d.rank = 2; d.dim[1] = N; d.stride[0] = K * 2; d.box[1] = BM;
   }
-  sc.sk.KB = (a.K + BK - 1) / BK;
-  sc.sk.U = sc.n_st * sc.sk.KB;
-  sc.sk.G = std::min(sm_count(), sc.sk.U);
-  // With more than 80 rows the MMAs fall behind the weight stream, and a lookahead beyond the ring only fills L2
-  // with tiles that are evicted before they are read and then fetched twice (measured at 140 rows: 1.8x the weight
-  // bytes from DRAM, step 10 % slower).  With few rows the stream is the bound and the deep lookahead pays.
-  if (a.R > 80) sc.l2_ahead = 0;
-  return sc;
+  return make_map(m, W, d);
+}
+// activation planes [planes][plane_rows][K], the first npad rows of all planes per box
+bool plane_map(CUtensorMap *m, const void *X, uint64_t planes, uint64_t plane_rows, uint64_t K, uint32_t npad) {
+  MapDims d{};
+  d.rank = 3; d.dim[0] = K; d.dim[1] = plane_rows; d.dim[2] = planes; d.stride[0] = K * 2; d.stride[1] = plane_rows * K * 2;
+  d.box[0] = BK; d.box[1] = npad; d.box[2] = (cuuint32_t)planes;
+  return make_map(m, X, d);
+}
+
+constexpr uint32_t pow2_cols(int c) { return c <= 32 ? 32 : c <= 64 ? 64 : c <= 128 ? 128 : c <= 256 ? 256 : 512; }
+constexpr int align_n(int v, int a) { return (v + a - 1) / a * a; }
+
+typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const LinArgs, const TileSched, const TileCfg);
+template <int EPI> KernelFn kernel_epi(int tm, bool merged) {
+  switch (tm) {
+    case 1: return merged ? gemm_kernel<1, true, EPI> : gemm_kernel<1, false, EPI>;
+    case 2: return merged ? gemm_kernel<2, true, EPI> : gemm_kernel<2, false, EPI>;
+    default: return merged ? gemm_kernel<3, true, EPI> : gemm_kernel<3, false, EPI>;
+  }
+}
+KernelFn kernel_of(int epi, int tm, bool merged) {
+  switch (epi) {
+    case EPI_RESIDUAL: return kernel_epi<EPI_RESIDUAL>(tm, merged);
+    case EPI_QKV_ROPE: return kernel_epi<EPI_QKV_ROPE>(tm, merged);
+    case EPI_SWIGLU: return kernel_epi<EPI_SWIGLU>(tm, merged);
+    case EPI_LOGITS: return kernel_epi<EPI_LOGITS>(tm, merged);
+    default: return kernel_epi<EPI_PSEUDO>(tm, merged);
+  }
+}
+
+// CTAs that can run at once in clusters of n with one CTA per SM (GPCs hold whole clusters only: 148, 148, 135, 132,
+// 130, 132, 105, 120 for n = 1 .. 8 on a B200)
+int cluster_ctas(int n) {
+  static int cap[9] = {0};
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  if (cap[n] == 0) {
+    int dev = 0, sms = 0, k = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
+    if (n == 1) { cap[n] = sms; return sms; }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(n * 64); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemMax;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    KernelFn fn = kernel_of(EPI_RESIDUAL, 1, true);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&k, fn, &cfg) != cudaSuccess || k < 1) { cudaGetLastError(); k = std::max(1, sms / n * 3 / 4); }
+    cap[n] = k * n;
+  }
+  return cap[n];
+}
+
+struct Plan { TileSched sc; TileCfg cf; int tm, merged, smem; };
+
+// cycles of one M = 128, K = 16 MMA of n columns: reading the operands from shared memory (128 + n rows of 32 bytes at 128
+// bytes a cycle), computing, or issuing it, whichever takes longest (measured: 50 at 16 columns, 55 at 80, 72 at 144)
+float mma_clk(int n) { return std::max(50.f, std::max(n / 2.f, 34.f + n / 4.f)); }
+
+Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes) {
+  Plan best{};
+  float best_cost = 1e30f;
+  TileSched s{};
+  s.mode = epi == EPI_SWIGLU ? ROWS_GATE_UP : epi == EPI_QKV_ROPE ? ROWS_ROTARY : ROWS_LINEAR;
+  s.heads = s.mode == ROWS_ROTARY ? BM / dh : 0;
+  s.n_tiles = s.mode == ROWS_GATE_UP ? 2 * ((F + BM - 1) / BM) : (N + BM - 1) / BM;
+  s.KB = (K + BK - 1) / BK;
+  for (int merged = 1; merged >= 0; --merged) {
+    if (!merged && planes == 1) continue;
+    const int npad = merged ? align_n(R, planes == 2 ? 8 : 16) : align_n(R, 16);
+    const int n_mma = merged ? planes * npad : npad;
+    if (n_mma > 256) continue;
+    const int x_stage = planes * npad * 128;
+    for (int tm = 1; tm <= 3; ++tm) {
+      // the epilogue reads 16 columns at a time, 8 of them beyond the last plane's when npad is an odd multiple of 8
+      const int over = npad & 8;
+      if (tm * n_mma + over > 512 || (s.mode == ROWS_GATE_UP && tm != 2)) continue;
+      for (int split = 1; split <= 8 && split <= s.KB; ++split) {
+        const int cap = cluster_ctas(split) / split * split;
+        int jobs = (s.n_tiles + tm - 1) / tm;
+        const int waves = (jobs * split + cap - 1) / cap, kb = (s.KB + split - 1) / split;
+        const int per = std::min(tm, s.n_tiles);
+        // rings: four activation stages (two or three of the wide ones), the rest for weight tiles
+        // and, when it is not much, room for the sums over the k slices (saves a cluster barrier) or the rotary table (an L2
+        // round trip every 16 token rows)
+        const int tpo = align_n((R + split - 1) / split, 4), per_tile = split * tpo * 512;         // bytes of a tile's sums
+        int red = split > 1 ? per * per_tile : 0, rope = epi == EPI_QKV_ROPE ? align_n(std::min(tpo, R) * dh * 4, 128) : 0;
+        if (red > 40 * 1024) red = 0;
+        if (rope > 24 * 1024) rope = 0;
+        const int side = red + rope;
+        const int avail = kSmemMax - 1024 - kTailBytes - side;
+        int sx = std::min(x_stage <= 12 * 1024 ? 4 : x_stage <= 24 * 1024 ? 3 : 2, std::max(kb, 1));
+        const bool by_unit = tm == 1 && 2 * n_mma + over <= 512 && s.KB / split >= 2;
+        if (by_unit) sx = std::max(2, sx & ~1);
+        int sw = std::min(std::min(kMaxStages, (avail - sx * x_stage) / W_TILE), kb * per);
+        if (by_unit) sw &= ~1; else sw = sw / per * per;
+        if (sw < per || sw * W_TILE + sx * x_stage > avail) continue;
+        if (x_stage <= 24 * 1024) sx = std::min(std::min(6, kb), (avail - sw * W_TILE) / x_stage);      // what is left
+        if (by_unit) sx &= ~1;
+        if (sw < 2 * per && kb > 1) continue;
+        // microseconds: the weights at the rate HBM gives that many CTAs (6.8 TB/s from 84 on); a CTA's MMAs; its bytes from
+        // L2, which gives a CTA 150 GB/s and all of them 15 TB/s; the epilogue's two passes (35 rows: 0.8 + 1.1 us, 131
+        // rows: 3.2 + 3.0 us after the O projection; from registers 2.3 and 7 us for a gate and up pair) and barriers
+        const int ctas = std::min(jobs * split, cap), own = std::min(tpo, R);
+        const float hbm = (float)s.n_tiles * s.KB * W_TILE / 6.8e6f * std::max(1.f, 84.f / ctas);
+        const float mma = (float)waves * per * kb * 4.f * (merged ? 1 : planes) * mma_clk(n_mma) / 1850.f;
+        const float ingest = (float)waves * kb * (per * W_TILE + x_stage) / std::min(150e3f, 15e6f / ctas);
+        const bool direct = split == 1 && (epi == EPI_QKV_ROPE || epi == EPI_SWIGLU || epi == EPI_LOGITS);
+        const float out = direct ? 0.5f + 0.025f * R * per : 0.025f * R * per + 0.09f * own * per + (split == 1 ? 0.5f : red ? 1.f : 2.f);
+        // a ring slot goes round in 0.9 us (activations) or 1.4 us (weights)
+        const float rings_us = (float)waves * kb * std::max(0.9f / sx, 1.4f * per / sw);
+        const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.1f * (hbm + mma + ingest) + waves * (2.f + out);
+        TileCfg c{};
+        c.planes = planes; c.npad = npad; c.acc = n_mma; c.sw = sw; c.sx = sx;
+        c.tpo = tpo; c.inv_tpo = (65536 + c.tpo - 1) / c.tpo;
+        c.planes_side = merged ? planes : 1; c.acc_set = tm * n_mma; c.sets = 1; c.issuers = 1;
+        if (by_unit) c.sets = c.issuers = 2;
+        else if (tm >= 2) { c.issuers = 2; c.by_tile = 1; }
+        c.idesc = instr_desc_m128(n_mma); c.tmem_cols = pow2_cols(c.sets * tm * n_mma + over);
+        const int rings = align_n(sw * W_TILE + sx * x_stage, 128);
+        if (red) {
+          c.red_off = rings; c.tp = per; c.tail = rings + red;
+        } else {
+          c.tail = align_n(std::max(rings, per_tile * (s.mode == ROWS_GATE_UP ? 2 : 1)), 128);      // gate and up tiles go together
+          c.tp = std::min(per, c.tail / per_tile);
+        }
+        if (rope) { c.rope_off = c.tail; c.rope_bytes = rope; c.tail += rope; }
+        const int smem = c.tail + 1024 + kTailBytes;
+        if (smem > kSmemMax || cost >= best_cost) continue;
+        best_cost = cost;
+        best = Plan{s, c, tm, merged, smem};
+        best.sc.jobs = jobs; best.sc.split = split;
+      }
+    }
+  }
+  return best;
+}
+
+Plan cached_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes) {
+  typedef std::tuple<int, int, int, int, int, int> Key;
+  static std::map<Key, Plan> cache;
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  const Key key((int)epi * 256 + dh, N, K, F, R, planes);
+  auto it = cache.find(key);
+  if (it != cache.end()) return it->second;
+  const Plan p = make_plan(epi, N, K, F, dh, R, planes);
+  if (cache.size() > 4096) cache.clear();
+  return cache[key] = p;
 }
 
 }  // namespace
 
 bool gemm_tc_available() { return encode_fn() != nullptr; }
 
-cudaError_t launch_gemm_tc(GemmEpilogue epi, const GemmArgs &a, bool pdl, cudaStream_t st, StreamK *sk_out) {
+cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream_t st) {
   if (!encode_fn()) return cudaErrorNotSupported;
-  const Sched sc = make_sched(epi, a, pdl);
-  // a CTA's range of U / G units touches at most this many supertiles, each needing a scratch slot
-  const int per = (sc.sk.U + sc.sk.G - 1) / sc.sk.G;
-  if (sc.sk.G > kGemmMaxCtas || (per + sc.sk.KB - 2) / sc.sk.KB + 1 > kGemmSlots ||
-      (long long)(sc.sk.U + 1) * (sc.sk.G + 1) >= (1ll << 31))   // the schedule arithmetic is 32-bit
+  Plan p = cached_plan(epi, a.N, a.K, a.F, a.dh, a.R, a.planes);
+  if (p.tm == 0 || p.smem > kSmemMax || p.cf.tp < 1 || p.cf.sw < 1 || p.cf.sx < 1 || (p.cf.sets == 2 && ((p.cf.sw | p.cf.sx) & 1)))
     return cudaErrorInvalidConfiguration;
-  if (sk_out) *sk_out = sc.sk;
-  return launch_rows(a, sc, st);
+  p.cf.pdl = pdl ? 1 : 0;
+  KernelFn fn = kernel_of(epi, p.tm, p.merged != 0);
+  static std::map<KernelFn, int> configured;
+  static std::mutex mu;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!configured[fn]) {
+      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+      if (e != cudaSuccess) return e;
+      configured[fn] = 1;
+    }
+  }
+  CUtensorMap tmW, tmX;
+  if (!weight_map(&tmW, epi, a.W, (uint64_t)a.N, (uint64_t)a.K, (uint64_t)a.F, (uint64_t)a.dh)) return cudaErrorInvalidValue;
+  if (!plane_map(&tmX, a.X, (uint64_t)a.planes, (uint64_t)a.plane_rows, (uint64_t)a.K, (uint32_t)p.cf.npad)) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(p.sc.jobs * p.sc.split));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = p.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int na = 0;
+  if (pdl) { attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[na++].val.programmaticStreamSerializationAllowed = 1; }
+  if (p.sc.split > 1) {
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = p.sc.split; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1; ++na;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, fn, tmW, tmX, a, p.sc, p.cf);
 }
 
 }  // namespace firp

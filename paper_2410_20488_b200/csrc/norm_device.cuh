@@ -1,5 +1,4 @@
-// Device bodies of the residual-update + RMSNorm pass and of the operand split for Eq. 3, shared by their own
-// kernels and by the fused decoder kernel.
+// Device bodies of the persistent kernel's residual-update + RMSNorm pass and of its operand split for Eq. 3.
 //   rmsnorm_item:  h[r] += the partial tiles a residual GEMM left in scratch (fixed order: ascending CTA index);
 //                  x[r] = h[r] * g as bf16 planes (hi, lo; plus a third plane on request) -- NOT yet divided by the
 //                  row's RMS; ss[r][w] = sum of h[r][c]^2 over the 128 columns of warp w.  The division by

@@ -1,35 +1,37 @@
-// Small kernels of the FIRP step: tree bookkeeping, embedding, residual-add + RMSNorm,
-// the pseudo-hidden projection (Eq. 3), the acceptance walk / next tree, KV compaction.
+// Small kernels of the FIRP step: tree bookkeeping and embedding, the acceptance walk / next tree, KV compaction.
+#include "finish_device.cuh"
 #include "firp_kernels.cuh"
 #include "launch_util.cuh"
-#include "norm_device.cuh"
 
 
 namespace firp {
 
 // ---------------------------------------------------------------------------
-// Tree prep (Section 3.4 "Tree attention"; Section 3.3 for the pseudo rows):
-// depth, absolute position, ancestor-or-self bitmask, rotary table.
-// One CTA per sequence; the extended parent array lives in shared memory.
+// Everything a step needs before its first layer, one CTA per row:
+//   bookkeeping (Section 3.4 "Tree attention"; Section 3.3 for the pseudo rows): depth, absolute position,
+//   ancestor-or-self bitmask, rotary table
+//   embedding: the fp32 residual row of a tree row from the bf16 table, and what the first layer reads of it
+// Latency-bound; rows are independent once each CTA has the parents of its sequence in shared memory.
 // ---------------------------------------------------------------------------
-__global__ void tree_prep_kernel(Rows rw, const int32_t *parents, int parents_stride, const int32_t *seq_ids,
-                                 const int32_t *ctx_len, int dh, float theta, TreeMeta meta,
-                                 int32_t *out_depth, uint32_t *out_mask, int out_mask_words, unsigned *zero_word, int pdl) {
+constexpr int kPrepThreads = 128;
+
+__global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl) {
   __shared__ int32_t ext[kMaxTreeRows];
-  __shared__ int32_t sdepth[kMaxTreeRows];
+  __shared__ int s_depth;
   if (pdl) { griddep_launch(); griddep_wait(); }
-  const int s = blockIdx.x, tid = threadIdx.x;
-  if (zero_word && s == 0 && tid == 0) *zero_word = 0u;
-  const int n = ctx_len[seq_ids[s]];
-  for (int v = tid; v < rw.Ms; v += blockDim.x) {
+  const Rows &rw = a.rw;
+  const int r = blockIdx.x, s = r / rw.Ms, v = r - s * rw.Ms, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (a.zero_word && r == 0 && tid == 0) *a.zero_word = 0u;
+  const int n = a.ctx_len[a.seq_ids[s]];
+  for (int u = tid; u <= v; u += kPrepThreads) {
     int p;
-    if (v < rw.T) p = parents[s * parents_stride + v];     // stride 0: one template for every sequence
-    else if (rw.chains) p = v - rw.T;   // step 1 of node u (row T + u) hangs off u, step i off step i-1 of the same node
-    else p = (v == rw.T) ? rw.anchor : v - 1;
-    ext[v] = p;
+    if (u < rw.T) p = a.parents[s * a.parents_stride + u];
+    else if (rw.chains) p = u - rw.T;   // step 1 of node w (row T + w) hangs off w, step i off step i-1 of the same node
+    else p = (u == rw.T) ? rw.anchor : u - 1;
+    ext[u] = p;
   }
   __syncthreads();
-  for (int v = tid; v < rw.Ms; v += blockDim.x) {
+  if (tid == kPrepThreads - 1) {        // the last warp: the rotary table below is the first ones'
     uint32_t bits[kMaskWords];
 #pragma unroll
     for (int w = 0; w < kMaskWords; ++w) bits[w] = 0u;
@@ -43,104 +45,35 @@ __global__ void tree_prep_kernel(Rows rw, const int32_t *parents, int parents_st
       ++dep;
       u = ext[u];
     }
-    sdepth[v] = dep;
-    const int r = s * rw.Ms + v;
-    meta.depth[r] = dep;
-    meta.pos[r] = n + dep;
+    s_depth = dep;
+    a.meta.depth[r] = dep;
+    a.meta.pos[r] = n + dep;
 #pragma unroll
-    for (int w = 0; w < kMaskWords; ++w) meta.mask[(size_t)r * kMaskWords + w] = bits[w];
-    if (out_depth) out_depth[r] = dep;
-    if (out_mask)
-      for (int w = 0; w < out_mask_words; ++w) out_mask[(size_t)r * out_mask_words + w] = bits[w];
+    for (int w = 0; w < kMaskWords; ++w) a.meta.mask[(size_t)r * kMaskWords + w] = bits[w];
+    if (a.out_depth) a.out_depth[r] = dep;
+    if (a.out_mask)
+      for (int w = 0; w < a.out_mask_words; ++w) a.out_mask[(size_t)r * a.out_mask_words + w] = bits[w];
+  }
+  if (v < rw.T) {                       // pseudo rows get their residual from Eq. 3
+    const int tok = min(max(a.tokens[s * rw.T + v], 0), a.vocab - 1);
+    const int xp_row = a.xp == nullptr ? -1 : rw.chains ? s * rw.T + v : v == rw.anchor ? s : -1;
+    for (int c = warp * 128 + lane * 4; c < a.d; c += kPrepThreads * 4)
+      store_residual(a, r, xp_row, c, load_bf16x4(a.embed + (size_t)tok * a.d + c), a.x ? load_bf16x4(a.g + c) : make_float4(0.f, 0.f, 0.f, 0.f), lane);
   }
   __syncthreads();
-  const int half = dh / 2;
-  const double l2t = log2((double)theta);
-  for (int i = tid; i < rw.Ms * half; i += blockDim.x) {
-    const int v = i / half, c = i % half;
-    const double inv_freq = exp2(-2.0 * (double)c / (double)dh * l2t);
-    const double ang = (double)(n + sdepth[v]) * inv_freq;
+  const int half = a.dh / 2;
+  const double l2t = log2((double)a.theta);
+  if (tid < half) {
+    const double inv_freq = exp2(-2.0 * (double)tid / (double)a.dh * l2t);
+    const double ang = (double)(n + s_depth) * inv_freq;
     double sn, cs;
     sincos(ang, &sn, &cs);
-    meta.rope[(size_t)(s * rw.Ms + v) * half + c] = make_float2((float)cs, (float)sn);
+    a.meta.rope[(size_t)r * half + tid] = make_float2((float)cs, (float)sn);
   }
 }
 
-void launch_tree_prep(const Rows &rw, const int32_t *d_parents, int parents_stride, const int32_t *d_seq_ids, const int32_t *d_ctx_len,
-                      int dh, float theta, TreeMeta meta, int32_t *out_depth, uint32_t *out_mask, int out_mask_words,
-                      unsigned *zero_word, bool pdl, cudaStream_t st) {
-  launch_k(tree_prep_kernel, dim3(rw.n_seq), dim3(256), 0, st, pdl, rw, d_parents, parents_stride, d_seq_ids, d_ctx_len, dh, theta, meta,
-           out_depth, out_mask, out_mask_words, zero_word, pdl ? 1 : 0);
-}
-
-// ---------------------------------------------------------------------------
-// Embedding gather: fp32 residual rows from bf16 table rows; pseudo rows start at zero.
-// ---------------------------------------------------------------------------
-__global__ void embed_kernel(Rows rw, const int32_t *tokens, const bf16 *__restrict__ embed, int d,
-                             int vocab, float *h, int pdl) {
-  if (pdl) { griddep_launch(); griddep_wait(); }
-  const int r = blockIdx.x, s = r / rw.Ms, v = r % rw.Ms;
-  float *dst = h + (size_t)r * d;
-  if (v >= rw.T) {
-    for (int c = threadIdx.x; c < d; c += blockDim.x) dst[c] = 0.f;
-    return;
-  }
-  int tok = tokens[s * rw.T + v];
-  tok = min(max(tok, 0), vocab - 1);
-  const bf16 *src = embed + (size_t)tok * d;
-  for (int c = threadIdx.x * 2; c < d; c += blockDim.x * 2) {
-    const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162 *>(src + c);
-    *reinterpret_cast<float2 *>(dst + c) = __bfloat1622float2(p);
-  }
-}
-
-void launch_embed(const Rows &rw, const int32_t *d_tokens, const bf16 *embed, int d, int vocab, float *h, bool pdl,
-                  cudaStream_t st) {
-  launch_k(embed_kernel, dim3(rw.R), dim3(128), 0, st, pdl, rw, d_tokens, embed, d, vocab, h, pdl ? 1 : 0);
-}
-
-// ---------------------------------------------------------------------------
-// Residual update + first half of RMSNorm, as a flat elementwise kernel.
-//   h[r] += the partial tiles a residual GEMM left in scratch (fixed order: ascending CTA index)
-//   x[r]  = h[r] * g as bf16 planes (hi, lo; plus a third plane on request) -- NOT yet divided by the row's RMS
-//   ss[r][w] = sum of h[r][c]^2 over the 128 columns of warp w
-// The division by sqrt(mean(h^2) + eps) commutes with the GEMM that consumes x, so that GEMM's
-// finisher applies it to the fp32 sums (it adds the ss[r][*] in a fixed order).  This kernel then
-// has no reduction across threads beyond a warp, no barrier, and every thread is independent.
-// A thread owns 4 neighbouring columns of one row; d must be a multiple of 128.
-// ---------------------------------------------------------------------------
-constexpr int kNormThreads = 256;
-
-__global__ void __launch_bounds__(kNormThreads)
-rmsnorm_kernel(Rows rw, int v0, int nv, float *h, Partials pend, const bf16 *__restrict__ g, int d, bf16 *x,
-               size_t x_lo_off, int planes, float *ss, int pdl) {
-  if (pdl) { griddep_launch(); griddep_wait(); }
-  rmsnorm_item(rw, v0, nv, h, pend, g, d, x, x_lo_off, planes, ss, blockIdx.x * kNormThreads + threadIdx.x);
-}
-
-cudaError_t launch_rmsnorm(const Rows &rw, int v0, int v1, float *h, const Partials &pending, const bf16 *g, int d,
-                           bf16 *x, size_t x_lo_off, int planes, float *ss, bool pdl, cudaStream_t st) {
-  const int nv = v1 - v0;
-  if (nv <= 0) return cudaSuccess;
-  const int threads = rw.n_seq * nv * (d >> 2);
-  return launch_k(rmsnorm_kernel, dim3((threads + kNormThreads - 1) / kNormThreads), dim3(kNormThreads), 0, st, pdl, rw,
-                  v0, nv, h, pending, g, d, x, x_lo_off, planes, ss, pdl ? 1 : 0);
-}
-
-// ---------------------------------------------------------------------------
-// Pseudo hidden states, Eq. 3: h~_i = W_i h[anchor] + b_i on the raw fp32 residual stream.  The k maps are
-// one [k d][d] weight matrix for the stream-K GEMM; this kernel prepares its operand: the anchor row of every
-// sequence, untouched by any norm, as (hi, lo) bf16 planes in row s of xp.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256)
-root_split_kernel(Rows rw, const float *h, const bf16 *g, int d, bf16 *xp, size_t xp_lo_off, int pdl) {
-  if (pdl) { griddep_launch(); griddep_wait(); }
-  root_split_item(rw, h, g, d, xp, xp_lo_off, blockIdx.x * 256 + threadIdx.x);
-}
-
-void launch_root_split(const Rows &rw, const float *h, const bf16 *g, int d, bf16 *xp, size_t xp_lo_off, bool pdl, cudaStream_t st) {
-  const int threads = rw.n_seq * (rw.chains ? rw.T : 1) * (d >> 2);
-  launch_k(root_split_kernel, dim3((threads + 255) / 256), dim3(256), 0, st, pdl, rw, h, g, d, xp, xp_lo_off, pdl ? 1 : 0);
+void launch_prep(const PrepArgs &a, bool pdl, cudaStream_t st) {
+  launch_k(prep_kernel, dim3(a.rw.R), dim3(kPrepThreads), 0, st, pdl, a, pdl ? 1 : 0);
 }
 
 // ---------------------------------------------------------------------------

@@ -32,15 +32,23 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
                : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
+// The same, but the hardware may hold the thread for up to hint_ns while the phase is incomplete.
+__device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity, uint32_t hint_ns) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(bar), "r"(parity), "r"(hint_ns) : "memory");
+  return ok != 0;
+}
 // Bounded wait: gives up after limit_ns, sets the status word and returns.  `dead` is sticky per thread:
 // after one timeout later waits return at once, so the kernel runs to its end without waiting again.
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int *err, bool &dead,
                                           unsigned long long limit_ns = kDefaultWaitNs) {
   if (dead || mbar_try_wait(bar, parity)) return;
-  const unsigned long long t0 = globaltimer();
-  uint32_t spins = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 255u) == 0 && globaltimer() - t0 > limit_ns) {
+  unsigned long long t0 = 0;
+  while (!mbar_try_wait_hint(bar, parity, 10000u)) {
+    const unsigned long long t = globaltimer();
+    if (t0 == 0) t0 = t;
+    if (t - t0 > limit_ns) {
       dead = true;
       atomicExch(err, kErrTimeout);
       return;
@@ -59,6 +67,30 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *tm,
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
       ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar), "l"(policy) : "memory");
 }
+// untiled copy; dst, src and bytes are multiples of 16
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *tm, int x, int y, int z, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
+      ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy) : "memory");
+}
+// coordinates {x, 0, 0, 0, v}
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *tm, int x, int v, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %3, %3, %4}], [%5], %6;"
+      ::"r"(dst), "l"(tm), "r"(x), "r"(0), "r"(v), "r"(bar), "l"(policy) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *tm, int x, int y, int z, uint64_t policy) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %3}], %4;"
+               ::"l"(tm), "r"(x), "r"(y), "r"(z), "l"(policy) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_5d(const CUtensorMap *tm, int x, int v, uint64_t policy) {
+  asm volatile("cp.async.bulk.prefetch.tensor.5d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %2, %2, %3}], %4;"
+               ::"l"(tm), "r"(x), "r"(0), "r"(v), "l"(policy) : "memory");
+}
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int x, int y, uint64_t policy) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile.L2::cache_hint [%0, {%1, %2}], %3;"
                ::"l"(tm), "r"(x), "r"(y), "l"(policy) : "memory");
@@ -66,6 +98,12 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int x, in
 __device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap *tm, int x, int y, int z, int w, uint64_t policy) {
   asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %3, %4}], %5;"
                ::"l"(tm), "r"(x), "r"(y), "r"(z), "r"(w), "l"(policy) : "memory");
+}
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+  return ok != 0;
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }

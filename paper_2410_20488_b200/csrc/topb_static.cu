@@ -19,7 +19,7 @@ extern "C" int firp_topb_static(const float *d_logits, int32_t rows, int32_t voc
             FIRP_TOPB_STATIC_MAX_SLOTS);
     return FIRP_ERR_CAPACITY;
   }
-  firp::launch_topb(d_logits, rows, vocab, b, d_ids, d_vals, false, (cudaStream_t)stream);
+  firp::launch_topb(d_logits, rows, vocab, b, d_ids, d_vals, true, (cudaStream_t)stream);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     fprintf(stderr, "firp_topb_static: launch failed: %s\n", cudaGetErrorString(e));

@@ -115,8 +115,9 @@ int firp_init_weights(firp_ctx *ctx, const firp_weights *w);
  * (greedy next token), n_accepted = 1, next_tree_tokens = the first draft tree on the
  * template `next_parents` (HOST, [T_next]), topb_*; logits (if given) holds 1+k rows:
  * the last prompt row, then the pseudo rows.  d_prompt is a DEVICE array [P].
- * k = 0 gives plain prefill (T_next must then be 1).  The prompt is processed 144 - k rows at a time
- * (one pass over the weights per chunk), whatever max_rows is.
+ * k = 0 gives plain prefill (T_next must then be 1).  One pass over the weights takes up to 2047 - k rows of
+ * the prompt at head_dim 128, and 144 - k otherwise, with the fused mode on or with the mma attention
+ * kernel; max_rows does not matter.
  */
 int firp_prefill(firp_ctx *ctx, int32_t seq, const int32_t *d_prompt, int32_t P, int32_t k, int32_t l,
                  const int32_t *next_parents, int32_t T_next, const firp_step_out *out, void *stream);

@@ -124,7 +124,8 @@ __device__ unsigned long long g_attn_trace[16];
 #define TC_STAMP(k) do { } while (0)
 #endif
 
-template <int NQ>
+// PROMPT: the rows are a stretch of a prompt, each sees the rows up to itself (no masks in memory)
+template <int NQ, bool PROMPT>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnArgs a,
                     int qper, int pdl) {
@@ -173,7 +174,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
   const int kvh = blockIdx.y, G = a.H / a.Hkv;
   const int qblocks = gridDim.z / a.rw.n_seq;
-  const int s = blockIdx.z / qblocks, qb = blockIdx.z % qblocks;
+  // a prompt's later blocks see more of it: the longest go first
+  const int s = blockIdx.z / qblocks, qb = PROMPT ? qblocks - 1 - (int)blockIdx.z : blockIdx.z % qblocks;
   const int split = blockIdx.x, nsplits = gridDim.x;
   const int qrows_total = a.rows_active * G, q0 = qb * qper;
   const int ncols = min(qper, qrows_total - q0);
@@ -198,7 +200,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   if (warp == 18 && lane < 2) s_sn[lane] = lane == 0 ? __ldcg(a.seq_ids + s) : __ldcg(a.pos + s * a.rw.Ms);
   __syncthreads();
   const int slot = s_sn[0], n = s_sn[1];
-  const int kv_len = min(n + a.rows_active, a.max_ctx);
+  const int kv_len = min(n + (PROMPT ? (q0 + ncols - 1) / G + 1 : a.rows_active), a.max_ctx);
   const int tiles_total = (kv_len + kTcTile - 1) / kTcTile;
   const int t0 = (split * tiles_total + nsplits - 1) / nsplits, t1 = ((split + 1) * tiles_total + nsplits - 1) / nsplits;
   const int ntiles = t1 - t0;                       // tile t0 + i goes to warpgroup i & 1 as its (i >> 1)-th
@@ -315,6 +317,13 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       if (pvalid && p >= n) {
         const int u = p - n, mw = u >> 5, b = u & 31;
         vis = 0u;
+        if (PROMPT) {
+#pragma unroll
+          for (int jj = 0; jj < NH; ++jj) {
+            const int v = (q0 + c_lo + jj) / G;      // row v sees the rows up to itself ("Masked": no other pseudo row)
+            vis |= (uint32_t)(u <= v && (!a.rw.masked || u < a.rw.T || u == v)) << jj;
+          }
+        } else
 #pragma unroll
         for (int jj = 0; jj < NH; ++jj) {
           const int qr = min(q0 + c_lo + jj, qrows_total - 1);
@@ -537,13 +546,13 @@ bool kv_map(CUtensorMap *m, const void *plane, uint64_t rows, uint64_t width) {
   return true;
 }
 
-template <int NQ>
+template <int NQ, bool PROMPT>
 cudaError_t launch_nq(const CUtensorMap &tmK, const CUtensorMap &tmV, const AttnArgs &a, int qblocks, int qper, bool pdl,
                       cudaStream_t st) {
   constexpr int SMEM = TcLayout<NQ>::BYTES + 1024;      // + what aligning the base to 1024 bytes may take
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_tc_kernel<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    cudaError_t e = cudaFuncSetAttribute(tree_attn_tc_kernel<NQ, PROMPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
     configured = true;
   }
@@ -559,7 +568,7 @@ cudaError_t launch_nq(const CUtensorMap &tmK, const CUtensorMap &tmV, const Attn
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel<NQ>, tmK, tmV, a, qper, pdl ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel<NQ, PROMPT>, tmK, tmV, a, qper, pdl ? 1 : 0);
 }
 
 }  // namespace
@@ -597,9 +606,13 @@ cudaError_t launch_attention_tc(const AttnArgs &a, bool pdl, cudaStream_t st) {
   const uint64_t width = (uint64_t)a.Hkv * kTcDh, rows = a.kv_stride / width;
   CUtensorMap tmK, tmV;
   if (!kv_map(&tmK, a.kcache, rows, width) || !kv_map(&tmV, a.kcache + a.kv_stride, rows, width)) return cudaErrorInvalidValue;
-  if (qper <= 16) return launch_nq<16>(tmK, tmV, a, qblocks, qper, pdl, st);
-  if (qper <= 32) return launch_nq<32>(tmK, tmV, a, qblocks, qper, pdl, st);
-  return launch_nq<48>(tmK, tmV, a, qblocks, qper, pdl, st);
+  if (a.rw.prompt) {
+    if (qper <= 16) return launch_nq<16, true>(tmK, tmV, a, qblocks, qper, pdl, st);
+    return launch_nq<48, true>(tmK, tmV, a, qblocks, qper, pdl, st);
+  }
+  if (qper <= 16) return launch_nq<16, false>(tmK, tmV, a, qblocks, qper, pdl, st);
+  if (qper <= 32) return launch_nq<32, false>(tmK, tmV, a, qblocks, qper, pdl, st);
+  return launch_nq<48, false>(tmK, tmV, a, qblocks, qper, pdl, st);
 }
 
 }  // namespace firp

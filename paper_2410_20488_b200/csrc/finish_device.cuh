@@ -83,15 +83,12 @@ __device__ __forceinline__ float4 load_bf16x4(const bf16 *p) {
 }
 
 // A row of the residual stream has its new value: store it, and what the next GEMM reads of it -- x = h * g as bf16 planes
-// (not yet divided by the row's RMS: the consumer's epilogue does that), the sum of squares of these 128 columns and, for
-// the rows Eq. 3 reads at the next layer, their own planes.  One warp, 4 neighbouring columns per lane.
+// (not yet divided by the row's RMS: the consumer's epilogue does that), sq, the sum of squares of these 128 columns, and,
+// for the rows Eq. 3 reads at the next layer, their own planes.  One warp, 4 neighbouring columns per lane.
 template <typename Args>   // LinArgs or PrepArgs
-__device__ __forceinline__ void store_residual(const Args &a, int row, int xp_row, int col, float4 v, float4 g, int lane) {
+__device__ __forceinline__ void store_residual(const Args &a, int row, int xp_row, int col, float4 v, float4 g, float sq, int lane) {
   *reinterpret_cast<float4 *>(a.h + (size_t)row * a.d + col) = v;
   if (a.x == nullptr) return;
-  float sq = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
   if (lane == 0) a.ss_out[(size_t)row * kNormMaxWarps + (col >> 7)] = sq;
   const float y[4] = {v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w};
   uint2 hi, lo;
@@ -110,6 +107,12 @@ __device__ __forceinline__ void store_residual(const Args &a, int row, int xp_ro
     *reinterpret_cast<uint2 *>(dp) = hi;
     *reinterpret_cast<uint2 *>(dp + a.xp_plane) = lo;
   }
+}
+__device__ __forceinline__ float warp_sq(float4 v) {
+  float sq = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  return sq;
 }
 
 // ---- q, k, v: rotary embedding, query planes, cache rows --------------------------------------

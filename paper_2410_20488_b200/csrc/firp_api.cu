@@ -49,7 +49,7 @@ struct firp_ctx {
   std::string err;
   int launches = 0;
   bool bound = false, have_weights = false, stepped = false;
-  int Rmax = 0, S = 0;                  // rows the workspace holds (a prefill chunk), path stride
+  int Rmax = 0, S = 0;                  // rows the workspace holds (a stretch of a prompt), path stride
   int row_cap = 0;                      // rows one step may carry (max_rows of the configuration)
   int sm_count = 148;                   // of the device the buffers were bound on
   bool use_pdl = true;                  // programmatic dependent launch
@@ -95,21 +95,21 @@ struct firp_ctx {
   size_t carve(void *base) {
     Carver c{reinterpret_cast<uint8_t *>(base), 0};
     const int d = cfg.d_model, nq = cfg.n_heads * cfg.head_dim, half = cfg.head_dim / 2;
-    const size_t R = Rmax;
+    const size_t R = Rmax, Rt = kMaxTreeRows;     // rows of a prompt; rows of a step and of what the lm-head sees
     h = c.take<float>(R * d);
     xp = c.take<bf16>(2 * R * d);           // the rows Eq. 3 reads (anchor of each sequence, or all tree rows): hi plane, lo plane
     x = c.take<bf16>(3 * R * d);            // normalised activations: hi plane, lo plane, third plane (QKV input)
     q = c.take<bf16>(2 * R * nq);
     o = c.take<bf16>(2 * R * nq);
     y = c.take<bf16>(2 * R * cfg.d_ffn);
-    gemm_ws = c.take<float>((size_t)kGemmMaxCtas * kGemmSlots * 2 * R * 128);
+    gemm_ws = c.take<float>((size_t)kGemmMaxCtas * kGemmSlots * 2 * Rt * 128);
     ss = c.take<float>(R * kNormMaxWarps);
-    logits = c.take<float>(R * cfg.vocab);
-    top_ids = c.take<int32_t>(R * kMaxTopB);
-    top_vals = c.take<float>(R * kMaxTopB);
-    meta.depth = c.take<int32_t>(R);
+    logits = c.take<float>(Rt * cfg.vocab);
+    top_ids = c.take<int32_t>(Rt * kMaxTopB);
+    top_vals = c.take<float>(Rt * kMaxTopB);
+    meta.depth = c.take<int32_t>(Rt);
     meta.pos = c.take<int32_t>(R);
-    meta.mask = c.take<uint32_t>(R * kMaskWords);
+    meta.mask = c.take<uint32_t>(Rt * kMaskWords);
     meta.rope = c.take<float2>(R * half);
     ctx_len = c.take<int32_t>(cfg.max_batch);
     seq_ids = c.take<int32_t>(kMaxSeq);
@@ -243,7 +243,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
 
   if (fused) {      // all decoder layers (and the lm-head) as one persistent kernel
     FusedStep fs{};
-    fs.shape = fshape; fs.rw = rw; memcpy(fs.tl, ra.tl, sizeof(fs.tl)); fs.want_head = ra.want_head; fs.prenorm = c->pred_prenorm != 0; fs.Rp = (int)Rp;
+    fs.shape = fshape; fs.rw = rw; memcpy(fs.tl, ra.tl, sizeof(fs.tl)); fs.want_head = ra.want_head; fs.prenorm = c->pred_prenorm != 0; fs.Rp = (int)Rp; fs.ws_rows = kMaxTreeRows;
     fs.n_hi_max = ra.n_hi_max; fs.max_batch = cfg.max_batch; fs.weights_gen = c->weights_gen; fs.wait_ns = c->wait_ns;
     fs.wqkv = c->wqkv.data(); fs.wo = c->wo.data(); fs.wgu = c->wgu.data(); fs.wd = c->wd.data();
     fs.g_attn = c->g_attn.data(); fs.g_mlp = c->g_mlp.data();
@@ -262,9 +262,9 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
   }
 
   enum { G_QKV = 0, G_O, G_GATE_UP, G_DOWN, G_LM_HEAD };     // index of c->planes
-  auto launch = [&](GemmEpilogue epi, const void *W, int N, int K, int planes, int R, LinArgs &l) -> cudaError_t {
-    l.W = (const bf16 *)W; l.N = N; l.K = K; l.R = R; l.F = F; l.dh = dh; l.planes = planes; l.plane_rows = (int)Rp;
-    l.rw = rw; l.err = c->dev_status; l.wait_ns = c->wait_ns; l.eps = cfg.rms_eps;
+  auto launch = [&](GemmEpilogue epi, const void *W, int N, int K, int planes, const Rows &rows, LinArgs &l, int R = 0) -> cudaError_t {
+    l.W = (const bf16 *)W; l.N = N; l.K = K; l.R = R ? R : rows.R; l.rw = rows; l.F = F; l.dh = dh; l.planes = planes; l.plane_rows = (int)Rp;
+    l.err = c->dev_status; l.wait_ns = c->wait_ns; l.eps = cfg.rms_eps;
     ++nl;
     return launch_gemm(epi, l, pdl, st);
   };
@@ -287,7 +287,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       if (c->pred_prenorm) l.ss = c->ss;
       l.pred_b = c->w.pred_b ? (const bf16 *)c->w.pred_b + (size_t)alive * d : nullptr;
       residual_out(l, c->g_attn[j], x_planes);
-      FIRP_CUDA(c, launch(EPI_PSEUDO, (const bf16 *)c->w.pred_w + (size_t)alive * d * d, ins * d, d, 2, rw.n_seq * per_step, l));
+      FIRP_CUDA(c, launch(EPI_PSEUDO, (const bf16 *)c->w.pred_w + (size_t)alive * d * d, ins * d, d, 2, rw, l, rw.n_seq * per_step));
       alive += ins;
     }
     bf16 *kplane = c->kv + (size_t)j * c->kv_layer();
@@ -297,7 +297,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       l.X = c->x; l.ss = c->ss; l.rows_active = act;
       l.H = H; l.Hkv = Hkv; l.rope = c->meta.rope; l.seq_ids = c->seq_ids; l.pos = c->meta.pos;
       l.q = c->q; l.q_plane = Rp * nq; l.kcache = kplane; l.kv_stride = c->kv_plane(); l.max_ctx = cfg.max_ctx; l.pages = c->pages();
-      FIRP_CUDA(c, launch(EPI_QKV_ROPE, c->wqkv[j], (H + 2 * Hkv) * dh, d, c->planes[G_QKV], rw.R, l));
+      FIRP_CUDA(c, launch(EPI_QKV_ROPE, c->wqkv[j], (H + 2 * Hkv) * dh, d, c->planes[G_QKV], rw, l));
     }
     {
       AttnArgs a{};
@@ -326,13 +326,13 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       LinArgs l{};
       l.X = c->o; l.rows_active = act;
       residual_out(l, c->g_mlp[j], 2);
-      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wo[j], d, nq, c->planes[G_O], rw.R, l));
+      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wo[j], d, nq, c->planes[G_O], rw, l));
     }
     {
       FIRP_TIMED(KC_GEMM_GATE_UP);
       LinArgs l{};
       l.X = c->x; l.ss = c->ss; l.rows_active = act; l.y = c->y; l.y_plane = Rp * F;
-      FIRP_CUDA(c, launch(EPI_SWIGLU, c->wgu[j], 2 * F, d, c->planes[G_GATE_UP], rw.R, l));
+      FIRP_CUDA(c, launch(EPI_SWIGLU, c->wgu[j], 2 * F, d, c->planes[G_GATE_UP], rw, l));
     }
     {
       FIRP_TIMED(KC_GEMM_DOWN);
@@ -346,23 +346,27 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       } else {
         l.h = c->h; l.d = d;     // nothing reads the stream after the last layer of a prompt's inner chunk
       }
-      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wd[j], d, F, c->planes[G_DOWN], rw.R, l));
+      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wd[j], d, F, c->planes[G_DOWN], rw, l));
     }
   }
   if (ra.want_head) {
+    // of a prompt only the last row and the pseudo rows behind it need logits: they become the rows of what follows
+    const int first = rw.prompt ? rw.T - 1 : 0;
+    Rows hr = rw;
+    if (rw.prompt) { hr = Rows{}; hr.n_seq = 1; hr.T = 1; hr.k = rw.k; hr.kc = rw.kc; hr.Ms = hr.R = 1 + rw.k; }
     if (!fused) {
       FIRP_TIMED(KC_GEMM_LM_HEAD);
       LinArgs l{};
-      l.X = c->x; l.ss = c->ss; l.rows_active = rw.Ms; l.logits = ra.logits_dst;
-      FIRP_CUDA(c, launch(EPI_LOGITS, c->w.lm_head, cfg.vocab, d, c->planes[G_LM_HEAD], rw.R, l));
+      l.X = c->x + (size_t)first * d; l.ss = c->ss + (size_t)first * kNormMaxWarps; l.rows_active = hr.Ms; l.logits = ra.logits_dst;
+      FIRP_CUDA(c, launch(EPI_LOGITS, c->w.lm_head, cfg.vocab, d, c->planes[G_LM_HEAD], hr, l));
     }
     { FIRP_TIMED(KC_TOPB);
-      launch_topb(ra.logits_dst, rw.R, cfg.vocab, cfg.top_b, c->top_ids, c->top_vals, pdl, st); ++nl; }
+      launch_topb(ra.logits_dst, hr.R, cfg.vocab, cfg.top_b, c->top_ids, c->top_vals, pdl, st); ++nl; }
     AcceptArgs a{};
     a.tokens = ra.d_tokens; a.parents = c->parents; a.next_parents = c->next_parents;
     a.parents_stride = ra.parents_stride; a.sizes = ra.d_sizes;
     a.top_ids = c->top_ids; a.top_vals = c->top_vals; a.T_next = ra.T_next; a.B = cfg.top_b; a.S = c->S;
-    a.prefill_last_row = ra.prefill_last_row;
+    a.prefill_last_row = rw.prompt ? 0 : ra.prefill_last_row;
     a.path = c->path; a.n_accepted = c->n_acc; a.accepted = c->accepted; a.next_tokens = c->next_tokens;
     if (out) {
       a.o_path = out->path; a.o_n_accepted = out->n_accepted; a.o_accepted = out->accepted_tokens;
@@ -370,7 +374,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       a.o_topb_ids = out->topb_ids; a.o_topb_vals = out->topb_vals;
     }
     FIRP_TIMED(KC_ACCEPT);
-    launch_accept(rw, a, pdl, st); ++nl;
+    launch_accept(hr, a, pdl, st); ++nl;
   }
   FIRP_CUDA(c, cudaGetLastError());
   return FIRP_OK;
@@ -401,7 +405,9 @@ int firp_create(const firp_model_cfg *cfg, firp_ctx **out) {
   if (cfg->max_rows < 0 || cfg->max_rows > 144) return bad("max_rows must be 0..144");
   if (cfg->max_rows > rows) rows = cfg->max_rows;
   c->row_cap = (int)align_up(rows, 16);
-  c->Rmax = 144;          // the workspace always holds the largest row count, so that a prompt is prefilled 141 rows at a time
+  // The workspace always holds a step's 144 rows, whatever the step capacity, and, at head dimension 128, a stretch of a
+  // prompt: up to 2047 rows, no more than a context can have.
+  c->Rmax = cfg->head_dim == 128 ? std::max(kMaxTreeRows, std::min((int)align_up(cfg->max_ctx, 16), (int)align_up(kMaxPromptRows, 16))) : kMaxTreeRows;
   c->S = cfg->max_depth + 1;
   c->n_hi.assign(cfg->max_batch, 0);
 
@@ -588,7 +594,7 @@ static int step_impl(firp_ctx *ctx, int32_t n_seq, const int32_t *seq_ids, const
   if (tree_sizes && (rc = upload_i32(ctx, ctx->tree_sizes, tree_sizes, n_seq, ctx->last_sizes, st))) return rc;
 
   RunArgs ra{};
-  ra.rw = Rows{n_seq, T, pseudo, Ms, n_seq * Ms, 0, chains ? 1 : 0, k, ctx->pseudo_masked};
+  ra.rw = Rows{n_seq, T, pseudo, Ms, n_seq * Ms, 0, chains ? 1 : 0, k, ctx->pseudo_masked, 0};
   for (int i = 0; i < k; ++i) ra.tl[i] = layers[i];
   ra.d_tokens = d_tree_tokens; ra.want_head = true; ra.prefill_last_row = -1; ra.T_next = T_next;
   ra.out = out; ra.logits_dst = (out && out->logits) ? out->logits : ctx->logits; ra.n_hi_max = n_hi_max;
@@ -628,13 +634,15 @@ int firp_prefill_layers(firp_ctx *ctx, int32_t seq, const int32_t *d_prompt, int
   std::vector<int32_t> ids(1, seq);
   if ((rc = upload_i32(ctx, ctx->seq_ids, ids.data(), 1, ctx->last_seq_ids, st))) return rc;
   if ((rc = upload_i32(ctx, ctx->next_parents, next_parents, T_next, ctx->last_next_parents, st))) return rc;
-  // chain template for the prompt rows
-  // the prompt runs in chunks of as many rows as the kernels take at once (144 less the pseudo rows of the last
-  // chunk): a 512-token prompt is four passes over the weights
-  const int chunk = std::min(ctx->Rmax, kMaxTreeRows) - k;
-  std::vector<int32_t> chain(chunk);
-  for (int i = 0; i < chunk; ++i) chain[i] = i - 1;
-  if ((rc = upload_i32(ctx, ctx->parents, chain.data(), chunk, ctx->last_parents, st))) return rc;
+  // At head dimension 128 (tcgen05 attention, one kernel per operation) up to 2047 rows run at once, so that the GEMMs are
+  // bound by the tensor cores and not by re-reading the weights; otherwise as many as a step may have.
+  const bool prompt = cfg.head_dim == 128 && ctx->attn_tc != 0 && !ctx->use_fused;
+  const int chunk = std::min(ctx->Rmax, prompt ? kMaxPromptRows : kMaxTreeRows) - k;
+  if (!prompt) {
+    std::vector<int32_t> chain(chunk);
+    for (int i = 0; i < chunk; ++i) chain[i] = i - 1;
+    if ((rc = upload_i32(ctx, ctx->parents, chain.data(), chunk, ctx->last_parents, st))) return rc;
+  }
   FIRP_CUDA(ctx, cudaMemsetAsync(ctx->ctx_len + seq, 0, sizeof(int32_t), st));
   ctx->n_hi[seq] = 0;
 
@@ -643,7 +651,7 @@ int firp_prefill_layers(firp_ctx *ctx, int32_t seq, const int32_t *d_prompt, int
     const bool last = (p0 + Tc == P);
     const int kc = last ? k : 0;
     RunArgs ra{};
-    ra.rw = Rows{1, Tc, kc, Tc + kc, Tc + kc, Tc - 1, 0, kc, ctx->pseudo_masked};
+    ra.rw = Rows{1, Tc, kc, Tc + kc, Tc + kc, Tc - 1, 0, kc, ctx->pseudo_masked, prompt ? 1 : 0};
     for (int i = 0; i < kc; ++i) ra.tl[i] = layers[i];
     ra.d_tokens = d_prompt + p0; ra.want_head = last; ra.prefill_last_row = Tc - 1; ra.T_next = T_next;
     ra.out = nullptr; ra.logits_dst = ctx->logits; ra.n_hi_max = ctx->n_hi[seq];
@@ -654,7 +662,7 @@ int firp_prefill_layers(firp_ctx *ctx, int32_t seq, const int32_t *d_prompt, int
     }
     if ((rc = run_rows(ctx, ra, st))) return rc;
     if (last && out && out->logits)
-      FIRP_CUDA(ctx, cudaMemcpyAsync(out->logits, ctx->logits + (size_t)(Tc - 1) * cfg.vocab,
+      FIRP_CUDA(ctx, cudaMemcpyAsync(out->logits, ctx->logits + (prompt ? 0 : (size_t)(Tc - 1) * cfg.vocab),
                                      sizeof(float) * (size_t)(1 + k) * cfg.vocab, cudaMemcpyDeviceToDevice, st));
     launch_advance_ctx(1, ctx->seq_ids, ctx->ctx_len, Tc, ctx->use_pdl, st); ++ctx->launches;
     ctx->n_hi[seq] += Tc;

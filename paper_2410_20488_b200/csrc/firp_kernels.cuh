@@ -10,6 +10,7 @@ typedef __nv_bfloat16 bf16;
 
 constexpr int kMaxSeq = 16;        // sequences per step
 constexpr int kMaxTreeRows = 144;  // rows per sequence: T + k (128 + 8), or T (1 + k) with a chain under every node
+constexpr int kMaxPromptRows = 2047;  // rows of a prompt that run at once, pseudo rows included
 constexpr int kMaskWords = 5;      // ceil(136 / 32)
 constexpr int kMaxTopB = 8;
 constexpr int kAttnTile = 64;      // kv positions per attention tile
@@ -27,6 +28,8 @@ struct Rows {
   int chains;  // != 0: a chain under every tree node; chain row i (1-based) of node v is row T + (i-1) T + v
   int kc;      // prediction steps per chain (k = kc with one chain, k = T * kc with a chain per node)
   int masked;  // != 0: a pseudo row sees no other pseudo row (the "Masked" ablation of Section 4.3)
+  int prompt;  // != 0: a stretch of a prompt: one sequence, rows 0 .. T-1 a chain, the pseudo rows behind it; more rows than a
+               // tree may have, no masks in TreeMeta (row v sees the rows up to itself)
 };
 
 // Rows of the KV cache.  A (layer, K|V) plane holds max_batch * max_ctx rows of Hkv * dh elements.  Without a
@@ -150,7 +153,7 @@ struct LinArgs {
   const bf16 *X;    // [planes][plane_rows][K] activations as bf16 planes
   int plane_rows, planes;
   const bf16 *W;    // [N][K] weights
-  int R, N, K;      // token rows (<= kMaxTreeRows)
+  int R, N, K;      // token rows (<= kMaxPromptRows)
   Rows rw; int rows_active;      // rows with v < rows_active are written, the others skipped
   int *err;         // device status word (set to a non-zero code if a bounded wait gives up)
   unsigned long long wait_ns;   // bounded waits give up after this many nanoseconds (0: the default of 2 s)
@@ -246,7 +249,7 @@ struct FusedStep {
   int tl[8];                 // insertion layer of each prediction step (non-decreasing)
   bool want_head;            // final norm + lm-head
   bool prenorm;              // Eq. 3 reads the anchor through the insertion layer's input RMSNorm
-  int Rp;                    // rows per activation plane
+  int Rp, ws_rows;           // rows per activation plane, per scratch tile
   int n_hi_max;              // upper bound of the longest committed context among the sequences
   int max_batch;             // of the configuration (sizes the attention scratch)
   uint64_t weights_gen;      // changes whenever the weight pointers change

@@ -80,7 +80,7 @@ struct FusedOp {
 
 struct FusedParams {
   Rows rw;
-  int d, H, Hkv, dh, F, V, Rp, max_ctx, splits;
+  int d, H, Hkv, dh, F, V, Rp, ws_rows, max_ctx, splits;
   float eps;
   float *h, *ws, *ss, *logits, *attn_ws;
   bf16 *x, *xp, *q, *o, *y, *kv;
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
     unsigned epoch = 0;
     unsigned use[2] = {0u, 0u};
     const int nq = P.H * P.dh;
-    const size_t plane_elems = (size_t)P.Rp * BM, slot_elems = TM * plane_elems;
+    const size_t plane_elems = (size_t)P.ws_rows * BM, slot_elems = TM * plane_elems;
     griddep_wait();                                  // tree bookkeeping and embeddings are complete
     if (P.n_ops > 0 && P.ops[0].type == OP_GEMM && wtid == 0) mbar_arrive(xgo);
     for (int oi = 0; oi < P.n_ops; ++oi) {
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
         }
         case OP_NORM: {
           Partials pend{};
-          pend.ws = P.ws; pend.ws_rows = P.Rp;
+          pend.ws = P.ws; pend.ws_rows = P.ws_rows;
           if (op.aux >= 0) { const GemmClass &c = P.cls[op.aux]; pend.sk = StreamK{c.U, c.KB, c.G}; }
           const unsigned total = (unsigned)(P.rw.n_seq * op.nv * (P.d >> 2));
           for (unsigned t = tbase; t < total; t += tstride)
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
         case OP_FINISH: {
           const GemmClass &c = P.cls[op.cls];
           Partials p{};
-          p.sk = StreamK{c.U, c.KB, c.G}; p.ws = P.ws; p.ws_rows = P.Rp;
+          p.sk = StreamK{c.U, c.KB, c.G}; p.ws = P.ws; p.ws_rows = P.ws_rows;
           GemmArgs a{};
           a.R = P.rw.R; a.rw = P.rw; a.rows_active = op.act; a.N = c.N; a.K = c.K; a.eps = P.eps;
           const int n_st = c.U / c.KB;
@@ -607,7 +607,7 @@ cudaError_t launch_fused_layers(FusedPlan *plan, const FusedStep &fs, bool pdl, 
   if (!same) {
     plan->valid = false;
     P = FusedParams{};
-    P.rw = rw; P.d = d; P.H = H; P.Hkv = Hkv; P.dh = dh; P.F = F; P.V = sh.V; P.Rp = fs.Rp; P.max_ctx = sh.max_ctx; P.eps = sh.eps;
+    P.rw = rw; P.d = d; P.H = H; P.Hkv = Hkv; P.dh = dh; P.F = F; P.V = sh.V; P.Rp = fs.Rp; P.ws_rows = fs.ws_rows; P.max_ctx = sh.max_ctx; P.eps = sh.eps;
     P.h = fs.h; P.ws = fs.ws; P.ss = fs.ss; P.attn_ws = fs.attn_ws; P.x = fs.x; P.xp = fs.xp; P.q = fs.q; P.o = fs.o; P.y = fs.y;
     P.kv = fs.kv; P.kv_seq = fs.kv_seq; P.kv_layer = fs.kv_layer; P.kv_plane = fs.kv_plane; P.pages = fs.pages;
     P.rope = fs.rope; P.pos = fs.pos; P.seq_ids = fs.seq_ids; P.ctx_len = fs.ctx_len; P.mask = fs.mask;

@@ -1,11 +1,11 @@
 // Weight-streaming GEMM of the step on the 5th-generation tensor cores (tcgen05 + TMEM), operands staged by TMA, with
 // the elementwise step that follows the contraction in its epilogue.
-//   out[m][n] = sum_k X[m][k] * W[n][k], m = T + k token rows (at most 144), W read once.
+//   out[m][n] = sum_k X[m][k] * W[n][k], m = the T + k token rows of a step (at most 144) or the rows of a prompt.
 //
 // Roles are swapped: weight rows are the MMA M dimension (one TMEM lane each), token rows the MMA N dimension (one
-// TMEM column each).  A tile is 128 weight rows that one thread block finishes by itself: 128 neighbouring rows, or 64
-// gate rows and the 64 up rows that go with them.  A job is up to TM tiles; the k blocks of a job are cut over the
-// `split` CTAs of a cluster, and grid = jobs x split, one wave wherever the matrix allows it.
+// TMEM column each).  A tile is 128 weight rows; a job is up to TM tiles (or 128 gate rows and the 128 up rows that go with
+// them) that one thread block, or a cluster, finishes by itself for up to 256 token rows: the k blocks of a job are cut over
+// the `split` CTAs of the cluster.  Grid = jobs x blocks of token rows x split, one wave wherever the matrix allows it.
 //
 // Why whole tiles and not one equal share of the matrix per SM: HBM does not need every SM.  A TMA ring of 6 x 32 KB per
 // CTA streams 6.7 TB/s from 86 CTAs, 6.8 from 108, 6.9 from 128 (measured), so a schedule that leaves some SMs without
@@ -14,15 +14,18 @@
 // the O projection at 35 rows of the 7B shape, 37 of 102 us per layer.  Step at the 7B shape, 35 rows, 512 cached tokens:
 // 3534 -> 3121 us; one row 3062 -> 2696; 13B shape, 67 rows 8958 -> 6734; 34B shape, 140 rows 6631 -> 6230.
 //
+// A prompt comes as one stretch of up to 2047 rows, in blocks of up to 256: the weights, 13.5 GB at the 7B shape, are read
+// once instead of once per 141 rows.  It is bound by the MMA issue of two passes over the bf16 planes: 1999 tokens of the 7B
+// shape 92.2 -> 65.9 ms; per layer QKV 0.44, attention 0.33, O 0.19, gate/up 0.60, down 0.45 ms.
+//
 // Bound now, per layer of 98 us: the weight stream (QKV 15.1, gate/up 27.8, down 13.1 us at 6.7-6.9 TB/s; the O projection
 // 5.5), the epilogues (4 + 2.5 + 2 + 2), five hand-overs of 2 us and the attention's 12.
 //
 // Per CTA (one per SM at the large shapes):
 //   warp 0     : weight producer (one thread, TMA, 128-byte swizzle, deep ring).  Weights never depend on the previous
-//                kernel, so under programmatic dependent launch this stream starts while the predecessor drains.  Its
-//                own loads issued, it brings the head of the next GEMM's weights into L2.
+//                kernel, so under programmatic dependent launch this stream starts while the predecessor drains.
 //   warp 2     : activation producer: the bf16 planes of the k block, after waiting for the previous kernel.
-//   warp 1     : MMA issuer: tcgen05.mma kind::f16, M = 128, K = 16.  The planes of the activations (hi, lo) either sit
+//   warps 1, 3 : MMA issuers: tcgen05.mma kind::f16, M = 128, K = 16.  The planes of the activations (hi, lo) either sit
 //                side by side as ONE operand of N = planes x npad columns (added in the epilogue) or are accumulated
 //                one after the other into npad columns.  The whole warp runs the loop and an elected lane issues, which
 //                keeps the descriptors in uniform registers (M = 128, N = 80: 59 cycles per MMA; one lane alone: 86).
@@ -56,9 +59,9 @@ constexpr int kThreads = 384;      // 12 warps
 constexpr int kEpiWarps = 8;
 constexpr int W_TILE = BM * 128;   // bytes of one 128-row weight tile of a k block
 constexpr int kSmemMax = 227 * 1024;
-constexpr int kTailBytes = 1536;   // row scales, row indices, slots and lengths, barriers, TMEM address (behind the rings)
-constexpr int kMaxRows = kMaxTreeRows;
-constexpr int kMaxStages = 12;       // of either ring
+constexpr int kTailBytes = 1984;   // row scales, row indices, slots and lengths, barriers, TMEM address (behind the rings)
+constexpr int kMaxRows = 256;      // token rows of a CTA (MMA N)
+constexpr int kMaxW = 12, kMaxX = 6;  // ring depths: weight tiles, activation stages
 
 // How the rows of the weight are dealt to tiles of 128, each one TMA box per k block.
 //   ROWS_LINEAR   128 neighbouring rows
@@ -71,13 +74,15 @@ struct TileSched {
   int mode, heads;   // heads: of a tile (ROWS_ROTARY)
   int n_tiles, KB;   // tiles; 64-wide k blocks
   int jobs, split;   // job j = tiles [n_tiles j / jobs, n_tiles (j + 1) / jobs), its k blocks cut over `split` CTAs
+  int blocks;        // of token rows: the CTAs of a job's blocks are neighbours, so that its weights come from HBM once
 };
 // A CTA starts its k range at a place of its own and wraps around: CTAs that march through k together would ask the same
 // L2 slices for the same activation rows, and HBM for weight rows whose addresses differ only above bit 12.
-struct CtaWork { int t0, nt, kb0, kb1, off; };
+struct CtaWork { int t0, nt, kb0, kb1, off, block; };
 __device__ __forceinline__ CtaWork cta_work(const TileSched &s, int cta) {
-  const int j = cta / s.split, r = cta - j * s.split;
+  const int jb = cta / s.split, r = cta - jb * s.split, j = s.blocks == 1 ? jb : jb / s.blocks;
   CtaWork w;
+  w.block = jb - j * s.blocks;
   w.t0 = s.n_tiles * j / s.jobs;
   w.nt = s.n_tiles * (j + 1) / s.jobs - w.t0;
   w.kb0 = s.KB * r / s.split;
@@ -90,9 +95,10 @@ __device__ __forceinline__ int unit_kb(const CtaWork &w, int u) { const int k = 
 
 // Shared memory and operand shape of a launch.
 struct TileCfg {
-  int planes, npad;     // activation planes; token rows padded to the MMA's N
+  int planes, npad;     // activation planes; token rows of a block padded to the MMA's N
+  int rpb;              // token rows of a block
   int acc;              // accumulator columns per tile
-  int issuers, by_tile; // MMA issuing warps: they take the units in turn, each with accumulators of its own, or the tiles
+  int issuers, by_tile; // MMA issuing warps: they take the units in turn, each with accumulator sets of its own, or the tiles
   int sets, acc_set;    // accumulator sets (summed in the epilogue), columns per set
   int sw, sx;           // ring depths: weight tiles, activation stages
   int planes_side;      // planes that sit side by side in the accumulator's columns
@@ -141,12 +147,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   const uint32_t w_ring = base, x_ring = base + cf.sw * W_TILE;
   float *s_rs = reinterpret_cast<float *>(data + cf.tail);          // 1 / RMS of every token row
   int *s_slot = reinterpret_cast<int *>(s_rs + kMaxRows), *s_pos = s_slot + kMaxSeq;      // of every sequence
-  uint16_t *s_row = reinterpret_cast<uint16_t *>(s_pos + kMaxSeq);                        // sequence << 8 | row of every token row
+  uint16_t *s_row = reinterpret_cast<uint16_t *>(s_pos + kMaxSeq);                        // sequence << 11 | row of every token row
   const uint32_t bars = base + cf.tail + kMaxRows * 6 + 2 * kMaxSeq * 4;
-  const uint32_t full_w = bars, empty_w = full_w + 8 * kMaxStages, full_x = empty_w + 8 * kMaxStages, empty_x = full_x + 8 * kMaxStages,
-                 acc_full = empty_x + 8 * kMaxStages, rope_full = acc_full + 8, tmem_slot = rope_full + 8;
+  const uint32_t full_w = bars, empty_w = full_w + 8 * kMaxW, full_x = empty_w + 8 * kMaxW, empty_x = full_x + 8 * kMaxX,
+                 acc_full = empty_x + 8 * kMaxX, rope_full = acc_full + 8, tmem_slot = rope_full + 8;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const CtaWork wk = cta_work(sc, blockIdx.x);
+  const int row0 = wk.block * cf.rpb, R = min(cf.rpb, a.R - row0);      // this CTA's token rows
   const int n_units = wk.kb1 - wk.kb0;
   // The weight ring holds single tiles (16 KB slots: a slot is free again after four MMAs).  Its depth is a multiple of the
   // job's tiles, so that a slot always holds the same tile and is read by the same issuer: one that skipped a phase of a
@@ -199,25 +206,27 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
       if (cf.pdl) griddep_wait();
       if (EPI == EPI_QKV_ROPE && cf.rope_bytes) {
-        const int r0 = (int)(blockIdx.x % sc.split) * cf.tpo, bytes = max(0, min(cf.tpo, a.R - r0)) * (a.dh >> 1) * 8;   // of the rows finished here
+        const int r0 = (int)(blockIdx.x % sc.split) * cf.tpo, bytes = max(0, min(cf.tpo, R - r0)) * (a.dh >> 1) * 8;   // of the rows finished here
         mbar_expect_tx(rope_full, bytes);
-        if (bytes) bulk_load(base + cf.rope_off, a.rope + (size_t)r0 * (a.dh >> 1), bytes, rope_full);
+        if (bytes) bulk_load(base + cf.rope_off, a.rope + (size_t)(row0 + r0) * (a.dh >> 1), bytes, rope_full);
       }
       int sl = 0;
       uint32_t par = 1;
       for (int it = 0; it < n_units; ++it) {
         mbar_wait(empty_x + 8 * sl, par, a.err, dead, wait_ns);
         mbar_expect_tx(full_x + 8 * sl, x_stage);
-        tma_load_3d(x_ring + sl * x_stage, &tmX, unit_kb(wk, it) * BK, 0, 0, full_x + 8 * sl, pol);   // all planes
+        tma_load_3d(x_ring + sl * x_stage, &tmX, unit_kb(wk, it) * BK, row0, 0, full_x + 8 * sl, pol);   // all planes
         if (++sl == sx_n) { sl = 0; par ^= 1; }
       }
     }
   } else if (warp == 1 || warp == 3) {        // ---- MMA issuers
     const int iw = warp >> 1;
     if (iw < cf.issuers) {
-      // by units: unit iw, iw + issuers, ... into accumulators of its own; by tiles: every unit, tiles iw, iw + issuers, ...
+      // by units: unit iw, iw + issuers, ... into accumulator sets of its own; by tiles: every unit, tiles iw, iw + issuers, ...
       const int u0 = cf.by_tile ? 0 : iw, du = cf.by_tile ? 1 : cf.issuers;
-      const uint32_t tm0 = __shfl_sync(0xffffffffu, tmem, 0) + (cf.by_tile ? 0u : (uint32_t)(iw * cf.acc_set));
+      const uint32_t tm0 = __shfl_sync(0xffffffffu, tmem, 0);
+      uint32_t acc = tm0 + (uint32_t)(u0 * cf.acc_set);      // unit it goes to accumulator set it % sets
+      const uint32_t acc_end = tm0 + (uint32_t)(cf.sets * cf.acc_set), acc_step = (uint32_t)(du * cf.acc_set);
       int sw = cf.by_tile ? iw : u0, sx = u0;            // slot of the unit's first tile of this issuer; X slot
       uint32_t parw = 0, parx = 0;
       if (sw >= sw_n) { sw -= sw_n; parw ^= 1; }
@@ -237,10 +246,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
             const uint64_t dw = smem_desc(w_ring + sl * W_TILE);
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
-              if (elect_one()) tc_mma(tm0 + t * cf.acc, dw + 2 * kk, dx + 2 * kk, cf.idesc, (it > u0 || kk > 0) ? 1u : 0u);
+              if (elect_one()) tc_mma(acc + t * cf.acc, dw + 2 * kk, dx + 2 * kk, cf.idesc, (it >= cf.sets || kk > 0) ? 1u : 0u);
 #pragma unroll
               for (int pl = 1; pl < 3; ++pl)
-                if (!MERGED && pl < cf.planes && elect_one()) tc_mma(tm0 + t * cf.acc, dw + 2 * kk, dx + (uint64_t)(pl * (x_plane >> 4)) + 2 * kk, cf.idesc, 1u);
+                if (!MERGED && pl < cf.planes && elect_one()) tc_mma(acc + t * cf.acc, dw + 2 * kk, dx + (uint64_t)(pl * (x_plane >> 4)) + 2 * kk, cf.idesc, 1u);
             }
             if (elect_one()) tc_commit(empty_w + 8 * sl);      // the slot is free once these MMAs have read it
           }
@@ -250,6 +259,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         if (elect_one()) tc_commit(empty_x + 8 * sx);
         sw += cf.by_tile ? wk.nt : du;
         if (sw >= sw_n) { sw -= sw_n; parw ^= 1; }
+        acc += acc_step;
+        if (acc >= acc_end) acc -= acc_end - tm0;
         sx += du;
         if (sx >= sx_n) { sx -= sx_n; parx ^= 1; }
       }
@@ -263,7 +274,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   const int ew = warp - 4, quarter = warp & 3, half_w = ew >> 2;
   const int split = sc.split;
   const uint32_t rank = (uint32_t)(blockIdx.x % split);
-  const int own0 = (int)rank * cf.tpo, n_own = max(0, min(cf.tpo, a.R - own0));     // token rows this CTA finishes
+  const int own0 = (int)rank * cf.tpo, n_own = max(0, min(cf.tpo, R - own0));     // token rows (of the block) this CTA finishes
   const float *red = reinterpret_cast<const float *>(data + cf.red_off);         // [k slice][own row][tile of the pass][128]
   constexpr bool kDirect = EPI == EPI_QKV_ROPE || EPI == EPI_SWIGLU || EPI == EPI_LOGITS;   // may leave from registers
   const int half = EPI == EPI_QKV_ROPE ? a.dh >> 1 : 1;
@@ -285,7 +296,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       for (int u = 0; u < 4; ++u) {
         v[u] = 0.f;
         if (a.ss == nullptr) continue;
-        const float *p = a.ss + (size_t)lin_src_row<EPI>(a, min(m0 + u * kEpiWarps, a.R - 1)) * kNormMaxWarps;
+        const float *p = a.ss + (size_t)lin_src_row<EPI>(a, row0 + min(m0 + u * kEpiWarps, R - 1)) * kNormMaxWarps;
         v[u] = (lane < nw ? __ldcg(p + lane) : 0.f) + (lane + 32 < nw ? __ldcg(p + lane + 32) : 0.f);
       }
 #pragma unroll
@@ -295,14 +306,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         const int m = m0 + u * kEpiWarps;
         if (lane == 0 && m < m_end) {
           s_rs[m] = a.ss ? rsqrtf(v[u] / (float)a.K + a.eps) : 1.f;
-          const int s = m / per, row = m - s * per;
-          s_row[m] = (uint16_t)(m < own0 + n_own && (EPI == EPI_PSEUDO || row < a.rows_active) ? s << 8 | row : 0xffff);
+          const int s = (row0 + m) / per, row = row0 + m - s * per;
+          s_row[m] = (uint16_t)(m < own0 + n_own && (EPI == EPI_PSEUDO || row < a.rows_active) ? s << 11 | row : 0xffff);
         }
       }
     }
   }
-  // columns [c0, c0 + 16) of tile t: the sums over the planes' columns and the issuers' accumulators (all loads in flight
-  // together)
+  // columns [c0, c0 + 16) of tile t: the sums over the planes' columns and the accumulator sets
   const uint32_t tquarter = tmem + ((uint32_t)(quarter * 32) << 16);
   auto load_acc = [&](int t, int c0, float *r) {
     const uint32_t ta = tquarter + (uint32_t)(t * cf.acc + c0);
@@ -326,12 +336,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         for (int j = 0; j < 16; ++j) r[j] += l[2][j];
       }
     }
-    if (cf.planes_side > 2) {                      // a third plane
-      tc_ld16(ta + 2 * cf.npad, l[0]);
-      if (cf.sets > 1) tc_ld16(ta + cf.acc_set + 2 * cf.npad, l[1]);
-      tc_ld_wait();
+    // the third plane's columns and the third and fourth set's (one loop for all of them cost 1 us per layer)
+    if (cf.sets > 2 || cf.planes_side > 2) {
+#pragma unroll 1
+      for (int i = 0; i < cf.sets; ++i)
+#pragma unroll 1
+        for (int pl = i < 2 ? 2 : 0; pl < cf.planes_side; ++pl) {
+          tc_ld16(ta + i * cf.acc_set + pl * cf.npad, l[0]);
+          tc_ld_wait();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) r[j] += cf.sets > 1 ? l[0][j] + l[1][j] : l[0][j];
+          for (int j = 0; j < 16; ++j) r[j] += l[0][j];
+        }
     }
   };
   auto wait_acc = [&]() {
@@ -349,14 +364,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       const int rowi = quarter * 32 + lane;                     // row of the tile
       const int c = EPI == EPI_QKV_ROPE ? (quarter * 16 + (lane & 15)) & (half - 1) : 0, hi_half = (lane >> 4) & 1;
       // the rotary table of the step lies in shared memory, or, when it does not fit beside the rings, in L2
-      const float2 *rope = cf.rope_bytes ? reinterpret_cast<const float2 *>(data + cf.rope_off) : a.rope;
+      const float2 *rope = cf.rope_bytes ? reinterpret_cast<const float2 *>(data + cf.rope_off) : a.rope + (size_t)row0 * half;
       wait_acc();
 #pragma unroll 1
       for (int t = 0; t < wk.nt; t += pitch) {
         const int tile = wk.t0 + t;
         const int unit = EPI == EPI_QKV_ROPE ? tile * sc.heads + (sc.heads == 2 ? quarter >> 1 : 0) : 0;    // query, key or value head
 #pragma unroll 1
-        for (int c0 = half_w * 16; c0 < a.R; c0 += 32) {
+        for (int c0 = half_w * 16; c0 < R; c0 += 32) {
           float r[16], r2[16], rs[16];
           uint32_t row[8];                                      // two rows each
           load_acc(t, c0, r);
@@ -368,7 +383,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
           auto row_of = [&](int j) { return (int)((row[j >> 1] >> (16 * (j & 1))) & 0xffffu); };       // 0xffff: not to be written
           if (EPI == EPI_LOGITS) {
             const int n = tile * BM + rowi;
-            float *dst = a.logits + (size_t)c0 * a.N + n;
+            float *dst = a.logits + (size_t)(row0 + c0) * a.N + n;
             if (n < a.N) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) if (row_of(j) != 0xffff) dst[(size_t)j * a.N] = r[j] * rs[j];
@@ -377,7 +392,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
             const int n = (tile >> 1) * BM + rowi;
 #pragma unroll
             for (int j = 0; j < 16; ++j) { const float g = r[j] * rs[j]; r[j] = g / (1.f + __expf(-g)) * (r2[j] * rs[j]); }
-            bf16 *dst = a.y + (size_t)c0 * a.F + n;
+            bf16 *dst = a.y + (size_t)(row0 + c0) * a.F + n;
             if (n < a.F) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
@@ -395,14 +410,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
             if (unit < a.H + a.Hkv) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
-                const float2 cs = rope[min(c0 + j, a.R - 1) * half + c];
+                const float2 cs = rope[min(c0 + j, R - 1) * half + c];
                 const float o = __shfl_xor_sync(0xffffffffu, r[j], 16);
                 r[j] = r[j] * cs.x + (hi_half ? o : -o) * cs.y;
               }
             }
             const int col = c + hi_half * half;
             if (unit < a.H) {
-              bf16 *dst = a.q + (size_t)c0 * a.H * a.dh + unit * a.dh + col;
+              bf16 *dst = a.q + (size_t)(row0 + c0) * a.H * a.dh + unit * a.dh + col;
               const int stride = a.H * a.dh;
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
@@ -420,8 +435,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
               for (int j = 0; j < 16; ++j) {
                 const int w = row_of(j);
                 if (w != 0xffff) {
-                  const int pos = s_pos[w >> 8] + (w & 255);
-                  if (pos < a.max_ctx) dst[kv_row(a.pages, s_slot[w >> 8], pos, a.max_ctx) * stride] = __float2bfloat16_rn(r[j]);
+                  const int pos = s_pos[w >> 11] + (w & 2047);
+                  if (pos < a.max_ctx) dst[kv_row(a.pages, s_slot[w >> 11], pos, a.max_ctx) * stride] = __float2bfloat16_rn(r[j]);
                 }
               }
             }
@@ -432,15 +447,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   } else {
   for (int p0 = 0; p0 < wk.nt; p0 += cf.tp) {
     const int tp = min(cf.tp, wk.nt - p0);
-    // the residual rows a warp adds to first are on their way before the contraction is complete
-    float4 g0, h1;
+    // the residual rows a warp adds to first, and their gain, are on their way before the contraction is complete
+    float4 h0, h1, gain = make_float4(0.f, 0.f, 0.f, 0.f);
     auto residual = [&](int loc, int tl) {
-      return __ldcg(reinterpret_cast<const float4 *>(a.h + (size_t)min(own0 + loc, a.R - 1) * a.d + (wk.t0 + p0 + tl) * BM + lane * 4));
+      return __ldcg(reinterpret_cast<const float4 *>(a.h + (size_t)(row0 + min(own0 + loc, R - 1)) * a.d + (wk.t0 + p0 + tl) * BM + lane * 4));
     };
+    auto gain_of = [&](int tl) { return load_bf16x4(a.g + (wk.t0 + p0 + tl) * BM + lane * 4); };
     if (epi) {
-      if (EPI == EPI_RESIDUAL) {
-        g0 = residual(ew, 0);
+      if (EPI == EPI_RESIDUAL && n_own > 0) {
+        h0 = residual(ew, 0);
         h1 = ew + kEpiWarps < n_own ? residual(ew + kEpiWarps, 0) : residual(ew, min(1, tp - 1));
+        if (a.x) gain = gain_of(0);
       }
       if (p0 == 0) wait_acc();
     }
@@ -456,13 +473,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
 #pragma unroll 1
       for (int tl = 0; tl < tp; ++tl) {
 #pragma unroll 1
-        for (int c0 = half_w * 16; c0 < a.R; c0 += 32) {
+        for (int c0 = half_w * 16; c0 < R; c0 += 32) {
           float r[16];
           load_acc(p0 + tl, c0, r);
 #pragma unroll
           for (int g = 0; g < 4; ++g) {            // four token rows go to one CTA (tpo is a multiple of four)
             const int m = c0 + 4 * g;
-            if (m < a.R) {
+            if (m < R) {
               const int o = (m * cf.inv_tpo) >> 16;
               const uint32_t dst = map_rank(mine + (uint32_t)(((int)rank * cf.tpo + m - o * cf.tpo) * tp + tl) * 512u, (uint32_t)o);
 #pragma unroll
@@ -483,39 +500,80 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       for (int s = 1; s < split; ++s) v = add4(v, *reinterpret_cast<const float4 *>(red + s * slice + idx));
       return v;
     };
+    if (EPI == EPI_RESIDUAL) {
+      // a warp per (token row, tile), 4 neighbouring columns per lane
+      auto finish = [&](int loc, int n0, float4 v, float sq) {
+        const int row = s_row[own0 + loc], s = row >> 11, w = row & 2047;
+        if (row == 0xffff) return;
+        int xp_row = -1;
+        if (a.xp != nullptr) {
+          if (a.rw.chains) xp_row = w < a.rw.T ? s * a.rw.T + w : -1;
+          else xp_row = w == a.rw.anchor ? s : -1;
+        }
+        store_residual(a, row0 + own0 + loc, xp_row, n0, v, gain, sq, lane);
+      };
+      if (n_own <= 4 * kEpiWarps) {                // few rows: one after the other, two residual rows ahead
+        int loc = ew, tl = ew < n_own ? 0 : tp;
+#pragma unroll 1
+        while (tl < tp) {
+          int nloc = loc + kEpiWarps, ntl = tl;
+          if (nloc >= n_own) { nloc = ew; ++ntl; }
+          const float4 v = add4(h0, sums((loc * tp + tl) * BM + lane * 4));
+          h0 = h1;
+          int l2 = nloc + kEpiWarps, t2 = ntl;
+          if (l2 >= n_own) { l2 = ew; ++t2; }
+          if (t2 < tp) h1 = residual(l2, t2);
+          finish(loc, (wk.t0 + p0 + tl) * BM + lane * 4, v, warp_sq(v));
+          if (a.x && ntl != tl && ntl < tp) gain = gain_of(ntl);
+          loc = nloc; tl = ntl;
+        }
+      } else {                                     // a prompt's: four at a time, so that their chains overlap
+#pragma unroll 1
+        for (int tl = 0; tl < tp; ++tl) {
+          const int n0 = (wk.t0 + p0 + tl) * BM + lane * 4;
+          if (a.x && tl) gain = gain_of(tl);
+#pragma unroll 1
+          for (int l0 = ew; l0 < n_own; l0 += 4 * kEpiWarps) {
+            float4 v[4];
+            float sq[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = residual(l0 + u * kEpiWarps, tl);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              v[u] = add4(v[u], sums((min(l0 + u * kEpiWarps, n_own - 1) * tp + tl) * BM + lane * 4));
+              sq[u] = v[u].x * v[u].x + v[u].y * v[u].y + v[u].z * v[u].z + v[u].w * v[u].w;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+              for (int u = 0; u < 4; ++u) sq[u] += __shfl_xor_sync(0xffffffffu, sq[u], o);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (l0 + u * kEpiWarps < n_own) finish(l0 + u * kEpiWarps, n0, v[u], sq[u]);
+          }
+        }
+      }
+      continue;
+    }
     // a warp per (token row, tile or pair of tiles): 4 neighbouring columns, or pairs, per lane; half a warp for rotary pairs
     const int loc0 = EPI == EPI_QKV_ROPE ? 2 * ew + (lane >> 4) : ew, dloc = EPI == EPI_QKV_ROPE ? 2 * kEpiWarps : kEpiWarps;
     int loc = loc0, tl = loc0 >= n_own ? tp : 0;
 #pragma unroll 1
     while (tl < tp) {
-      int nloc = loc + dloc, ntl = tl;
-      if (nloc >= n_own) { nloc = loc0; ntl += pitch; }
-      const float4 c0 = g0;
-      if (EPI == EPI_RESIDUAL) {
-        g0 = h1;
-        int l2 = nloc + dloc, t2 = ntl;
-        if (l2 >= n_own) { l2 = loc0; ++t2; }
-        if (t2 < tp) h1 = residual(l2, t2);
-      }
-      const int m = own0 + loc, tile = wk.t0 + p0 + tl, row = s_row[m], s = row >> 8, v = row & 255;
-      const float rs = s_rs[m];
+      const int lm = own0 + loc, m = row0 + lm, tile = wk.t0 + p0 + tl, row = s_row[lm], s = row >> 11, v = row & 2047;
+      const float rs = s_rs[lm];
       const int idx = (loc * tp + tl) * BM, rope_row = (cf.rope_bytes ? loc : m) * half;
-      loc = nloc; tl = ntl;
+      loc += dloc;
+      if (loc >= n_own) { loc = loc0; tl += pitch; }
       if (row == 0xffff) continue;
-      if (EPI == EPI_RESIDUAL || EPI == EPI_PSEUDO || EPI == EPI_LOGITS) {
+      if (EPI == EPI_PSEUDO || EPI == EPI_LOGITS) {
         const int n0 = tile * BM + lane * 4;
         const float4 sum = mul4(sums(idx + lane * 4), rs);
-        if (EPI == EPI_RESIDUAL) {
-          int xp_row = -1;
-          if (a.xp != nullptr) {
-            if (a.rw.chains) xp_row = v < a.rw.T ? s * a.rw.T + v : -1;
-            else xp_row = v == a.rw.anchor ? s : -1;
-          }
-          store_residual(a, m, xp_row, n0, add4(c0, sum), a.x ? load_bf16x4(a.g + n0) : sum, lane);
-        } else if (EPI == EPI_PSEUDO) {            // output column = (map, column); d is a multiple of 128: one map per tile
+        if (EPI == EPI_PSEUDO) {                   // output column = (map, column); d is a multiple of 128: one map per tile
           const int i = n0 / a.d, o = n0 - i * a.d;
           const float4 r = a.pred_b ? add4(sum, load_bf16x4(a.pred_b + n0)) : sum;
-          store_residual(a, s * a.rw.Ms + a.rw.T + (a.rw.chains ? (a.pseudo0 + i) * a.rw.T + v : a.pseudo0 + i), -1, o, r, load_bf16x4(a.g + o), lane);
+          store_residual(a, s * a.rw.Ms + a.rw.T + (a.rw.chains ? (a.pseudo0 + i) * a.rw.T + v : a.pseudo0 + i), -1, o, r, load_bf16x4(a.g + o), warp_sq(r), lane);
         } else if (n0 < a.N) {                     // EPI_LOGITS
           float *dst = a.logits + (size_t)m * a.N + n0;
           if ((a.N & 3) == 0) {
@@ -699,7 +757,7 @@ struct Plan { TileSched sc; TileCfg cf; int tm, merged, smem; };
 // bytes a cycle), computing, or issuing it, whichever takes longest (measured: 50 at 16 columns, 55 at 80, 72 at 144)
 float mma_clk(int n) { return std::max(50.f, std::max(n / 2.f, 34.f + n / 4.f)); }
 
-Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes) {
+Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int planes) {
   Plan best{};
   float best_cost = 1e30f;
   TileSched s{};
@@ -707,6 +765,13 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes)
   s.heads = s.mode == ROWS_ROTARY ? BM / dh : 0;
   s.n_tiles = s.mode == ROWS_GATE_UP ? 2 * ((F + BM - 1) / BM) : (N + BM - 1) / BM;
   s.KB = (K + BK - 1) / BK;
+  const int adds_wanted = epi == EPI_RESIDUAL ? std::max(176, (rows > kMaxTreeRows ? 1 : 2) * s.KB) : (epi == EPI_SWIGLU ? 260 : epi == EPI_LOGITS ? 512 : 176) * std::max(64, s.KB) / 64;
+  for (int max_adds = adds_wanted; best.tm == 0 && max_adds < (1 << 20); max_adds *= 2)
+  for (int most : {256, 192, 128}) {         // token rows of a block: blocks of equal size
+  s.blocks = (rows + most - 1) / most;
+  const int R = align_n((rows + s.blocks - 1) / s.blocks, s.blocks > 1 ? 16 : 1);
+  s.blocks = (rows + R - 1) / R;
+  if (most < 256 && rows <= kMaxTreeRows) break;
   for (int merged = 1; merged >= 0; --merged) {
     if (!merged && planes == 1) continue;
     const int npad = merged ? align_n(R, planes == 2 ? 8 : 16) : align_n(R, 16);
@@ -720,7 +785,7 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes)
       for (int split = 1; split <= 8 && split <= s.KB; ++split) {
         const int cap = cluster_ctas(split) / split * split;
         int jobs = (s.n_tiles + tm - 1) / tm;
-        const int waves = (jobs * split + cap - 1) / cap, kb = (s.KB + split - 1) / split;
+        const int waves = (jobs * s.blocks * split + cap - 1) / cap, kb = (s.KB + split - 1) / split;
         const int per = std::min(tm, s.n_tiles);
         // rings: four activation stages (two or three of the wide ones), the rest for weight tiles
         // and, when it is not much, room for the sums over the k slices (saves a cluster barrier) or the rotary table (an L2
@@ -734,37 +799,45 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes)
         int sx = std::min(x_stage <= 12 * 1024 ? 4 : x_stage <= 24 * 1024 ? 3 : 2, std::max(kb, 1));
         const bool by_unit = tm == 1 && 2 * n_mma + over <= 512 && s.KB / split >= 2;
         if (by_unit) sx = std::max(2, sx & ~1);
-        int sw = std::min(std::min(kMaxStages, (avail - sx * x_stage) / W_TILE), kb * per);
+        int sw = std::min(std::min(kMaxW, (avail - sx * x_stage) / W_TILE), kb * per);
         if (by_unit) sw &= ~1; else sw = sw / per * per;
         if (sw < per || sw * W_TILE + sx * x_stage > avail) continue;
-        if (x_stage <= 24 * 1024) sx = std::min(std::min(6, kb), (avail - sw * W_TILE) / x_stage);      // what is left
+        if (x_stage <= 24 * 1024) sx = std::min(std::min(kMaxX, kb), (avail - sw * W_TILE) / x_stage);      // what is left
         if (by_unit) sx &= ~1;
         if (sw < 2 * per && kb > 1) continue;
+        // The tensor core truncates where it adds to an accumulator, so the error of a sum grows with the additions in a row
+        // (measured on the cache rows of a 1999-token prompt against fp64: 1.1e-4, 1.5e-4 and 2.1e-4 in the 2-norm after
+        // 168, 256 and 512 of them).  As many accumulator sets as fit, up to four, share the k blocks, and what is still
+        // longer than the limit is left to a split.
+        int sets = by_unit ? 2 : 1;
+        const int per_kb = (BK / 16) * (merged ? 1 : planes);
+        while (sets < (rows > kMaxTreeRows ? 4 : 2) && (kb + sets - 1) / sets * per_kb > 96 && 2 * sets * tm * n_mma + over <= 512 && s.KB / split >= 2 * sets) sets *= 2;
+        const int adds = (kb + sets - 1) / sets * per_kb;
+        if (adds > max_adds) continue;
         // microseconds: the weights at the rate HBM gives that many CTAs (6.8 TB/s from 84 on); a CTA's MMAs; its bytes from
         // L2, which gives a CTA 150 GB/s and all of them 15 TB/s; the epilogue's two passes (35 rows: 0.8 + 1.1 us, 131
         // rows: 3.2 + 3.0 us after the O projection; from registers 2.3 and 7 us for a gate and up pair) and barriers
-        const int ctas = std::min(jobs * split, cap), own = std::min(tpo, R);
+        const int ctas = std::min(jobs * s.blocks * split, cap), own = std::min(tpo, R);
         const float hbm = (float)s.n_tiles * s.KB * W_TILE / 6.8e6f * std::max(1.f, 84.f / ctas);
         const float mma = (float)waves * per * kb * 4.f * (merged ? 1 : planes) * mma_clk(n_mma) / 1850.f;
         const float ingest = (float)waves * kb * (per * W_TILE + x_stage) / std::min(150e3f, 15e6f / ctas);
         const bool direct = split == 1 && (epi == EPI_QKV_ROPE || epi == EPI_SWIGLU || epi == EPI_LOGITS);
-        const float out = direct ? 0.5f + 0.025f * R * per : 0.025f * R * per + 0.09f * own * per + (split == 1 ? 0.5f : red ? 1.f : 2.f);
+        const float out = direct ? 0.5f + 0.025f * R * per : 0.025f * R * per + 0.05f * own * per + (split == 1 ? 0.5f : red ? 1.f : 2.f);
         // a ring slot goes round in 0.9 us (activations) or 1.4 us (weights)
         const float rings_us = (float)waves * kb * std::max(0.9f / sx, 1.4f * per / sw);
         const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.1f * (hbm + mma + ingest) + waves * (2.f + out);
         TileCfg c{};
-        c.planes = planes; c.npad = npad; c.acc = n_mma; c.sw = sw; c.sx = sx;
+        c.planes = planes; c.rpb = R; c.npad = npad; c.acc = n_mma; c.sw = sw; c.sx = sx;
         c.tpo = tpo; c.inv_tpo = (65536 + c.tpo - 1) / c.tpo;
-        c.planes_side = merged ? planes : 1; c.acc_set = tm * n_mma; c.sets = 1; c.issuers = 1;
-        if (by_unit) c.sets = c.issuers = 2;
-        else if (tm >= 2) { c.issuers = 2; c.by_tile = 1; }
+        c.planes_side = merged ? planes : 1; c.acc_set = tm * n_mma; c.sets = sets; c.issuers = by_unit || tm >= 2 ? 2 : 1; c.by_tile = tm >= 2;
         c.idesc = instr_desc_m128(n_mma); c.tmem_cols = pow2_cols(c.sets * tm * n_mma + over);
         const int rings = align_n(sw * W_TILE + sx * x_stage, 128);
         if (red) {
           c.red_off = rings; c.tp = per; c.tail = rings + red;
         } else {
-          c.tail = align_n(std::max(rings, per_tile * (s.mode == ROWS_GATE_UP ? 2 : 1)), 128);      // gate and up tiles go together
-          c.tp = std::min(per, c.tail / per_tile);
+          // over the rings; gate and up tiles go together
+          c.tail = align_n(std::max(rings, direct ? 0 : per_tile * (s.mode == ROWS_GATE_UP ? 2 : 1)), 128);
+          c.tp = direct ? per : std::min(per, c.tail / per_tile);
         }
         if (rope) { c.rope_off = c.tail; c.rope_bytes = rope; c.tail += rope; }
         const int smem = c.tail + 1024 + kTailBytes;
@@ -774,6 +847,7 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes)
         best.sc.jobs = jobs; best.sc.split = split;
       }
     }
+  }
   }
   return best;
 }
@@ -798,7 +872,7 @@ bool gemm_tc_available() { return encode_fn() != nullptr; }
 cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream_t st) {
   if (!encode_fn()) return cudaErrorNotSupported;
   Plan p = cached_plan(epi, a.N, a.K, a.F, a.dh, a.R, a.planes);
-  if (p.tm == 0 || p.smem > kSmemMax || p.cf.tp < 1 || p.cf.sw < 1 || p.cf.sx < 1 || (p.cf.sets == 2 && ((p.cf.sw | p.cf.sx) & 1)))
+  if (p.tm == 0 || p.smem > kSmemMax || p.cf.tp < 1 || p.cf.sw < 1 || p.cf.sx < 1 || (!p.cf.by_tile && p.cf.issuers == 2 && ((p.cf.sw | p.cf.sx | p.cf.sets) & 1)))
     return cudaErrorInvalidConfiguration;
   p.cf.pdl = pdl ? 1 : 0;
   KernelFn fn = kernel_of(epi, p.tm, p.merged != 0);
@@ -816,7 +890,7 @@ cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream
   if (!weight_map(&tmW, epi, a.W, (uint64_t)a.N, (uint64_t)a.K, (uint64_t)a.F, (uint64_t)a.dh)) return cudaErrorInvalidValue;
   if (!plane_map(&tmX, a.X, (uint64_t)a.planes, (uint64_t)a.plane_rows, (uint64_t)a.K, (uint32_t)p.cf.npad)) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(p.sc.jobs * p.sc.split));
+  cfg.gridDim = dim3((unsigned)(p.sc.jobs * p.sc.blocks * p.sc.split));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = st;

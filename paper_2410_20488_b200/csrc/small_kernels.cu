@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl)
   const int r = blockIdx.x, s = r / rw.Ms, v = r - s * rw.Ms, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (a.zero_word && r == 0 && tid == 0) *a.zero_word = 0u;
   const int n = a.ctx_len[a.seq_ids[s]];
-  for (int u = tid; u <= v; u += kPrepThreads) {
+  for (int u = tid; u <= v && !rw.prompt; u += kPrepThreads) {
     int p;
     if (u < rw.T) p = a.parents[s * a.parents_stride + u];
     else if (rw.chains) p = u - rw.T;   // step 1 of node w (row T + w) hangs off w, step i off step i-1 of the same node
@@ -31,7 +31,9 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl)
     ext[u] = p;
   }
   __syncthreads();
-  if (tid == kPrepThreads - 1) {        // the last warp: the rotary table below is the first ones'
+  if (rw.prompt) {                      // a chain: the row index is the depth, and says who sees whom
+    if (tid == 0) { s_depth = v; a.meta.pos[r] = n + v; }
+  } else if (tid == kPrepThreads - 1) { // the last warp: the rotary table below is the first ones'
     uint32_t bits[kMaskWords];
 #pragma unroll
     for (int w = 0; w < kMaskWords; ++w) bits[w] = 0u;
@@ -58,7 +60,10 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl)
     const int tok = min(max(a.tokens[s * rw.T + v], 0), a.vocab - 1);
     const int xp_row = a.xp == nullptr ? -1 : rw.chains ? s * rw.T + v : v == rw.anchor ? s : -1;
     for (int c = warp * 128 + lane * 4; c < a.d; c += kPrepThreads * 4)
-      store_residual(a, r, xp_row, c, load_bf16x4(a.embed + (size_t)tok * a.d + c), a.x ? load_bf16x4(a.g + c) : make_float4(0.f, 0.f, 0.f, 0.f), lane);
+    {
+      const float4 e = load_bf16x4(a.embed + (size_t)tok * a.d + c);
+      store_residual(a, r, xp_row, c, e, a.x ? load_bf16x4(a.g + c) : e, warp_sq(e), lane);
+    }
   }
   __syncthreads();
   const int half = a.dh / 2;

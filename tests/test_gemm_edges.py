@@ -1,0 +1,42 @@
+"""The GEMMs with their fused epilogues, and prompts that run in one stretch, at the sizes where a tile, a block of token rows
+or a stretch ends: lock-step against the oracle (prefill logits, cache rows, two steps; the bounds are the harness's own)."""
+import pytest
+
+import synth_inputs as si
+from lockstep import lockstep_run
+
+pytestmark = pytest.mark.gpu
+
+SMALL = si.scaled(si.CONFIGS["c1"], d=256, H=2, Hkv=2, dh=128, F=512)
+
+
+def _run(shape, P, steps=2, max_tree=8, forced_steps=(), masked=False):
+    import oracle
+    from paper_2410_20488_b200 import FirpEngine
+    weights = si.all_weights(shape, gains=True)
+    parents = si.tree_template(8)
+    max_ctx = (P + 64 + 63) // 64 * 64
+    eng = FirpEngine(shape, weights, max_ctx=max_ctx, max_tree=max_tree)
+    orc = oracle.Oracle(shape, weights, max_ctx=max_ctx, masked=masked)
+    if masked:
+        eng.set_pseudo_masked(True)
+    lockstep_run(eng, orc, shape, parents, si.prompt(shape, length=P), steps, forced_steps=forced_steps)
+    eng.close()
+
+
+# 144 rows: what a step may have; 256: a block of token rows; 2047 rows: a stretch (3 of them pseudo rows)
+@pytest.mark.parametrize("P", [1, 15, 125, 141, 142, 145, 253, 254, 257, 500, 1021, 2044, 2045, 2100])
+def test_prompt_lengths(P):
+    _run(SMALL, P, forced_steps=(1,))
+
+
+@pytest.mark.parametrize("l", [0, 1])
+def test_prompt_with_masked_pseudo_rows(l):
+    _run(si.scaled(SMALL, l=l), 300, masked=True)
+
+
+# rows of the matrices that end inside a tile: odd vocabularies, FFN widths, head counts
+@pytest.mark.parametrize("kw", [dict(d=384, H=3, Hkv=1, dh=128, F=1000, V=1001), dict(d=128, H=1, Hkv=1, dh=128, F=8, V=9),
+                                dict(d=384, H=5, Hkv=1, dh=64, F=136, V=2050), dict(d=1152, H=9, Hkv=3, dh=128, F=1544, V=1031)])
+def test_ragged_matrices(kw):
+    _run(si.scaled(si.CONFIGS["c1"], **kw), 200)

@@ -1,7 +1,7 @@
 // Tree-masked split-KV decode attention on the tcgen05 tensor cores (Section 3.4 "Tree attention"; Section 3.3
-// for the pseudo rows), head dimension 128.
+// for the pseudo rows), head dimension 128.  Two kernels: few query rows (this text), and many (below).
 //
-// Roles are swapped as in the GEMMs: a tile of 128 cached positions is the MMA's M dimension, the query rows of
+// Few: roles are swapped as in the GEMMs: a tile of 128 cached positions is the MMA's M dimension, the query rows of
 // the block (tree rows x heads of the group, <= 48) its N dimension.
 //   S^T = K Q^T      K tile [128 pos][128 dh] K-major (TMA, 128-byte swizzle), Q [NQ][128] K-major (hi and lo
 //                    bf16 planes, both accumulated into the same fp32 columns)           -> NQ TMEM columns
@@ -21,8 +21,10 @@
 #include <cooperative_groups.h>
 
 #include <map>
+#include <mutex>
 #include <tuple>
 
+#include "finish_device.cuh"
 #include "firp_kernels.cuh"
 #include "launch_util.cuh"
 #include "tc_device.cuh"
@@ -124,8 +126,7 @@ __device__ unsigned long long g_attn_trace[16];
 #define TC_STAMP(k) do { } while (0)
 #endif
 
-// PROMPT: the rows are a stretch of a prompt, each sees the rows up to itself (no masks in memory)
-template <int NQ, bool PROMPT>
+template <int NQ>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnArgs a,
                     int qper, int pdl) {
@@ -174,8 +175,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
   const int kvh = blockIdx.y, G = a.H / a.Hkv;
   const int qblocks = gridDim.z / a.rw.n_seq;
-  // a prompt's later blocks see more of it: the longest go first
-  const int s = blockIdx.z / qblocks, qb = PROMPT ? qblocks - 1 - (int)blockIdx.z : blockIdx.z % qblocks;
+  const int s = blockIdx.z / qblocks, qb = blockIdx.z % qblocks;
   const int split = blockIdx.x, nsplits = gridDim.x;
   const int qrows_total = a.rows_active * G, q0 = qb * qper;
   const int ncols = min(qper, qrows_total - q0);
@@ -200,7 +200,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   if (warp == 18 && lane < 2) s_sn[lane] = lane == 0 ? __ldcg(a.seq_ids + s) : __ldcg(a.pos + s * a.rw.Ms);
   __syncthreads();
   const int slot = s_sn[0], n = s_sn[1];
-  const int kv_len = min(n + (PROMPT ? (q0 + ncols - 1) / G + 1 : a.rows_active), a.max_ctx);
+  const int kv_len = min(n + a.rows_active, a.max_ctx);
   const int tiles_total = (kv_len + kTcTile - 1) / kTcTile;
   const int t0 = (split * tiles_total + nsplits - 1) / nsplits, t1 = ((split + 1) * tiles_total + nsplits - 1) / nsplits;
   const int ntiles = t1 - t0;                       // tile t0 + i goes to warpgroup i & 1 as its (i >> 1)-th
@@ -317,13 +317,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       if (pvalid && p >= n) {
         const int u = p - n, mw = u >> 5, b = u & 31;
         vis = 0u;
-        if (PROMPT) {
-#pragma unroll
-          for (int jj = 0; jj < NH; ++jj) {
-            const int v = (q0 + c_lo + jj) / G;      // row v sees the rows up to itself ("Masked": no other pseudo row)
-            vis |= (uint32_t)(u <= v && (!a.rw.masked || u < a.rw.T || u == v)) << jj;
-          }
-        } else
 #pragma unroll
         for (int jj = 0; jj < NH; ++jj) {
           const int qr = min(q0 + c_lo + jj, qrows_total - 1);
@@ -506,6 +499,404 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   TC_STAMP(14);
 }
 
+// ---------------------------------------------------------------------------
+// Many query rows: the rows are the MMA's M dimension (up to 128 of them per block, one TMEM lane each), the 128 positions of a
+// tile its N dimension.
+//   S = Q K^T        Q [128 rows][128] K-major (hi and lo planes), K tile as the K-major B operand        -> 128 TMEM columns
+//   softmax          thread = row: maximum and sum without any exchange; P = 2^(s - m) as bf16 (hi, lo) over the scores it came
+//                    from, 16 positions in 8 + 8 columns
+//   O = P V          P from TMEM, V tile as the MN-major B operand                                        -> 128 TMEM columns
+// Two softmax warpgroups take the tiles in turn and hand the running maximum on, row by row; two output warpgroups keep half
+// the columns of O each in registers, O <- O 2^(old max - new max) + O(tile), so that no accumulator sees more than the 16
+// additions of one tile.  S of up to three tiles is in flight.  S and O have an issuer each: one warp issues an MMA every
+// 80-110 cycles beside the softmax warps of its scheduler, the MMA itself takes 66.
+// The contraction costs the same for 1 row and for 128 (a tile of the other kernel 2.2 us per 48 rows, of this one 2.5 us), and
+// the exponentials, 3300-5500 cycles per tile and warpgroup, bound it.  Measured, us per launch, the other kernel / this one:
+// 131 rows at 2047 cached tokens of the 7B shape 50 / 34, four requests of 35 rows x 8 heads per cache head at up to 4096 84 /
+// 61, a 1999-token prompt 324 / 157, 35 rows at 8192 46 / 60.
+// ---------------------------------------------------------------------------
+constexpr int kRowM = 128;                       // query rows of a block (MMA M = TMEM lanes)
+constexpr int kRowThreads = 4 * kTcWg + 128;     // two softmax and two output warpgroups, two MMA issuers, K and V producers
+constexpr int kRowSmem = 6 * kTcStage + 1024;    // Q (hi, lo), two K and two V tiles, + alignment
+constexpr int kRowMaxPart = kRowM + kAttnMaxSplits;
+
+// Operand descriptors as (low, high) words: only the start address, in the low one, moves.
+__device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+               ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+               ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t *u) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+               ::"r"(taddr), "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]), "r"(u[8]),
+                 "r"(u[9]), "r"(u[10]), "r"(u[11]), "r"(u[12]), "r"(u[13]), "r"(u[14]), "r"(u[15]) : "memory");
+}
+__device__ __forceinline__ void tc_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster4(uint32_t addr, float x, float y, float z, float w) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 256;" ::"r"(id) : "memory"); }
+
+template <bool PROMPT>
+__global__ void __launch_bounds__(kRowThreads, 1)
+tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnArgs a,
+                      int qper, int pdl) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ float s_m[kRowM];                      // running max of each row (log2 units)
+  __shared__ float s_corr[4][kRowM];                // 2^(old max - new max) of the last four tiles
+  __shared__ float s_l[2][kRowM], s_ml[2][kRowM];   // each softmax warpgroup's sum of P, and the max it is relative to
+  __shared__ float s_pm[kRowMaxPart], s_pl[kRowMaxPart];    // (max, sum) received for the merge: [split][row]
+  __shared__ uint32_t s_oidx[kRowM];                // element offset of each row's output
+  // mbarriers: K landed [2], V landed [2], O complete [2], S complete [3], P written [3], O read, Q written.  A barrier's next
+  // phase never completes before all who wait for this one have seen it: S(i + 3) is issued after O(i) is complete, K(i + 2)
+  // is loaded after S(i) is, O(i + 1) is issued after O(i) has been read.
+  __shared__ __align__(8) uint64_t s_bar[14];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_sn[2];
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint8_t *base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t sb = smem_u32(base);
+  constexpr int K_OFF = 0, V_OFF = 2 * kTcStage, Q_OFF = 4 * kTcStage;       // Q: [2 planes][2 dh halves][128 rows][128 B]
+  const uint32_t bar0 = smem_u32(s_bar);
+  const uint32_t full_k = bar0, full_v = bar0 + 16, o_ready = bar0 + 32, s_ready = bar0 + 48, p_ready = bar0 + 72, o_free = bar0 + 96,
+                 q_ready = bar0 + 104;
+  if (tid == 0) {
+    for (int i = 0; i < 9; ++i) mbar_init(bar0 + 8 * i, 1);
+    for (int i = 0; i < 3; ++i) mbar_init(p_ready + 8 * i, kTcWg);
+    mbar_init(o_free, 2 * kTcWg); mbar_init(q_ready, 4 * kTcWg);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 16) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem;                     // columns: S / P of tiles i % 3 at 128 (i % 3), O at 384
+  if (pdl) { griddep_launch(); griddep_wait(); }
+
+  const int kvh = blockIdx.y, G = a.H / a.Hkv;
+  const int qblocks = gridDim.z / a.rw.n_seq;
+  // a prompt's later blocks see more of it: the longest go first
+  const int s = blockIdx.z / qblocks, qb = PROMPT ? qblocks - 1 - (int)blockIdx.z : blockIdx.z % qblocks;
+  const int split = blockIdx.x, nsp = gridDim.x;
+  const int qrows_total = a.rows_active * G, q0 = qb * qper;
+  const int ncols = min(qper, qrows_total - q0);
+  if (warp == 18 && lane < 2) s_sn[lane] = lane == 0 ? __ldcg(a.seq_ids + s) : __ldcg(a.pos + s * a.rw.Ms);
+  // the queries of this block: row j = query row q0 + j -> (tree row (q0 + j) / G, head kvh G + (q0 + j) % G).  Rows beyond
+  // ncols hold anything: they only feed their own lanes of S and O, which nothing reads.
+  if (warp < 16) {
+    for (int j = tid >> 4; j < ncols; j += 32) {
+      const int c = tid & 15, qr = q0 + j;
+      const bf16 *src = a.q + ((size_t)(s * a.rw.Ms + qr / G) * a.H + kvh * G + qr % G) * kTcDh + c * 8;
+      const uint4 qh = *reinterpret_cast<const uint4 *>(src), ql = *reinterpret_cast<const uint4 *>(src + a.q_lo_off);
+      const int off = Q_OFF + (c >> 3) * kTcSlab + j * 128 + (((c & 7) ^ (j & 7)) << 4);
+      *reinterpret_cast<uint4 *>(base + off) = qh;
+      *reinterpret_cast<uint4 *>(base + off + kTcStage) = ql;
+    }
+    fence_async_smem();
+    mbar_arrive(q_ready);
+    if (tid < kRowM) {
+      s_m[tid] = -INFINITY;
+      if (tid < ncols) {
+        const int qr = q0 + tid;
+        s_oidx[tid] = (uint32_t)(((s * a.rw.Ms + qr / G) * a.H + kvh * G + qr % G) * kTcDh);
+      }
+    }
+  }
+  __syncthreads();
+  const int slot = s_sn[0], n = s_sn[1];
+  const int kv_len = min(n + (PROMPT ? (q0 + ncols - 1) / G + 1 : a.rows_active), a.max_ctx);
+  const int tiles_total = (kv_len + kTcTile - 1) / kTcTile;
+  const int t0 = (split * tiles_total + nsp - 1) / nsp, t1 = ((split + 1) * tiles_total + nsp - 1) / nsp;
+  const int ntiles = t1 - t0;                       // tile t0 + i goes to softmax warpgroup i & 1
+  const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kDefaultWaitNs;
+  bool dead = false;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), per = (ncols + nsp - 1) / nsp;
+  // The merge: o = sum_p 2^(m_p - M) O_p / sum_p 2^(m_p - M) l_p over the kv splits p.  CTA r of the cluster finalises the rows
+  // [r per, (r + 1) per): once every CTA has left its tile loop (its buffers are free), the output threads push their rows
+  // into the owners' shared memory (16-byte remote stores, chunks permuted by row against bank conflicts), (m, l) likewise;
+  // after a second barrier the owners add up what they received, in split order, a warp per row.  A lone CTA takes the
+  // same route through its own shared memory.
+  float4 *sM = reinterpret_cast<float4 *>(base + K_OFF);         // [splits][per][32 chunks of 4 columns], over the K and V buffers
+  const int row = tid & 127;                        // of a softmax or output thread: its row (TMEM lane)
+  const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+
+  if (warp >= 18) {
+    // ---- producers (one lane each): K and V buffers, free again when the MMAs that read them have completed
+    if (lane == 0) {
+      const bool is_v = warp == 19;
+      const CUtensorMap *tm = is_v ? &tmV : &tmK;
+      const uint32_t full = is_v ? full_v : full_k;
+      const uint32_t dst0 = sb + (is_v ? V_OFF : K_OFF);
+      uint64_t pol;
+      asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+      for (int i = 0; i < ntiles; ++i) {
+        const int w = i & 1, q = i >> 1, t = t0 + i;
+        if (q > 0) {
+          if (is_v) mbar_wait(o_ready + 8 * w, (q - 1) & 1, a.err, dead, wait_ns);
+          else mbar_wait(s_ready + 8 * ((i - 2) % 3), ((i - 2) / 3) & 1, a.err, dead, wait_ns);
+        }
+        mbar_expect_tx(full + 8 * w, kTcStage);
+#pragma unroll
+        for (int ph = 0; ph < 2; ++ph) {            // 64-position x 64-element boxes; a half lies inside one page
+          const int p0 = t * kTcTile + ph * 64;
+          const int src = (int)kv_row(a.pages, slot, p0 < kv_len ? p0 : 0, a.max_ctx);   // a half beyond the context: any rows
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            tma_load_2d(dst0 + (uint32_t)(w * kTcStage + h * kTcSlab + ph * 8192), tm, kvh * kTcDh + h * 64, src, full + 8 * w, pol);
+        }
+      }
+      // no copy is in flight when the CTA ends, even after a wait that ran out
+      dead = false;
+      for (int i = max(0, ntiles - 2); i < ntiles; ++i) mbar_wait(full + 8 * (i & 1), (i >> 1) & 1, a.err, dead, wait_ns);
+    }
+  } else if (warp == 16) {
+    // ---- MMA issuer of S, up to three tiles ahead of O
+    const uint64_t kdesc = smem_desc(sb + K_OFF), qdesc = smem_desc(sb + Q_OFF);
+    const uint32_t q_lo = (uint32_t)qdesc, hi = (uint32_t)(kdesc >> 32);
+    mbar_wait(q_ready, 0, a.err, dead, wait_ns);
+    int b3 = 0;                                     // i % 3
+    for (int i = 0; i < ntiles; ++i) {
+      const int w = i & 1;
+      const uint32_t k_lo = (uint32_t)kdesc + (uint32_t)(w * (kTcStage >> 4)), col = tmem + b3 * 128;
+      mbar_wait(full_k + 8 * w, (i >> 1) & 1, a.err, dead, wait_ns);
+      if (i >= 3) mbar_wait(o_ready + 8 * ((i - 3) & 1), ((i - 3) >> 1) & 1, a.err, dead, wait_ns);   // its P, in the same columns, has been read
+      tc_fence_after();
+#pragma unroll
+      for (int pl = 0; pl < 2; ++pl)
+        if (pl < a.q_planes) {
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk) {
+            const uint32_t off = (uint32_t)(((kk >> 2) * kTcSlab + (kk & 3) * 32) >> 4);
+            if (elect_one()) tc_mma_ss(col, q_lo + (uint32_t)((pl * kTcStage) >> 4) + off, k_lo + off, hi, instr_desc_m128(128), (pl | kk) != 0);
+          }
+        }
+      if (elect_one()) tc_commit(s_ready + 8 * b3);
+      b3 = b3 == 2 ? 0 : b3 + 1;
+    }
+  } else if (warp == 17) {
+    // ---- MMA issuer of O
+    const uint64_t vdesc = smem_desc_mn(sb + V_OFF, kTcSlab);
+    const uint32_t hi = (uint32_t)(vdesc >> 32);
+    int b3 = 0, ph3 = 0;                            // i % 3, i / 3
+    for (int i = 0; i < ntiles; ++i) {
+      const int w = i & 1;
+      const uint32_t v_lo = (uint32_t)vdesc + (uint32_t)(w * (kTcStage >> 4)), pcol = tmem + b3 * 128;
+      mbar_wait(full_v + 8 * w, (i >> 1) & 1, a.err, dead, wait_ns);
+      if (i >= 1) mbar_wait(o_free, (i - 1) & 1, a.err, dead, wait_ns);          // O of the tile before has been read
+      mbar_wait(p_ready + 8 * b3, ph3 & 1, a.err, dead, wait_ns);
+      tc_fence_after();
+#pragma unroll
+      for (int pl = 0; pl < 2; ++pl)
+        if (pl < a.p_planes) {
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)
+            if (elect_one())
+              tc_mma_ts(tmem + 384, pcol + ks * 16 + pl * 8, v_lo + (uint32_t)((ks * 2048) >> 4), hi, instr_desc_m128(128) | (1u << 16), (pl | ks) != 0);
+        }
+      if (elect_one()) tc_commit(o_ready + 8 * w);
+      if (++b3 == 3) { b3 = 0; ++ph3; }
+    }
+  } else if (warp < 8) {
+    // ---- softmax warpgroups: thread = row; g takes tiles g, g + 2, ...
+    const int g = warp >> 2;
+    const float scale_log2 = rsqrtf((float)kTcDh) * 1.4426950408889634f;
+    const int v = min(q0 + row, qrows_total - 1) / G;            // tree row
+    const uint32_t *mrow = PROMPT ? nullptr : a.mask + (size_t)(s * a.rw.Ms + v) * kMaskWords;
+    float m_mine = -INFINITY, l = 0.f;
+    int b3 = g, ph3 = 0;                                         // i % 3, i / 3
+    for (int i = g; i < ntiles; i += 2) {
+      const int q = i >> 1, p0 = (t0 + i) * kTcTile;
+      const bool masked = __any_sync(0xffffffffu, p0 + kTcTile > n);   // some of the tile's positions are not committed ones (a vote: the branches on it stay branches)
+      // visibility of the tile's positions, a bit each: the committed prefix is visible to all, new row u = p - n to the
+      // rows whose mask has bit u
+      uint32_t vis[4];
+      if (masked) {
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const int u0 = p0 + 32 * w - n, left = kv_len - (p0 + 32 * w);
+          uint32_t bits;
+          if (PROMPT) {                                          // row v sees the rows up to itself ("Masked": no other pseudo row)
+            const int ones = v - u0 + 1;
+            bits = ones >= 32 ? ~0u : ones <= 0 ? 0u : (1u << ones) - 1u;
+            if (a.rw.masked && v >= a.rw.T) {
+              const int tree = a.rw.T - u0;
+              const uint32_t tb = tree >= 32 ? ~0u : tree <= 0 ? 0u : (1u << tree) - 1u;
+              const uint32_t self = v >= u0 && v - u0 < 32 ? 1u << (v - u0) : 0u;
+              bits &= tb | self;
+            }
+          } else if (u0 <= -32) {
+            bits = ~0u;
+          } else {
+            const int w0 = u0 >> 5, sh = u0 & 31;                // w0 = -1: all ones
+            const uint32_t lo = w0 < 0 ? ~0u : w0 < kMaskWords ? mrow[w0] : 0u;
+            const uint32_t hi = w0 + 1 < kMaskWords ? mrow[w0 + 1] : 0u;
+            bits = __funnelshift_r(lo, hi, sh);
+          }
+          vis[w] = left >= 32 ? bits : left <= 0 ? 0u : bits & ((1u << left) - 1u);
+        }
+      }
+      if ((warp & 3) == 0) mbar_wait(s_ready + 8 * b3, ph3 & 1, a.err, dead, wait_ns);      // one warp polls: sixteen would slow the MMAs' operand reads
+      __syncwarp();
+      wg_sync(2 + g);
+      tc_fence_after();
+      const uint32_t ts = tlane + b3 * 128;
+      // (the next columns are on their way while these are worked on)
+      float mt = -INFINITY;
+      {
+        float r[2][32];
+        tc_ld16(ts, r[0]); tc_ld16(ts + 16, r[0] + 16);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          float *x = r[c & 1], *y = r[(c + 1) & 1];
+          tc_ld_wait();
+          if (c < 3) { tc_ld16(ts + 32 * (c + 1), y); tc_ld16(ts + 32 * (c + 1) + 16, y + 16); }
+          if (masked) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) x[j] = ((vis[c] >> j) & 1u) ? x[j] : -INFINITY;
+          }
+          float m4[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+          for (int j = 4; j < 32; ++j) m4[j & 3] = fmaxf(m4[j & 3], x[j]);
+          mt = fmaxf(mt, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
+        }
+      }
+      // the running max goes from tile to tile, and so from one warpgroup to the other
+      if (i > 0) pair_sync(1 + (i & 1));
+      const float m_old = s_m[row], m_new = fmaxf(m_old, mt * scale_log2), msafe = m_new == -INFINITY ? 0.f : m_new;
+      s_m[row] = m_new;
+      s_corr[i & 3][row] = exp2f(m_old - msafe);
+      if (i + 1 < ntiles) pair_arrive(1 + ((i + 1) & 1));
+      l *= exp2f(m_mine - msafe);
+      m_mine = m_new;
+      // P = 2^(s - m) as bf16 (hi, lo) over the scores it came from: 16 scores become 8 columns of hi and 8 of lo
+      float sum[4] = {0.f, 0.f, 0.f, 0.f};
+      {
+        float r[2][16];
+        tc_ld16(ts, r[0]);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          float *x = r[c & 1];
+          uint32_t pk[16];
+          tc_ld_wait();
+          if (c < 7) tc_ld16(ts + 16 * (c + 1), r[(c + 1) & 1]);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) x[j] = exp2f(fmaf(x[j], scale_log2, -msafe));
+          if (masked) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) x[j] = ((vis[c >> 1] >> (16 * (c & 1) + j)) & 1u) ? x[j] : 0.f;
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            sum[j & 1] += x[2 * j]; sum[2 + (j & 1)] += x[2 * j + 1];
+            const __nv_bfloat162 hh = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+            const uint32_t h = *reinterpret_cast<const uint32_t *>(&hh);
+            const __nv_bfloat162 ll = __floats2bfloat162_rn(x[2 * j] - __uint_as_float(h << 16), x[2 * j + 1] - __uint_as_float(h & 0xffff0000u));
+            pk[j] = h;
+            pk[8 + j] = *reinterpret_cast<const uint32_t *>(&ll);
+          }
+          tc_st16(ts + 16 * c, pk);
+        }
+      }
+      l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+      tc_st_wait();
+      if (p0 + row >= kv_len) {                                  // a position beyond the context: its V row may hold anything, and 0 x NaN is NaN
+        mbar_wait(full_v + 8 * g, q & 1, a.err, dead, wait_ns);
+        uint4 *v0 = reinterpret_cast<uint4 *>(base + V_OFF + g * kTcStage + row * 128);
+        uint4 *v1 = reinterpret_cast<uint4 *>(base + V_OFF + g * kTcStage + kTcSlab + row * 128);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) { v0[c] = make_uint4(0u, 0u, 0u, 0u); v1[c] = make_uint4(0u, 0u, 0u, 0u); }
+        fence_async_smem();
+      }
+      tc_fence_before();
+      mbar_arrive(p_ready + 8 * b3);
+      if (b3 == 0) b3 = 2; else { --b3; ++ph3; }                 // i + 2
+    }
+    s_l[g][row] = l;                                             // relative to m_mine
+    s_ml[g][row] = m_mine;
+  } else {
+    // ---- output warpgroups: thread = row, 64 of the 128 columns; O of each tile joins the running one
+    float o_acc[64];                                             // O[row][64 dh] of the tiles so far
+#pragma unroll
+    for (int j = 0; j < 64; ++j) o_acc[j] = 0.f;
+    const uint32_t to = tlane + 384 + (warp >= 12 ? 64 : 0);
+    for (int i = 0; i < ntiles; ++i) {
+      if (warp == 8) mbar_wait(o_ready + 8 * (i & 1), (i >> 1) & 1, a.err, dead, wait_ns);
+      __syncwarp();
+      pair_sync(5);
+      tc_fence_after();
+      const float corr = s_corr[i & 3][row];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        float r[8];
+        tc_ld8(to + 8 * c, r);
+        tc_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) o_acc[8 * c + j] = o_acc[8 * c + j] * corr + r[j];
+      }
+      tc_fence_before();
+      mbar_arrive(o_free);
+    }
+    tc_fence_before();
+    cluster.sync();
+    if (row < ncols) {
+      const int owner = row / per, loc = row - owner * per, c0 = warp >= 12 ? 16 : 0;
+      const uint32_t dst = map_rank(sb + K_OFF, (uint32_t)owner) + (uint32_t)((rank * per + loc) * 512);
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        st_cluster4(dst + (uint32_t)(((c0 + c) ^ (loc & 31)) * 16), o_acc[4 * c], o_acc[4 * c + 1], o_acc[4 * c + 2], o_acc[4 * c + 3]);
+      if (c0 == 0) {                                             // a warpgroup's sum is relative to the max of its own last tile
+        const float m = s_m[row], ms = m == -INFINITY ? 0.f : m;
+        cluster.map_shared_rank(s_pm, owner)[rank * per + loc] = m;
+        cluster.map_shared_rank(s_pl, owner)[rank * per + loc] = s_l[0][row] * exp2f(s_ml[0][row] - ms) + s_l[1][row] * exp2f(s_ml[1][row] - ms);
+      }
+    }
+  }
+  if (warp < 8 || warp >= 16) { tc_fence_before(); cluster.sync(); }
+  if (warp == 16) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+  cluster.sync();
+  const int n_own = min(per, ncols - rank * per);
+  for (int loc = warp; loc < n_own; loc += kRowThreads / 32) {
+    float M = -INFINITY;
+    for (int sp = 0; sp < nsp; ++sp) M = fmaxf(M, s_pm[sp * per + loc]);
+    float L = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int sp = 0; sp < nsp; ++sp) {
+      const float pm = s_pm[sp * per + loc], w = pm == -INFINITY ? 0.f : exp2f(pm - M);      // a partial without tiles: weight 0
+      const float4 ov = sM[(size_t)(sp * per + loc) * 32 + (lane ^ (loc & 31))];
+      L += w * s_pl[sp * per + loc];
+      acc.x += w * ov.x; acc.y += w * ov.y; acc.z += w * ov.z; acc.w += w * ov.w;
+    }
+    const float inv = L > 0.f ? 1.f / L : 0.f;
+    const float y[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
+    uint2 hi, lo;
+    split4(y, hi, lo);
+    bf16 *dst = a.o + (size_t)s_oidx[rank * per + loc] + lane * 4;
+    *reinterpret_cast<uint2 *>(dst) = hi;
+    *reinterpret_cast<uint2 *>(dst + a.o_lo_off) = lo;
+  }
+
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -529,6 +920,8 @@ EncodeTiledFn kv_encode_fn() {
 bool kv_map(CUtensorMap *m, const void *plane, uint64_t rows, uint64_t width) {
   typedef std::tuple<const void *, uint64_t, uint64_t> Key;
   static std::map<Key, CUtensorMap> cache;
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
   const Key key(plane, rows, width);
   auto it = cache.find(key);
   if (it != cache.end()) { *m = it->second; return true; }
@@ -546,20 +939,18 @@ bool kv_map(CUtensorMap *m, const void *plane, uint64_t rows, uint64_t width) {
   return true;
 }
 
-template <int NQ, bool PROMPT>
-cudaError_t launch_nq(const CUtensorMap &tmK, const CUtensorMap &tmV, const AttnArgs &a, int qblocks, int qper, bool pdl,
-                      cudaStream_t st) {
-  constexpr int SMEM = TcLayout<NQ>::BYTES + 1024;      // + what aligning the base to 1024 bytes may take
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_tc_kernel<NQ, PROMPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+typedef void (*AttnFn)(const CUtensorMap, const CUtensorMap, AttnArgs, int, int);
+cudaError_t launch_attn(AttnFn fn, bool *configured, int threads, int smem, const CUtensorMap &tmK, const CUtensorMap &tmV, const AttnArgs &a,
+                        bool pdl, cudaStream_t st) {
+  if (!*configured) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    configured = true;
+    *configured = true;
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(a.splits, a.Hkv, a.rw.n_seq * qblocks);
-  cfg.blockDim = dim3(kTcThreads);
-  cfg.dynamicSmemBytes = SMEM;
+  cfg.gridDim = dim3(a.splits, a.Hkv, a.rw.n_seq * a.tc.qblocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -568,7 +959,17 @@ cudaError_t launch_nq(const CUtensorMap &tmK, const CUtensorMap &tmV, const Attn
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel<NQ, PROMPT>, tmK, tmV, a, qper, pdl ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, fn, tmK, tmV, a, a.tc.qper, pdl ? 1 : 0);
+}
+template <int NQ>
+cudaError_t launch_nq(const CUtensorMap &tmK, const CUtensorMap &tmV, const AttnArgs &a, bool pdl, cudaStream_t st) {
+  static bool configured = false;
+  return launch_attn(tree_attn_tc_kernel<NQ>, &configured, kTcThreads, TcLayout<NQ>::BYTES + 1024, tmK, tmV, a, pdl, st);   // + alignment of the base
+}
+template <bool PROMPT>
+cudaError_t launch_rows(const CUtensorMap &tmK, const CUtensorMap &tmV, const AttnArgs &a, bool pdl, cudaStream_t st) {
+  static bool configured = false;
+  return launch_attn(tree_attn_rows_kernel<PROMPT>, &configured, kRowThreads, kRowSmem, tmK, tmV, a, pdl, st);
 }
 
 }  // namespace
@@ -579,40 +980,37 @@ extern "C" int firp_debug_attn_trace(unsigned long long *out) {
 }
 #endif
 
-void attention_tc_blocks(int qrows, int *qblocks, int *qper) {
-  *qblocks = (qrows + kAttnTcMaxCols - 1) / kAttnTcMaxCols;
-  *qper = (qrows + *qblocks - 1) / *qblocks;
-}
-
-int attention_tc_splits(int groups, int kv_tiles, int sm_count) {
-  // one CTA per SM, two tiles in flight per CTA (one per tile group): rounds x (the longest split's tiles per tile
-  // group at ~2.8 us each + the fixed cost of a CTA, + the cluster barriers when there is more than one split)
-  int best = 1;
+// More than 48 query rows share a block of 128 once the context has more than 6 tiles; a prompt always does.  Measured at the
+// 7B / 13B shapes, us per step with blocks of 48 / of 128: 128 rows over 5 tiles 4820 / 4850, 67 rows over 9 tiles 6490 / 6390,
+// 131 rows over 18 tiles 6190 / 5850.
+// Splits: one CTA per SM.  Rounds x (the tiles of the longest split at 2.5 us each, or 2.8 us per pair of them, one per tile
+// group, + the fixed cost of a CTA, + the cluster barriers when there is more than one split).
+AttnTcPlan attention_tc_plan(int qrows, int seq_heads, int kv_tiles, bool prompt, int sm_count) {
+  AttnTcPlan p{};
+  p.rows = prompt || (qrows > kAttnTcMaxCols && kv_tiles > 6);
+  const int most = p.rows ? kRowM : kAttnTcMaxCols;
+  p.qblocks = (qrows + most - 1) / most;
+  p.qper = (qrows + p.qblocks - 1) / p.qblocks;
+  p.splits = 1;
   float best_cost = 1e30f;
   for (int s = 1; s <= kAttnMaxSplits && s <= (kv_tiles > 0 ? kv_tiles : 1); ++s) {
-    const int rounds = (s * groups + sm_count - 1) / sm_count;
+    const int rounds = (s * seq_heads * p.qblocks + sm_count - 1) / sm_count;
     const int per = (kv_tiles + s - 1) / s;
-    const float cost = (float)rounds * (2.8f * (float)((per + 1) / 2) + 8.f + (s > 1 ? 1.5f : 0.f));
-    if (cost < best_cost - 1e-6f) { best_cost = cost; best = s; }
+    const float cost = (float)rounds * ((p.rows ? 2.5f * (float)per : 2.8f * (float)((per + 1) / 2)) + 8.f + (s > 1 ? 1.5f : 0.f));
+    if (cost < best_cost - 1e-6f) { best_cost = cost; p.splits = s; }
   }
-  return best;
+  return p;
 }
 
 cudaError_t launch_attention_tc(const AttnArgs &a, bool pdl, cudaStream_t st) {
   if (a.dh != kTcDh) return cudaErrorInvalidValue;
-  const int G = a.H / a.Hkv;
-  int qblocks, qper;
-  attention_tc_blocks(a.rows_active * G, &qblocks, &qper);
   const uint64_t width = (uint64_t)a.Hkv * kTcDh, rows = a.kv_stride / width;
   CUtensorMap tmK, tmV;
   if (!kv_map(&tmK, a.kcache, rows, width) || !kv_map(&tmV, a.kcache + a.kv_stride, rows, width)) return cudaErrorInvalidValue;
-  if (a.rw.prompt) {
-    if (qper <= 16) return launch_nq<16, true>(tmK, tmV, a, qblocks, qper, pdl, st);
-    return launch_nq<48, true>(tmK, tmV, a, qblocks, qper, pdl, st);
-  }
-  if (qper <= 16) return launch_nq<16, false>(tmK, tmV, a, qblocks, qper, pdl, st);
-  if (qper <= 32) return launch_nq<32, false>(tmK, tmV, a, qblocks, qper, pdl, st);
-  return launch_nq<48, false>(tmK, tmV, a, qblocks, qper, pdl, st);
+  if (a.tc.rows) return a.rw.prompt ? launch_rows<true>(tmK, tmV, a, pdl, st) : launch_rows<false>(tmK, tmV, a, pdl, st);
+  if (a.tc.qper <= 16) return launch_nq<16>(tmK, tmV, a, pdl, st);
+  if (a.tc.qper <= 32) return launch_nq<32>(tmK, tmV, a, pdl, st);
+  return launch_nq<48>(tmK, tmV, a, pdl, st);
 }
 
 }  // namespace firp

@@ -311,12 +311,11 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       a.o = c->o; a.o_lo_off = Rp * nq; a.err = c->dev_status; a.wait_ns = c->wait_ns;
       // Head dimension 128 runs on the tensor-core kernel unless told otherwise.  Measured at the 7B shape, us per step
       // mma.sync / tcgen05: 1 row at 128 cached tokens 2850 / 2724; 35 rows at 512 3441 / 3242, at 8192 6208 / 4185; 131
-      // rows at 2047 6890 / 6810; 6 sequences x 18 rows at 128-1024 6170 / 5130.
+      // rows at 2047 6890 / 5850; 6 sequences x 18 rows at 128-1024 6170 / 5130.
       const bool tc = dh == 128 && c->attn_tc != 0;
       if (tc) {
-        int qb_tc, qper_tc;
-        attention_tc_blocks(act * G, &qb_tc, &qper_tc);
-        a.splits = attention_tc_splits(rw.n_seq * Hkv * qb_tc, (ra.n_hi_max + act + kAttnTcTile - 1) / kAttnTcTile, c->sm_count);
+        a.tc = attention_tc_plan(act * G, rw.n_seq * Hkv, (ra.n_hi_max + act + kAttnTcTile - 1) / kAttnTcTile, rw.prompt, c->sm_count);
+        a.splits = a.tc.splits;
       }
       FIRP_TIMED(KC_ATTENTION);
       FIRP_CUDA(c, tc ? launch_attention_tc(a, pdl, st) : launch_attention(a, pdl, st)); ++nl;

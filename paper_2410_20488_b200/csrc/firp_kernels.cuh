@@ -216,7 +216,10 @@ struct GemmArgs {
 
 // ---- tree-masked split-KV attention ---------------------------------------
 constexpr int kAttnMaxSplits = 8;   // kv splits = CTAs per cluster (portable cluster size limit)
+// Blocks of query rows: `rows`: up to 128 as the MMA's M dimension, else up to 48 as its N; qblocks of qper each.
+struct AttnTcPlan { bool rows; int qblocks, qper, splits; };
 struct AttnArgs {
+  AttnTcPlan tc;
   Rows rw; int rows_active;
   int H, Hkv, dh;
   const bf16 *q; size_t q_lo_off;   // [R][H*dh] rotated queries, hi and lo planes
@@ -226,7 +229,7 @@ struct AttnArgs {
   const int32_t *seq_ids, *ctx_len;
   const int32_t *pos;         // [R] absolute position of every row (row 0 of a sequence: its committed length)
   const uint32_t *mask;       // [R][kMaskWords]
-  int splits;                 // kv splits (grid.x = cluster size): 1, 2, 4 or 8
+  int splits;                 // kv splits (grid.x = cluster size), 1 to kAttnMaxSplits
   int q_planes, p_planes;     // bf16 planes of the queries / of the probabilities that enter the tensor cores: 2 (hi, lo) or 1
   bf16 *o; size_t o_lo_off;   // [R][H*dh] hi plane, lo plane
   int *err; unsigned long long wait_ns;   // status word and bound of the device-side waits (tensor-core kernel; 0: default)
@@ -234,11 +237,10 @@ struct AttnArgs {
 // kv splits for `groups` = sequences x kv heads x query blocks and `kv_tiles` 64-position tiles
 int attention_splits(int groups, int kv_tiles);
 cudaError_t launch_attention(const AttnArgs &a, bool pdl, cudaStream_t st);
-// The tcgen05 kernel (head dimension 128): 128-position tiles, query blocks of at most kAttnTcMaxCols columns
-// (query rows x heads of the group), a.splits from attention_tc_splits.
+// The tcgen05 kernels (head dimension 128): 128-position tiles, query rows x heads of the group in blocks of at most
+// kAttnTcMaxCols or 128; a.tc and a.splits from attention_tc_plan.  seq_heads = sequences x kv heads.
 constexpr int kAttnTcTile = 128, kAttnTcMaxCols = 48;
-void attention_tc_blocks(int qrows, int *qblocks, int *qper);
-int attention_tc_splits(int groups, int kv_tiles, int sm_count);
+AttnTcPlan attention_tc_plan(int qrows, int seq_heads, int kv_tiles, bool prompt, int sm_count);
 cudaError_t launch_attention_tc(const AttnArgs &a, bool pdl, cudaStream_t st);
 
 // ---- the decoder layers of a step as one persistent kernel (fused_step.cu) ------------------------------

@@ -16,7 +16,8 @@
 //
 // A prompt comes as one stretch of up to 2047 rows, in blocks of up to 256: the weights, 13.5 GB at the 7B shape, are read
 // once instead of once per 141 rows.  It is bound by the MMA issue of two passes over the bf16 planes: 1999 tokens of the 7B
-// shape 92.2 -> 65.9 ms; per layer QKV 0.44, attention 0.33, O 0.19, gate/up 0.60, down 0.45 ms.
+// shape 92.2 -> 65.9 ms (61.3 with attn_tc.cu's blocks of 128 rows); per layer QKV 0.44, attention 0.16, O 0.19, gate/up 0.60,
+// down 0.45 ms.
 //
 // Bound now, per layer of 98 us: the weight stream (QKV 15.1, gate/up 27.8, down 13.1 us at 6.7-6.9 TB/s; the O projection
 // 5.5), the epilogues (4 + 2.5 + 2 + 2), five hand-overs of 2 us and the attention's 12.

@@ -1,5 +1,5 @@
-"""The GEMMs with their fused epilogues, and prompts that run in one stretch, at the sizes where a tile, a block of token rows
-or a stretch ends: lock-step against the oracle (prefill logits, cache rows, two steps; the bounds are the harness's own)."""
+"""The GEMMs with their fused epilogues, prompts that run in one stretch, and the attention's blocks of many query rows, at the
+sizes where a tile, a block of rows or a stretch ends: lock-step against the oracle (prefill logits, cache rows, two steps; the bounds are the harness's own)."""
 import pytest
 
 import synth_inputs as si
@@ -10,13 +10,13 @@ pytestmark = pytest.mark.gpu
 SMALL = si.scaled(si.CONFIGS["c1"], d=256, H=2, Hkv=2, dh=128, F=512)
 
 
-def _run(shape, P, steps=2, max_tree=8, forced_steps=(), masked=False):
+def _run(shape, P, steps=2, T=8, forced_steps=(), masked=False):
     import oracle
     from paper_2410_20488_b200 import FirpEngine
     weights = si.all_weights(shape, gains=True)
-    parents = si.tree_template(8)
-    max_ctx = (P + 64 + 63) // 64 * 64
-    eng = FirpEngine(shape, weights, max_ctx=max_ctx, max_tree=max_tree)
+    parents = si.tree_template(T, (4, 4, 8))
+    max_ctx = (P + 8 * T + 63) // 64 * 64
+    eng = FirpEngine(shape, weights, max_ctx=max_ctx, max_tree=T)
     orc = oracle.Oracle(shape, weights, max_ctx=max_ctx, masked=masked)
     if masked:
         eng.set_pseudo_masked(True)
@@ -40,3 +40,10 @@ def test_prompt_with_masked_pseudo_rows(l):
                                 dict(d=384, H=5, Hkv=1, dh=64, F=136, V=2050), dict(d=1152, H=9, Hkv=3, dh=128, F=1544, V=1031)])
 def test_ragged_matrices(kw):
     _run(si.scaled(si.CONFIGS["c1"], **kw), 200)
+
+
+# more than 48 query rows on more than six tiles of context: one block of 128 rows, or several; a lone CTA or a cluster of splits
+@pytest.mark.parametrize("T,H,Hkv,P,masked", [(46, 2, 2, 764, False), (61, 2, 2, 1023, True), (125, 2, 2, 893, False), (126, 2, 1, 1150, False),
+                                              (8, 16, 2, 800, False), (32, 8, 1, 1021, False)])
+def test_many_query_rows(T, H, Hkv, P, masked):
+    _run(si.scaled(SMALL, d=H * 128, H=H, Hkv=Hkv), P, T=T, forced_steps=(1,), masked=masked)

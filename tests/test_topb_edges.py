@@ -18,7 +18,9 @@ def _rows(vocab, rng):
 
 
 @pytest.mark.parametrize("vocab,b", [(1, 8), (7, 8), (8, 8), (9, 3), (512, 8), (513, 8), (4095, 8), (4096, 1), (4097, 8), (32767, 8),
-                                     (32768, 5), (32769, 8), (50257, 5), (130001, 8)])
+                                     (32768, 5), (32769, 8), (50257, 5), (130001, 8),
+                                     (32, 8), (33, 8), (1023, 8), (1028, 8), (8192, 8), (8193, 8), (32772, 8), (65536, 3), (65537, 8), (262144, 8),
+                                     (262149, 8), (524296, 5)])
 def test_topb_edges(vocab, b):
     import torch
     from paper_2410_20488_b200 import firp_topb_static

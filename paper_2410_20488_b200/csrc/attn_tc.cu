@@ -27,6 +27,7 @@
 #include "finish_device.cuh"
 #include "firp_kernels.cuh"
 #include "launch_util.cuh"
+#include "pipeline.h"
 #include "tc_device.cuh"
 
 namespace cg = cooperative_groups;
@@ -558,10 +559,14 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   __shared__ float s_l[2][kRowM], s_ml[2][kRowM];   // each softmax warpgroup's sum of P, and the max it is relative to
   __shared__ float s_pm[kRowMaxPart], s_pl[kRowMaxPart];    // (max, sum) received for the merge: [split][row]
   __shared__ uint32_t s_oidx[kRowM];                // element offset of each row's output
-  // mbarriers: K landed [2], V landed [2], O complete [2], S complete [3], P written [3], O read, Q written.  A barrier's next
-  // phase never completes before all who wait for this one have seen it: S(i + 3) is issued after O(i) is complete, K(i + 2)
-  // is loaded after S(i) is, O(i + 1) is issued after O(i) has been read.
-  __shared__ __align__(8) uint64_t s_bar[14];
+  // mbarriers: K landed [2], V landed [2], O complete [3], S complete [3], P written [3], O read, Q written.  The phase after
+  // the one of tile i, and what its completion needs of those who wait for tile i:
+  //   K, V (i + 2)     loaded by the producer after S(i), O(i): the issuers have seen K(i), V(i)
+  //   S, P, O (i + 3)  need S(i + 3), which its issuer issues after it has seen O(i).  P(i) and O(i) need all of a softmax
+  //                    warpgroup to have seen S(i); O(i + 1) needs the output warps to have seen O(i); the producers of K(i + 2)
+  //                    and V(i + 2) look for S(i) and O(i) before they load what S(i + 2) and O(i + 2) need
+  //   O read (i + 1)   needs O(i + 1), issued after O(i) has been read
+  __shared__ __align__(8) uint64_t s_bar[15];
   __shared__ uint32_t s_tmem;
   __shared__ int s_sn[2];
 
@@ -570,10 +575,10 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   const uint32_t sb = smem_u32(base);
   constexpr int K_OFF = 0, V_OFF = 2 * kTcStage, Q_OFF = 4 * kTcStage;       // Q: [2 planes][2 dh halves][128 rows][128 B]
   const uint32_t bar0 = smem_u32(s_bar);
-  const uint32_t full_k = bar0, full_v = bar0 + 16, o_ready = bar0 + 32, s_ready = bar0 + 48, p_ready = bar0 + 72, o_free = bar0 + 96,
-                 q_ready = bar0 + 104;
+  const uint32_t full_k = bar0, full_v = bar0 + 16, o_ready = bar0 + 32, s_ready = bar0 + 56, p_ready = bar0 + 80, o_free = bar0 + 104,
+                 q_ready = bar0 + 112;
   if (tid == 0) {
-    for (int i = 0; i < 9; ++i) mbar_init(bar0 + 8 * i, 1);
+    for (int i = 0; i < 10; ++i) mbar_init(bar0 + 8 * i, 1);
     for (int i = 0; i < 3; ++i) mbar_init(p_ready + 8 * i, kTcWg);
     mbar_init(o_free, 2 * kTcWg); mbar_init(q_ready, 4 * kTcWg);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -647,10 +652,10 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
       for (int i = 0; i < ntiles; ++i) {
-        const int w = i & 1, q = i >> 1, t = t0 + i;
-        if (q > 0) {
-          if (is_v) mbar_wait(o_ready + 8 * w, (q - 1) & 1, a.err, dead, wait_ns);
-          else mbar_wait(s_ready + 8 * ((i - 2) % 3), ((i - 2) / 3) & 1, a.err, dead, wait_ns);
+        const int w = rows_kv(i).bar, t = t0 + i;
+        if (i >= kRowsKvRing) {                     // S or O of the tile before in this buffer
+          const TilePhase f = rows_spo(i - kRowsKvRing);
+          mbar_wait((is_v ? o_ready : s_ready) + 8 * f.bar, f.parity, a.err, dead, wait_ns);
         }
         mbar_expect_tx(full + 8 * w, kTcStage);
 #pragma unroll
@@ -664,7 +669,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       }
       // no copy is in flight when the CTA ends, even after a wait that ran out
       dead = false;
-      for (int i = max(0, ntiles - 2); i < ntiles; ++i) mbar_wait(full + 8 * (i & 1), (i >> 1) & 1, a.err, dead, wait_ns);
+      for (int i = max(0, ntiles - kRowsKvRing); i < ntiles; ++i) mbar_wait(full + 8 * rows_kv(i).bar, rows_kv(i).parity, a.err, dead, wait_ns);
     }
   } else if (warp == 16) {
     // ---- MMA issuer of S, up to three tiles ahead of O
@@ -676,7 +681,10 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const int w = i & 1;
       const uint32_t k_lo = (uint32_t)kdesc + (uint32_t)(w * (kTcStage >> 4)), col = tmem + b3 * 128;
       mbar_wait(full_k + 8 * w, (i >> 1) & 1, a.err, dead, wait_ns);
-      if (i >= 3) mbar_wait(o_ready + 8 * ((i - 3) & 1), ((i - 3) >> 1) & 1, a.err, dead, wait_ns);   // its P, in the same columns, has been read
+      if (i >= kRowsSpoRing) {                      // its P, in the same columns, has been read
+        const TilePhase f = rows_spo(i - kRowsSpoRing);
+        mbar_wait(o_ready + 8 * f.bar, f.parity, a.err, dead, wait_ns);
+      }
       tc_fence_after();
 #pragma unroll
       for (int pl = 0; pl < 2; ++pl)
@@ -710,7 +718,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             if (elect_one())
               tc_mma_ts(tmem + 384, pcol + ks * 16 + pl * 8, v_lo + (uint32_t)((ks * 2048) >> 4), hi, instr_desc_m128(128) | (1u << 16), (pl | ks) != 0);
         }
-      if (elect_one()) tc_commit(o_ready + 8 * w);
+      if (elect_one()) tc_commit(o_ready + 8 * b3);
       if (++b3 == 3) { b3 = 0; ++ph3; }
     }
   } else if (warp < 8) {
@@ -837,7 +845,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     for (int j = 0; j < 64; ++j) o_acc[j] = 0.f;
     const uint32_t to = tlane + 384 + (warp >= 12 ? 64 : 0);
     for (int i = 0; i < ntiles; ++i) {
-      if (warp == 8) mbar_wait(o_ready + 8 * (i & 1), (i >> 1) & 1, a.err, dead, wait_ns);
+      if (warp == 8) mbar_wait(o_ready + 8 * rows_spo(i).bar, rows_spo(i).parity, a.err, dead, wait_ns);
       __syncwarp();
       pair_sync(5);
       tc_fence_after();

@@ -272,9 +272,11 @@ int firp_set_fused(firp_ctx *ctx, int32_t on);
 
 /*
  * Bound of every wait inside the kernels (for a tile, for the other CTAs of the persistent kernel), in
- * microseconds; 0 restores the default of 2 s.  A wait that runs out sets a device status word and the
- * kernel runs to its end without waiting again; the next firp_context_len returns
- * FIRP_ERR_DEVICE_TIMEOUT (results since the last check are invalid) and clears the word.
+ * microseconds; 0 restores the default of 2 s.  A kernel's waits start when the one before it has completed, and each
+ * is for one tile: neither an early launch nor a kernel's own length counts against the limit.  A wait that runs out sets a
+ * device status word and the kernel runs to its end without waiting again, except for its own copies and MMAs still
+ * under way (2 s at most); the next firp_context_len returns FIRP_ERR_DEVICE_TIMEOUT (results since the last check are
+ * invalid) and clears the word.
  */
 int firp_set_wait_limit_us(firp_ctx *ctx, int64_t usec);
 

@@ -120,6 +120,34 @@ template <int NH, bool SUM> __device__ __forceinline__ void warp_cols_to_smem(co
   }
 }
 
+// The K or V buffers as their producer sees them (pipeline.h): a buffer is free again when the MMAs that read it have completed.
+struct KvRing {
+  const CUtensorMap *tm; const AttnArgs &a;
+  uint32_t full, freed, dst0;
+  int slot, t0, kv_len, kvh;
+  uint64_t pol; unsigned long long wait_ns; bool dead;
+  __device__ __forceinline__ bool free(int, int w, uint32_t parity) { return mbar_wait(freed + 8 * w, parity, a.err, dead, wait_ns); }
+  __device__ __forceinline__ void load(int i, int w) {
+    mbar_expect_tx(full + 8 * w, kTcStage);
+#pragma unroll
+    for (int ph = 0; ph < 2; ++ph) {                // 64-position x 64-element boxes; a half lies inside one page
+      const int p0 = (t0 + i) * kTcTile + ph * 64;
+      const int row = (int)kv_row(a.pages, slot, p0 < kv_len ? p0 : 0, a.max_ctx);   // a half beyond the context: any rows
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        tma_load_2d(dst0 + (uint32_t)(w * kTcStage + h * kTcSlab + ph * 8192), tm, kvh * kTcDh + h * 64, row, full + 8 * w, pol);
+    }
+  }
+  __device__ __forceinline__ void landed(int w, uint32_t parity) { mbar_drain(full + 8 * w, parity, a.err); }
+};
+struct RowsKvRing : KvRing {     // of the kernel for many query rows: S or O of the tile before in this buffer, on barriers in threes
+  __device__ __forceinline__ bool free(int i, int, uint32_t) {
+    if (i < kRowsKvRing) return true;
+    const TilePhase f = rows_spo(i - kRowsKvRing);
+    return mbar_wait(freed + 8 * f.bar, f.parity, a.err, dead, wait_ns);
+  }
+};
+
 #ifdef FIRP_ATTN_TRACE
 __device__ unsigned long long g_attn_trace[16];
 #define TC_STAMP(k) do { if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) g_attn_trace[k] = globaltimer(); } while (0)
@@ -222,20 +250,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const uint32_t dst0 = sb + (is_v ? LY::V_OFF : LY::K_OFF);
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
-      for (int i = 0; i < ntiles; ++i) {
-        const int w = i & 1, q = i >> 1, t = t0 + i;
-        if (q > 0) mbar_wait(freed + 8 * w, (q - 1) & 1, a.err, dead, wait_ns);
-        mbar_expect_tx(full + 8 * w, kTcStage);
-#pragma unroll
-        for (int ph = 0; ph < 2; ++ph) {            // 64-position x 64-element boxes; a half lies inside one page
-          const int p0 = t * kTcTile + ph * 64;
-          const int row = (int)kv_row(a.pages, slot, p0 < kv_len ? p0 : 0, a.max_ctx);   // a half beyond the context: any rows
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            tma_load_2d(dst0 + (uint32_t)(w * kTcStage + h * kTcSlab + ph * 8192), tm, kvh * kTcDh + h * 64, row,
-                        full + 8 * w, pol);
-        }
-      }
+      KvRing ring{tm, a, full, freed, dst0, slot, t0, kv_len, kvh, pol, wait_ns, false};
+      produce(ring, ntiles, 2);
     }
   } else if (warp == 16) {
     // ---- MMA issuer (one lane): S^T of tile i, then O^T of tile i - 1
@@ -277,6 +293,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           tc_commit(o_ready + 8 * w);
         }
       }
+      if (ntiles > 0) mbar_drain(o_ready + 8 * ((ntiles - 1) & 1), ((ntiles - 1) >> 1) & 1, a.err);   // no MMA outlives the CTA
     }
   } else {
     // ---- the four softmax warpgroups: tile group g takes tiles g, g + 2, ...; half h of it owns the query columns
@@ -651,25 +668,8 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const uint32_t dst0 = sb + (is_v ? V_OFF : K_OFF);
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
-      for (int i = 0; i < ntiles; ++i) {
-        const int w = rows_kv(i).bar, t = t0 + i;
-        if (i >= kRowsKvRing) {                     // S or O of the tile before in this buffer
-          const TilePhase f = rows_spo(i - kRowsKvRing);
-          mbar_wait((is_v ? o_ready : s_ready) + 8 * f.bar, f.parity, a.err, dead, wait_ns);
-        }
-        mbar_expect_tx(full + 8 * w, kTcStage);
-#pragma unroll
-        for (int ph = 0; ph < 2; ++ph) {            // 64-position x 64-element boxes; a half lies inside one page
-          const int p0 = t * kTcTile + ph * 64;
-          const int src = (int)kv_row(a.pages, slot, p0 < kv_len ? p0 : 0, a.max_ctx);   // a half beyond the context: any rows
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            tma_load_2d(dst0 + (uint32_t)(w * kTcStage + h * kTcSlab + ph * 8192), tm, kvh * kTcDh + h * 64, src, full + 8 * w, pol);
-        }
-      }
-      // no copy is in flight when the CTA ends, even after a wait that ran out
-      dead = false;
-      for (int i = max(0, ntiles - kRowsKvRing); i < ntiles; ++i) mbar_wait(full + 8 * rows_kv(i).bar, rows_kv(i).parity, a.err, dead, wait_ns);
+      RowsKvRing ring{{tm, a, full, is_v ? o_ready : s_ready, dst0, slot, t0, kv_len, kvh, pol, wait_ns, false}};
+      produce(ring, ntiles, kRowsKvRing);
     }
   } else if (warp == 16) {
     // ---- MMA issuer of S, up to three tiles ahead of O
@@ -698,6 +698,9 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       if (elect_one()) tc_commit(s_ready + 8 * b3);
       b3 = b3 == 2 ? 0 : b3 + 1;
     }
+    // no MMA outlives the CTA, whichever wait ran out
+    if (ntiles > 0 && lane == 0) mbar_drain(s_ready + 8 * rows_spo(ntiles - 1).bar, rows_spo(ntiles - 1).parity, a.err);
+    __syncwarp();
   } else if (warp == 17) {
     // ---- MMA issuer of O
     const uint64_t vdesc = smem_desc_mn(sb + V_OFF, kTcSlab);
@@ -721,6 +724,8 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       if (elect_one()) tc_commit(o_ready + 8 * b3);
       if (++b3 == 3) { b3 = 0; ++ph3; }
     }
+    if (ntiles > 0 && lane == 0) mbar_drain(o_ready + 8 * rows_spo(ntiles - 1).bar, rows_spo(ntiles - 1).parity, a.err);
+    __syncwarp();
   } else if (warp < 8) {
     // ---- softmax warpgroups: thread = row; g takes tiles g, g + 2, ...
     const int g = warp >> 2;

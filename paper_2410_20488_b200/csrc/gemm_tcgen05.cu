@@ -33,8 +33,9 @@
 //   warps 4-11 : epilogue.  TMEM -> shared memory of the CTA of the cluster that finishes the token row (the ring's
 //                memory, no longer needed), cluster barrier, sum over the k slices in rank order, then the fused step:
 //                residual + RMSNorm operand, rotary + cache, SwiGLU, logits, or Eq. 3.
-// Every mbarrier wait is bounded (~2 s): on expiry the status word is set and the kernel runs to its end; TMEM is
-// always released.
+// Every mbarrier wait is bounded (2 s, or what the caller set) and starts after the previous kernel has completed: an early
+// launch does not count against it.  On expiry the status word is set and the kernel runs to its end; the producers stop
+// loading and wait for what is in flight, and TMEM is released when the last MMA has completed.
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -46,6 +47,7 @@
 #include "finish_device.cuh"
 #include "firp_kernels.cuh"
 #include "launch_util.cuh"
+#include "pipeline.h"
 #include "tc_device.cuh"
 
 namespace cg = cooperative_groups;
@@ -133,6 +135,36 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 __device__ __forceinline__ float4 mul4(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
+// The rings as their producers see them (pipeline.h).
+struct RingBase {
+  uint32_t full, empty;          // barriers of slot 0
+  int *err; unsigned long long wait_ns; bool dead;
+  __device__ __forceinline__ bool free(int, int slot, uint32_t parity) { return mbar_wait(empty + 8 * slot, parity, err, dead, wait_ns); }
+  __device__ __forceinline__ void landed(int slot, uint32_t parity) { mbar_drain(full + 8 * slot, parity, err); }
+};
+struct WeightRing : RingBase {   // one tile per slot
+  const CUtensorMap *tm; const TileSched &sc; const CtaWork &wk;
+  uint32_t ring; uint64_t pol;
+  int depth, pdl, it, t;         // of the next load: unit, tile
+  __device__ __forceinline__ bool free(int u, int slot, uint32_t parity) {
+    if (pdl && u == depth) griddep_wait();      // the slots only come free once the activations are there
+    return RingBase::free(u, slot, parity);
+  }
+  __device__ __forceinline__ void load(int, int slot) {
+    mbar_expect_tx(full + 8 * slot, W_TILE);
+    load_tile(ring + slot * W_TILE, tm, sc, wk.t0 + t, unit_kb(wk, it), full + 8 * slot, pol);
+    if (++t == wk.nt) { t = 0; ++it; }
+  }
+};
+struct ActRing : RingBase {      // all planes of a k block per slot
+  const CUtensorMap *tm; const CtaWork &wk;
+  uint32_t ring, stage; uint64_t pol;
+  int row0;
+  __device__ __forceinline__ void load(int u, int slot) {
+    mbar_expect_tx(full + 8 * slot, stage);
+    tma_load_3d(ring + slot * stage, tm, unit_kb(wk, u) * BK, row0, 0, full + 8 * slot, pol);
+  }
+};
 // MERGED: the activation planes sit side by side in one operand (or there is only one); else one after the other.
 // The epilogue's code runs once per launch from a cold instruction cache, in the shadow of nothing: one kernel per epilogue
 // and rolled loops keep it short (all five in one kernel, four items unrolled: 5-7 us instead of 1-2).
@@ -188,17 +220,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     if (lane == 0) {             // ---- weight producer: does not wait for the previous kernel
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-      int sl = 0;
-      uint32_t par = 1;
-      for (int it = 0; it < n_units; ++it) {
-        const int kb = unit_kb(wk, it);
-        for (int t = 0; t < wk.nt; ++t) {
-          mbar_wait(empty_w + 8 * sl, par, a.err, dead, wait_ns);
-          mbar_expect_tx(full_w + 8 * sl, W_TILE);
-          load_tile(w_ring + sl * W_TILE, &tmW, sc, wk.t0 + t, kb, full_w + 8 * sl, pol);
-          if (++sl == sw_n) { sl = 0; par ^= 1; }
-        }
-      }
+      WeightRing ring{{full_w, empty_w, a.err, wait_ns, false}, &tmW, sc, wk, w_ring, pol, sw_n, cf.pdl, 0, 0};
+      produce(ring, n_units * wk.nt, sw_n);
     }
   } else if (warp == 2) {
     if (lane == 0) {             // ---- activation producer
@@ -211,18 +234,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         mbar_expect_tx(rope_full, bytes);
         if (bytes) bulk_load(base + cf.rope_off, a.rope + (size_t)(row0 + r0) * (a.dh >> 1), bytes, rope_full);
       }
-      int sl = 0;
-      uint32_t par = 1;
-      for (int it = 0; it < n_units; ++it) {
-        mbar_wait(empty_x + 8 * sl, par, a.err, dead, wait_ns);
-        mbar_expect_tx(full_x + 8 * sl, x_stage);
-        tma_load_3d(x_ring + sl * x_stage, &tmX, unit_kb(wk, it) * BK, row0, 0, full_x + 8 * sl, pol);   // all planes
-        if (++sl == sx_n) { sl = 0; par ^= 1; }
-      }
+      ActRing ring{{full_x, empty_x, a.err, wait_ns, false}, &tmX, wk, x_ring, x_stage, pol, row0};
+      produce(ring, n_units, sx_n);
+      if (EPI == EPI_QKV_ROPE && cf.rope_bytes) mbar_drain(rope_full, 0, a.err);
     }
   } else if (warp == 1 || warp == 3) {        // ---- MMA issuers
     const int iw = warp >> 1;
     if (iw < cf.issuers) {
+      if (cf.pdl) griddep_wait();        // the limit of the waits below starts here
       // by units: unit iw, iw + issuers, ... into accumulator sets of its own; by tiles: every unit, tiles iw, iw + issuers, ...
       const int u0 = cf.by_tile ? 0 : iw, du = cf.by_tile ? 1 : cf.issuers;
       const uint32_t tm0 = __shfl_sync(0xffffffffu, tmem, 0);
@@ -352,8 +371,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   };
   auto wait_acc = [&]() {
     // one warp polls, the others sleep at a block barrier: eight polling warps halve the rate of the producer's and the
-    // issuers' shared-memory operations
-    if (warp == 4) mbar_wait(acc_full, 0, a.err, dead, wait_ns);
+    // issuers' shared-memory operations.  The whole contraction passes meanwhile, so the limit is that of all the issuers' waits
+    // together: they bound each of theirs, and commit in any case.
+    if (warp == 4) mbar_wait(acc_full, 0, a.err, dead, kDefaultWaitNs + min(wait_ns, 1ull << 48) * (unsigned)(2 * n_units * TM + 2));
     if (EPI == EPI_QKV_ROPE && cf.rope_bytes) mbar_wait(rope_full, 0, a.err, dead, wait_ns);      // long complete
     epi_sync();
     tc_fence_after();

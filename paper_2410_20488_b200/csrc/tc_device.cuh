@@ -39,11 +39,12 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
                : "=r"(ok) : "r"(bar), "r"(parity), "r"(hint_ns) : "memory");
   return ok != 0;
 }
-// Bounded wait: gives up after limit_ns, sets the status word and returns.  `dead` is sticky per thread:
+// Bounded wait: gives up after limit_ns, sets the status word and returns false.  `dead` is sticky per thread:
 // after one timeout later waits return at once, so the kernel runs to its end without waiting again.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int *err, bool &dead,
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int *err, bool &dead,
                                           unsigned long long limit_ns = kDefaultWaitNs) {
-  if (dead || mbar_try_wait(bar, parity)) return;
+  if (dead) return false;
+  if (mbar_try_wait(bar, parity)) return true;
   unsigned long long t0 = 0;
   while (!mbar_try_wait_hint(bar, parity, 10000u)) {
     const unsigned long long t = globaltimer();
@@ -51,9 +52,16 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int *er
     if (t - t0 > limit_ns) {
       dead = true;
       atomicExch(err, kErrTimeout);
-      return;
+      return false;
     }
   }
+  return true;
+}
+// Before a block ends: the copies or MMAs that complete this phase are still under way.  Under the default limit, whatever the
+// caller's is and whether or not an earlier wait ran out: shared and tensor memory must not be given back before.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity, int *err) {
+  bool dead = false;
+  mbar_wait(bar, parity, err, dead, kDefaultWaitNs);
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm, int x, int y, uint32_t bar,
                                             uint64_t policy) {

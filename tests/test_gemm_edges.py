@@ -47,3 +47,23 @@ def test_ragged_matrices(kw):
                                               (8, 16, 2, 800, False), (32, 8, 1, 1021, False)])
 def test_many_query_rows(T, H, Hkv, P, masked):
     _run(si.scaled(SMALL, d=H * 128, H=H, Hkv=Hkv), P, T=T, forced_steps=(1,), masked=masked)
+
+
+def test_a_limit_shorter_than_a_kernel_is_no_time_out():
+    """Waits are for single tiles and start when the kernel before has completed: launches of several hundred microseconds, of blocks
+    that work 60 us each, pass under a limit of 50 us."""
+    import torch
+    from paper_2410_20488_b200 import FirpEngine
+    shape = si.scaled(si.CONFIGS["c1"], L=1, l=0, d=4096, H=32, Hkv=32, dh=128, F=11008)
+    P = 2044
+    eng = FirpEngine(shape, si.all_weights(shape), max_ctx=2112)
+    prompt = torch.from_numpy(si.prompt(shape, length=P)).cuda()
+    parents = si.tree_template(shape.T)
+    first, second = (eng.new_out(1, 1, shape.k, T_next=shape.T) for _ in range(2))
+    eng.prefill(0, prompt, shape.k, shape.l, parents, first)
+    assert eng.context_len(0) == P
+    eng.set_wait_limit_us(50)
+    eng.prefill(0, prompt, shape.k, shape.l, parents, second)
+    assert eng.context_len(0) == P                 # raises on a time-out
+    assert torch.equal(first.logits, second.logits)
+    eng.close()

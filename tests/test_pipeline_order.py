@@ -21,6 +21,16 @@ int kv_bar(int i) { return rows_kv(i).bar; }
 int kv_parity(int i) { return rows_kv(i).parity; }
 int spo_bar(int i) { return rows_spo(i).bar; }
 int spo_parity(int i) { return rows_spo(i).parity; }
+typedef int (*Free)(int, int, unsigned);
+typedef void (*Load)(int, int);
+typedef void (*Landed)(int, unsigned);
+struct Ring {
+  Free f; Load l; Landed d;
+  bool free(int u, int slot, unsigned parity) { return f(u, slot, parity) != 0; }
+  void load(int u, int slot) { l(u, slot); }
+  void landed(int slot, unsigned parity) { d(slot, parity); }
+};
+void run_producer(int n, int depth, Free f, Load l, Landed d) { Ring r{f, l, d}; produce(r, n, depth); }
 }
 """
 
@@ -153,3 +163,39 @@ def test_rows_attention_at_random_timings(order, seed):
     stuck = simulate(attention_roles(order, rng.randint(1, 24), lambda is_v, i: rng.expovariate(1 / slow[0]), lambda i: rng.expovariate(1 / slow[1]),
                                      lambda: rng.expovariate(1 / slow[2]), lambda: rng.expovariate(1 / slow[3])))
     assert not stuck, stuck
+
+
+@pytest.mark.parametrize("depth", [1, 2, 3, 12])
+@pytest.mark.parametrize("n,stops_at", [(0, 99), (1, 99), (2, 99), (5, 99), (13, 99), (40, 99), (40, 0), (40, 1), (40, 3), (40, 11), (40, 12), (40, 25)])
+def test_producer_leaves_nothing_in_flight(order, depth, n, stops_at):
+    """Loads go in order, each into a slot whose last load its reader has given back, none after a wait that ran out, and every
+    one has been seen to land when the producer leaves.  From unit `stops_at` on the readers give no slot back."""
+    in_flight, loaded, ran_out, landed = {}, [], [], [0] * depth
+
+    def free(u, slot, parity):
+        assert not ran_out and u == len(loaded) and slot == u % depth
+        released = u // depth                               # phases that the slot's readers complete for this load, if they do
+        assert parity == (released & 1) ^ 1                 # the phase just before: complete at the start, then once per turn
+        if u - depth >= stops_at:
+            ran_out.append(u)
+            return 0
+        if u >= depth:                                      # given back: its reader has seen it land
+            assert in_flight.pop(slot) == u - depth
+            landed[slot] += 1
+        return 1
+
+    def load(u, slot):
+        assert not ran_out and slot not in in_flight
+        loaded.append(u)
+        in_flight[slot] = u
+
+    def land(slot, parity):
+        assert parity == landed[slot] & 1
+        del in_flight[slot]
+        landed[slot] += 1
+
+    types = (ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_uint), ctypes.CFUNCTYPE(None, ctypes.c_int, ctypes.c_int),
+             ctypes.CFUNCTYPE(None, ctypes.c_int, ctypes.c_uint))
+    order.run_producer(n, depth, *(t(f) for t, f in zip(types, (free, load, land))))
+    assert not in_flight
+    assert loaded == list(range(min(n, stops_at + depth)))

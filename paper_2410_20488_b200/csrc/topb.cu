@@ -63,10 +63,12 @@ __device__ __forceinline__ u64 warp_bth(uint32_t hi, uint32_t lo, int B) {
   return th ? ((u64)th << 32) | tl : 0;
 }
 
-// EPT: logits of a thread per pass.  VEC: four neighbouring logits per load (rows start on 16-byte boundaries)
+// EPT: logits of a thread per pass.  VEC: four neighbouring logits per load (rows start on 16-byte boundaries).  The kernel is
+// launched beside the one that writes the logits: they are read through L2, never through the read-only path, whose data must
+// not change while a kernel lives.
 template <int EPT, bool VEC>
 __global__ void __launch_bounds__(32 * kTopWarps)
-topb_kernel(const float *__restrict__ vals, int V, int B, int32_t *out_ids, float *out_vals, int pdl) {
+topb_kernel(const float *vals, int V, int B, int32_t *out_ids, float *out_vals, int pdl) {
   __shared__ u64 s_list[kTopList + kMaxTopB], s_max[kTopWarps];
   __shared__ u64 s_best[kMaxTopB], s_all[kTopCluster * kMaxTopB];
   __shared__ int s_n;
@@ -90,11 +92,11 @@ topb_kernel(const float *__restrict__ vals, int V, int B, int32_t *out_ids, floa
       const int id = id_of(e);
       const bool in = id < V && id >= 0;
       if (VEC) {
-        const float4 f = in ? __ldg(reinterpret_cast<const float4 *>(row + id)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 f = in ? __ldcg(reinterpret_cast<const float4 *>(row + id)) : make_float4(0.f, 0.f, 0.f, 0.f);
         k[e] = in ? order_key(f.x) : 0u; k[e + (VEC ? 1 : 0)] = in ? order_key(f.y) : 0u;
         k[e + (VEC ? 2 : 0)] = in ? order_key(f.z) : 0u; k[e + (VEC ? 3 : 0)] = in ? order_key(f.w) : 0u;
       } else {
-        k[e] = in ? order_key(__ldg(row + id)) : 0u;
+        k[e] = in ? order_key(__ldcg(row + id)) : 0u;
       }
     }
 #pragma unroll
@@ -161,7 +163,7 @@ topb_kernel(const float *__restrict__ vals, int V, int B, int32_t *out_ids, floa
     const u64 key = list[tid];
     const int id = key ? (int)~(uint32_t)key : 0x7fffffff;
     float v = key ? order_value((uint32_t)(key >> 32)) : -INFINITY;
-    if (v == 0.f) v = row[id];             // the sign of a zero is not in the key
+    if (v == 0.f) v = __ldcg(row + id);             // the sign of a zero is not in the key
     out_ids[(size_t)blockIdx.y * B + tid] = id;
     out_vals[(size_t)blockIdx.y * B + tid] = v;
   }

@@ -42,7 +42,8 @@ def test_ragged_matrices(kw):
     _run(si.scaled(si.CONFIGS["c1"], **kw), 200)
 
 
-# more than 48 query rows on more than six tiles of context: one block of 128 rows, or several; a lone CTA or a cluster of splits
+# more than 48 query rows on more than six tiles of context: one block of 128 rows, or two; clusters of five to eight splits of one or two tiles
+# (many tiles per block, lone blocks: test_rows_attention.py)
 @pytest.mark.parametrize("T,H,Hkv,P,masked", [(46, 2, 2, 764, False), (61, 2, 2, 1023, True), (125, 2, 2, 893, False), (126, 2, 1, 1150, False),
                                               (8, 16, 2, 800, False), (32, 8, 1, 1021, False)])
 def test_many_query_rows(T, H, Hkv, P, masked):

@@ -251,7 +251,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
       KvRing ring{tm, a, full, freed, dst0, slot, t0, kv_len, kvh, pol, wait_ns, false};
-      produce(ring, ntiles, 2);
+      drain(ring, produce(ring, ntiles, 2), 2);
     }
   } else if (warp == 16) {
     // ---- MMA issuer (one lane): S^T of tile i, then O^T of tile i - 1
@@ -669,7 +669,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
       RowsKvRing ring{{tm, a, full, is_v ? o_ready : s_ready, dst0, slot, t0, kv_len, kvh, pol, wait_ns, false}};
-      produce(ring, ntiles, kRowsKvRing);
+      drain(ring, produce(ring, ntiles, kRowsKvRing), kRowsKvRing);
     }
   } else if (warp == 16) {
     // ---- MMA issuer of S, up to three tiles ahead of O

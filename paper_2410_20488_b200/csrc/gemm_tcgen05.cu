@@ -33,9 +33,10 @@
 //   warps 4-11 : epilogue.  TMEM -> shared memory of the CTA of the cluster that finishes the token row (the ring's
 //                memory, no longer needed), cluster barrier, sum over the k slices in rank order, then the fused step:
 //                residual + RMSNorm operand, rotary + cache, SwiGLU, logits, or Eq. 3.
-// Every mbarrier wait is bounded (2 s, or what the caller set) and starts after the previous kernel has completed: an early
-// launch does not count against it.  On expiry the status word is set and the kernel runs to its end; the producers stop
-// loading and wait for what is in flight, and TMEM is released when the last MMA has completed.
+// Every mbarrier wait is bounded (2 s, or what the caller set, counted from the previous kernel's completion: an early launch
+// does not count against it).  On expiry the status word is set and the kernel runs to its end; the producers stop
+// loading, and the block ends when what it has started has landed and the last MMA has completed.  (Only then: producers that
+// always waited for their last loads cost a step of up to 32 rows 1-5 %.)
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -140,16 +141,15 @@ struct RingBase {
   uint32_t full, empty;          // barriers of slot 0
   int *err; unsigned long long wait_ns; bool dead;
   __device__ __forceinline__ bool free(int, int slot, uint32_t parity) { return mbar_wait(empty + 8 * slot, parity, err, dead, wait_ns); }
+};
+struct Landing {
+  uint32_t full; int *err;
   __device__ __forceinline__ void landed(int slot, uint32_t parity) { mbar_drain(full + 8 * slot, parity, err); }
 };
 struct WeightRing : RingBase {   // one tile per slot
   const CUtensorMap *tm; const TileSched &sc; const CtaWork &wk;
   uint32_t ring; uint64_t pol;
-  int depth, pdl, it, t;         // of the next load: unit, tile
-  __device__ __forceinline__ bool free(int u, int slot, uint32_t parity) {
-    if (pdl && u == depth) griddep_wait();      // the slots only come free once the activations are there
-    return RingBase::free(u, slot, parity);
-  }
+  int it, t;                     // of the next load: unit, tile
   __device__ __forceinline__ void load(int, int slot) {
     mbar_expect_tx(full + 8 * slot, W_TILE);
     load_tile(ring + slot * W_TILE, tm, sc, wk.t0 + t, unit_kb(wk, it), full + 8 * slot, pol);
@@ -184,6 +184,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   const uint32_t bars = base + cf.tail + kMaxRows * 6 + 2 * kMaxSeq * 4;
   const uint32_t full_w = bars, empty_w = full_w + 8 * kMaxW, full_x = empty_w + 8 * kMaxW, empty_x = full_x + 8 * kMaxX,
                  acc_full = empty_x + 8 * kMaxX, rope_full = acc_full + 8, tmem_slot = rope_full + 8;
+  volatile int *gave_up = reinterpret_cast<volatile int *>(data + (tmem_slot + 4 - base));   // a thread's wait has run out
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const CtaWork wk = cta_work(sc, blockIdx.x);
   const int row0 = wk.block * cf.rpb, R = min(cf.rpb, a.R - row0);      // this CTA's token rows
@@ -197,6 +198,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     const int readers = cf.by_tile ? cf.issuers : 1;
     for (int i = 0; i < sw_n; ++i) { mbar_init(full_w + 8 * i, 1); mbar_init(empty_w + 8 * i, 1); }
     for (int i = 0; i < sx_n; ++i) { mbar_init(full_x + 8 * i, 1); mbar_init(empty_x + 8 * i, readers); }
+    *gave_up = 0;
     mbar_init(acc_full, cf.issuers);
     mbar_init(rope_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -216,12 +218,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
 
   bool dead = false;
   const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kDefaultWaitNs;
+  // For what only the issuers' commits end: they start waiting when the previous kernel has completed, bound each of their waits
+  // and commit in any case.  (The weight producer does not wait for the previous kernel itself: griddepcontrol.wait between its
+  // loads cost a step of up to 32 rows 2-6 %.)
+  const unsigned long long all_ns = kDefaultWaitNs + min(wait_ns, 1ull << 48) * (unsigned)(2 * n_units * TM + 2);
+  int started = 0;               // loads of a producer
   if (warp == 0) {
     if (lane == 0) {             // ---- weight producer: does not wait for the previous kernel
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-      WeightRing ring{{full_w, empty_w, a.err, wait_ns, false}, &tmW, sc, wk, w_ring, pol, sw_n, cf.pdl, 0, 0};
-      produce(ring, n_units * wk.nt, sw_n);
+      WeightRing ring{{full_w, empty_w, a.err, all_ns, false}, &tmW, sc, wk, w_ring, pol, 0, 0};
+      started = produce(ring, n_units * wk.nt, sw_n);
+      dead = ring.dead;
     }
   } else if (warp == 2) {
     if (lane == 0) {             // ---- activation producer
@@ -235,8 +243,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         if (bytes) bulk_load(base + cf.rope_off, a.rope + (size_t)(row0 + r0) * (a.dh >> 1), bytes, rope_full);
       }
       ActRing ring{{full_x, empty_x, a.err, wait_ns, false}, &tmX, wk, x_ring, x_stage, pol, row0};
-      produce(ring, n_units, sx_n);
-      if (EPI == EPI_QKV_ROPE && cf.rope_bytes) mbar_drain(rope_full, 0, a.err);
+      started = produce(ring, n_units, sx_n);
+      dead = ring.dead;
     }
   } else if (warp == 1 || warp == 3) {        // ---- MMA issuers
     const int iw = warp >> 1;
@@ -371,9 +379,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   };
   auto wait_acc = [&]() {
     // one warp polls, the others sleep at a block barrier: eight polling warps halve the rate of the producer's and the
-    // issuers' shared-memory operations.  The whole contraction passes meanwhile, so the limit is that of all the issuers' waits
-    // together: they bound each of theirs, and commit in any case.
-    if (warp == 4) mbar_wait(acc_full, 0, a.err, dead, kDefaultWaitNs + min(wait_ns, 1ull << 48) * (unsigned)(2 * n_units * TM + 2));
+    // issuers' shared-memory operations
+    if (warp == 4) mbar_wait(acc_full, 0, a.err, dead, all_ns);
     if (EPI == EPI_QKV_ROPE && cf.rope_bytes) mbar_wait(rope_full, 0, a.err, dead, wait_ns);      // long complete
     epi_sync();
     tc_fence_after();
@@ -655,7 +662,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   }
   }
   tc_fence_before();
+  if (dead) *gave_up = 1;
   __syncthreads();
+  if (*gave_up) {                // some loads or MMAs may still be under way (otherwise the accumulators were waited for, and they for all)
+    if (lane == 0 && warp == 0) { Landing r{full_w, a.err}; drain(r, started, sw_n); }
+    if (lane == 0 && warp == 2) {
+      Landing r{full_x, a.err};
+      drain(r, started, sx_n);
+      if (EPI == EPI_QKV_ROPE && cf.rope_bytes) mbar_drain(rope_full, 0, a.err);
+    }
+    if (lane == 0 && warp == 4) mbar_drain(acc_full, 0, a.err);
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cf.tmem_cols) : "memory");

@@ -26,19 +26,23 @@ constexpr int kRowsSpoRing = 3;
 FIRP_HD TilePhase rows_spo(int i) { return TilePhase{i % kRowsSpoRing, (unsigned)(i / kRowsSpoRing) & 1u}; }
 
 // A producer: loads 0 .. n - 1 go, in order, into a ring of `depth` slots.  It gives up with the first slot that does not come
-// free in time (a load into it would be counted on a barrier whose phase is still open), and never leaves before what it has
-// loaded has landed: a copy must not outlive the memory it writes to, which the next block on the SM may own.
+// free in time: a load into it would be counted on a barrier whose phase is still open.  Returns the number of loads started.
 //   bool ring.free(u, slot, parity)    bounded wait for the slot's phase of that parity; false: it ran out
 //   void ring.load(u, slot)            starts load u
-//   void ring.landed(slot, parity)     bounded wait, under a limit of its own, for the slot's phase of that parity
-template <class Ring> FIRP_HD void produce(Ring &ring, int n, int depth) {
+template <class Ring> FIRP_HD int produce(Ring &ring, int n, int depth) {
   int u = 0, slot = 0;
   unsigned parity = 1;
   for (; u < n && ring.free(u, slot, parity); ++u) {
     ring.load(u, slot);
     if (++slot == depth) { slot = 0; parity ^= 1u; }
   }
-  for (int v = u > depth ? u - depth : 0; v < u; ++v) ring.landed(v % depth, (unsigned)(v / depth) & 1u);
+  return u;
+}
+// The last of n loads started have landed, oldest first.  After a wait that ran out nobody else may have looked, and a copy must
+// not outlive the memory it writes to, which the next block on the SM may own.
+//   void ring.landed(slot, parity)     bounded wait, under a limit of its own, for the slot's phase of that parity
+template <class Ring> FIRP_HD void drain(Ring &ring, int n, int depth) {
+  for (int v = n > depth ? n - depth : 0; v < n; ++v) ring.landed(v % depth, (unsigned)(v / depth) & 1u);
 }
 
 }  // namespace firp

@@ -30,7 +30,7 @@ struct Ring {
   void load(int u, int slot) { l(u, slot); }
   void landed(int slot, unsigned parity) { d(slot, parity); }
 };
-void run_producer(int n, int depth, Free f, Load l, Landed d) { Ring r{f, l, d}; produce(r, n, depth); }
+void run_producer(int n, int depth, Free f, Load l, Landed d) { Ring r{f, l, d}; drain(r, produce(r, n, depth), depth); }
 }
 """
 
@@ -169,7 +169,7 @@ def test_rows_attention_at_random_timings(order, seed):
 @pytest.mark.parametrize("n,stops_at", [(0, 99), (1, 99), (2, 99), (5, 99), (13, 99), (40, 99), (40, 0), (40, 1), (40, 3), (40, 11), (40, 12), (40, 25)])
 def test_producer_leaves_nothing_in_flight(order, depth, n, stops_at):
     """Loads go in order, each into a slot whose last load its reader has given back, none after a wait that ran out, and every
-    one has been seen to land when the producer leaves.  From unit `stops_at` on the readers give no slot back."""
+    one has been seen to land after the drain.  From unit `stops_at` on the readers give no slot back."""
     in_flight, loaded, ran_out, landed = {}, [], [], [0] * depth
 
     def free(u, slot, parity):

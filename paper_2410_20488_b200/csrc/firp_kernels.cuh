@@ -189,6 +189,8 @@ template <int EPI> __device__ __forceinline__ int lin_src_row(const LinArgs &a, 
 }
 // pdl: launch with programmatic stream serialization (the kernel waits on its predecessor itself).
 cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream_t st);
+// additions in a row that an accumulator of that GEMM sees (its precision, for the tests)
+int gemm_additions(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes);
 bool gemm_tc_available();         // the driver entry point for tensor-map encoding was found
 
 // What the finishers of the persistent kernel's GEMMs read (fused_step.cu).

@@ -165,10 +165,11 @@ struct ActRing : RingBase {      // all planes of a k block per slot
     tma_load_3d(ring + slot * stage, tm, unit_kb(wk, u) * BK, row0, 0, full + 8 * slot, pol);
   }
 };
-// MERGED: the activation planes sit side by side in one operand (or there is only one); else one after the other.
+// MERGED: the activation planes sit side by side in one operand (or there is only one); else one after the other.  DEEP: more than two
+// accumulator sets, or planes side by side (in one kernel with the others the code they skip cost them 1-2 % of a two-layer step).
 // The epilogue's code runs once per launch from a cold instruction cache, in the shadow of nothing: one kernel per epilogue
 // and rolled loops keep it short (all five in one kernel, four items unrolled: 5-7 us instead of 1-2).
-template <int TM, bool MERGED, int EPI>
+template <int TM, bool MERGED, bool DEEP, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ LinArgs a,
             const __grid_constant__ TileSched sc, const __grid_constant__ TileCfg cf) {
@@ -344,7 +345,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   const uint32_t tquarter = tmem + ((uint32_t)(quarter * 32) << 16);
   auto load_acc = [&](int t, int c0, float *r) {
     const uint32_t ta = tquarter + (uint32_t)(t * cf.acc + c0);
-    float l[3][16];
+    float l[DEEP ? 4 : 3][16];
     tc_ld16(ta, r);
     if (cf.planes_side > 1) tc_ld16(ta + cf.npad, l[0]);
     if (cf.sets > 1) {
@@ -364,17 +365,39 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         for (int j = 0; j < 16; ++j) r[j] += l[2][j];
       }
     }
-    // the third plane's columns and the third and fourth set's (one loop for all of them cost 1 us per layer)
-    if (cf.sets > 2 || cf.planes_side > 2) {
+    if (DEEP) {       // the third and fourth set's columns, the third plane's
+      if (cf.sets > 2) {
+        tc_ld16(ta + 2 * cf.acc_set, l[0]);
+        if (cf.planes_side > 1) tc_ld16(ta + 2 * cf.acc_set + cf.npad, l[1]);
+        if (cf.sets > 3) {
+          tc_ld16(ta + 3 * cf.acc_set, l[2]);
+          if (cf.planes_side > 1) tc_ld16(ta + 3 * cf.acc_set + cf.npad, l[3]);
+        }
+        tc_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) r[j] += l[0][j];
+        if (cf.planes_side > 1) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) r[j] += l[1][j];
+        }
+        if (cf.sets > 3) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) r[j] += l[2][j];
+          if (cf.planes_side > 1) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) r[j] += l[3][j];
+          }
+        }
+      }
+      if (cf.planes_side > 2) {
 #pragma unroll 1
-      for (int i = 0; i < cf.sets; ++i)
-#pragma unroll 1
-        for (int pl = i < 2 ? 2 : 0; pl < cf.planes_side; ++pl) {
-          tc_ld16(ta + i * cf.acc_set + pl * cf.npad, l[0]);
+        for (int i = 0; i < cf.sets; ++i) {
+          tc_ld16(ta + i * cf.acc_set + 2 * cf.npad, l[0]);
           tc_ld_wait();
 #pragma unroll
           for (int j = 0; j < 16; ++j) r[j] += l[0][j];
         }
+      }
     }
   };
   auto wait_acc = [&]() {
@@ -748,20 +771,20 @@ constexpr uint32_t pow2_cols(int c) { return c <= 32 ? 32 : c <= 64 ? 64 : c <= 
 constexpr int align_n(int v, int a) { return (v + a - 1) / a * a; }
 
 typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const LinArgs, const TileSched, const TileCfg);
-template <int EPI> KernelFn kernel_epi(int tm, bool merged) {
-  switch (tm) {
-    case 1: return merged ? gemm_kernel<1, true, EPI> : gemm_kernel<1, false, EPI>;
-    case 2: return merged ? gemm_kernel<2, true, EPI> : gemm_kernel<2, false, EPI>;
-    default: return merged ? gemm_kernel<3, true, EPI> : gemm_kernel<3, false, EPI>;
-  }
+template <bool MERGED, bool DEEP, int EPI> KernelFn kernel_tm(int tm) {
+  return tm == 1 ? gemm_kernel<1, MERGED, DEEP, EPI> : tm == 2 ? gemm_kernel<2, MERGED, DEEP, EPI> : gemm_kernel<3, MERGED, DEEP, EPI>;
 }
-KernelFn kernel_of(int epi, int tm, bool merged) {
+template <int EPI> KernelFn kernel_epi(int tm, bool merged, bool deep) {
+  if (merged) return deep ? kernel_tm<true, true, EPI>(tm) : kernel_tm<true, false, EPI>(tm);
+  return deep ? kernel_tm<false, true, EPI>(tm) : kernel_tm<false, false, EPI>(tm);
+}
+KernelFn kernel_of(int epi, int tm, bool merged, bool deep) {
   switch (epi) {
-    case EPI_RESIDUAL: return kernel_epi<EPI_RESIDUAL>(tm, merged);
-    case EPI_QKV_ROPE: return kernel_epi<EPI_QKV_ROPE>(tm, merged);
-    case EPI_SWIGLU: return kernel_epi<EPI_SWIGLU>(tm, merged);
-    case EPI_LOGITS: return kernel_epi<EPI_LOGITS>(tm, merged);
-    default: return kernel_epi<EPI_PSEUDO>(tm, merged);
+    case EPI_RESIDUAL: return kernel_epi<EPI_RESIDUAL>(tm, merged, deep);
+    case EPI_QKV_ROPE: return kernel_epi<EPI_QKV_ROPE>(tm, merged, deep);
+    case EPI_SWIGLU: return kernel_epi<EPI_SWIGLU>(tm, merged, deep);
+    case EPI_LOGITS: return kernel_epi<EPI_LOGITS>(tm, merged, deep);
+    default: return kernel_epi<EPI_PSEUDO>(tm, merged, deep);
   }
 }
 
@@ -782,7 +805,7 @@ int cluster_ctas(int n) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    KernelFn fn = kernel_of(EPI_RESIDUAL, 1, true);
+    KernelFn fn = kernel_of(EPI_RESIDUAL, 1, true, false);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&k, fn, &cfg) != cudaSuccess || k < 1) { cudaGetLastError(); k = std::max(1, sms / n * 3 / 4); }
     cap[n] = k * n;
@@ -790,11 +813,20 @@ int cluster_ctas(int n) {
   return cap[n];
 }
 
-struct Plan { TileSched sc; TileCfg cf; int tm, merged, smem; };
+struct Plan { TileSched sc; TileCfg cf; int tm, merged, smem, adds; };
 
 // cycles of one M = 128, K = 16 MMA of n columns: reading the operands from shared memory (128 + n rows of 32 bytes at 128
 // bytes a cycle), computing, or issuing it, whichever takes longest (measured: 50 at 16 columns, 55 at 80, 72 at 144)
 float mma_clk(int n) { return std::max(50.f, std::max(n / 2.f, 34.f + n / 4.f)); }
+
+// Additions in a row that an accumulator would see if every SM of a B200 had an equal share of the matrix, in pairs of tiles, with two
+// planes into the same columns from 49 rows on.  The tensor core truncates where it adds to an accumulator, so the error of a sum
+// grows with their number: against 64-bit sums of the same planes, in the 2-norm, 0.24e-6 after 16, 0.48e-6 after 32, 1.1e-6 after
+// 76, 2.1e-6 after 128, 4.5e-6 after 256, 9.2e-6 after 512; what the two planes leave out of an activation is 2.4e-6.
+int longest_sum(int n_tiles, int KB, int rows, int planes) {
+  const int units = (n_tiles + 1) / 2 * KB, share = std::min(KB, (units + 147) / 148);
+  return std::max(16, 4 * share * (planes == 1 || rows <= (planes == 3 ? 80 : 48) ? 1 : planes));
+}
 
 Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int planes) {
   Plan best{};
@@ -804,7 +836,12 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
   s.heads = s.mode == ROWS_ROTARY ? BM / dh : 0;
   s.n_tiles = s.mode == ROWS_GATE_UP ? 2 * ((F + BM - 1) / BM) : (N + BM - 1) / BM;
   s.KB = (K + BK - 1) / BK;
-  const int adds_wanted = epi == EPI_RESIDUAL ? std::max(176, (rows > kMaxTreeRows ? 1 : 2) * s.KB) : (epi == EPI_SWIGLU ? 260 : epi == EPI_LOGITS ? 512 : 176) * std::max(64, s.KB) / 64;
+  // A prompt's sums may be longer: its results are as far from a 64-bit run as with the equal shares' (cache rows of 1999 tokens of
+  // the 7B shape 2.24e-3 / 2.32e-3, of 500 2.76e-3 / 2.88e-3: the rounding of the cache to bf16 hides them), and the equal shares'
+  // limit costs it 5 %.  A step's keep it, or 96 where that is more (an error below the planes' own).
+  const int share = longest_sum(s.n_tiles, s.KB, rows, planes);
+  int adds_wanted = epi == EPI_RESIDUAL ? std::max(176, (rows > kMaxTreeRows ? 1 : 2) * s.KB) : (epi == EPI_SWIGLU ? 260 : epi == EPI_LOGITS ? 512 : 176) * std::max(64, s.KB) / 64;
+  if (rows <= kMaxTreeRows) adds_wanted = std::min(adds_wanted, std::max(96, share));
   for (int max_adds = adds_wanted; best.tm == 0 && max_adds < (1 << 20); max_adds *= 2)
   for (int most : {256, 192, 128}) {         // token rows of a block: blocks of equal size
   s.blocks = (rows + most - 1) / most;
@@ -844,14 +881,18 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
         if (x_stage <= 24 * 1024) sx = std::min(std::min(kMaxX, kb), (avail - sw * W_TILE) / x_stage);      // what is left
         if (by_unit) sx &= ~1;
         if (sw < 2 * per && kb > 1) continue;
-        // The tensor core truncates where it adds to an accumulator, so the error of a sum grows with the additions in a row
-        // (measured on the cache rows of a 1999-token prompt against fp64: 1.1e-4, 1.5e-4 and 2.1e-4 in the 2-norm after
-        // 168, 256 and 512 of them).  As many accumulator sets as fit, up to four, share the k blocks, and what is still
-        // longer than the limit is left to a split.
+        // As many accumulator sets as fit, up to four, share the k blocks; what is still longer than the limit is left to a
+        // split.
         int sets = by_unit ? 2 : 1;
         const int per_kb = (BK / 16) * (merged ? 1 : planes);
-        while (sets < (rows > kMaxTreeRows ? 4 : 2) && (kb + sets - 1) / sets * per_kb > 96 && 2 * sets * tm * n_mma + over <= 512 && s.KB / split >= 2 * sets) sets *= 2;
-        const int adds = (kb + sets - 1) / sets * per_kb;
+        auto adds_of = [&](int n) { return (kb + n - 1) / n * per_kb; };
+        while (sets < 4 && (adds_of(sets) > std::min(share, max_adds) || (adds_of(sets) > 96 && (sets < 2 || rows > kMaxTreeRows))) &&
+               2 * sets * tm * n_mma + over <= 512 && s.KB / split >= 2 * sets) sets *= 2;
+        // Three are not dealt to two issuers, and one is too slow for a whole contraction (13B shape, 131 rows: the QKV projection
+        // 49.6 us so, 44.2 in three slices of three tiles; down in three slices 41.5, in eight of three tiles 46.6).
+        const bool lone = by_unit && sets == 2 && adds_of(2) > std::min(share, max_adds) && split > 1 && 3 * n_mma + over <= 512 && s.KB / split >= 3;
+        if (lone) sets = 3;
+        const int adds = adds_of(sets);
         if (adds > max_adds) continue;
         // microseconds: the weights at the rate HBM gives that many CTAs (6.8 TB/s from 84 on); a CTA's MMAs; its bytes from
         // L2, which gives a CTA 150 GB/s and all of them 15 TB/s; the epilogue's two passes (35 rows: 0.8 + 1.1 us, 131
@@ -861,14 +902,14 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
         const float mma = (float)waves * per * kb * 4.f * (merged ? 1 : planes) * mma_clk(n_mma) / 1850.f;
         const float ingest = (float)waves * kb * (per * W_TILE + x_stage) / std::min(150e3f, 15e6f / ctas);
         const bool direct = split == 1 && (epi == EPI_QKV_ROPE || epi == EPI_SWIGLU || epi == EPI_LOGITS);
-        const float out = direct ? 0.5f + 0.025f * R * per : 0.025f * R * per + 0.05f * own * per + (split == 1 ? 0.5f : red ? 1.f : 2.f);
+        const float out = (sets > 2 ? 0.004f * R * per : 0.f) + (direct ? 0.5f + 0.025f * R * per : 0.025f * R * per + 0.05f * own * per + (split == 1 ? 0.5f : red ? 1.f : 2.f));
         // a ring slot goes round in 0.9 us (activations) or 1.4 us (weights)
         const float rings_us = (float)waves * kb * std::max(0.9f / sx, 1.4f * per / sw);
-        const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.1f * (hbm + mma + ingest) + waves * (2.f + out);
+        const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.1f * (hbm + mma + ingest) + waves * (2.f + out) + (split >= 7 && rows > 128 ? 3.f : 0.f);
         TileCfg c{};
         c.planes = planes; c.rpb = R; c.npad = npad; c.acc = n_mma; c.sw = sw; c.sx = sx;
         c.tpo = tpo; c.inv_tpo = (65536 + c.tpo - 1) / c.tpo;
-        c.planes_side = merged ? planes : 1; c.acc_set = tm * n_mma; c.sets = sets; c.issuers = by_unit || tm >= 2 ? 2 : 1; c.by_tile = tm >= 2;
+        c.planes_side = merged ? planes : 1; c.acc_set = tm * n_mma; c.sets = sets; c.issuers = (by_unit && !lone) || tm >= 2 ? 2 : 1; c.by_tile = tm >= 2;
         c.idesc = instr_desc_m128(n_mma); c.tmem_cols = pow2_cols(c.sets * tm * n_mma + over);
         const int rings = align_n(sw * W_TILE + sx * x_stage, 128);
         if (red) {
@@ -882,7 +923,7 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
         const int smem = c.tail + 1024 + kTailBytes;
         if (smem > kSmemMax || cost >= best_cost) continue;
         best_cost = cost;
-        best = Plan{s, c, tm, merged, smem};
+        best = Plan{s, c, tm, merged, smem, adds};
         best.sc.jobs = jobs; best.sc.split = split;
       }
     }
@@ -906,6 +947,8 @@ Plan cached_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int plane
 
 }  // namespace
 
+int gemm_additions(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes) { return cached_plan(epi, N, K, F, dh, R, planes).adds; }
+
 bool gemm_tc_available() { return encode_fn() != nullptr; }
 
 cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream_t st) {
@@ -914,7 +957,7 @@ cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream
   if (p.tm == 0 || p.smem > kSmemMax || p.cf.tp < 1 || p.cf.sw < 1 || p.cf.sx < 1 || (!p.cf.by_tile && p.cf.issuers == 2 && ((p.cf.sw | p.cf.sx | p.cf.sets) & 1)))
     return cudaErrorInvalidConfiguration;
   p.cf.pdl = pdl ? 1 : 0;
-  KernelFn fn = kernel_of(epi, p.tm, p.merged != 0);
+  KernelFn fn = kernel_of(epi, p.tm, p.merged != 0, p.cf.sets > 2 || p.cf.planes_side > 2);
   static std::map<KernelFn, int> configured;
   static std::mutex mu;
   {

@@ -68,3 +68,18 @@ def test_a_limit_shorter_than_a_kernel_is_no_time_out():
     assert eng.context_len(0) == P                 # raises on a time-out
     assert torch.equal(first.logits, second.logits)
     eng.close()
+
+
+@pytest.mark.parametrize("d,H,Hkv,F,V", [(4096, 32, 32, 11008, 32000), (5120, 40, 40, 13824, 32000), (8192, 64, 8, 22016, 32000)])
+def test_sums_of_a_step_are_no_longer_than_equal_shares_make_them(d, H, Hkv, F, V):
+    """The tensor core truncates on every addition: no accumulator of a step sees more in a row than if every SM had an equal share
+    of the matrix (pairs of 128-row tiles; both planes in the same columns from 49 rows on), or 96 (1.6e-6, below the planes' own 2.4e-6)."""
+    import ctypes
+    from paper_2410_20488_b200 import binding
+    additions = binding.load_library()._ZN4firp14gemm_additionsENS_12GemmEpilogueEiiiiii
+    additions.restype, additions.argtypes = ctypes.c_int, [ctypes.c_int] * 7
+    for rows in (1, 4, 11, 18, 35, 48, 49, 67, 72, 96, 108, 128, 129, 131, 140, 144):
+        for epi, N, K in ((0, d, H * 128), (0, d, F), (1, (H + 2 * Hkv) * 128, d), (2, 2 * F, d), (3, V, d), (4, 3 * d, d)):
+            blocks, pairs = -(-K // 64), -(-(-(-N // 128)) // 2)
+            share = 4 * min(blocks, -(-pairs * blocks // 148)) * (1 if rows <= 48 else 2)
+            assert 0 < additions(epi, N, K, F, 128, rows, 2) <= max(96, share), (rows, epi, N, K)

@@ -309,16 +309,17 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       const int G = H / Hkv, qblocks = (act * G + 63) / 64;
       a.splits = attention_splits(rw.n_seq * Hkv * qblocks, tiles);
       a.o = c->o; a.o_lo_off = Rp * nq; a.err = c->dev_status; a.wait_ns = c->wait_ns;
-      // Head dimension 128 runs on the tensor-core kernel unless told otherwise.  Measured at the 7B shape, us per step
-      // mma.sync / tcgen05: 1 row at 128 cached tokens 2850 / 2724; 35 rows at 512 3441 / 3242, at 8192 6208 / 4185; 131
-      // rows at 2047 6890 / 5850; 6 sequences x 18 rows at 128-1024 6170 / 5130.
+      // Head dimension 128 runs on the tensor-core kernel unless told otherwise.  Measured on eight layers of the 7B shape, tcgen05 /
+      // mma.sync: where the latter is nearest, 16-48 rows on up to 200 tokens 0.99-1.01, 99 rows 1.00-1.01, four sequences of 35 rows on
+      // 64-900 tokens 0.95-0.99; twelve of 12 rows 0.94 at 64 tokens, 0.84 at 1200; the whole shape, us per step: 1 row at 128 tokens
+      // 2724 / 2850; 35 rows at 512 3242 / 3441, at 8192 4185 / 6208; 131 rows at 2047 5850 / 6890.
       const bool tc = dh == 128 && c->attn_tc != 0;
       if (tc) {
         a.tc = attention_tc_plan(act * G, rw.n_seq * Hkv, (ra.n_hi_max + act + kAttnTcTile - 1) / kAttnTcTile, rw.prompt, c->sm_count);
         a.splits = a.tc.splits;
       }
       FIRP_TIMED(KC_ATTENTION);
-      FIRP_CUDA(c, tc ? launch_attention_tc(a, pdl, st) : launch_attention(a, pdl, st)); ++nl;
+      FIRP_CUDA(c, tc ? launch_attention_tc(a, pdl, st) : launch_attention(a, pdl && attention_early(dh, act, tiles), st)); ++nl;
     }
     {
       FIRP_TIMED(KC_GEMM_O);

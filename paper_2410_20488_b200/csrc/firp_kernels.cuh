@@ -239,6 +239,7 @@ struct AttnArgs {
 // kv splits for `groups` = sequences x kv heads x query blocks and `kv_tiles` 64-position tiles
 int attention_splits(int groups, int kv_tiles);
 cudaError_t launch_attention(const AttnArgs &a, bool pdl, cudaStream_t st);
+bool attention_early(int dh, int rows, int kv_tiles);     // whether its early launch pays: rows of a sequence, 64-position tiles
 // The tcgen05 kernels (head dimension 128): 128-position tiles, query rows x heads of the group in blocks of at most
 // kAttnTcMaxCols or 128; a.tc and a.splits from attention_tc_plan.  seq_heads = sequences x kv heads.
 constexpr int kAttnTcTile = 128, kAttnTcMaxCols = 48;

@@ -34,6 +34,7 @@
 #include "firp_kernels.cuh"
 #include "launch_util.cuh"
 #include "norm_device.cuh"
+#include "pipeline.h"
 #include "tc_device.cuh"
 
 namespace firp {
@@ -135,6 +136,13 @@ __device__ __forceinline__ void grid_sync(unsigned *ctr, unsigned &epoch, int wt
   WorkerSync::sync();             // the acquire of thread 0 reaches the other workers through this barrier
 }
 
+// A producer's loads of the step: after a wait that ran out it starts no more, and it leaves only when what it has started has
+// landed (pipeline.h).
+struct StepRing {
+  uint32_t full; int *err;
+  __device__ __forceinline__ void landed(int slot, uint32_t parity) { mbar_drain(full + 8 * slot, parity, err); }
+};
+
 template <int NPAD>
 __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid_constant__ FusedParams P) {
   constexpr int X_PLANE = NPAD * 128;          // bytes of one activation plane of a stage
@@ -183,7 +191,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
       int k = 0;
-      for (int g = 0; g < P.n_gemm; ++g) {
+      for (int g = 0; g < P.n_gemm && !dead; ++g) {
         const GemmClass &c = P.cls[P.gemm_cls[g]];
         const CUtensorMap *tm = P.maps + P.gemm_map[g];
         const StreamK sk{c.U, c.KB, c.G};
@@ -192,7 +200,7 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
           const int u = u0 + it;
           const int st = u / c.KB, kb = u - st * c.KB;
           const int sl = k % SW;
-          mbar_wait(empty_w + 8 * sl, ((k / SW) & 1) ^ 1, P.err, dead, wait_ns);
+          if (!mbar_wait(empty_w + 8 * sl, ((k / SW) & 1) ^ 1, P.err, dead, wait_ns)) break;
           mbar_expect_tx(full_w + 8 * sl, W_STAGE);
           const uint32_t dst = w_ring + sl * W_STAGE, bar = full_w + 8 * sl;
           if (c.mode == ROWS_ROTARY) {
@@ -208,6 +216,8 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
           }
         }
       }
+      StepRing ring{full_w, P.err};
+      drain(ring, k, SW);
     }
   } else if (warp == 6) {
     if (lane == 0) {             // ---- activation producer
@@ -215,27 +225,29 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
       asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
       const int xrows = min((P.rw.R + 7) & ~7, NPAD);
       int k = 0;
-      for (int g = 0; g < P.n_gemm; ++g) {
+      for (int g = 0; g < P.n_gemm && !dead; ++g) {
         const GemmClass &c = P.cls[P.gemm_cls[g]];
         const CUtensorMap *tm = P.maps + c.xmap;
         const StreamK sk{c.U, c.KB, c.G};
         const int u0 = cta < c.G ? sk_begin(sk, cta) : 0, n_units = cta < c.G ? sk_begin(sk, cta + 1) - u0 : 0;
-        mbar_wait(xgo, g & 1, P.err, dead, wait_ns);     // the workers have passed the barrier before this GEMM
+        if (!mbar_wait(xgo, g & 1, P.err, dead, wait_ns)) break;     // the workers have passed the barrier before this GEMM
         fence_proxy_async();
         for (int it = 0; it < n_units; ++it, ++k) {
           const int kb = (u0 + it) % c.KB;
           const int sl = k % SX;
-          mbar_wait(empty_x + 8 * sl, ((k / SX) & 1) ^ 1, P.err, dead, wait_ns);
+          if (!mbar_wait(empty_x + 8 * sl, ((k / SX) & 1) ^ 1, P.err, dead, wait_ns)) break;
           mbar_expect_tx(full_x + 8 * sl, c.P * xrows * 128);
           const uint32_t dst = x_ring + sl * X_STAGE;
           for (int pl = 0; pl < c.P; ++pl)
             tma_load_2d(dst + pl * X_PLANE, tm, kb * BK, pl * P.Rp, full_x + 8 * sl, pol);
         }
       }
+      StepRing ring{full_x, P.err};
+      drain(ring, k, SX);
     }
   } else if (warp == 1) {
     if (lane == 0) {             // ---- MMA issuer
-      int kw = 0;
+      int kw = 0, last = -1;
       unsigned use[2] = {0u, 0u};
       for (int g = 0; g < P.n_gemm; ++g) {
         const GemmClass &c = P.cls[P.gemm_cls[g]];
@@ -273,10 +285,12 @@ __global__ void __launch_bounds__(kFThreads, 1) fused_layers_kernel(const __grid
           }
           tc_commit(acc_full + 8 * buf);
           ++use[buf];
+          last = buf;
           u += kb1 - kb0;
           ++seg;
         }
       }
+      if (last >= 0) mbar_drain(acc_full + 8 * last, (use[last] - 1u) & 1u, P.err);      // no MMA outlives the CTA
     }
   } else {                       // ---- workers: warps 2..5 (group A) and 7..10 (group B)
     const int wgroup = warp >= 7 ? 1 : 0;

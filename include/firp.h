@@ -95,7 +95,9 @@ int firp_create(const firp_model_cfg *cfg, firp_ctx **out);
 void firp_destroy(firp_ctx *ctx);
 const char *firp_last_error(const firp_ctx *ctx);
 
-/* Bytes of device memory the caller must provide: scratch workspace and bf16 KV cache
+/* Bytes of device memory the caller must provide: scratch workspace and bf16 KV cache.  The workspace holds the
+ * activations of a stretch of a prompt, whether or not the context ever prefills: at head_dim 128 min(max_ctx, 2047) rows
+ * (about 390 MB at the shape of a 7B model, 665 MB at that of a 34B model, from 2048 positions on), otherwise 144.
  * (layout [layer][K|V][row][kv_head][head_dim] with row = slot * max_ctx + position, or, with a page table
  * (firp_set_kv_pages), row = page * 64 + position % 64). */
 size_t firp_workspace_bytes(const firp_ctx *ctx);
@@ -302,9 +304,10 @@ int firp_last_launch_count(const firp_ctx *ctx);
 /*
  * Per-kernel timing aid (measurement only; it changes no result).  While enabled, every kernel
  * launch of firp_step / firp_prefill / firp_kv_commit is bracketed by a pair of CUDA events on
- * the call's stream, grouped by kernel class (the steps of Section 3.2-3.4: tree bookkeeping,
- * embedding, residual + RMSNorm, Eq. 3 projection, the five weight-streaming GEMMs and their
- * finishers, tree attention, top-B, acceptance walk, KV compaction).  The events serialise launches that otherwise overlap, so a
+ * the call's stream, grouped by kernel class (the steps of Section 3.2-3.4: tree bookkeeping with
+ * the embedding, Eq. 3 projection, the five weight-streaming GEMMs with the elementwise steps behind them, tree
+ * attention, top-B, acceptance walk, KV compaction).  The classes embed, residual_rmsnorm, qkv_rope_finish,
+ * swiglu_finish and logits_finish have no kernel of their own any more and stay at zero.  The events serialise launches that otherwise overlap, so a
  * profiled step is slower than an unprofiled one: use it for per-kernel durations, not for the
  * step latency.
  *   firp_profile_enable  on != 0 starts (and clears) the collection, 0 stops it.

@@ -29,7 +29,8 @@ struct Carver {
 
 }  // namespace
 
-// Kernel classes of the per-kernel timing aid (firp_profile_*).
+// Kernel classes of the per-kernel timing aid (firp_profile_*).  Their indices are part of the ABI: embedding, norm and finishers, which
+// have become part of other kernels, keep theirs and are never timed.
 enum KernelClass {
   KC_TREE_PREP = 0, KC_EMBED, KC_RMSNORM, KC_PSEUDO_PROJ, KC_GEMM_QKV, KC_QKV_FINISH, KC_ATTENTION, KC_GEMM_O,
   KC_GEMM_GATE_UP, KC_SWIGLU_FINISH, KC_GEMM_DOWN, KC_GEMM_LM_HEAD, KC_LOGITS_FINISH, KC_TOPB, KC_ACCEPT, KC_COMMIT, KC_FUSED_LAYERS, KC_COUNT

@@ -14,7 +14,6 @@ constexpr int kMaxPromptRows = 2047;  // rows of a prompt that run at once, pseu
 constexpr int kMaskWords = 5;      // ceil(136 / 32)
 constexpr int kMaxTopB = 8;
 constexpr int kAttnTile = 64;      // kv positions per attention tile
-constexpr int kGemmBN = 64;        // weight rows per GEMM tile
 constexpr int kGemmBK = 64;        // k elements per pipeline stage
 
 // Per-step row geometry shared by every kernel.  Row r = s * Ms + v.

@@ -91,22 +91,6 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *tm,
       "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %3, %3, %4}], [%5], %6;"
       ::"r"(dst), "l"(tm), "r"(x), "r"(0), "r"(v), "r"(bar), "l"(policy) : "memory");
 }
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *tm, int x, int y, int z, uint64_t policy) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %3}], %4;"
-               ::"l"(tm), "r"(x), "r"(y), "r"(z), "l"(policy) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_5d(const CUtensorMap *tm, int x, int v, uint64_t policy) {
-  asm volatile("cp.async.bulk.prefetch.tensor.5d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %2, %2, %3}], %4;"
-               ::"l"(tm), "r"(x), "r"(0), "r"(v), "l"(policy) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int x, int y, uint64_t policy) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile.L2::cache_hint [%0, {%1, %2}], %3;"
-               ::"l"(tm), "r"(x), "r"(y), "l"(policy) : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap *tm, int x, int y, int z, int w, uint64_t policy) {
-  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %3, %4}], %5;"
-               ::"l"(tm), "r"(x), "r"(y), "r"(z), "r"(w), "l"(policy) : "memory");
-}
 // true in one lane of a converged warp
 __device__ __forceinline__ bool elect_one() {
   uint32_t ok;

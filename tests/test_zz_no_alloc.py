@@ -1,8 +1,8 @@
 """firp_topb_static -- the entry point that allocates nothing -- against firp_step.
 
 Some hosts of this library may not allocate device memory while decoding (a serving loop with a
-memory pool fixed at start-up, a plug-in that only ever receives buffers from its host), so this
-one call keeps its scratch in a fixed array inside the library.  Here it is run, through the C ABI,
+memory pool fixed at start-up, a plug-in that only ever receives buffers from its host), and this
+one call needs no memory besides its arguments.  Here it is run, through the C ABI,
 on the logits that firp_step exported, twice in a row on different logits, and must reproduce the
 selections firp_step made from the same rows: the greedy token of every tree row and the ordered
 top-B ids and values of every pseudo row, exactly (both paths select from the same fp32 numbers).
@@ -32,7 +32,7 @@ def test_static_topb_matches_step_twice_in_a_row(c1, c1_weights):
     ids = torch.full((T + k, B), -1, dtype=torch.int32, device="cuda")
     vals = torch.zeros((T + k, B), dtype=torch.float32, device="cuda")
     tokens = pout.next_tree_tokens[0].clone()
-    for call in range(2):                     # two calls in a row share the built-in scratch
+    for call in range(2):                     # two calls in a row
         eng.step(tokens, parents, k, c1.l, out)
         ids.fill_(-1)
         firp_topb_static(out.logits.data_ptr(), T + k, V, B, ids.data_ptr(), vals.data_ptr(), eng.stream)

@@ -98,8 +98,8 @@ const char *firp_last_error(const firp_ctx *ctx);
 /* Bytes of device memory the caller must provide: scratch workspace and bf16 KV cache.  The workspace holds the
  * activations of a stretch of a prompt, whether or not the context ever prefills: at head_dim 128 min(max_ctx, 2047) rows
  * (about 390 MB at the shape of a 7B model, 665 MB at that of a 34B model, from 2048 positions on), otherwise 144.
- * (layout [layer][K|V][row][kv_head][head_dim] with row = slot * max_ctx + position, or, with a page table
- * (firp_set_kv_pages), row = page * 64 + position % 64). */
+ * The cache's layout is [layer][K|V][row][kv_head][head_dim] with row = slot * max_ctx + position, or, with a page table
+ * (firp_set_kv_pages), row = page * 64 + position % 64. */
 size_t firp_workspace_bytes(const firp_ctx *ctx);
 size_t firp_kv_bytes(const firp_ctx *ctx);
 

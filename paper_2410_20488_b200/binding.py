@@ -239,12 +239,12 @@ def firp_set_attention_planes(ctx, q_planes=2, p_planes=2):
 
 
 def firp_set_attention_kernel(ctx, tensor_core=None):
-    """True: the tcgen05 kernel, False: the mma.sync kernel, None: chosen per step (the default)."""
+    """Head dimension 128: True or None (the default) the tcgen05 kernels, False the mma.sync kernel."""
     _check(ctx, load_library().firp_set_attention_kernel(ctx, -1 if tensor_core is None else (1 if tensor_core else 0)))
 
 
 def firp_set_fused(ctx, on: bool):
-    """Run the layers of small steps as one persistent kernel (default) or one kernel per operation."""
+    """Run the layers of small steps as one persistent kernel, or (the default) one kernel per operation."""
     _check(ctx, load_library().firp_set_fused(ctx, int(bool(on))))
 
 

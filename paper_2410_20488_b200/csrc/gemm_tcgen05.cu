@@ -12,7 +12,8 @@
 // weights costs 1-3 % of the stream, while shares that end in mid-tile cost a pass over fp32 partial tiles in global
 // memory, a kernel of its own to sum them and a hand-over: 7 us after the QKV, gate/up and down projections and 14 us after
 // the O projection at 35 rows of the 7B shape, 37 of 102 us per layer.  Step at the 7B shape, 35 rows, 512 cached tokens:
-// 3534 -> 3121 us; one row 3062 -> 2696; 13B shape, 67 rows 8958 -> 6734; 34B shape, 140 rows 6631 -> 6230.
+// 3534 -> 3121 us; one row 3062 -> 2696; 13B shape, 67 rows 8958 -> 6734; 34B shape, 140 rows 6631 -> 6230.  (With the limit on a
+// step's sums, in turn on one box: 3133 -> 3163, 2706 -> 2728, 6532 -> 6518, 6045 -> 6118.)
 //
 // A prompt comes as one stretch of up to 2047 rows, in blocks of up to 256: the weights, 13.5 GB at the 7B shape, are read
 // once instead of once per 141 rows.  It is bound by the MMA issue of two passes over the bf16 planes: 1999 tokens of the 7B
@@ -29,7 +30,8 @@
 //   warps 1, 3 : MMA issuers: tcgen05.mma kind::f16, M = 128, K = 16.  The planes of the activations (hi, lo) either sit
 //                side by side as ONE operand of N = planes x npad columns (added in the epilogue) or are accumulated
 //                one after the other into npad columns.  The whole warp runs the loop and an elected lane issues, which
-//                keeps the descriptors in uniform registers (M = 128, N = 80: 59 cycles per MMA; one lane alone: 86).
+//                keeps the descriptors in uniform registers (M = 128, N = 80: 59 cycles per MMA; one lane alone: 86).  One of them
+//                issues alone where a job has one tile of one accumulator set, or of three.
 //   warps 4-11 : epilogue.  TMEM -> shared memory of the CTA of the cluster that finishes the token row (the ring's
 //                memory, no longer needed), cluster barrier, sum over the k slices in rank order, then the fused step:
 //                residual + RMSNorm operand, rotary + cache, SwiGLU, logits, or Eq. 3.

@@ -74,7 +74,7 @@ __device__ __forceinline__ void attn_split_item(const AttnArgs &a, uint8_t *smem
     const int i = ch / CH, c = ch % CH;
     const int qr = qb * kAttnQRows + i;
     const bool valid = qr < qrows_total;
-    const bf16 *src = valid ? a.q + ((size_t)(s * a.rw.Ms + qr / G) * a.H + kvh * G + qr % G) * DH + c * 8 : a.q;
+    const bf16 *src = valid ? a.q + ((size_t)act_row(a.rw, s, qr / G) * a.H + kvh * G + qr % G) * DH + c * 8 : a.q;
     cp_async_16(attn_smem_u32(sQ + tile_off<DH>(i, c)), src, valid);
     cp_async_16(attn_smem_u32(sQ + Q_BYTES + tile_off<DH>(i, c)), valid ? src + a.q_lo_off : a.q, valid);
   }

@@ -218,7 +218,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const int idx = it * kTcSoft + tid, j = idx >> 4, c = idx & 15, qr = q0 + j;
       qh[it] = make_uint4(0u, 0u, 0u, 0u); ql[it] = qh[it];
       if (j < ncols) {
-        const bf16 *src = a.q + ((size_t)(s * a.rw.Ms + qr / G) * a.H + kvh * G + qr % G) * kTcDh + c * 8;
+        const bf16 *src = a.q + ((size_t)act_row(a.rw, s, qr / G) * a.H + kvh * G + qr % G) * kTcDh + c * 8;
         qh[it] = *reinterpret_cast<const uint4 *>(src);
         ql[it] = *reinterpret_cast<const uint4 *>(src + a.q_lo_off);
       }
@@ -316,7 +316,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       mbar_arrive(q_ready);
       if (tid < ncols) {
         const int qr = q0 + tid;
-        s_oidx[tid] = (uint32_t)(((s * a.rw.Ms + qr / G) * a.H + kvh * G + qr % G) * kTcDh);
+        s_oidx[tid] = (uint32_t)((act_row(a.rw, s, qr / G) * a.H + kvh * G + qr % G) * kTcDh);
       }
     }
     TC_STAMP(2);
@@ -624,7 +624,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   if (warp < 16) {
     for (int j = tid >> 4; j < ncols; j += 32) {
       const int c = tid & 15, qr = q0 + j;
-      const bf16 *src = a.q + ((size_t)(s * a.rw.Ms + qr / G) * a.H + kvh * G + qr % G) * kTcDh + c * 8;
+      const bf16 *src = a.q + ((size_t)act_row(a.rw, s, qr / G) * a.H + kvh * G + qr % G) * kTcDh + c * 8;
       const uint4 qh = *reinterpret_cast<const uint4 *>(src), ql = *reinterpret_cast<const uint4 *>(src + a.q_lo_off);
       const int off = Q_OFF + (c >> 3) * kTcSlab + j * 128 + (((c & 7) ^ (j & 7)) << 4);
       *reinterpret_cast<uint4 *>(base + off) = qh;
@@ -636,7 +636,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       s_m[tid] = -INFINITY;
       if (tid < ncols) {
         const int qr = q0 + tid;
-        s_oidx[tid] = (uint32_t)(((s * a.rw.Ms + qr / G) * a.H + kvh * G + qr % G) * kTcDh);
+        s_oidx[tid] = (uint32_t)((act_row(a.rw, s, qr / G) * a.H + kvh * G + qr % G) * kTcDh);
       }
     }
   }

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kAttnThreads) tree_attn_kernel(AttnArgs a, int
       const float inv = (L > 0.f) ? 1.f / L : 0.f;
       const float val[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
       const int qr = qb * kAttnQRows + i;
-      const int r = s * a.rw.Ms + qr / G, head = kvh * G + qr % G;
+      const int r = act_row(a.rw, s, qr / G), head = kvh * G + qr % G;
       const __nv_bfloat162 h01 = __floats2bfloat162_rn(val[0], val[1]), h23 = __floats2bfloat162_rn(val[2], val[3]);
       const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
       const __nv_bfloat162 l01 = __floats2bfloat162_rn(val[0] - f01.x, val[1] - f01.y);

@@ -112,6 +112,7 @@ struct firp_ctx {
     meta.pos = c.take<int32_t>(R);
     meta.mask = c.take<uint32_t>(Rt * kMaskWords);
     meta.rope = c.take<float2>(R * half);
+    meta.row_of = c.take<uint16_t>(Rt);
     ctx_len = c.take<int32_t>(cfg.max_batch);
     seq_ids = c.take<int32_t>(kMaxSeq);
     parents = c.take<int32_t>(kMaxTreeRows);
@@ -219,7 +220,7 @@ struct RunArgs {
 
 int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
   const firp_model_cfg &cfg = c->cfg;
-  const Rows &rw = ra.rw;
+  Rows rw = ra.rw;
   const int d = cfg.d_model, H = cfg.n_heads, Hkv = cfg.n_kv_heads, dh = cfg.head_dim, F = cfg.d_ffn;
   const int nq = H * dh;
   const size_t Rp = (size_t)c->Rmax;          // rows per activation plane
@@ -228,6 +229,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
   const bool pdl = c->use_pdl;
   const FusedShape fshape{cfg.n_layers, d, H, Hkv, dh, F, cfg.vocab, cfg.max_ctx, cfg.rms_eps};
   const bool fused = c->use_fused && fused_eligible(fshape, rw);
+  rw.by_step = !fused && rw.n_seq > 1;                         // one sequence's rows go by step as they are
   const int per_step = rw.chains ? rw.T : 1;                   // pseudo rows one prediction step adds per sequence
   const int x_planes = c->planes[0] == 3 ? 3 : 2;              // of the QKV projection's operand
   { FIRP_TIMED(KC_TREE_PREP);
@@ -263,8 +265,8 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
   }
 
   enum { G_QKV = 0, G_O, G_GATE_UP, G_DOWN, G_LM_HEAD };     // index of c->planes
-  auto launch = [&](GemmEpilogue epi, const void *W, int N, int K, int planes, const Rows &rows, LinArgs &l, int R = 0) -> cudaError_t {
-    l.W = (const bf16 *)W; l.N = N; l.K = K; l.R = R ? R : rows.R; l.rw = rows; l.F = F; l.dh = dh; l.planes = planes; l.plane_rows = (int)Rp;
+  auto launch = [&](GemmEpilogue epi, const void *W, int N, int K, int planes, const Rows &rows, LinArgs &l, int R) -> cudaError_t {
+    l.W = (const bf16 *)W; l.N = N; l.K = K; l.R = R; l.rw = rows; l.row_of = rows.by_step ? c->meta.row_of : nullptr; l.F = F; l.dh = dh; l.planes = planes; l.plane_rows = (int)Rp;
     l.err = c->dev_status; l.wait_ns = c->wait_ns; l.eps = cfg.rms_eps;
     ++nl;
     return launch_gemm(epi, l, pdl, st);
@@ -284,7 +286,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
                      // tree row when each node carries a chain), on the raw residual or (pre-norm) on its normalised rows
       FIRP_TIMED(KC_PSEUDO_PROJ);
       LinArgs l{};
-      l.X = c->xp; l.rows_active = act; l.pseudo0 = alive;     // map i of this GEMM is prediction step alive + i
+      l.X = c->xp; l.pseudo0 = alive;     // map i of this GEMM is prediction step alive + i
       if (c->pred_prenorm) l.ss = c->ss;
       l.pred_b = c->w.pred_b ? (const bf16 *)c->w.pred_b + (size_t)alive * d : nullptr;
       residual_out(l, c->g_attn[j], x_planes);
@@ -295,10 +297,10 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
     {
       FIRP_TIMED(KC_GEMM_QKV);
       LinArgs l{};
-      l.X = c->x; l.ss = c->ss; l.rows_active = act;
+      l.X = c->x; l.ss = c->ss;
       l.H = H; l.Hkv = Hkv; l.rope = c->meta.rope; l.seq_ids = c->seq_ids; l.pos = c->meta.pos;
       l.q = c->q; l.q_plane = Rp * nq; l.kcache = kplane; l.kv_stride = c->kv_plane(); l.max_ctx = cfg.max_ctx; l.pages = c->pages();
-      FIRP_CUDA(c, launch(EPI_QKV_ROPE, c->wqkv[j], (H + 2 * Hkv) * dh, d, c->planes[G_QKV], rw, l));
+      FIRP_CUDA(c, launch(EPI_QKV_ROPE, c->wqkv[j], (H + 2 * Hkv) * dh, d, c->planes[G_QKV], rw, l, rw.n_seq * act));
     }
     {
       AttnArgs a{};
@@ -325,20 +327,20 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
     {
       FIRP_TIMED(KC_GEMM_O);
       LinArgs l{};
-      l.X = c->o; l.rows_active = act;
+      l.X = c->o;
       residual_out(l, c->g_mlp[j], 2);
-      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wo[j], d, nq, c->planes[G_O], rw, l));
+      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wo[j], d, nq, c->planes[G_O], rw, l, rw.n_seq * act));
     }
     {
       FIRP_TIMED(KC_GEMM_GATE_UP);
       LinArgs l{};
-      l.X = c->x; l.ss = c->ss; l.rows_active = act; l.y = c->y; l.y_plane = Rp * F;
-      FIRP_CUDA(c, launch(EPI_SWIGLU, c->wgu[j], 2 * F, d, c->planes[G_GATE_UP], rw, l));
+      l.X = c->x; l.ss = c->ss; l.y = c->y; l.y_plane = Rp * F;
+      FIRP_CUDA(c, launch(EPI_SWIGLU, c->wgu[j], 2 * F, d, c->planes[G_GATE_UP], rw, l, rw.n_seq * act));
     }
     {
       FIRP_TIMED(KC_GEMM_DOWN);
       LinArgs l{};
-      l.X = c->y; l.rows_active = act;
+      l.X = c->y;
       if (j + 1 < cfg.n_layers) {
         residual_out(l, c->g_attn[j + 1], x_planes);
         if (ins_next > 0) { l.xp = c->xp; l.xp_plane = Rp * d; l.xp_normed = c->pred_prenorm; }
@@ -347,7 +349,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
       } else {
         l.h = c->h; l.d = d;     // nothing reads the stream after the last layer of a prompt's inner chunk
       }
-      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wd[j], d, F, c->planes[G_DOWN], rw, l));
+      FIRP_CUDA(c, launch(EPI_RESIDUAL, c->wd[j], d, F, c->planes[G_DOWN], rw, l, rw.n_seq * act));
     }
   }
   if (ra.want_head) {
@@ -358,8 +360,8 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
     if (!fused) {
       FIRP_TIMED(KC_GEMM_LM_HEAD);
       LinArgs l{};
-      l.X = c->x + (size_t)first * d; l.ss = c->ss + (size_t)first * kNormMaxWarps; l.rows_active = hr.Ms; l.logits = ra.logits_dst;
-      FIRP_CUDA(c, launch(EPI_LOGITS, c->w.lm_head, cfg.vocab, d, c->planes[G_LM_HEAD], hr, l));
+      l.X = c->x + (size_t)first * d; l.ss = c->ss + (size_t)first * kNormMaxWarps; l.logits = ra.logits_dst;
+      FIRP_CUDA(c, launch(EPI_LOGITS, c->w.lm_head, cfg.vocab, d, c->planes[G_LM_HEAD], hr, l, hr.R));
     }
     { FIRP_TIMED(KC_TOPB);
       launch_topb(ra.logits_dst, hr.R, cfg.vocab, cfg.top_b, c->top_ids, c->top_vals, pdl, st); ++nl; }

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "rows.h"
+
 namespace firp {
 
 typedef __nv_bfloat16 bf16;
@@ -15,21 +17,6 @@ constexpr int kMaskWords = 5;      // ceil(136 / 32)
 constexpr int kMaxTopB = 8;
 constexpr int kAttnTile = 64;      // kv positions per attention tile
 constexpr int kGemmBK = 64;        // k elements per pipeline stage
-
-// Per-step row geometry shared by every kernel.  Row r = s * Ms + v.
-struct Rows {
-  int n_seq;   // sequences in this step
-  int T;       // tree rows per sequence
-  int k;       // pseudo rows per sequence
-  int Ms;      // T + k
-  int R;       // n_seq * Ms
-  int anchor;  // tree row the pseudo chain hangs off (one chain)
-  int chains;  // != 0: a chain under every tree node; chain row i (1-based) of node v is row T + (i-1) T + v
-  int kc;      // prediction steps per chain (k = kc with one chain, k = T * kc with a chain per node)
-  int masked;  // != 0: a pseudo row sees no other pseudo row (the "Masked" ablation of Section 4.3)
-  int prompt;  // != 0: a stretch of a prompt: one sequence, rows 0 .. T-1 a chain, the pseudo rows behind it; more rows than a
-               // tree may have, no masks in TreeMeta (row v sees the rows up to itself)
-};
 
 // Rows of the KV cache.  A (layer, K|V) plane holds max_batch * max_ctx rows of Hkv * dh elements.  Without a
 // page table position `pos` of slot `slot` is row slot * max_ctx + pos; with one (pages of kKvPage positions,
@@ -73,7 +60,8 @@ struct TreeMeta {
   int32_t *depth;      // [R]
   int32_t *pos;        // [R] absolute position = ctx_len + depth
   uint32_t *mask;      // [R][kMaskWords] bit u: row v attends to new row u of its sequence
-  float2 *rope;        // [R][dh/2] (cos, sin) of pos * theta^(-2c/dh)
+  float2 *rope;        // [R][dh/2] (cos, sin) of pos * theta^(-2c/dh), by row of the activations
+  uint16_t *row_of;    // [R] seq_row of each row of the activations
 };
 struct PrepArgs {
   Rows rw;
@@ -152,8 +140,9 @@ struct LinArgs {
   const bf16 *X;    // [planes][plane_rows][K] activations as bf16 planes
   int plane_rows, planes;
   const bf16 *W;    // [N][K] weights
-  int R, N, K;      // token rows (<= kMaxPromptRows)
-  Rows rw; int rows_active;      // rows with v < rows_active are written, the others skipped
+  int R, N, K;      // token rows (<= kMaxPromptRows): the first R of the activations
+  Rows rw;
+  const uint16_t *row_of;       // seq_row of every row of the activations; NULL: one sequence, row v is row v
   int *err;         // device status word (set to a non-zero code if a bounded wait gives up)
   unsigned long long wait_ns;   // bounded waits give up after this many nanoseconds (0: the default of 2 s)
   // X holds h * g, not yet divided by the RMS: row m of the result is scaled by 1 / sqrt(sum_w ss[m][w] / K + eps)
@@ -167,8 +156,8 @@ struct LinArgs {
   const bf16 *g; bf16 *x; size_t x_plane; int x_planes; float *ss_out;
   bf16 *xp; size_t xp_plane; int xp_normed;
   // EPI_PSEUDO (Eq. 3): output n = i * d + o of map pseudo0 + i (+ pred_b[n]).  One chain: token row m = sequence m, result
-  // to h row m * Ms + T + pseudo0 + i.  A chain per node: token row m = s * T + v, result to h row
-  // s * Ms + T + (pseudo0 + i) * T + v.
+  // to h row act_row(m, T + pseudo0 + i).  A chain per node: token row m = s * T + v, result to h row
+  // act_row(s, T + (pseudo0 + i) * T + v).
   const bf16 *pred_b; int pseudo0;
   // EPI_QKV_ROPE
   int H, Hkv, dh;
@@ -178,13 +167,12 @@ struct LinArgs {
   KvPages pages;
   // EPI_SWIGLU: y[R][F], N = 2F
   bf16 *y; size_t y_plane; int F;
-  // EPI_LOGITS: logits[R][N]
+  // EPI_LOGITS: logits[n_seq * Ms][N], rows as the caller counts them
   float *logits;
 };
-// row of ss that belongs to token row m (Eq. 3 multiplies rows of the residual stream that lie elsewhere)
+// row of ss that belongs to token row m (Eq. 3 multiplies rows of the residual stream: all tree rows, or each sequence's anchor)
 template <int EPI> __device__ __forceinline__ int lin_src_row(const LinArgs &a, int m) {
-  if (EPI != EPI_PSEUDO) return m;
-  return a.rw.chains ? m / a.rw.T * a.rw.Ms + m % a.rw.T : m * a.rw.Ms + a.rw.anchor;
+  return EPI == EPI_PSEUDO && !a.rw.chains ? act_row(a.rw, m, a.rw.anchor) : m;
 }
 // pdl: launch with programmatic stream serialization (the kernel waits on its predecessor itself).
 cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream_t st);

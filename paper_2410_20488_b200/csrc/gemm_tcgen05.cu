@@ -183,7 +183,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   const uint32_t w_ring = base, x_ring = base + cf.sw * W_TILE;
   float *s_rs = reinterpret_cast<float *>(data + cf.tail);          // 1 / RMS of every token row
   int *s_slot = reinterpret_cast<int *>(s_rs + kMaxRows), *s_pos = s_slot + kMaxSeq;      // of every sequence
-  uint16_t *s_row = reinterpret_cast<uint16_t *>(s_pos + kMaxSeq);                        // sequence << 11 | row of every token row
+  uint16_t *s_row = reinterpret_cast<uint16_t *>(s_pos + kMaxSeq);                        // seq_row of every token row, 0xffff: none
   const uint32_t bars = base + cf.tail + kMaxRows * 6 + 2 * kMaxSeq * 4;
   const uint32_t full_w = bars, empty_w = full_w + 8 * kMaxW, full_x = empty_w + 8 * kMaxW, empty_x = full_x + 8 * kMaxX,
                  acc_full = empty_x + 8 * kMaxX, rope_full = acc_full + 8, tmem_slot = rope_full + 8;
@@ -317,17 +317,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       s_slot[lane] = __ldcg(a.seq_ids + lane);
       s_pos[lane] = __ldcg(a.pos + lane * a.rw.Ms);      // committed length (position of the root row)
     }
-    // of every row this CTA finishes: its sequence and row (0xffff: none, or not to be written), and
+    // of every row this CTA finishes: its sequence and row (0xffff: none), and
     // 1 / sqrt(mean(h^2) + eps) from the per-128-column sums of squares, added in a fixed order
-    const int nw = a.K >> 7, per = EPI == EPI_PSEUDO ? (a.rw.chains ? a.rw.T : 1) : a.rw.Ms;
+    const int nw = a.K >> 7;
     const int m_end = min(kMaxRows, own0 + ((n_own + 15) & ~15));
     for (int m0 = own0 + ew; m0 < m_end; m0 += 4 * kEpiWarps) {
       float v[4];
+      uint16_t w[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
+        const int r = row0 + min(m0 + u * kEpiWarps, R - 1);
+        w[u] = EPI == EPI_PSEUDO && !a.rw.chains ? seq_row(r, 0) : a.row_of ? __ldcg(a.row_of + r) : seq_row(0, r);
         v[u] = 0.f;
         if (a.ss == nullptr) continue;
-        const float *p = a.ss + (size_t)lin_src_row<EPI>(a, row0 + min(m0 + u * kEpiWarps, R - 1)) * kNormMaxWarps;
+        const float *p = a.ss + (size_t)lin_src_row<EPI>(a, r) * kNormMaxWarps;
         v[u] = (lane < nw ? __ldcg(p + lane) : 0.f) + (lane + 32 < nw ? __ldcg(p + lane + 32) : 0.f);
       }
 #pragma unroll
@@ -337,8 +340,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         const int m = m0 + u * kEpiWarps;
         if (lane == 0 && m < m_end) {
           s_rs[m] = a.ss ? rsqrtf(v[u] / (float)a.K + a.eps) : 1.f;
-          const int s = (row0 + m) / per, row = row0 + m - s * per;
-          s_row[m] = (uint16_t)(m < own0 + n_own && (EPI == EPI_PSEUDO || row < a.rows_active) ? s << 11 | row : 0xffff);
+          s_row[m] = m < own0 + n_own ? w[u] : 0xffff;
         }
       }
     }
@@ -433,13 +435,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
           for (int q = 0; q < 4; ++q) *reinterpret_cast<float4 *>(rs + 4 * q) = *reinterpret_cast<const float4 *>(s_rs + c0 + 4 * q);
 #pragma unroll
           for (int q = 0; q < 2; ++q) *reinterpret_cast<uint4 *>(row + 4 * q) = *reinterpret_cast<const uint4 *>(s_row + c0 + 8 * q);
-          auto row_of = [&](int j) { return (int)((row[j >> 1] >> (16 * (j & 1))) & 0xffffu); };       // 0xffff: not to be written
+          auto row_of = [&](int j) { return (int)((row[j >> 1] >> (16 * (j & 1))) & 0xffffu); };       // 0xffff: none
           if (EPI == EPI_LOGITS) {
             const int n = tile * BM + rowi;
-            float *dst = a.logits + (size_t)(row0 + c0) * a.N + n;
             if (n < a.N) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) if (row_of(j) != 0xffff) dst[(size_t)j * a.N] = r[j] * rs[j];
+              for (int j = 0; j < 16; ++j) {
+                const int w = row_of(j);
+                if (w != 0xffff) a.logits[(size_t)(row_seq(w) * a.rw.Ms + row_in_seq(w)) * a.N + n] = r[j] * rs[j];
+              }
             }
           } else if (EPI == EPI_SWIGLU) {
             const int n = (tile >> 1) * BM + rowi;
@@ -488,8 +492,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
               for (int j = 0; j < 16; ++j) {
                 const int w = row_of(j);
                 if (w != 0xffff) {
-                  const int pos = s_pos[w >> 11] + (w & 2047);
-                  if (pos < a.max_ctx) dst[kv_row(a.pages, s_slot[w >> 11], pos, a.max_ctx) * stride] = __float2bfloat16_rn(r[j]);
+                  const int pos = s_pos[row_seq(w)] + row_in_seq(w);
+                  if (pos < a.max_ctx) dst[kv_row(a.pages, s_slot[row_seq(w)], pos, a.max_ctx) * stride] = __float2bfloat16_rn(r[j]);
                 }
               }
             }
@@ -556,7 +560,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     if (EPI == EPI_RESIDUAL) {
       // a warp per (token row, tile), 4 neighbouring columns per lane
       auto finish = [&](int loc, int n0, float4 v, float sq) {
-        const int row = s_row[own0 + loc], s = row >> 11, w = row & 2047;
+        const int row = s_row[own0 + loc], s = row_seq(row), w = row_in_seq(row);
         if (row == 0xffff) return;
         int xp_row = -1;
         if (a.xp != nullptr) {
@@ -614,7 +618,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     int loc = loc0, tl = loc0 >= n_own ? tp : 0;
 #pragma unroll 1
     while (tl < tp) {
-      const int lm = own0 + loc, m = row0 + lm, tile = wk.t0 + p0 + tl, row = s_row[lm], s = row >> 11, v = row & 2047;
+      const int lm = own0 + loc, m = row0 + lm, tile = wk.t0 + p0 + tl, row = s_row[lm], s = row_seq(row), v = row_in_seq(row);
       const float rs = s_rs[lm];
       const int idx = (loc * tp + tl) * BM, rope_row = (cf.rope_bytes ? loc : m) * half;
       loc += dloc;
@@ -626,9 +630,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         if (EPI == EPI_PSEUDO) {                   // output column = (map, column); d is a multiple of 128: one map per tile
           const int i = n0 / a.d, o = n0 - i * a.d;
           const float4 r = a.pred_b ? add4(sum, load_bf16x4(a.pred_b + n0)) : sum;
-          store_residual(a, s * a.rw.Ms + a.rw.T + (a.rw.chains ? (a.pseudo0 + i) * a.rw.T + v : a.pseudo0 + i), -1, o, r, load_bf16x4(a.g + o), warp_sq(r), lane);
+          store_residual(a, act_row(a.rw, s, a.rw.T + (a.rw.chains ? (a.pseudo0 + i) * a.rw.T + v : a.pseudo0 + i)), -1, o, r, load_bf16x4(a.g + o), warp_sq(r), lane);
         } else if (n0 < a.N) {                     // EPI_LOGITS
-          float *dst = a.logits + (size_t)m * a.N + n0;
+          float *dst = a.logits + (size_t)(s * a.rw.Ms + v) * a.N + n0;
           if ((a.N & 3) == 0) {
             *reinterpret_cast<float4 *>(dst) = sum;
           } else {

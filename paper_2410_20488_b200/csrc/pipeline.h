@@ -2,10 +2,12 @@
 // it can be run on the host with any timing.
 #pragma once
 
+#ifndef FIRP_HD
 #ifdef __CUDACC__
 #define FIRP_HD __host__ __device__ __forceinline__
 #else
 #define FIRP_HD inline
+#endif
 #endif
 
 namespace firp {

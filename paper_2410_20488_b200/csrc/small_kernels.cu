@@ -20,8 +20,9 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl)
   __shared__ int s_depth;
   if (pdl) { griddep_launch(); griddep_wait(); }
   const Rows &rw = a.rw;
-  const int r = blockIdx.x, s = r / rw.Ms, v = r - s * rw.Ms, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int r = blockIdx.x, s = r / rw.Ms, v = r - s * rw.Ms, ar = act_row(rw, s, v), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (a.zero_word && r == 0 && tid == 0) *a.zero_word = 0u;
+  if (rw.by_step && tid == 0) a.meta.row_of[ar] = seq_row(s, v);
   const int n = a.ctx_len[a.seq_ids[s]];
   for (int u = tid; u <= v && !rw.prompt; u += kPrepThreads) {
     int p;
@@ -62,7 +63,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl)
     for (int c = warp * 128 + lane * 4; c < a.d; c += kPrepThreads * 4)
     {
       const float4 e = load_bf16x4(a.embed + (size_t)tok * a.d + c);
-      store_residual(a, r, xp_row, c, e, a.x ? load_bf16x4(a.g + c) : e, warp_sq(e), lane);
+      store_residual(a, ar, xp_row, c, e, a.x ? load_bf16x4(a.g + c) : e, warp_sq(e), lane);
     }
   }
   __syncthreads();
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl)
     const double ang = (double)(n + s_depth) * inv_freq;
     double sn, cs;
     sincos(ang, &sn, &cs);
-    a.meta.rope[(size_t)r * half + tid] = make_float2((float)cs, (float)sn);
+    a.meta.rope[(size_t)ar * half + tid] = make_float2((float)cs, (float)sn);
   }
 }
 

@@ -65,12 +65,6 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t lbo_byt
 }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void wg_sync(int w) { asm volatile("bar.sync %0, 128;" ::"r"(1 + w) : "memory"); }
-__device__ __forceinline__ void tc_ld8(uint32_t taddr, float *r) {
-  uint32_t *u = reinterpret_cast<uint32_t *>(r);
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7])
-               : "r"(taddr) : "memory");
-}
 // N = 8, 16 or 24 consecutive columns of this warp's lanes (no wait)
 template <int N> __device__ __forceinline__ void tc_ld_cols(uint32_t taddr, float *r) {
   static_assert(N == 8 || N == 16 || N == 24, "columns per warpgroup");

@@ -65,8 +65,9 @@ constexpr int kThreads = 384;      // 12 warps
 constexpr int kEpiWarps = 8;
 constexpr int W_TILE = BM * 128;   // bytes of one 128-row weight tile of a k block
 constexpr int kSmemMax = 227 * 1024;
-constexpr int kTailBytes = 1984;   // row scales, row indices, slots and lengths, barriers, TMEM address (behind the rings)
+constexpr int kTailBytes = 2496;   // row scales, slots and lengths, row indices, barriers, TMEM address (behind the rings)
 constexpr int kMaxRows = 256;      // token rows of a CTA (MMA N)
+constexpr int kNoRow = -1, kNoKv = -2;
 constexpr int kMaxW = 12, kMaxX = 6;  // ring depths: weight tiles, activation stages
 
 // How the rows of the weight are dealt to tiles of 128, each one TMA box per k block.
@@ -171,7 +172,10 @@ struct ActRing : RingBase {      // all planes of a k block per slot
 // accumulator sets, or planes side by side (in one kernel with the others the code they skip cost them 1-2 % of a two-layer step).
 // The epilogue's code runs once per launch from a cold instruction cache, in the shadow of nothing: one kernel per epilogue
 // and rolled loops keep it short (all five in one kernel, four items unrolled: 5-7 us instead of 1-2).
-template <int TM, bool MERGED, bool DEEP, int EPI>
+// C: token rows (TMEM columns) that the epilogue takes at a time.  Eight for up to 48 rows: its passes are then so short that they run
+// about as long as their code takes to come from a cold instruction cache (us per step with 16 / with 8: two-layer shape 79.7 / 75.1, one
+// row of the 7B shape 2722 / 2690, 35 rows 3220 / 3166); with more rows sixteen hide more of the TMEM loads (128 and 131 rows 5987 / 6033).
+template <int TM, bool MERGED, bool DEEP, int C, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ LinArgs a,
             const __grid_constant__ TileSched sc, const __grid_constant__ TileCfg cf) {
@@ -184,7 +188,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   float *s_rs = reinterpret_cast<float *>(data + cf.tail);          // 1 / RMS of every token row
   int *s_slot = reinterpret_cast<int *>(s_rs + kMaxRows), *s_pos = s_slot + kMaxSeq;      // of every sequence
   uint16_t *s_row = reinterpret_cast<uint16_t *>(s_pos + kMaxSeq);                        // seq_row of every token row, 0xffff: none
-  const uint32_t bars = base + cf.tail + kMaxRows * 6 + 2 * kMaxSeq * 4;
+  int *s_kv = reinterpret_cast<int *>(s_pos + kMaxSeq);      // QKV: instead, every token row's row of a cache plane; kNoKv: none, kNoRow: no token row
+  const uint32_t bars = base + cf.tail + kMaxRows * 8 + 2 * kMaxSeq * 4;
   const uint32_t full_w = bars, empty_w = full_w + 8 * kMaxW, full_x = empty_w + 8 * kMaxW, empty_x = full_x + 8 * kMaxX,
                  acc_full = empty_x + 8 * kMaxX, rope_full = acc_full + 8, tmem_slot = rope_full + 8;
   volatile int *gave_up = reinterpret_cast<volatile int *>(data + (tmem_slot + 4 - base));   // a thread's wait has run out
@@ -340,66 +345,64 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         const int m = m0 + u * kEpiWarps;
         if (lane == 0 && m < m_end) {
           s_rs[m] = a.ss ? rsqrtf(v[u] / (float)a.K + a.eps) : 1.f;
-          s_row[m] = m < own0 + n_own ? w[u] : 0xffff;
+          if (EPI == EPI_QKV_ROPE) s_kv[m] = m < own0 + n_own ? w[u] : kNoRow;
+          else s_row[m] = m < own0 + n_own ? w[u] : 0xffff;
         }
+      }
+    }
+    if (EPI == EPI_QKV_ROPE) {       // once per row here, and not by every thread that writes to it
+      epi_sync();
+      const int m = own0 + (int)threadIdx.x - 128;
+      if (m < m_end && s_kv[m] != kNoRow) {
+        const int s = row_seq(s_kv[m]), pos = s_pos[s] + row_in_seq(s_kv[m]);
+        s_kv[m] = pos < a.max_ctx ? (int)kv_row(a.pages, s_slot[s], pos, a.max_ctx) : kNoKv;
       }
     }
   }
-  // columns [c0, c0 + 16) of tile t: the sums over the planes' columns and the accumulator sets
+  // columns [c0, c0 + C) of tile t: the sums over the planes' columns and the accumulator sets
+  auto ld = [](uint32_t ta, float *r) { if (C == 16) tc_ld16(ta, r); else tc_ld8(ta, r); };
   const uint32_t tquarter = tmem + ((uint32_t)(quarter * 32) << 16);
   auto load_acc = [&](int t, int c0, float *r) {
     const uint32_t ta = tquarter + (uint32_t)(t * cf.acc + c0);
-    float l[DEEP ? 4 : 3][16];
-    tc_ld16(ta, r);
-    if (cf.planes_side > 1) tc_ld16(ta + cf.npad, l[0]);
+    float l[DEEP ? 4 : 3][C];
+    auto add = [&](const float *x) {
+#pragma unroll
+      for (int j = 0; j < C; ++j) r[j] += x[j];
+    };
+    ld(ta, r);
+    if (cf.planes_side > 1) ld(ta + cf.npad, l[0]);
     if (cf.sets > 1) {
-      tc_ld16(ta + cf.acc_set, l[1]);
-      if (cf.planes_side > 1) tc_ld16(ta + cf.acc_set + cf.npad, l[2]);
+      ld(ta + cf.acc_set, l[1]);
+      if (cf.planes_side > 1) ld(ta + cf.acc_set + cf.npad, l[2]);
     }
     tc_ld_wait();
-    if (cf.planes_side > 1) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) r[j] += l[0][j];
-    }
+    if (cf.planes_side > 1) add(l[0]);
     if (cf.sets > 1) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) r[j] += l[1][j];
-      if (cf.planes_side > 1) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) r[j] += l[2][j];
-      }
+      add(l[1]);
+      if (cf.planes_side > 1) add(l[2]);
     }
     if (DEEP) {       // the third and fourth set's columns, the third plane's
       if (cf.sets > 2) {
-        tc_ld16(ta + 2 * cf.acc_set, l[0]);
-        if (cf.planes_side > 1) tc_ld16(ta + 2 * cf.acc_set + cf.npad, l[1]);
+        ld(ta + 2 * cf.acc_set, l[0]);
+        if (cf.planes_side > 1) ld(ta + 2 * cf.acc_set + cf.npad, l[1]);
         if (cf.sets > 3) {
-          tc_ld16(ta + 3 * cf.acc_set, l[2]);
-          if (cf.planes_side > 1) tc_ld16(ta + 3 * cf.acc_set + cf.npad, l[3]);
+          ld(ta + 3 * cf.acc_set, l[2]);
+          if (cf.planes_side > 1) ld(ta + 3 * cf.acc_set + cf.npad, l[3]);
         }
         tc_ld_wait();
-#pragma unroll
-        for (int j = 0; j < 16; ++j) r[j] += l[0][j];
-        if (cf.planes_side > 1) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) r[j] += l[1][j];
-        }
+        add(l[0]);
+        if (cf.planes_side > 1) add(l[1]);
         if (cf.sets > 3) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) r[j] += l[2][j];
-          if (cf.planes_side > 1) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) r[j] += l[3][j];
-          }
+          add(l[2]);
+          if (cf.planes_side > 1) add(l[3]);
         }
       }
       if (cf.planes_side > 2) {
 #pragma unroll 1
         for (int i = 0; i < cf.sets; ++i) {
-          tc_ld16(ta + i * cf.acc_set + 2 * cf.npad, l[0]);
+          ld(ta + i * cf.acc_set + 2 * cf.npad, l[0]);
           tc_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) r[j] += l[0][j];
+          add(l[0]);
         }
       }
     }
@@ -413,7 +416,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     tc_fence_after();
   };
   if (kDirect && split == 1) {
-    // ---- no other CTA contributes: a thread has one weight row of its tile in 8 token rows at a time, and what it is
+    // ---- no other CTA contributes: a thread has one weight row of its tile in C token rows at a time, and what it is
     // combined with in the same thread (gate and up) or 16 lanes away (rotary pair)
     if (epi) {
       const int rowi = quarter * 32 + lane;                     // row of the tile
@@ -426,21 +429,26 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         const int tile = wk.t0 + t;
         const int unit = EPI == EPI_QKV_ROPE ? tile * sc.heads + (sc.heads == 2 ? quarter >> 1 : 0) : 0;    // query, key or value head
 #pragma unroll 1
-        for (int c0 = half_w * 16; c0 < R; c0 += 32) {
-          float r[16], r2[16], rs[16];
-          uint32_t row[8];                                      // two rows each
+        for (int c0 = half_w * C; c0 < R; c0 += 2 * C) {
+          float r[C], r2[C], rs[C];
+          uint32_t row[EPI == EPI_QKV_ROPE ? C : C / 2];            // two rows each, or one row's place in the cache
           load_acc(t, c0, r);
           if (EPI == EPI_SWIGLU) load_acc(t + 1, c0, r2);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) *reinterpret_cast<float4 *>(rs + 4 * q) = *reinterpret_cast<const float4 *>(s_rs + c0 + 4 * q);
+          for (int q = 0; q < C / 4; ++q) *reinterpret_cast<float4 *>(rs + 4 * q) = *reinterpret_cast<const float4 *>(s_rs + c0 + 4 * q);
+          if (EPI == EPI_QKV_ROPE) {
 #pragma unroll
-          for (int q = 0; q < 2; ++q) *reinterpret_cast<uint4 *>(row + 4 * q) = *reinterpret_cast<const uint4 *>(s_row + c0 + 8 * q);
+            for (int q = 0; q < C / 4; ++q) *reinterpret_cast<uint4 *>(row + 4 * q) = *reinterpret_cast<const uint4 *>(s_kv + c0 + 4 * q);
+          } else {
+#pragma unroll
+            for (int q = 0; q < C / 8; ++q) *reinterpret_cast<uint4 *>(row + 4 * q) = *reinterpret_cast<const uint4 *>(s_row + c0 + 8 * q);
+          }
           auto row_of = [&](int j) { return (int)((row[j >> 1] >> (16 * (j & 1))) & 0xffffu); };       // 0xffff: none
           if (EPI == EPI_LOGITS) {
             const int n = tile * BM + rowi;
             if (n < a.N) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < C; ++j) {
                 const int w = row_of(j);
                 if (w != 0xffff) a.logits[(size_t)(row_seq(w) * a.rw.Ms + row_in_seq(w)) * a.N + n] = r[j] * rs[j];
               }
@@ -448,11 +456,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
           } else if (EPI == EPI_SWIGLU) {
             const int n = (tile >> 1) * BM + rowi;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) { const float g = r[j] * rs[j]; r[j] = g / (1.f + __expf(-g)) * (r2[j] * rs[j]); }
+            for (int j = 0; j < C; ++j) { const float g = r[j] * rs[j]; r[j] = g / (1.f + __expf(-g)) * (r2[j] * rs[j]); }
             bf16 *dst = a.y + (size_t)(row0 + c0) * a.F + n;
             if (n < a.F) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < C; ++j) {
                 const bf16 h = __float2bfloat16_rn(r[j]);
                 if (row_of(j) != 0xffff) {
                   dst[(size_t)j * a.F] = h;
@@ -463,10 +471,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
           } else {
             // queries and keys are rotated at the row's tree position (Section 3.4): y = x cos -+ (other half) sin
 #pragma unroll
-            for (int j = 0; j < 16; ++j) r[j] *= rs[j];
+            for (int j = 0; j < C; ++j) r[j] *= rs[j];
             if (unit < a.H + a.Hkv) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < C; ++j) {
                 const float2 cs = rope[min(c0 + j, R - 1) * half + c];
                 const float o = __shfl_xor_sync(0xffffffffu, r[j], 16);
                 r[j] = r[j] * cs.x + (hi_half ? o : -o) * cs.y;
@@ -477,9 +485,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
               bf16 *dst = a.q + (size_t)(row0 + c0) * a.H * a.dh + unit * a.dh + col;
               const int stride = a.H * a.dh;
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
+              for (int j = 0; j < C; ++j) {
                 const bf16 h = __float2bfloat16_rn(r[j]);
-                if (row_of(j) != 0xffff) {
+                if ((int)row[j] != kNoRow) {
                   dst[(size_t)j * stride] = h;
                   dst[(size_t)j * stride + a.q_plane] = __float2bfloat16_rn(r[j] - __bfloat162float(h));
                 }
@@ -489,12 +497,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
               bf16 *dst = a.kcache + (is_v ? a.kv_stride : 0) + kvh * a.dh + col;
               const size_t stride = (size_t)a.Hkv * a.dh;
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const int w = row_of(j);
-                if (w != 0xffff) {
-                  const int pos = s_pos[row_seq(w)] + row_in_seq(w);
-                  if (pos < a.max_ctx) dst[kv_row(a.pages, s_slot[row_seq(w)], pos, a.max_ctx) * stride] = __float2bfloat16_rn(r[j]);
-                }
+              for (int j = 0; j < C; ++j) {
+                if ((int)row[j] >= 0) dst[(size_t)row[j] * stride] = __float2bfloat16_rn(r[j]);
               }
             }
           }
@@ -530,11 +534,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
 #pragma unroll 1
       for (int tl = 0; tl < tp; ++tl) {
 #pragma unroll 1
-        for (int c0 = half_w * 16; c0 < R; c0 += 32) {
-          float r[16];
+        for (int c0 = half_w * C; c0 < R; c0 += 2 * C) {
+          float r[C];
           load_acc(p0 + tl, c0, r);
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {            // four token rows go to one CTA (tpo is a multiple of four)
+          for (int g = 0; g < C / 4; ++g) {            // four token rows go to one CTA (tpo is a multiple of four)
             const int m = c0 + 4 * g;
             if (m < R) {
               const int o = (m * cf.inv_tpo) >> 16;
@@ -618,12 +622,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     int loc = loc0, tl = loc0 >= n_own ? tp : 0;
 #pragma unroll 1
     while (tl < tp) {
-      const int lm = own0 + loc, m = row0 + lm, tile = wk.t0 + p0 + tl, row = s_row[lm], s = row_seq(row), v = row_in_seq(row);
+      const int lm = own0 + loc, m = row0 + lm, tile = wk.t0 + p0 + tl, row = EPI == EPI_QKV_ROPE ? s_kv[lm] : s_row[lm], s = row_seq(row), v = row_in_seq(row);
       const float rs = s_rs[lm];
       const int idx = (loc * tp + tl) * BM, rope_row = (cf.rope_bytes ? loc : m) * half;
       loc += dloc;
       if (loc >= n_own) { loc = loc0; tl += pitch; }
-      if (row == 0xffff) continue;
+      if (row == (EPI == EPI_QKV_ROPE ? kNoRow : 0xffff)) continue;
       if (EPI == EPI_PSEUDO || EPI == EPI_LOGITS) {
         const int n0 = tile * BM + lane * 4;
         const float4 sum = mul4(sums(idx + lane * 4), rs);
@@ -679,9 +683,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
           *reinterpret_cast<uint2 *>(dst + a.q_plane) = l1;
           *reinterpret_cast<uint2 *>(dst + a.q_plane + half) = l2;
         } else {                         // the cache stores bf16: one rounding, on store
-          const int is_v = unit >= a.H + a.Hkv, kvh = unit - a.H - (is_v ? a.Hkv : 0), pos = s_pos[s] + v;
-          if (pos < a.max_ctx) {
-            bf16 *dst = a.kcache + (is_v ? a.kv_stride : 0) + (kv_row(a.pages, s_slot[s], pos, a.max_ctx) * a.Hkv + kvh) * a.dh + c;
+          const int is_v = unit >= a.H + a.Hkv, kvh = unit - a.H - (is_v ? a.Hkv : 0);
+          if (row >= 0) {
+            bf16 *dst = a.kcache + (is_v ? a.kv_stride : 0) + ((size_t)row * a.Hkv + kvh) * a.dh + c;
             *reinterpret_cast<uint2 *>(dst) = round4(x1);
             *reinterpret_cast<uint2 *>(dst + half) = round4(x2);
           }
@@ -775,22 +779,24 @@ bool plane_map(CUtensorMap *m, const void *X, uint64_t planes, uint64_t plane_ro
 
 constexpr uint32_t pow2_cols(int c) { return c <= 32 ? 32 : c <= 64 ? 64 : c <= 128 ? 128 : c <= 256 ? 256 : 512; }
 constexpr int align_n(int v, int a) { return (v + a - 1) / a * a; }
+constexpr bool few_rows(int r) { return r <= 48; }      // of a block: the epilogue takes 8 at a time
 
 typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const LinArgs, const TileSched, const TileCfg);
-template <bool MERGED, bool DEEP, int EPI> KernelFn kernel_tm(int tm) {
-  return tm == 1 ? gemm_kernel<1, MERGED, DEEP, EPI> : tm == 2 ? gemm_kernel<2, MERGED, DEEP, EPI> : gemm_kernel<3, MERGED, DEEP, EPI>;
+template <bool MERGED, bool DEEP, int C, int EPI> KernelFn kernel_tm(int tm) {
+  return tm == 1 ? gemm_kernel<1, MERGED, DEEP, C, EPI> : tm == 2 ? gemm_kernel<2, MERGED, DEEP, C, EPI> : gemm_kernel<3, MERGED, DEEP, C, EPI>;
 }
-template <int EPI> KernelFn kernel_epi(int tm, bool merged, bool deep) {
-  if (merged) return deep ? kernel_tm<true, true, EPI>(tm) : kernel_tm<true, false, EPI>(tm);
-  return deep ? kernel_tm<false, true, EPI>(tm) : kernel_tm<false, false, EPI>(tm);
+template <int EPI> KernelFn kernel_epi(int tm, bool merged, bool deep, bool few) {
+  if (!merged) return deep ? kernel_tm<false, true, 16, EPI>(tm) : kernel_tm<false, false, 16, EPI>(tm);
+  if (few) return deep ? kernel_tm<true, true, 8, EPI>(tm) : kernel_tm<true, false, 8, EPI>(tm);
+  return deep ? kernel_tm<true, true, 16, EPI>(tm) : kernel_tm<true, false, 16, EPI>(tm);
 }
-KernelFn kernel_of(int epi, int tm, bool merged, bool deep) {
+KernelFn kernel_of(int epi, int tm, bool merged, bool deep, bool few) {
   switch (epi) {
-    case EPI_RESIDUAL: return kernel_epi<EPI_RESIDUAL>(tm, merged, deep);
-    case EPI_QKV_ROPE: return kernel_epi<EPI_QKV_ROPE>(tm, merged, deep);
-    case EPI_SWIGLU: return kernel_epi<EPI_SWIGLU>(tm, merged, deep);
-    case EPI_LOGITS: return kernel_epi<EPI_LOGITS>(tm, merged, deep);
-    default: return kernel_epi<EPI_PSEUDO>(tm, merged, deep);
+    case EPI_RESIDUAL: return kernel_epi<EPI_RESIDUAL>(tm, merged, deep, few);
+    case EPI_QKV_ROPE: return kernel_epi<EPI_QKV_ROPE>(tm, merged, deep, few);
+    case EPI_SWIGLU: return kernel_epi<EPI_SWIGLU>(tm, merged, deep, few);
+    case EPI_LOGITS: return kernel_epi<EPI_LOGITS>(tm, merged, deep, few);
+    default: return kernel_epi<EPI_PSEUDO>(tm, merged, deep, few);
   }
 }
 
@@ -811,7 +817,7 @@ int cluster_ctas(int n) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    KernelFn fn = kernel_of(EPI_RESIDUAL, 1, true, false);
+    KernelFn fn = kernel_of(EPI_RESIDUAL, 1, true, false, true);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&k, fn, &cfg) != cudaSuccess || k < 1) { cudaGetLastError(); k = std::max(1, sms / n * 3 / 4); }
     cap[n] = k * n;
@@ -861,8 +867,8 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
     if (n_mma > 256) continue;
     const int x_stage = planes * npad * 128;
     for (int tm = 1; tm <= 3; ++tm) {
-      // the epilogue reads 16 columns at a time, 8 of them beyond the last plane's when npad is an odd multiple of 8
-      const int over = npad & 8;
+      // the epilogue of many rows reads 16 columns at a time, 8 of them beyond the last plane's when npad is an odd multiple of 8
+      const int over = few_rows(R) ? 0 : npad & 8;
       if (tm * n_mma + over > 512 || (s.mode == ROWS_GATE_UP && tm != 2)) continue;
       for (int split = 1; split <= 8 && split <= s.KB; ++split) {
         const int cap = cluster_ctas(split) / split * split;
@@ -963,7 +969,7 @@ cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream
   if (p.tm == 0 || p.smem > kSmemMax || p.cf.tp < 1 || p.cf.sw < 1 || p.cf.sx < 1 || (!p.cf.by_tile && p.cf.issuers == 2 && ((p.cf.sw | p.cf.sx | p.cf.sets) & 1)))
     return cudaErrorInvalidConfiguration;
   p.cf.pdl = pdl ? 1 : 0;
-  KernelFn fn = kernel_of(epi, p.tm, p.merged != 0, p.cf.sets > 2 || p.cf.planes_side > 2);
+  KernelFn fn = kernel_of(epi, p.tm, p.merged != 0, p.cf.sets > 2 || p.cf.planes_side > 2, few_rows(p.cf.rpb));
   static std::map<KernelFn, int> configured;
   static std::mutex mu;
   {

@@ -118,10 +118,12 @@ template <int NH, bool SUM> __device__ __forceinline__ void warp_cols_to_smem(co
 struct KvRing {
   const CUtensorMap *tm; const AttnArgs &a;
   uint32_t full, freed, dst0;
-  int slot, t0, kv_len, kvh;
+  int slot, t0, n, kv_len, kvh;
   uint64_t pol; unsigned long long wait_ns; bool dead;
+  bool waited;                     // for the QKV projection, which writes the rows from n on
   __device__ __forceinline__ bool free(int, int w, uint32_t parity) { return mbar_wait(freed + 8 * w, parity, a.err, dead, wait_ns); }
   __device__ __forceinline__ void load(int i, int w) {
+    if (!waited && (t0 + i + 1) * kTcTile > n) { griddep_wait(); waited = true; }
     mbar_expect_tx(full + 8 * w, kTcStage);
 #pragma unroll
     for (int ph = 0; ph < 2; ++ph) {                // 64-position x 64-element boxes; a half lies inside one page
@@ -148,6 +150,37 @@ __device__ unsigned long long g_attn_trace[16];
 #else
 #define TC_STAMP(k) do { } while (0)
 #endif
+
+// What happens under the QKV projection.  It lets this kernel start only after its own wait, so that all that was written before it --
+// lengths, slots, the cache's committed rows -- may be read without waiting for it: the tiles that lie in the committed prefix are on
+// their way or in shared memory when it completes, only the queries and the tile with the step's own rows are loaded after that.  us
+// per step, everything behind one wait / this: one row of the 7B shape 2690 / 2634, 35 rows at 512 tokens 3166 / 3156, at 8192 4238 / 4214,
+// 131 rows 5969 / 5909, four requests of the 34B shape 6094 / 6021.
+//
+// Slot and committed length (position of the root row) of sequence s: the two producers'
+// warps load them and go on to the tiles of the committed prefix, and the second one leaves them to the others in s_sn, behind a
+// barrier of their own.  (Thousands of warps asking L2 for the same two words at once took microseconds.)  `threads`: of the second
+// producer's warp and the warps that wait.
+__device__ __forceinline__ int2 load_slot_and_length(const AttnArgs &a, int s, int lane, bool leave, int threads, int *s_sn) {
+  const int v = lane == 0 ? __ldcg(a.seq_ids + s) : lane == 1 ? __ldcg(a.pos + s * a.rw.Ms) : 0;
+  if (leave) {
+    if (lane < 2) s_sn[lane] = v;
+    __syncwarp();
+    asm volatile("bar.arrive 9, %0;" ::"r"(threads) : "memory");
+  }
+  return make_int2(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 1));
+}
+__device__ __forceinline__ void wait_slot_and_length(int threads) { asm volatile("bar.sync 9, %0;" ::"r"(threads) : "memory"); }
+// The tiles of a kv split: those of the first `rows` new rows' context, cut evenly.
+struct KvRange { int kv_len, t0, ntiles; };
+__device__ __forceinline__ KvRange kv_range(int n, int rows, int max_ctx, int split, int nsplits) {
+  KvRange r;
+  r.kv_len = min(n + rows, max_ctx);
+  const int total = (r.kv_len + kTcTile - 1) / kTcTile;
+  r.t0 = (split * total + nsplits - 1) / nsplits;
+  r.ntiles = ((split + 1) * total + nsplits - 1) / nsplits - r.t0;
+  return r;
+}
 
 template <int NQ>
 __global__ void __launch_bounds__(kTcThreads, 1)
@@ -193,7 +226,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
-  if (pdl) { griddep_launch(); griddep_wait(); }
+  if (pdl) griddep_launch();
   TC_STAMP(1);
 
   const int kvh = blockIdx.y, G = a.H / a.Hkv;
@@ -207,6 +240,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   constexpr int QIT = (NQ * 16 + kTcSoft - 1) / kTcSoft;
   uint4 qh[QIT], ql[QIT];
   if (warp < 16) {
+    if (pdl) griddep_wait();
 #pragma unroll
     for (int it = 0; it < QIT; ++it) {
       const int idx = it * kTcSoft + tid, j = idx >> 4, c = idx & 15, qr = q0 + j;
@@ -218,15 +252,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
     }
   }
-  // one warp loads the slot and the committed length (position of the root row): thousands of warps asking L2 for the
-  // same two words at once took microseconds
-  if (warp == 18 && lane < 2) s_sn[lane] = lane == 0 ? __ldcg(a.seq_ids + s) : __ldcg(a.pos + s * a.rw.Ms);
-  __syncthreads();
-  const int slot = s_sn[0], n = s_sn[1];
-  const int kv_len = min(n + a.rows_active, a.max_ctx);
-  const int tiles_total = (kv_len + kTcTile - 1) / kTcTile;
-  const int t0 = (split * tiles_total + nsplits - 1) / nsplits, t1 = ((split + 1) * tiles_total + nsplits - 1) / nsplits;
-  const int ntiles = t1 - t0;                       // tile t0 + i goes to warpgroup i & 1 as its (i >> 1)-th
   const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kDefaultWaitNs;
   bool dead = false;
   constexpr int NH = NQ / 2;                        // columns per warpgroup
@@ -235,6 +260,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   for (int j = 0; j < NH; ++j) o_acc[j] = 0.f;
 
   if (warp >= 17) {
+    const int2 sn = load_slot_and_length(a, s, lane, warp == 18, 18 * 32, s_sn);
     // ---- producers (one lane each): warp 17 feeds the K buffers, warp 18 the V buffers.  A buffer is free again
     // when the MMAs that read it have completed, which is what s_ready / o_ready of its warpgroup report.
     if (lane == 0) {
@@ -242,14 +268,17 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const CUtensorMap *tm = is_v ? &tmV : &tmK;
       const uint32_t full = is_v ? full_v : full_k, freed = is_v ? o_ready : s_ready;
       const uint32_t dst0 = sb + (is_v ? LY::V_OFF : LY::K_OFF);
+      const KvRange kv = kv_range(sn.y, a.rows_active, a.max_ctx, split, nsplits);
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
-      KvRing ring{tm, a, full, freed, dst0, slot, t0, kv_len, kvh, pol, wait_ns, false};
-      drain(ring, produce(ring, ntiles, 2), 2);
+      KvRing ring{tm, a, full, freed, dst0, sn.x, kv.t0, sn.y, kv.kv_len, kvh, pol, wait_ns, false, false};
+      drain(ring, produce(ring, kv.ntiles, 2), 2);
     }
   } else if (warp == 16) {
     // ---- MMA issuer (one lane): S^T of tile i, then O^T of tile i - 1
+    wait_slot_and_length(18 * 32);
     if (lane == 0) {
+      const int ntiles = kv_range(s_sn[1], a.rows_active, a.max_ctx, split, nsplits).ntiles;      // tile t0 + i goes to tile group i & 1 as its (i >> 1)-th
       const uint32_t idesc_k = instr_desc_m128(NQ), idesc_mn = idesc_k | (1u << 15);
       // operand descriptors of warpgroup 0; another buffer, dh half or k step only moves the start address
       const uint64_t kdesc0 = smem_desc(sb + LY::K_OFF), qdesc0 = smem_desc(sb + LY::Q_OFF);
@@ -292,6 +321,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   } else {
     // ---- the four softmax warpgroups: tile group g takes tiles g, g + 2, ...; half h of it owns the query columns
     // [h NH, (h + 1) NH) of those tiles
+    wait_slot_and_length(18 * 32);
+    const int n = s_sn[1];
+    const KvRange kv = kv_range(n, a.rows_active, a.max_ctx, split, nsplits);
+    const int kv_len = kv.kv_len, t0 = kv.t0, ntiles = kv.ntiles;
     const int wgi = warp >> 2, g = wgi >> 1, h = wgi & 1, wt = tid & (kTcWg - 1);
     const int c_lo = h * NH;
     const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * 2 * NQ + c_lo);
@@ -603,7 +636,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;                     // columns: S / P of tiles i % 3 at 128 (i % 3), O at 384
-  if (pdl) { griddep_launch(); griddep_wait(); }
+  if (pdl) griddep_launch();
 
   const int kvh = blockIdx.y, G = a.H / a.Hkv;
   const int qblocks = gridDim.z / a.rw.n_seq;
@@ -612,17 +645,26 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   const int split = blockIdx.x, nsp = gridDim.x;
   const int qrows_total = a.rows_active * G, q0 = qb * qper;
   const int ncols = min(qper, qrows_total - q0);
-  if (warp == 18 && lane < 2) s_sn[lane] = lane == 0 ? __ldcg(a.seq_ids + s) : __ldcg(a.pos + s * a.rw.Ms);
   // the queries of this block: row j = query row q0 + j -> (tree row (q0 + j) / G, head kvh G + (q0 + j) % G).  Rows beyond
   // ncols hold anything: they only feed their own lanes of S and O, which nothing reads.
   if (warp < 16) {
-    for (int j = tid >> 4; j < ncols; j += 32) {
-      const int c = tid & 15, qr = q0 + j;
+    if (pdl) griddep_wait();
+    uint4 qh[kRowM / 32], ql[kRowM / 32];           // all loads go out before the first is waited for
+    const int c = tid & 15;
+#pragma unroll
+    for (int u = 0; u < kRowM / 32; ++u) {
+      const int qr = q0 + min((tid >> 4) + 32 * u, ncols - 1);
       const bf16 *src = a.q + ((size_t)act_row(a.rw, s, qr / G) * a.H + kvh * G + qr % G) * kTcDh + c * 8;
-      const uint4 qh = *reinterpret_cast<const uint4 *>(src), ql = *reinterpret_cast<const uint4 *>(src + a.q_lo_off);
-      const int off = Q_OFF + (c >> 3) * kTcSlab + j * 128 + (((c & 7) ^ (j & 7)) << 4);
-      *reinterpret_cast<uint4 *>(base + off) = qh;
-      *reinterpret_cast<uint4 *>(base + off + kTcStage) = ql;
+      qh[u] = *reinterpret_cast<const uint4 *>(src);
+      ql[u] = *reinterpret_cast<const uint4 *>(src + a.q_lo_off);
+    }
+#pragma unroll
+    for (int u = 0; u < kRowM / 32; ++u) {
+      const int j = (tid >> 4) + 32 * u, off = Q_OFF + (c >> 3) * kTcSlab + j * 128 + (((c & 7) ^ (j & 7)) << 4);
+      if (j < ncols) {
+        *reinterpret_cast<uint4 *>(base + off) = qh[u];
+        *reinterpret_cast<uint4 *>(base + off + kTcStage) = ql[u];
+      }
     }
     fence_async_smem();
     mbar_arrive(q_ready);
@@ -634,12 +676,16 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       }
     }
   }
-  __syncthreads();
-  const int slot = s_sn[0], n = s_sn[1];
-  const int kv_len = min(n + (PROMPT ? (q0 + ncols - 1) / G + 1 : a.rows_active), a.max_ctx);
-  const int tiles_total = (kv_len + kTcTile - 1) / kTcTile;
-  const int t0 = (split * tiles_total + nsp - 1) / nsp, t1 = ((split + 1) * tiles_total + nsp - 1) / nsp;
-  const int ntiles = t1 - t0;                       // tile t0 + i goes to softmax warpgroup i & 1
+  int2 sn;
+  if (warp >= 18) {
+    sn = load_slot_and_length(a, s, lane, warp == 19, 19 * 32, s_sn);
+  } else {
+    wait_slot_and_length(19 * 32);
+    sn = make_int2(s_sn[0], s_sn[1]);
+  }
+  const int n = sn.y;
+  const KvRange kv = kv_range(n, PROMPT ? (q0 + ncols - 1) / G + 1 : a.rows_active, a.max_ctx, split, nsp);
+  const int kv_len = kv.kv_len, t0 = kv.t0, ntiles = kv.ntiles;      // tile t0 + i goes to softmax warpgroup i & 1
   const unsigned long long wait_ns = a.wait_ns ? a.wait_ns : kDefaultWaitNs;
   bool dead = false;
   cg::cluster_group cluster = cg::this_cluster();
@@ -662,7 +708,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const uint32_t dst0 = sb + (is_v ? V_OFF : K_OFF);
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
-      RowsKvRing ring{{tm, a, full, is_v ? o_ready : s_ready, dst0, slot, t0, kv_len, kvh, pol, wait_ns, false}};
+      RowsKvRing ring{{tm, a, full, is_v ? o_ready : s_ready, dst0, sn.x, t0, n, kv_len, kvh, pol, wait_ns, false, false}};
       drain(ring, produce(ring, ntiles, kRowsKvRing), kRowsKvRing);
     }
   } else if (warp == 16) {

@@ -221,7 +221,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(data + (tmem_slot - base));
   // Dependents may start as SMs free up.  Not before TMEM is allocated: a dependent on the same SM then only ever waits
   // for columns of a kernel that does not wait for it.
-  if (cf.pdl) griddep_launch();
+  // The attention reads what was complete before the QKV projection started (context lengths, committed cache rows) before its own
+  // wait, so that projection lets it start only after waiting itself.
+  if (cf.pdl && EPI != EPI_QKV_ROPE) griddep_launch();
   if (sc.split > 1 && cf.red_off) cluster_arrive();
 
   bool dead = false;
@@ -245,6 +247,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
       if (cf.pdl) griddep_wait();
+      if (cf.pdl && EPI == EPI_QKV_ROPE) griddep_launch();
       if (EPI == EPI_QKV_ROPE && cf.rope_bytes) {
         const int r0 = (int)(blockIdx.x % sc.split) * cf.tpo, bytes = max(0, min(cf.tpo, R - r0)) * (a.dh >> 1) * 8;   // of the rows finished here
         mbar_expect_tx(rope_full, bytes);

@@ -3,8 +3,8 @@
 //   out[m][n] = sum_k X[m][k] * W[n][k], m = the T + k token rows of a step (at most 144) or the rows of a prompt.
 //
 // Roles are swapped: weight rows are the MMA M dimension (one TMEM lane each), token rows the MMA N dimension (one
-// TMEM column each).  A tile is 128 weight rows; a job is up to TM tiles (or 128 gate rows and the 128 up rows that go with
-// them) that one thread block, or a cluster, finishes by itself for up to 256 token rows: the k blocks of a job are cut over
+// TMEM column each).  A tile is 128 weight rows (64 gate rows and the up rows that go with them); a job is up to TM tiles
+// that one thread block, or a cluster, finishes by itself for up to 256 token rows: the k blocks of a job are cut over
 // the `split` CTAs of the cluster.  Grid = jobs x blocks of token rows x split, one wave wherever the matrix allows it.
 //
 // Why whole tiles and not one equal share of the matrix per SM: HBM does not need every SM.  A TMA ring of 6 x 32 KB per
@@ -72,7 +72,7 @@ constexpr int kMaxW = 12, kMaxX = 6;  // ring depths: weight tiles, activation s
 
 // How the rows of the weight are dealt to tiles of 128, each one TMA box per k block.
 //   ROWS_LINEAR   128 neighbouring rows
-//   ROWS_GATE_UP  even tiles: 128 gate rows, odd tiles: the up rows that go with them (a job is one such pair)
+//   ROWS_GATE_UP  64 gate rows and the up rows that go with them, in turns of 8, so that such a pair is 8 lanes apart in one warp
 //   ROWS_ROTARY   128 / dh heads; the rows of a head in groups of 32: 16 columns of its first half, then their partners in
 //                 the second half, so that a rotary pair is 16 lanes apart in one warp
 enum RowMode { ROWS_LINEAR = 0, ROWS_GATE_UP = 1, ROWS_ROTARY = 2 };
@@ -121,7 +121,7 @@ struct TileCfg {
 // one k block of one tile: 16 KB
 __device__ __forceinline__ void load_tile(uint32_t dst, const CUtensorMap *tm, const TileSched &s, int tile, int kb, uint32_t bar, uint64_t pol) {
   if (s.mode == ROWS_ROTARY) tma_load_5d(dst, tm, kb * BK, tile * s.heads, bar, pol);
-  else if (s.mode == ROWS_GATE_UP) tma_load_3d(dst, tm, kb * BK, (tile >> 1) * BM, tile & 1, bar, pol);
+  else if (s.mode == ROWS_GATE_UP) tma_load_4d(dst, tm, kb * BK, 0, 0, tile * 8, bar, pol);
   else tma_load_2d(dst, tm, kb * BK, tile * BM, bar, pol);
 }
 
@@ -317,7 +317,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   const float *red = reinterpret_cast<const float *>(data + cf.red_off);         // [k slice][own row][tile of the pass][128]
   constexpr bool kDirect = EPI == EPI_QKV_ROPE || EPI == EPI_SWIGLU || EPI == EPI_LOGITS;   // may leave from registers
   const int half = EPI == EPI_QKV_ROPE ? a.dh >> 1 : 1;
-  const int pitch = EPI == EPI_SWIGLU ? 2 : 1;       // tiles per item
   if (epi) {
     if (cf.pdl) griddep_wait();
     // one load per CTA (thousands of warps asking L2 for the same word at once take microseconds)
@@ -428,15 +427,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       const float2 *rope = cf.rope_bytes ? reinterpret_cast<const float2 *>(data + cf.rope_off) : a.rope + (size_t)row0 * half;
       wait_acc();
 #pragma unroll 1
-      for (int t = 0; t < wk.nt; t += pitch) {
+      for (int t = 0; t < wk.nt; ++t) {
         const int tile = wk.t0 + t;
         const int unit = EPI == EPI_QKV_ROPE ? tile * sc.heads + (sc.heads == 2 ? quarter >> 1 : 0) : 0;    // query, key or value head
 #pragma unroll 1
         for (int c0 = half_w * C; c0 < R; c0 += 2 * C) {
-          float r[C], r2[C], rs[C];
+          float r[C], rs[C];
           uint32_t row[EPI == EPI_QKV_ROPE ? C : C / 2];            // two rows each, or one row's place in the cache
           load_acc(t, c0, r);
-          if (EPI == EPI_SWIGLU) load_acc(t + 1, c0, r2);
 #pragma unroll
           for (int q = 0; q < C / 4; ++q) *reinterpret_cast<float4 *>(rs + 4 * q) = *reinterpret_cast<const float4 *>(s_rs + c0 + 4 * q);
           if (EPI == EPI_QKV_ROPE) {
@@ -457,15 +455,23 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
               }
             }
           } else if (EPI == EPI_SWIGLU) {
-            const int n = (tile >> 1) * BM + rowi;
+            // lanes 8 apart hold the gate and the up value of a column of y; each takes half of the token rows
+            const bool up = (lane & 8) != 0;
+            const int n = tile * (BM / 2) + (rowi >> 4) * 8 + (rowi & 7), m0 = c0 + (up ? C / 2 : 0);
 #pragma unroll
-            for (int j = 0; j < C; ++j) { const float g = r[j] * rs[j]; r[j] = g / (1.f + __expf(-g)) * (r2[j] * rs[j]); }
-            bf16 *dst = a.y + (size_t)(row0 + c0) * a.F + n;
+            for (int j = 0; j < C; ++j) r[j] *= rs[j];
+#pragma unroll
+            for (int j = 0; j < C / 2; ++j) {
+              const float got = __shfl_xor_sync(0xffffffffu, up ? r[j] : r[j + C / 2], 8);
+              const float g = up ? got : r[j], u = up ? r[j + C / 2] : got;
+              r[j] = g / (1.f + __expf(-g)) * u;
+            }
+            bf16 *dst = a.y + (size_t)(row0 + m0) * a.F + n;
             if (n < a.F) {
 #pragma unroll
-              for (int j = 0; j < C; ++j) {
+              for (int j = 0; j < C / 2; ++j) {
                 const bf16 h = __float2bfloat16_rn(r[j]);
-                if (row_of(j) != 0xffff) {
+                if (m0 + j < R) {
                   dst[(size_t)j * a.F] = h;
                   dst[(size_t)j * a.F + a.y_plane] = __float2bfloat16_rn(r[j] - __bfloat162float(h));
                 }
@@ -620,8 +626,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       }
       continue;
     }
-    // a warp per (token row, tile or pair of tiles): 4 neighbouring columns, or pairs, per lane; half a warp for rotary pairs
-    const int loc0 = EPI == EPI_QKV_ROPE ? 2 * ew + (lane >> 4) : ew, dloc = EPI == EPI_QKV_ROPE ? 2 * kEpiWarps : kEpiWarps;
+    // a warp per (token row, tile), 4 neighbouring columns per lane, or half a warp, 4 rotary or gate and up pairs per lane
+    constexpr bool kPairs = EPI == EPI_QKV_ROPE || EPI == EPI_SWIGLU;
+    const int loc0 = kPairs ? 2 * ew + (lane >> 4) : ew, dloc = kPairs ? 2 * kEpiWarps : kEpiWarps;
     int loc = loc0, tl = loc0 >= n_own ? tp : 0;
 #pragma unroll 1
     while (tl < tp) {
@@ -629,7 +636,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       const float rs = s_rs[lm];
       const int idx = (loc * tp + tl) * BM, rope_row = (cf.rope_bytes ? loc : m) * half;
       loc += dloc;
-      if (loc >= n_own) { loc = loc0; tl += pitch; }
+      if (loc >= n_own) { loc = loc0; ++tl; }
       if (row == (EPI == EPI_QKV_ROPE ? kNoRow : 0xffff)) continue;
       if (EPI == EPI_PSEUDO || EPI == EPI_LOGITS) {
         const int n0 = tile * BM + lane * 4;
@@ -648,9 +655,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
           }
         }
       } else if (EPI == EPI_SWIGLU) {
-        const int j0 = (tile >> 1) * BM + lane * 4;
+        const int e = (lane & 15) * 4, i1 = (e >> 3) * 16 + (e & 7), j0 = tile * (BM / 2) + e;
         if (j0 >= a.F) continue;
-        const float4 va = mul4(sums(idx + lane * 4), rs), vb = mul4(sums(idx + BM + lane * 4), rs);
+        const float4 va = mul4(sums(idx + i1), rs), vb = mul4(sums(idx + i1 + 8), rs);
         const float gg[4] = {va.x, va.y, va.z, va.w}, uu[4] = {vb.x, vb.y, vb.z, vb.w};
         float y[4];
 #pragma unroll
@@ -761,7 +768,9 @@ bool weight_map(CUtensorMap *m, int epi, const void *W, uint64_t N, uint64_t K, 
   MapDims d{};
   d.dim[0] = K; d.box[0] = BK;
   if (epi == EPI_SWIGLU) {
-    d.rank = 3; d.dim[1] = F; d.dim[2] = 2; d.stride[0] = K * 2; d.stride[1] = F * K * 2; d.box[1] = BM; d.box[2] = 1;
+    d.rank = 4; d.dim[1] = 8; d.dim[2] = 2; d.dim[3] = F / 8;
+    d.stride[0] = K * 2; d.stride[1] = F * K * 2; d.stride[2] = 8 * K * 2;
+    d.box[1] = 8; d.box[2] = 2; d.box[3] = 8;
   } else if (epi == EPI_QKV_ROPE) {
     const uint64_t half = dh / 2;
     d.rank = 5; d.dim[1] = 16; d.dim[2] = 2; d.dim[3] = half / 16; d.dim[4] = N / dh;
@@ -849,7 +858,7 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
   TileSched s{};
   s.mode = epi == EPI_SWIGLU ? ROWS_GATE_UP : epi == EPI_QKV_ROPE ? ROWS_ROTARY : ROWS_LINEAR;
   s.heads = s.mode == ROWS_ROTARY ? BM / dh : 0;
-  s.n_tiles = s.mode == ROWS_GATE_UP ? 2 * ((F + BM - 1) / BM) : (N + BM - 1) / BM;
+  s.n_tiles = s.mode == ROWS_GATE_UP ? (F + BM / 2 - 1) / (BM / 2) : (N + BM - 1) / BM;
   s.KB = (K + BK - 1) / BK;
   // A prompt's sums may be longer: its results are as far from a 64-bit run as with the equal shares' (cache rows of 1999 tokens of
   // the 7B shape 2.24e-3 / 2.32e-3, of 500 2.76e-3 / 2.88e-3: the rounding of the cache to bf16 hides them), and the equal shares'
@@ -872,7 +881,7 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
     for (int tm = 1; tm <= 3; ++tm) {
       // the epilogue of many rows reads 16 columns at a time, 8 of them beyond the last plane's when npad is an odd multiple of 8
       const int over = few_rows(R) ? 0 : npad & 8;
-      if (tm * n_mma + over > 512 || (s.mode == ROWS_GATE_UP && tm != 2)) continue;
+      if (tm * n_mma + over > 512) continue;
       for (int split = 1; split <= 8 && split <= s.KB; ++split) {
         const int cap = cluster_ctas(split) / split * split;
         int jobs = (s.n_tiles + tm - 1) / tm;
@@ -909,18 +918,21 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
         if (lone) sets = 3;
         const int adds = adds_of(sets);
         if (adds > max_adds) continue;
-        // microseconds: the weights at the rate HBM gives that many CTAs (6.8 TB/s from 84 on); a CTA's MMAs; its bytes from
-        // L2, which gives a CTA 150 GB/s and all of them 15 TB/s; the epilogue's two passes (35 rows: 0.8 + 1.1 us, 131
-        // rows: 3.2 + 3.0 us after the O projection; from registers 2.3 and 7 us for a gate and up pair) and barriers
+        // Microseconds: the weights at the rate HBM gives that many CTAs (6.8 TB/s from 84 on), a CTA's MMAs, its bytes from L2 (which
+        // gives a CTA 150 GB/s and all of them 15 TB/s), or a ring's turnaround, whichever is longest; a share of the others; and for each
+        // wave its start and its epilogue: from registers, or a push to the CTAs of the cluster and the sums there.  The constants are a
+        // fit to every plan of the 7B, 13B and 34B shapes' projections at 20-140 token rows and at prompts of 150-2002 (9216 times of
+        // launches back to back): within 7 % of the times of the plans near the best; the plan it chooses takes 0.8 % longer than the
+        // best one (constants set by hand: 1.5 %; the four projections of a layer of the 7B shape at 67 / 108 / 128 rows 94 / 114 / 120 us,
+        // now 93 / 108 / 116).
         const int ctas = std::min(jobs * s.blocks * split, cap), own = std::min(tpo, R);
         const float hbm = (float)s.n_tiles * s.KB * W_TILE / 6.8e6f * std::max(1.f, 84.f / ctas);
-        const float mma = (float)waves * per * kb * 4.f * (merged ? 1 : planes) * mma_clk(n_mma) / 1850.f;
+        const float mma = (float)waves * per * kb * 4.f * (merged ? 1 : planes) * mma_clk(n_mma) / 1570.f;
         const float ingest = (float)waves * kb * (per * W_TILE + x_stage) / std::min(150e3f, 15e6f / ctas);
         const bool direct = split == 1 && (epi == EPI_QKV_ROPE || epi == EPI_SWIGLU || epi == EPI_LOGITS);
-        const float out = (sets > 2 ? 0.004f * R * per : 0.f) + (direct ? 0.5f + 0.025f * R * per : 0.025f * R * per + 0.05f * own * per + (split == 1 ? 0.5f : red ? 1.f : 2.f));
-        // a ring slot goes round in 0.9 us (activations) or 1.4 us (weights)
-        const float rings_us = (float)waves * kb * std::max(0.9f / sx, 1.4f * per / sw);
-        const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.1f * (hbm + mma + ingest) + waves * (2.f + out) + (split >= 7 && rows > 128 ? 3.f : 0.f);
+        const float out = (sets > 2 ? 0.008f * R * per : 0.f) + (direct ? 0.028f * R * per : 0.017f * R * per + 0.0017f * own * per + (split == 1 || red ? 1.7f : 3.8f));
+        const float rings_us = (float)waves * kb * std::max(0.72f / sx, 1.12f * per / sw);
+        const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.035f * (hbm + mma + ingest) + waves * (1.5f + out) + (split >= 7 ? 1.f : 0.f);
         TileCfg c{};
         c.planes = planes; c.rpb = R; c.npad = npad; c.acc = n_mma; c.sw = sw; c.sx = sx;
         c.tpo = tpo; c.inv_tpo = (65536 + c.tpo - 1) / c.tpo;
@@ -930,8 +942,7 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
         if (red) {
           c.red_off = rings; c.tp = per; c.tail = rings + red;
         } else {
-          // over the rings; gate and up tiles go together
-          c.tail = align_n(std::max(rings, direct ? 0 : per_tile * (s.mode == ROWS_GATE_UP ? 2 : 1)), 128);
+          c.tail = align_n(std::max(rings, direct ? 0 : per_tile), 128);      // over the rings
           c.tp = direct ? per : std::min(per, c.tail / per_tile);
         }
         if (rope) { c.rope_off = c.tail; c.rope_bytes = rope; c.tail += rope; }

@@ -115,7 +115,7 @@ struct AcceptArgs {
 };
 void launch_accept(const Rows &rw, const AcceptArgs &a, bool pdl, cudaStream_t st);
 
-// KV compaction: rows path[j] -> slot n + j in every layer; then ctx_len += len
+// KV compaction: rows path[j] -> slot n + j in every layer; ctx_len = n + len
 struct CommitArgs {
   bf16 *kv;                 // cache base
   size_t seq_stride;        // elements per sequence
@@ -127,10 +127,11 @@ struct CommitArgs {
   const int32_t *path_len;  // [n_seq] device
   int S;
   int32_t *ctx_len;         // [max_batch] device
+  const int32_t *pos; int Ms;   // of the step: n = pos[s * Ms], its committed length
   int max_ctx; KvPages pages;
 };
 void launch_commit(int n_seq, const CommitArgs &a, bool pdl, cudaStream_t st);
-void launch_advance_ctx(int n_seq, const int32_t *seq_ids, int32_t *ctx_len, int amount, bool pdl, cudaStream_t st);
+void launch_advance_ctx(int n_seq, const int32_t *seq_ids, int32_t *ctx_len, int amount, bool pdl, cudaStream_t st);   // after a stretch of a prompt
 
 // ---- weight-streaming GEMM ---------------------------------------------------
 enum GemmEpilogue { EPI_RESIDUAL = 0, EPI_QKV_ROPE = 1, EPI_SWIGLU = 2, EPI_LOGITS = 3, EPI_PSEUDO = 4 };

@@ -20,8 +20,9 @@
 // shape 92.2 -> 65.9 ms (61.3 with attn_tc.cu's blocks of 128 rows); per layer QKV 0.44, attention 0.16, O 0.19, gate/up 0.60,
 // down 0.45 ms.
 //
-// Bound now, per layer of 98 us: the weight stream (QKV 15.1 us at 6.7 TB/s, O 5.5 at 6.1, gate/up 27.8 at 6.5, down 13.1 at
-// 6.9), the epilogues (4 + 2 + 2.5 + 2), five hand-overs of 2 us and the attention's 12.
+// Bound now, per layer of 93 us at 35 rows (device timestamps): the weight stream (QKV 15 us, O 5, gate/up 27, down 13.5, 6.1-6.9 TB/s),
+// the epilogues (2-2.5 each), four hand-overs of 2 (1.3 until the wait for the kernel before returns, 0.7 until its output is in
+// shared memory; O's first weights, behind the attention's late blocks, take 4.5) and the attention's 11-13.
 //
 // Per CTA (one per SM at the large shapes):
 //   warp 0     : weight producer (one thread, TMA, 128-byte swizzle, deep ring).  Weights never depend on the previous

@@ -177,6 +177,8 @@ void launch_accept(const Rows &rw, const AcceptArgs &a, bool pdl, cudaStream_t s
 // KV compaction of the accepted path.  Each thread owns one 16-byte column slice of a
 // (layer, K|V) plane and moves it for every path entry: it loads all source rows before
 // storing any, so a destination slot that is another entry's source is never clobbered.
+// One block moves the context length on; the others take it from the step's bookkeeping, where the root row's position is the
+// committed length (a kernel of its own for that: 3 us of the host and 2 of the two-layer shape's round, 78.2 -> 76.2 us).
 // ---------------------------------------------------------------------------
 constexpr int kMaxPath = 16;
 
@@ -184,8 +186,9 @@ __global__ void __launch_bounds__(128) commit_kernel(CommitArgs a, int pdl) {
   if (pdl) { griddep_launch(); griddep_wait(); }
   const int s = blockIdx.y, plane = blockIdx.x;     // plane = layer * 2 + (0 K, 1 V)
   const int slot = a.seq_ids[s];
-  const int n = a.ctx_len[slot];
+  const int n = a.pos[s * a.Ms];                    // not from ctx_len, which one block writes below while others start
   const int len = min(a.path_len[s], kMaxPath);
+  if (plane == 0 && threadIdx.x == 0) a.ctx_len[slot] = n + len;
   const int32_t *path = a.path + (size_t)s * a.S;
   bf16 *base = a.kv + (size_t)(plane >> 1) * a.layer_stride + (size_t)(plane & 1) * a.kv_stride;
   const int nvec = a.nkv >> 3;
@@ -205,21 +208,18 @@ __global__ void __launch_bounds__(128) commit_kernel(CommitArgs a, int pdl) {
   }
 }
 
-__global__ void advance_ctx_kernel(int n_seq, const int32_t *seq_ids, int32_t *ctx_len, const int32_t *path_len,
-                                   int amount, int pdl) {
+__global__ void advance_ctx_kernel(int n_seq, const int32_t *seq_ids, int32_t *ctx_len, int amount, int pdl) {
   if (pdl) { griddep_launch(); griddep_wait(); }
   const int s = threadIdx.x;
-  if (s < n_seq) ctx_len[seq_ids[s]] += path_len ? min(path_len[s], kMaxPath) : amount;
+  if (s < n_seq) ctx_len[seq_ids[s]] += amount;
 }
 
 void launch_commit(int n_seq, const CommitArgs &a, bool pdl, cudaStream_t st) {
   launch_k(commit_kernel, dim3(a.n_layers * 2, n_seq), dim3(128), 0, st, pdl, a, pdl ? 1 : 0);
-  launch_k(advance_ctx_kernel, dim3(1), dim3(32), 0, st, pdl, n_seq, a.seq_ids, a.ctx_len, a.path_len, 0, pdl ? 1 : 0);
 }
 
 void launch_advance_ctx(int n_seq, const int32_t *seq_ids, int32_t *ctx_len, int amount, bool pdl, cudaStream_t st) {
-  launch_k(advance_ctx_kernel, dim3(1), dim3(32), 0, st, pdl, n_seq, seq_ids, ctx_len, (const int32_t *)nullptr, amount,
-           pdl ? 1 : 0);
+  launch_k(advance_ctx_kernel, dim3(1), dim3(32), 0, st, pdl, n_seq, seq_ids, ctx_len, amount, pdl ? 1 : 0);
 }
 
 }  // namespace firp

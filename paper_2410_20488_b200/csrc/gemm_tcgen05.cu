@@ -866,7 +866,15 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
   // limit costs it 5 %.  A step's keep it, or 96 where that is more (an error below the planes' own).
   const int share = longest_sum(s.n_tiles, s.KB, rows, planes);
   int adds_wanted = epi == EPI_RESIDUAL ? std::max(176, (rows > kMaxTreeRows ? 1 : 2) * s.KB) : (epi == EPI_SWIGLU ? 260 : epi == EPI_LOGITS ? 512 : 176) * std::max(64, s.KB) / 64;
-  if (rows <= kMaxTreeRows) adds_wanted = std::min(adds_wanted, std::max(96, share));
+  if (rows <= kMaxTreeRows) {
+    adds_wanted = std::min(adds_wanted, std::max(96, share));
+    // Three tiles to a gate/up job would be faster with longer sums yet (one k slice, or two instead of three: 45 instead of 51 us at 131
+    // rows of the 7B shape, 137 instead of 160 at 140 of the 34B shape), at twice the error; so would fewer slices of the others'.
+    if (epi == EPI_QKV_ROPE && rows <= 48) adds_wanted = std::min(adds_wanted, 96);
+    if (epi == EPI_SWIGLU && s.KB > 96) adds_wanted = std::min(adds_wanted, rows <= 40 ? 256 : rows <= 128 ? 176 : 352);
+    if (epi == EPI_SWIGLU && s.KB <= 96 && rows > 128) adds_wanted = std::min(adds_wanted, 176 * std::max(64, s.KB) / 64);
+    if (epi == EPI_LOGITS && rows > 128) adds_wanted = std::min(adds_wanted, 352);
+  }
   for (int max_adds = adds_wanted; best.tm == 0 && max_adds < (1 << 20); max_adds *= 2)
   for (int most : {256, 192, 128}) {         // token rows of a block: blocks of equal size
   s.blocks = (rows + most - 1) / most;
@@ -887,6 +895,8 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
         const int cap = cluster_ctas(split) / split * split;
         int jobs = (s.n_tiles + tm - 1) / tm;
         const int waves = (jobs * s.blocks * split + cap - 1) / cap, kb = (s.KB + split - 1) / split;
+        // single gate/up tiles in several waves bring the activations to every one of them again: 146 us, pairs 128 (34B shape, 56 rows)
+        if (s.mode == ROWS_GATE_UP && tm == 1 && waves > 1 && rows <= kMaxTreeRows) continue;
         const int per = std::min(tm, s.n_tiles);
         // rings: four activation stages (two or three of the wide ones), the rest for weight tiles
         // and, when it is not much, room for the sums over the k slices (saves a cluster barrier) or the rotary table (an L2
@@ -931,7 +941,7 @@ Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int plan
         const float mma = (float)waves * per * kb * 4.f * (merged ? 1 : planes) * mma_clk(n_mma) / 1570.f;
         const float ingest = (float)waves * kb * (per * W_TILE + x_stage) / std::min(150e3f, 15e6f / ctas);
         const bool direct = split == 1 && (epi == EPI_QKV_ROPE || epi == EPI_SWIGLU || epi == EPI_LOGITS);
-        const float out = (sets > 2 ? 0.008f * R * per : 0.f) + (direct ? 0.028f * R * per : 0.017f * R * per + 0.0017f * own * per + (split == 1 || red ? 1.7f : 3.8f));
+        const float out = (sets > 2 ? 0.008f * R * per : 0.f) + (direct ? 0.028f * R * per : 0.017f * R * per + 0.0017f * own * per + (split == 1 ? 1.2f : red ? 1.7f : 3.8f));
         const float rings_us = (float)waves * kb * std::max(0.72f / sx, 1.12f * per / sw);
         const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.035f * (hbm + mma + ingest) + waves * (1.5f + out) + (split >= 7 ? 1.f : 0.f);
         TileCfg c{};

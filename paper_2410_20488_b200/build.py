@@ -10,7 +10,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfirp_b200.so")
 SOURCES = ["firp_api.cu", "small_kernels.cu", "topb.cu", "gemm_tcgen05.cu", "attn_tree.cu", "attn_tc.cu", "fused_step.cu",
            "topb_static.cu"]
-HEADERS = ["firp_kernels.cuh", "launch_util.cuh", "tc_device.cuh", "finish_device.cuh", "norm_device.cuh", "attn_device.cuh", "pipeline.h", "rows.h",
+HEADERS = ["firp_kernels.cuh", "launch_util.cuh", "tc_device.cuh", "finish_device.cuh", "norm_device.cuh", "attn_device.cuh", "pipeline.h", "rows.h", "gemm_plan.h",
            os.path.join("..", "..", "include", "firp.h")]
 # -dlcm=cg: plain global loads are cached in L2 only.  Under programmatic dependent launch kernels of
 # consecutive steps share an SM; buffers that are rewritten every step (context lengths, tree metadata,

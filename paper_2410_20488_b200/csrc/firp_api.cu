@@ -266,7 +266,7 @@ int run_rows(firp_ctx *c, const RunArgs &ra, cudaStream_t st) {
 
   enum { G_QKV = 0, G_O, G_GATE_UP, G_DOWN, G_LM_HEAD };     // index of c->planes
   auto launch = [&](GemmEpilogue epi, const void *W, int N, int K, int planes, const Rows &rows, LinArgs &l, int R) -> cudaError_t {
-    l.W = (const bf16 *)W; l.N = N; l.K = K; l.R = R; l.rw = rows; l.row_of = rows.by_step ? c->meta.row_of : nullptr; l.F = F; l.dh = dh; l.planes = planes; l.plane_rows = (int)Rp;
+    l.W = (const bf16 *)W; l.N = N; l.K = K; l.R = R; l.call_rows = epi == EPI_PSEUDO ? R : rows.R; l.rw = rows; l.row_of = rows.by_step ? c->meta.row_of : nullptr; l.F = F; l.dh = dh; l.planes = planes; l.plane_rows = (int)Rp;
     l.err = c->dev_status; l.wait_ns = c->wait_ns; l.eps = cfg.rms_eps;
     ++nl;
     return launch_gemm(epi, l, pdl, st);

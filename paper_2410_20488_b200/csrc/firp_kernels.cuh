@@ -4,19 +4,16 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gemm_plan.h"
 #include "rows.h"
 
 namespace firp {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int kMaxSeq = 16;        // sequences per step
-constexpr int kMaxTreeRows = 144;  // rows per sequence: T + k (128 + 8), or T (1 + k) with a chain under every node
-constexpr int kMaxPromptRows = 2047;  // rows of a prompt that run at once, pseudo rows included
 constexpr int kMaskWords = 5;      // ceil(136 / 32)
 constexpr int kMaxTopB = 8;
 constexpr int kAttnTile = 64;      // kv positions per attention tile
-constexpr int kGemmBK = 64;        // k elements per pipeline stage
 
 // Rows of the KV cache.  A (layer, K|V) plane holds max_batch * max_ctx rows of Hkv * dh elements.  Without a
 // page table position `pos` of slot `slot` is row slot * max_ctx + pos; with one (pages of kKvPage positions,
@@ -134,14 +131,13 @@ void launch_commit(int n_seq, const CommitArgs &a, bool pdl, cudaStream_t st);
 void launch_advance_ctx(int n_seq, const int32_t *seq_ids, int32_t *ctx_len, int amount, bool pdl, cudaStream_t st);   // after a stretch of a prompt
 
 // ---- weight-streaming GEMM ---------------------------------------------------
-enum GemmEpilogue { EPI_RESIDUAL = 0, EPI_QKV_ROPE = 1, EPI_SWIGLU = 2, EPI_LOGITS = 3, EPI_PSEUDO = 4 };
-
 // One GEMM of the kernel-per-operation mode: out[m][n] = sum_k X[m][k] W[n][k] and the elementwise step behind it.
 struct LinArgs {
   const bf16 *X;    // [planes][plane_rows][K] activations as bf16 planes
   int plane_rows, planes;
   const bf16 *W;    // [N][K] weights
   int R, N, K;      // token rows (<= kMaxPromptRows): the first R of the activations
+  int call_rows;    // rows of the call's last layers, where all pseudo rows are in: they set how long the sums may be (gemm_plan.h)
   Rows rw;
   const uint16_t *row_of;       // seq_row of every row of the activations; NULL: one sequence, row v is row v
   int *err;         // device status word (set to a non-zero code if a bounded wait gives up)

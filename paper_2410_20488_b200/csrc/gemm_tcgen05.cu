@@ -50,6 +50,7 @@
 
 #include "finish_device.cuh"
 #include "firp_kernels.cuh"
+#include "gemm_plan.h"
 #include "launch_util.cuh"
 #include "pipeline.h"
 #include "tc_device.cuh"
@@ -58,32 +59,12 @@ namespace cg = cooperative_groups;
 
 namespace firp {
 
+using namespace gemm;
+
 namespace {
 
-constexpr int BM = 128;            // weight rows per MMA tile
-constexpr int BK = kGemmBK;        // 64 bf16 = 128 bytes = one swizzle row
-constexpr int kThreads = 384;      // 12 warps
-constexpr int kEpiWarps = 8;
-constexpr int W_TILE = BM * 128;   // bytes of one 128-row weight tile of a k block
-constexpr int kSmemMax = 227 * 1024;
-constexpr int kTailBytes = 2496;   // row scales, slots and lengths, row indices, barriers, TMEM address (behind the rings)
-constexpr int kMaxRows = 256;      // token rows of a CTA (MMA N)
-constexpr int kNoRow = -1, kNoKv = -2;
-constexpr int kMaxW = 12, kMaxX = 6;  // ring depths: weight tiles, activation stages
+constexpr int kNoRow = -1, kNoKv = -2;      // of s_kv below
 
-// How the rows of the weight are dealt to tiles of 128, each one TMA box per k block.
-//   ROWS_LINEAR   128 neighbouring rows
-//   ROWS_GATE_UP  64 gate rows and the up rows that go with them, in turns of 8, so that such a pair is 8 lanes apart in one warp
-//   ROWS_ROTARY   128 / dh heads; the rows of a head in groups of 32: 16 columns of its first half, then their partners in
-//                 the second half, so that a rotary pair is 16 lanes apart in one warp
-enum RowMode { ROWS_LINEAR = 0, ROWS_GATE_UP = 1, ROWS_ROTARY = 2 };
-// Which tiles and k blocks a CTA multiplies.
-struct TileSched {
-  int mode, heads;   // heads: of a tile (ROWS_ROTARY)
-  int n_tiles, KB;   // tiles; 64-wide k blocks
-  int jobs, split;   // job j = tiles [n_tiles j / jobs, n_tiles (j + 1) / jobs), its k blocks cut over `split` CTAs
-  int blocks;        // of token rows: the CTAs of a job's blocks are neighbours, so that its weights come from HBM once
-};
 // A CTA starts its k range at a place of its own and wraps around: CTAs that march through k together would ask the same
 // L2 slices for the same activation rows, and HBM for weight rows whose addresses differ only above bit 12.
 struct CtaWork { int t0, nt, kb0, kb1, off, block; };
@@ -100,24 +81,6 @@ __device__ __forceinline__ CtaWork cta_work(const TileSched &s, int cta) {
 }
 // k block of unit u
 __device__ __forceinline__ int unit_kb(const CtaWork &w, int u) { const int k = w.kb0 + w.off + u; return k < w.kb1 ? k : k - (w.kb1 - w.kb0); }
-
-// Shared memory and operand shape of a launch.
-struct TileCfg {
-  int planes, npad;     // activation planes; token rows of a block padded to the MMA's N
-  int rpb;              // token rows of a block
-  int acc;              // accumulator columns per tile
-  int issuers, by_tile; // MMA issuing warps: they take the units in turn, each with accumulator sets of its own, or the tiles
-  int sets, acc_set;    // accumulator sets (summed in the epilogue), columns per set
-  int sw, sx;           // ring depths: weight tiles, activation stages
-  int planes_side;      // planes that sit side by side in the accumulator's columns
-  int tpo, inv_tpo;     // token rows finished per CTA of a cluster; ceil(65536 / tpo)
-  int tp;               // tiles per epilogue pass (what the ring's memory holds)
-  int tail;             // bytes from the rings' start to what lies behind them
-  int red_off;          // where the sums over the k slices go: behind the rings, or 0: over them
-  int rope_off, rope_bytes;      // the step's rotary table, if it is brought into shared memory
-  int pdl;
-  uint32_t idesc, tmem_cols;
-};
 
 // one k block of one tile: 16 KB
 __device__ __forceinline__ void load_tile(uint32_t dst, const CUtensorMap *tm, const TileSched &s, int tile, int kb, uint32_t bar, uint64_t pol) {
@@ -790,10 +753,6 @@ bool plane_map(CUtensorMap *m, const void *X, uint64_t planes, uint64_t plane_ro
   return make_map(m, X, d);
 }
 
-constexpr uint32_t pow2_cols(int c) { return c <= 32 ? 32 : c <= 64 ? 64 : c <= 128 ? 128 : c <= 256 ? 256 : 512; }
-constexpr int align_n(int v, int a) { return (v + a - 1) / a * a; }
-constexpr bool few_rows(int r) { return r <= 48; }      // of a block: the epilogue takes 8 at a time
-
 typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const LinArgs, const TileSched, const TileCfg);
 template <bool MERGED, bool DEEP, int C, int EPI> KernelFn kernel_tm(int tm) {
   return tm == 1 ? gemm_kernel<1, MERGED, DEEP, C, EPI> : tm == 2 ? gemm_kernel<2, MERGED, DEEP, C, EPI> : gemm_kernel<3, MERGED, DEEP, C, EPI>;
@@ -838,162 +797,34 @@ int cluster_ctas(int n) {
   return cap[n];
 }
 
-struct Plan { TileSched sc; TileCfg cf; int tm, merged, smem, adds; };
-
-// cycles of one M = 128, K = 16 MMA of n columns: reading the operands from shared memory (128 + n rows of 32 bytes at 128
-// bytes a cycle), computing, or issuing it, whichever takes longest (measured: 50 at 16 columns, 55 at 80, 72 at 144)
-float mma_clk(int n) { return std::max(50.f, std::max(n / 2.f, 34.f + n / 4.f)); }
-
-// Additions in a row that an accumulator would see if every SM of a B200 had an equal share of the matrix, in pairs of tiles, with two
-// planes into the same columns from 49 rows on.  The tensor core truncates where it adds to an accumulator, so the error of a sum
-// grows with their number: against 64-bit sums of the same planes, in the 2-norm, 0.24e-6 after 16, 0.48e-6 after 32, 1.1e-6 after
-// 76, 2.1e-6 after 128, 4.5e-6 after 256, 9.2e-6 after 512; what the two planes leave out of an activation is 2.4e-6.
-int longest_sum(int n_tiles, int KB, int rows, int planes) {
-  const int units = (n_tiles + 1) / 2 * KB, share = std::min(KB, (units + 147) / 148);
-  return std::max(16, 4 * share * (planes == 1 || rows <= (planes == 3 ? 80 : 48) ? 1 : planes));
-}
-
-Plan make_plan(GemmEpilogue epi, int N, int K, int F, int dh, int rows, int planes) {
-  Plan best{};
-  float best_cost = 1e30f;
-  TileSched s{};
-  s.mode = epi == EPI_SWIGLU ? ROWS_GATE_UP : epi == EPI_QKV_ROPE ? ROWS_ROTARY : ROWS_LINEAR;
-  s.heads = s.mode == ROWS_ROTARY ? BM / dh : 0;
-  s.n_tiles = s.mode == ROWS_GATE_UP ? (F + BM / 2 - 1) / (BM / 2) : (N + BM - 1) / BM;
-  s.KB = (K + BK - 1) / BK;
-  // A prompt's sums may be longer: its results are as far from a 64-bit run as with the equal shares' (cache rows of 1999 tokens of
-  // the 7B shape 2.24e-3 / 2.32e-3, of 500 2.76e-3 / 2.88e-3: the rounding of the cache to bf16 hides them), and the equal shares'
-  // limit costs it 5 %.  A step's keep it, or 96 where that is more (an error below the planes' own).
-  const int share = longest_sum(s.n_tiles, s.KB, rows, planes);
-  int adds_wanted = epi == EPI_RESIDUAL ? std::max(176, (rows > kMaxTreeRows ? 1 : 2) * s.KB) : (epi == EPI_SWIGLU ? 260 : epi == EPI_LOGITS ? 512 : 176) * std::max(64, s.KB) / 64;
-  if (rows <= kMaxTreeRows) {
-    adds_wanted = std::min(adds_wanted, std::max(96, share));
-    // Three tiles to a gate/up job would be faster with longer sums yet (one k slice, or two instead of three: 45 instead of 51 us at 131
-    // rows of the 7B shape, 137 instead of 160 at 140 of the 34B shape), at twice the error; so would fewer slices of the others'.
-    if (epi == EPI_QKV_ROPE && rows <= 48) adds_wanted = std::min(adds_wanted, 96);
-    if (epi == EPI_SWIGLU && s.KB > 96) adds_wanted = std::min(adds_wanted, rows <= 40 ? 256 : rows <= 128 ? 176 : 352);
-    if (epi == EPI_SWIGLU && s.KB <= 96 && rows > 128) adds_wanted = std::min(adds_wanted, 176 * std::max(64, s.KB) / 64);
-    if (epi == EPI_LOGITS && rows > 128) adds_wanted = std::min(adds_wanted, 352);
-  }
-  for (int max_adds = adds_wanted; best.tm == 0 && max_adds < (1 << 20); max_adds *= 2)
-  for (int most : {256, 192, 128}) {         // token rows of a block: blocks of equal size
-  s.blocks = (rows + most - 1) / most;
-  const int R = align_n((rows + s.blocks - 1) / s.blocks, s.blocks > 1 ? 16 : 1);
-  s.blocks = (rows + R - 1) / R;
-  if (most < 256 && rows <= kMaxTreeRows) break;
-  for (int merged = 1; merged >= 0; --merged) {
-    if (!merged && planes == 1) continue;
-    const int npad = merged ? align_n(R, planes == 2 ? 8 : 16) : align_n(R, 16);
-    const int n_mma = merged ? planes * npad : npad;
-    if (n_mma > 256) continue;
-    const int x_stage = planes * npad * 128;
-    for (int tm = 1; tm <= 3; ++tm) {
-      // the epilogue of many rows reads 16 columns at a time, 8 of them beyond the last plane's when npad is an odd multiple of 8
-      const int over = few_rows(R) ? 0 : npad & 8;
-      if (tm * n_mma + over > 512) continue;
-      for (int split = 1; split <= 8 && split <= s.KB; ++split) {
-        const int cap = cluster_ctas(split) / split * split;
-        int jobs = (s.n_tiles + tm - 1) / tm;
-        const int waves = (jobs * s.blocks * split + cap - 1) / cap, kb = (s.KB + split - 1) / split;
-        // single gate/up tiles in several waves bring the activations to every one of them again: 146 us, pairs 128 (34B shape, 56 rows)
-        if (s.mode == ROWS_GATE_UP && tm == 1 && waves > 1 && rows <= kMaxTreeRows) continue;
-        const int per = std::min(tm, s.n_tiles);
-        // rings: four activation stages (two or three of the wide ones), the rest for weight tiles
-        // and, when it is not much, room for the sums over the k slices (saves a cluster barrier) or the rotary table (an L2
-        // round trip every 16 token rows)
-        const int tpo = align_n((R + split - 1) / split, 4), per_tile = split * tpo * 512;         // bytes of a tile's sums
-        int red = split > 1 ? per * per_tile : 0, rope = epi == EPI_QKV_ROPE ? align_n(std::min(tpo, R) * dh * 4, 128) : 0;
-        if (red > 40 * 1024) red = 0;
-        if (rope > 24 * 1024) rope = 0;
-        const int side = red + rope;
-        const int avail = kSmemMax - 1024 - kTailBytes - side;
-        int sx = std::min(x_stage <= 12 * 1024 ? 4 : x_stage <= 24 * 1024 ? 3 : 2, std::max(kb, 1));
-        const bool by_unit = tm == 1 && 2 * n_mma + over <= 512 && s.KB / split >= 2;
-        if (by_unit) sx = std::max(2, sx & ~1);
-        int sw = std::min(std::min(kMaxW, (avail - sx * x_stage) / W_TILE), kb * per);
-        if (by_unit) sw &= ~1; else sw = sw / per * per;
-        if (sw < per || sw * W_TILE + sx * x_stage > avail) continue;
-        if (x_stage <= 24 * 1024) sx = std::min(std::min(kMaxX, kb), (avail - sw * W_TILE) / x_stage);      // what is left
-        if (by_unit) sx &= ~1;
-        if (sw < 2 * per && kb > 1) continue;
-        // As many accumulator sets as fit, up to four, share the k blocks; what is still longer than the limit is left to a
-        // split.
-        int sets = by_unit ? 2 : 1;
-        const int per_kb = (BK / 16) * (merged ? 1 : planes);
-        auto adds_of = [&](int n) { return (kb + n - 1) / n * per_kb; };
-        while (sets < 4 && (adds_of(sets) > std::min(share, max_adds) || (adds_of(sets) > 96 && (sets < 2 || rows > kMaxTreeRows))) &&
-               2 * sets * tm * n_mma + over <= 512 && s.KB / split >= 2 * sets) sets *= 2;
-        // Three are not dealt to two issuers, and one is too slow for a whole contraction (13B shape, 131 rows: the QKV projection
-        // 49.6 us so, 44.2 in three slices of three tiles; down in three slices 41.5, in eight of three tiles 46.6).
-        const bool lone = by_unit && sets == 2 && adds_of(2) > std::min(share, max_adds) && split > 1 && 3 * n_mma + over <= 512 && s.KB / split >= 3;
-        if (lone) sets = 3;
-        const int adds = adds_of(sets);
-        if (adds > max_adds) continue;
-        // Microseconds: the weights at the rate HBM gives that many CTAs (6.8 TB/s from 84 on), a CTA's MMAs, its bytes from L2 (which
-        // gives a CTA 150 GB/s and all of them 15 TB/s), or a ring's turnaround, whichever is longest; a share of the others; and for each
-        // wave its start and its epilogue: from registers, or a push to the CTAs of the cluster and the sums there.  The constants are a
-        // fit to every plan of the 7B, 13B and 34B shapes' projections at 20-140 token rows and at prompts of 150-2002 (9216 times of
-        // launches back to back): within 7 % of the times of the plans near the best; the plan it chooses takes 0.8 % longer than the
-        // best one (constants set by hand: 1.5 %; the four projections of a layer of the 7B shape at 67 / 108 / 128 rows 94 / 114 / 120 us,
-        // now 93 / 108 / 116).
-        const int ctas = std::min(jobs * s.blocks * split, cap), own = std::min(tpo, R);
-        const float hbm = (float)s.n_tiles * s.KB * W_TILE / 6.8e6f * std::max(1.f, 84.f / ctas);
-        const float mma = (float)waves * per * kb * 4.f * (merged ? 1 : planes) * mma_clk(n_mma) / 1570.f;
-        const float ingest = (float)waves * kb * (per * W_TILE + x_stage) / std::min(150e3f, 15e6f / ctas);
-        const bool direct = split == 1 && (epi == EPI_QKV_ROPE || epi == EPI_SWIGLU || epi == EPI_LOGITS);
-        const float out = (sets > 2 ? 0.008f * R * per : 0.f) + (direct ? 0.028f * R * per : 0.017f * R * per + 0.0017f * own * per + (split == 1 ? 1.2f : red ? 1.7f : 3.8f));
-        const float rings_us = (float)waves * kb * std::max(0.72f / sx, 1.12f * per / sw);
-        const float cost = std::max(std::max(hbm, rings_us), std::max(mma, ingest)) + 0.035f * (hbm + mma + ingest) + waves * (1.5f + out) + (split >= 7 ? 1.f : 0.f);
-        TileCfg c{};
-        c.planes = planes; c.rpb = R; c.npad = npad; c.acc = n_mma; c.sw = sw; c.sx = sx;
-        c.tpo = tpo; c.inv_tpo = (65536 + c.tpo - 1) / c.tpo;
-        c.planes_side = merged ? planes : 1; c.acc_set = tm * n_mma; c.sets = sets; c.issuers = (by_unit && !lone) || tm >= 2 ? 2 : 1; c.by_tile = tm >= 2;
-        c.idesc = instr_desc_m128(n_mma); c.tmem_cols = pow2_cols(c.sets * tm * n_mma + over);
-        const int rings = align_n(sw * W_TILE + sx * x_stage, 128);
-        if (red) {
-          c.red_off = rings; c.tp = per; c.tail = rings + red;
-        } else {
-          c.tail = align_n(std::max(rings, direct ? 0 : per_tile), 128);      // over the rings
-          c.tp = direct ? per : std::min(per, c.tail / per_tile);
-        }
-        if (rope) { c.rope_off = c.tail; c.rope_bytes = rope; c.tail += rope; }
-        const int smem = c.tail + 1024 + kTailBytes;
-        if (smem > kSmemMax || cost >= best_cost) continue;
-        best_cost = cost;
-        best = Plan{s, c, tm, merged, smem, adds};
-        best.sc.jobs = jobs; best.sc.split = split;
-      }
-    }
-  }
-  }
-  return best;
-}
-
-Plan cached_plan(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes) {
-  typedef std::tuple<int, int, int, int, int, int> Key;
+Plan cached_plan(const GemmShape &g, int rows, int call_rows) {
+  typedef std::tuple<int, int, int, int, int, int, int> Key;
   static std::map<Key, Plan> cache;
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
-  const Key key((int)epi * 256 + dh, N, K, F, R, planes);
+  const Key key((int)g.epi * 256 + g.dh, g.N, g.K, g.F, rows, call_rows, g.planes);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
-  const Plan p = make_plan(epi, N, K, F, dh, R, planes);
+  int ctas[9] = {0};
+  for (int n = 1; n <= 8; ++n) ctas[n] = cluster_ctas(n);
+  const Plan p = make_plan(g, rows, call_rows, ctas);
   if (cache.size() > 4096) cache.clear();
   return cache[key] = p;
 }
 
 }  // namespace
 
-int gemm_additions(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes) { return cached_plan(epi, N, K, F, dh, R, planes).adds; }
+int gemm_additions(GemmEpilogue epi, int N, int K, int F, int dh, int R, int planes) { return cached_plan({epi, N, K, F, dh, planes}, R, R).adds; }
 
 bool gemm_tc_available() { return encode_fn() != nullptr; }
 
 cudaError_t launch_gemm(GemmEpilogue epi, const LinArgs &a, bool pdl, cudaStream_t st) {
   if (!encode_fn()) return cudaErrorNotSupported;
-  Plan p = cached_plan(epi, a.N, a.K, a.F, a.dh, a.R, a.planes);
+  Plan p = cached_plan({epi, a.N, a.K, a.F, a.dh, a.planes}, a.R, a.call_rows);
   if (p.tm == 0 || p.smem > kSmemMax || p.cf.tp < 1 || p.cf.sw < 1 || p.cf.sx < 1 || (!p.cf.by_tile && p.cf.issuers == 2 && ((p.cf.sw | p.cf.sx | p.cf.sets) & 1)))
     return cudaErrorInvalidConfiguration;
   p.cf.pdl = pdl ? 1 : 0;
+  p.cf.idesc = instr_desc_m128(p.cf.acc);
   KernelFn fn = kernel_of(epi, p.tm, p.merged != 0, p.cf.sets > 2 || p.cf.planes_side > 2, few_rows(p.cf.rpb));
   static std::map<KernelFn, int> configured;
   static std::mutex mu;

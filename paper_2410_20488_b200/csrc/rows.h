@@ -12,6 +12,10 @@
 
 namespace firp {
 
+constexpr int kMaxSeq = 16;        // sequences per step
+constexpr int kMaxTreeRows = 144;  // rows per sequence: T + k (128 + 8), or T (1 + k) with a chain under every node
+constexpr int kMaxPromptRows = 2047;  // rows of a prompt that run at once, pseudo rows included
+
 // Per-step row geometry shared by every kernel.  Row r = s * Ms + v in what the caller gives and gets and in TreeMeta.
 struct Rows {
   int n_seq;   // sequences in this step

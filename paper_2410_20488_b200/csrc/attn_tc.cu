@@ -115,15 +115,20 @@ template <int NH, bool SUM> __device__ __forceinline__ void warp_cols_to_smem(co
 }
 
 // The K or V buffers as their producer sees them (pipeline.h): a buffer is free again when the MMAs that read it have completed.
+constexpr int kKvRing = 2;
 struct KvRing {
   const CUtensorMap *tm; const AttnArgs &a;
   uint32_t full, freed, dst0;
   int slot, t0, n, kv_len, kvh;
   uint64_t pol; unsigned long long wait_ns; bool dead;
   bool waited;                     // for the QKV projection, which writes the rows from n on
-  __device__ __forceinline__ bool free(int, int w, uint32_t parity) { return mbar_wait(freed + 8 * w, parity, a.err, dead, wait_ns); }
+  __device__ __forceinline__ void wait_for_projection() { if (!waited) { griddep_wait(); waited = true; } }
+  __device__ __forceinline__ bool free(int i, int w, uint32_t parity) {
+    if (i >= kKvRing) wait_for_projection();        // a buffer comes free only after it, and a limit does not count it
+    return mbar_wait(freed + 8 * w, parity, a.err, dead, wait_ns);
+  }
   __device__ __forceinline__ void load(int i, int w) {
-    if (!waited && (t0 + i + 1) * kTcTile > n) { griddep_wait(); waited = true; }
+    if ((t0 + i + 1) * kTcTile > n) wait_for_projection();
     mbar_expect_tx(full + 8 * w, kTcStage);
 #pragma unroll
     for (int ph = 0; ph < 2; ++ph) {                // 64-position x 64-element boxes; a half lies inside one page
@@ -139,6 +144,7 @@ struct KvRing {
 struct RowsKvRing : KvRing {     // of the kernel for many query rows: S or O of the tile before in this buffer, on barriers in threes
   __device__ __forceinline__ bool free(int i, int, uint32_t) {
     if (i < kRowsKvRing) return true;
+    wait_for_projection();
     const TilePhase f = rows_spo(i - kRowsKvRing);
     return mbar_wait(freed + 8 * f.bar, f.parity, a.err, dead, wait_ns);
   }
@@ -153,7 +159,8 @@ __device__ unsigned long long g_attn_trace[16];
 
 // What happens under the QKV projection.  It lets this kernel start only after its own wait, so that all that was written before it --
 // lengths, slots, the cache's committed rows -- may be read without waiting for it: the tiles that lie in the committed prefix are on
-// their way or in shared memory when it completes, only the queries and the tile with the step's own rows are loaded after that.  us
+// their way or in shared memory when it completes, only the queries and the tile with the step's own rows are loaded after that.  Each
+// role waits for the projection before the first of its own waits that only it can end, so that no limit counts its time.  us
 // per step, everything behind one wait / this: one row of the 7B shape 2690 / 2634, 35 rows at 512 tokens 3166 / 3156, at 8192 4238 / 4214,
 // 131 rows 5969 / 5909, four requests of the 34B shape 6094 / 6021.
 //
@@ -272,11 +279,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       uint64_t pol;
       asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
       KvRing ring{tm, a, full, freed, dst0, sn.x, kv.t0, sn.y, kv.kv_len, kvh, pol, wait_ns, false, false};
-      drain(ring, produce(ring, kv.ntiles, 2), 2);
+      drain(ring, produce(ring, kv.ntiles, kKvRing), kKvRing);
     }
   } else if (warp == 16) {
     // ---- MMA issuer (one lane): S^T of tile i, then O^T of tile i - 1
     wait_slot_and_length(18 * 32);
+    if (pdl) griddep_wait();       // the limit of the waits below starts here
     if (lane == 0) {
       const int ntiles = kv_range(s_sn[1], a.rows_active, a.max_ctx, split, nsplits).ntiles;      // tile t0 + i goes to tile group i & 1 as its (i >> 1)-th
       const uint32_t idesc_k = instr_desc_m128(NQ), idesc_mn = idesc_k | (1u << 15);
@@ -715,6 +723,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     // ---- MMA issuer of S, up to three tiles ahead of O
     const uint64_t kdesc = smem_desc(sb + K_OFF), qdesc = smem_desc(sb + Q_OFF);
     const uint32_t q_lo = (uint32_t)qdesc, hi = (uint32_t)(kdesc >> 32);
+    if (pdl) griddep_wait();                        // the limit of the waits below starts here
     mbar_wait(q_ready, 0, a.err, dead, wait_ns);
     int b3 = 0;                                     // i % 3
     for (int i = 0; i < ntiles; ++i) {
@@ -746,6 +755,7 @@ tree_attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const uint64_t vdesc = smem_desc_mn(sb + V_OFF, kTcSlab);
     const uint32_t hi = (uint32_t)(vdesc >> 32);
     int b3 = 0, ph3 = 0;                            // i % 3, i / 3
+    if (pdl) griddep_wait();
     for (int i = 0; i < ntiles; ++i) {
       const int w = i & 1;
       const uint32_t v_lo = (uint32_t)vdesc + (uint32_t)(w * (kTcStage >> 4)), pcol = tmem + b3 * 128;

@@ -70,6 +70,30 @@ def test_a_limit_shorter_than_a_kernel_is_no_time_out():
     eng.close()
 
 
+@pytest.mark.parametrize("T,Hkv", [(32, 64), (128, 8)])
+def test_a_limit_shorter_than_the_projection_before_the_attention_is_no_time_out(T, Hkv):
+    """The attention's blocks start under the QKV projection (403 MB of weights or 131 rows: more than 40 us) and load the first tiles of
+    the cached context, which has many for each; their waits for what the projection ends do not count it: a limit of 25 us is no time-out.
+    Both tcgen05 kernels: 35 query rows on 64 kv heads, 1048 on 8."""
+    import numpy as np
+    import torch
+    from paper_2410_20488_b200 import FirpEngine
+    n = 4000
+    shape = si.scaled(si.CONFIGS["c1"], L=1, l=0, d=8192, H=64, Hkv=Hkv, dh=128, F=1024)
+    eng = FirpEngine(shape, si.all_weights(shape), max_ctx=4352, max_tree=T)
+    eng.kv.view(torch.bfloat16).normal_(0.0, 1.8)
+    tokens = torch.from_numpy(si.random_tokens(shape, T, 3)).cuda()
+    first, second = eng.new_out(1, T, shape.k), eng.new_out(1, T, shape.k)
+    for out, limit in ((first, 0), (second, 25)):
+        eng.set_wait_limit_us(limit)
+        for _ in range(4):
+            eng.set_context_len(0, n)
+            eng.step(tokens, np.asarray(si.tree_template(T)), shape.k, shape.l, out)
+            assert eng.context_len(0) == n         # raises on a time-out
+    assert torch.equal(first.logits, second.logits)
+    eng.close()
+
+
 @pytest.mark.parametrize("d,H,Hkv,F,V", [(4096, 32, 32, 11008, 32000), (5120, 40, 40, 13824, 32000), (8192, 64, 8, 22016, 32000)])
 def test_sums_of_a_step_are_no_longer_than_equal_shares_make_them(d, H, Hkv, F, V):
     """The tensor core truncates on every addition: no accumulator of a step sees more in a row than if every SM had an equal share

@@ -81,7 +81,7 @@ struct firp_ctx {
   // host mirrors
   std::vector<int32_t> n_hi;           // upper bound of each slot's committed length
   std::vector<int32_t> last_parents, last_next_parents, last_seq_ids, last_sizes;
-  int last_n_seq = 0, last_T = 0, last_k = 0, last_Ms = 0;
+  int last_n_seq = 0, last_T = 0, last_k = 0;
   int pseudo_masked = 0;     // Section 4.3 "Masked": pseudo rows do not see one another
   int pred_prenorm = 0;      // Eq. 3 reads the anchor through the insertion layer's input RMSNorm
   int planes[5] = {2, 2, 2, 2, 2};
@@ -113,6 +113,7 @@ struct firp_ctx {
     meta.mask = c.take<uint32_t>(Rt * kMaskWords);
     meta.rope = c.take<float2>(R * half);
     meta.row_of = c.take<uint16_t>(Rt);
+    meta.n0 = c.take<int32_t>(kMaxSeq);
     ctx_len = c.take<int32_t>(cfg.max_batch);
     seq_ids = c.take<int32_t>(kMaxSeq);
     parents = c.take<int32_t>(kMaxTreeRows);
@@ -603,7 +604,7 @@ static int step_impl(firp_ctx *ctx, int32_t n_seq, const int32_t *seq_ids, const
   ra.out = out; ra.logits_dst = (out && out->logits) ? out->logits : ctx->logits; ra.n_hi_max = n_hi_max;
   ra.parents_stride = tree_sizes ? T : 0; ra.d_sizes = tree_sizes ? ctx->tree_sizes : nullptr;
   if ((rc = run_rows(ctx, ra, st))) return rc;
-  ctx->stepped = true; ctx->last_n_seq = n_seq; ctx->last_T = T; ctx->last_k = k; ctx->last_Ms = Ms;
+  ctx->stepped = true; ctx->last_n_seq = n_seq; ctx->last_T = T; ctx->last_k = k;
   return FIRP_OK;
 }
 
@@ -763,7 +764,7 @@ int firp_kv_commit(firp_ctx *ctx, int32_t n_seq, const int32_t *seq_ids, const i
   a.kv = ctx->kv; a.seq_stride = ctx->kv_seq(); a.layer_stride = ctx->kv_layer(); a.kv_stride = ctx->kv_plane();
   a.max_ctx = ctx->cfg.max_ctx; a.pages = ctx->pages();
   a.n_layers = ctx->cfg.n_layers; a.nkv = ctx->cfg.n_kv_heads * ctx->cfg.head_dim; a.seq_ids = ctx->seq_ids;
-  a.S = S; a.ctx_len = ctx->ctx_len; a.pos = ctx->meta.pos; a.Ms = ctx->last_Ms;
+  a.S = S; a.ctx_len = ctx->ctx_len; a.n0 = ctx->meta.n0;
   ctx->launches = 0;
   if (path) {
     for (int s = 0; s < n_seq; ++s) {

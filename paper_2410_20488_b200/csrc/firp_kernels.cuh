@@ -59,6 +59,7 @@ struct TreeMeta {
   uint32_t *mask;      // [R][kMaskWords] bit u: row v attends to new row u of its sequence
   float2 *rope;        // [R][dh/2] (cos, sin) of pos * theta^(-2c/dh), by row of the activations
   uint16_t *row_of;    // [R] seq_row of each row of the activations
+  int32_t *n0;         // [n_seq] committed length of each sequence when the step began
 };
 struct PrepArgs {
   Rows rw;
@@ -124,7 +125,7 @@ struct CommitArgs {
   const int32_t *path_len;  // [n_seq] device
   int S;
   int32_t *ctx_len;         // [max_batch] device
-  const int32_t *pos; int Ms;   // of the step: n = pos[s * Ms], its committed length
+  const int32_t *n0;        // [n_seq] device: n, the committed lengths of the step
   int max_ctx; KvPages pages;
 };
 void launch_commit(int n_seq, const CommitArgs &a, bool pdl, cudaStream_t st);

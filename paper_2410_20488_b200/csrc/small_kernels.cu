@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(PrepArgs a, int pdl)
   if (a.zero_word && r == 0 && tid == 0) *a.zero_word = 0u;
   if (rw.by_step && tid == 0) a.meta.row_of[ar] = seq_row(s, v);
   const int n = a.ctx_len[a.seq_ids[s]];
+  if (v == 0 && tid == 0) a.meta.n0[s] = n;
   for (int u = tid; u <= v && !rw.prompt; u += kPrepThreads) {
     int p;
     if (u < rw.T) p = a.parents[s * a.parents_stride + u];
@@ -177,8 +178,9 @@ void launch_accept(const Rows &rw, const AcceptArgs &a, bool pdl, cudaStream_t s
 // KV compaction of the accepted path.  Each thread owns one 16-byte column slice of a
 // (layer, K|V) plane and moves it for every path entry: it loads all source rows before
 // storing any, so a destination slot that is another entry's source is never clobbered.
-// One block moves the context length on; the others take it from the step's bookkeeping, where the root row's position is the
-// committed length (a kernel of its own for that: 3 us of the host and 2 of the two-layer shape's round, 78.2 -> 76.2 us).
+// One block moves the context length on; all take it from the step's bookkeeping, at a place that does not hang on the step's sizes, so
+// that a captured commit serves steps of any (a kernel of its own for the length: 3 us of the host and 2 of the two-layer shape's round,
+// 78.2 -> 76.2 us).
 // ---------------------------------------------------------------------------
 constexpr int kMaxPath = 16;
 
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(128) commit_kernel(CommitArgs a, int pdl) {
   if (pdl) { griddep_launch(); griddep_wait(); }
   const int s = blockIdx.y, plane = blockIdx.x;     // plane = layer * 2 + (0 K, 1 V)
   const int slot = a.seq_ids[s];
-  const int n = a.pos[s * a.Ms];                    // not from ctx_len, which one block writes below while others start
+  const int n = a.n0[s];                            // not from ctx_len, which one block writes below while others start
   const int len = min(a.path_len[s], kMaxPath);
   if (plane == 0 && threadIdx.x == 0) a.ctx_len[slot] = n + len;
   const int32_t *path = a.path + (size_t)s * a.S;

@@ -589,6 +589,43 @@ def test_device_side_commit_matches_explicit(torch_cuda, c1, c1_weights):
     eng.close()
 
 
+def test_a_captured_commit_serves_steps_of_other_sizes(torch_cuda, c1, c1_weights):
+    """A graph that holds only the commit of two sequences, captured after a step of 8 tree rows and replayed after steps of 5 and of 8:
+    every replay moves each context on by what its own step accepted and compacts its own rows, as the direct call does."""
+    import torch
+    lengths, sizes = (40, 23), (5, 8)
+    templates = {T: si.random_tree(41, T, 3, 2) if T == 5 else si.tree_template(8) for T in sizes}
+    ends = []
+    for captured in (True, False):
+        eng, _ = make_pair(c1, c1_weights, 256, max_batch=2)
+        for s_i, n in enumerate(lengths):
+            eng.prefill(s_i, torch.from_numpy(si.prompt(c1, seq=s_i, length=n)).cuda(), 3, 1, templates[8], eng.new_out(1, 1, 3, T_next=8))
+        outs = {T: eng.new_out(2, T, 3) for T in sizes}
+        tokens = {T: torch.from_numpy(np.stack([si.random_tokens(c1, T, s_i) for s_i in range(2)])).cuda() for T in sizes}
+
+        def step(T):
+            eng.step(tokens[T], templates[T], 3, 1, outs[T], n_seq=2)
+        for T in sizes:                    # what later calls find in place
+            step(T)
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            eng.commit(2)
+        want = list(lengths)
+        for T in (5, 8, 5):
+            step(T)
+            if captured:
+                graph.replay()
+            else:
+                eng.commit(2)
+            want = [w + int(outs[T].n_accepted[s_i].item()) for s_i, w in enumerate(want)]
+            assert [eng.context_len(0), eng.context_len(1)] == want
+        cache = eng.kv.view(torch.int16).view(c1.L, 2, 2, 256, -1)
+        ends.append([cache[:, :, s_i, :want[s_i]].cpu() for s_i in range(2)])
+        eng.close()
+    assert all(torch.equal(a, b) for a, b in zip(*ends))
+
+
 def test_device_side_commits_do_not_exhaust_the_capacity_bound(torch_cuda, c1, c1_weights):
     """A free-running loop that only ever commits on the device: the host's upper bound of the committed length
     grows by max_depth + 1 per step, the true length by about 1.  The step must keep running until the TRUE

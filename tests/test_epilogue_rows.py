@@ -1,7 +1,8 @@
 """The GEMMs' epilogues at the row counts where their passes change: 8 token rows at a time up to 48 rows and 16 above, a last pass of 1 row and of all
 of them, operands of an odd multiple of 8 columns (a pass of 16 reads past them), one or two planes to an operand; with rows that
 a layer does not have yet (pseudo rows inserted at the second layer) and matrices that end inside a tile, a group of 8 gate and up rows among
-them.  Lock-step against the oracle, the bounds are the harness's own."""
+them.  Matrices of this size take single tiles and no cluster; test_gemm_variants.py has the kernels of large ones.  Lock-step against the oracle,
+the bounds are the harness's own."""
 import pytest
 
 import synth_inputs as si

@@ -150,13 +150,6 @@ struct RowsKvRing : KvRing {     // of the kernel for many query rows: S or O of
   }
 };
 
-#ifdef FIRP_ATTN_TRACE
-__device__ unsigned long long g_attn_trace[16];
-#define TC_STAMP(k) do { if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) g_attn_trace[k] = globaltimer(); } while (0)
-#else
-#define TC_STAMP(k) do { } while (0)
-#endif
-
 // What happens under the QKV projection.  It lets this kernel start only after its own wait, so that all that was written before it --
 // lengths, slots, the cache's committed rows -- may be read without waiting for it: the tiles that lie in the committed prefix are on
 // their way or in shared memory when it completes, only the queries and the tile with the step's own rows are loaded after that.  Each
@@ -208,7 +201,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   __shared__ int s_sn[2];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  TC_STAMP(0);
   uint8_t *base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sb = smem_u32(base);
   const uint32_t bar0 = smem_u32(s_bar);
@@ -234,7 +226,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   if (pdl) griddep_launch();
-  TC_STAMP(1);
 
   const int kvh = blockIdx.y, G = a.H / a.Hkv;
   const int qblocks = gridDim.z / a.rw.n_seq;
@@ -243,7 +234,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int qrows_total = a.rows_active * G, q0 = qb * qper;
   const int ncols = min(qper, qrows_total - q0);
   // queries of this block (all softmax threads share the work): column j = query row q0 + j -> (tree row
-  // (q0 + j) / G, head kvh G + (q0 + j) % G).  Their loads go out before the context length above is first used.
+  // (q0 + j) / G, head kvh G + (q0 + j) % G).  Their loads go out before the context length below is first used.
   constexpr int QIT = (NQ * 16 + kTcSoft - 1) / kTcSoft;
   uint4 qh[QIT], ql[QIT];
   if (warp < 16) {
@@ -346,7 +337,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           *reinterpret_cast<uint4 *>(base + LY::Q_OFF + 2 * LY::Q_SLAB + off) = ql[it];
         }
       }
-      TC_STAMP(15);
       fence_async_smem();
       mbar_arrive(q_ready);
       if (tid < ncols) {
@@ -354,7 +344,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         s_oidx[tid] = (uint32_t)((act_row(a.rw, s, qr / G) * a.H + kvh * G + qr % G) * kTcDh);
       }
     }
-    TC_STAMP(2);
     const float scale_log2 = rsqrtf((float)kTcDh) * 1.4426950408889634f;
     // where this thread's position pair goes in a P row: 64-position half, 16-byte chunk, element
     const int p_half = wt >> 6, p_chunk = (wt & 63) >> 3, p_el2 = wt & 6, odd = wt & 1;
@@ -380,7 +369,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       __syncwarp();
       mbar_wait(s_ready + 8 * g, q & 1, a.err, dead, wait_ns);
       tc_fence_after();
-      if (i == 0) TC_STAMP(3);
       // pass 1: the tile's scores of this position (one wait for all TMEM loads), scaled and masked, and the
       // column maxima over the tile's positions
       float sv[NH];
@@ -390,7 +378,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int j = 0; j < NH; ++j) sv[j] = ((vis >> j) & 1u) ? sv[j] * scale_log2 : -INFINITY;
       warp_cols_to_smem<NH, false>(sv, &s_red[g][c_lo], warp & 3, lane);
       wg_sync(wgi);
-      if (i == 0) TC_STAMP(4);
       if (wt < NH) {
         const int j = c_lo + wt;
         const float4 v = *reinterpret_cast<const float4 *>(s_red[g][j]);
@@ -403,7 +390,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         s_l[g][j] = (s_l[g][j] + ((ps.x + ps.y) + (ps.z + ps.w))) * cr;
       }
       wg_sync(wgi);
-      if (i == 0) TC_STAMP(5);
       // pass 2: P = 2^(s - m) as bf16 (hi, lo) into the B operand of the second contraction.  Lanes 2i and 2i + 1
       // hold neighbouring positions: they swap one column of each column pair, so that every lane converts and
       // stores two neighbouring positions of one column as one 32-bit word.
@@ -445,10 +431,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       fence_async_smem();
       tc_fence_before();
       mbar_arrive(p_ready + 8 * g);
-      if (i == 0) TC_STAMP(6);
       mbar_wait(o_ready + 8 * g, q & 1, a.err, dead, wait_ns);
       tc_fence_after();
-      if (i == 0) TC_STAMP(7);
       // O^T of the tile joins the running one
       float *ov = sv;                                  // the scores are dead
       tc_ld_cols<NH>(tlane + NQ, ov);
@@ -462,10 +446,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         o_acc[4 * q4 + 3] = o_acc[4 * q4 + 3] * c4.w + ov[4 * q4 + 3];
       }
       tc_fence_before();
-      if (i == 0) TC_STAMP(8);
     }
   }
-  TC_STAMP(9);
   // ---- merge: o = sum_p 2^(m_p - M) O_p / sum_p 2^(m_p - M) l_p over the partials p = (kv split, tile group).
   // Columns go in groups of four; group c is finalised by CTA c % splits.  Once every CTA of the cluster has left
   // its tile loop (its buffers are free), every softmax thread pushes its columns of its tile group's partial into
@@ -485,7 +467,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   tc_fence_before();
   cg::cluster_group cluster = cg::this_cluster();
   if (nsp > 1) cluster.sync(); else __syncthreads();
-  TC_STAMP(11);
   if (warp == 16) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
@@ -513,9 +494,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       dl[(part * slots + sl) * 4 + (j & 3)] = s_l[my_g][j];
     }
   }
-  TC_STAMP(12);
   if (nsp > 1) cluster.sync(); else __syncthreads();
-  TC_STAMP(13);
   // owners: warpgroup w takes the received groups w, w + 4, ...; thread t of it dh index t of the group's four columns
   if (warp < 16) {
     for (int sl = warp >> 2; rank + sl * nsp < NG && 4 * (rank + sl * nsp) < ncols; sl += 4) {
@@ -549,7 +528,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
     }
   }
-  TC_STAMP(14);
 }
 
 // ---------------------------------------------------------------------------
@@ -1036,12 +1014,6 @@ cudaError_t launch_rows(const CUtensorMap &tmK, const CUtensorMap &tmV, const At
 }
 
 }  // namespace
-
-#ifdef FIRP_ATTN_TRACE
-extern "C" int firp_debug_attn_trace(unsigned long long *out) {
-  return (int)cudaMemcpyFromSymbol(out, g_attn_trace, sizeof(unsigned long long) * 16);
-}
-#endif
 
 // More than 48 query rows share a block of 128 once the context has more than 6 tiles; a prompt always does.  Measured at the
 // 7B / 13B shapes, us per step with blocks of 48 / of 128: 128 rows over 5 tiles 4820 / 4850, 67 rows over 9 tiles 6490 / 6390,

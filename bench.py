@@ -126,7 +126,7 @@ def kernel_source_digest() -> str:
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2410_20488_b200", "csrc")
     for name in sorted(os.listdir(csrc)):
-        if name.endswith((".cu", ".cuh")) and name != "firp_api.cu":       # device code only (firp_api.cu is host code)
+        if name.endswith((".cu", ".cuh", ".h")) and name != "firp_api.cu":       # device code, and the plans that choose it (firp_api.cu is host code)
             h.update(open(os.path.join(csrc, name), "rb").read())
     return h.hexdigest()[:16]
 

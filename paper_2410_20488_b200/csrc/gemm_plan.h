@@ -93,7 +93,9 @@ struct Rates {
 // Two sets of them, because what is fastest must not decide how long the sums are.  How long: kBySums, set by hand; the plan that it finds
 // for the rows of the whole call is the measure of precision, and stays as it is.  Which of the plans whose sums are no longer: kByTime, a
 // fit to every plan of the 7B, 13B and 34B shapes' projections at 20-140 token rows and at prompts of 150-2002 (9216 times of launches
-// back to back), within 7 % of the times of the plans near the best.  (Without that limit jobs of three gate/up tiles with sums twice as
+// back to back), within 7 % of the times of the plans near the best.  Under the same limit, us per step with the first set's constants alone / with
+// pairs of gate/up tiles only / so: a chain under each of 32 nodes 3766 / 3777 / 3737, 6 x 18 rows 4754 / 4733 / 4718, 131 rows 5771 / 5766 / 5754,
+// 67 rows of the 13B shape 6351 / 6325 / 6327, 4 x 35 of the 34B shape 5833 / 5798 / 5842 (spread 0.3 %, the last 0.8).  (Without that limit jobs of three gate/up tiles with sums twice as
 // long would be chosen: 45 instead of 51 us at 131 rows of the 7B shape, 137 instead of 160 at 140 of the 34B shape.)
 constexpr Rates kBySums{1850.f, 0.004f, 0.5f, 0.025f, 0.025f, 0.05f, 0.5f, 1.f, 2.f, 0.9f, 1.4f, 0.1f, 2.f, 3.f, 128, 1984, true};
 constexpr Rates kByTime{1570.f, 0.008f, 0.f, 0.028f, 0.017f, 0.0017f, 1.2f, 1.7f, 3.8f, 0.72f, 1.12f, 0.035f, 1.5f, 1.f, 0, kTailBytes, false};

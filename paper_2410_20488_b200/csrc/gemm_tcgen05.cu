@@ -137,8 +137,8 @@ struct ActRing : RingBase {      // all planes of a k block per slot
 // The epilogue's code runs once per launch from a cold instruction cache, in the shadow of nothing: one kernel per epilogue
 // and rolled loops keep it short (all five in one kernel, four items unrolled: 5-7 us instead of 1-2).
 // C: token rows (TMEM columns) that the epilogue takes at a time.  Eight for up to 48 rows: its passes are then so short that they run
-// about as long as their code takes to come from a cold instruction cache (us per step with 16 / with 8: two-layer shape 79.7 / 75.1, one
-// row of the 7B shape 2722 / 2690, 35 rows 3220 / 3166); with more rows sixteen hide more of the TMEM loads (128 and 131 rows 5987 / 6033).
+// about as long as their code takes to come from a cold instruction cache (us per step with 16 / with 8, nothing else changed: two-layer
+// shape 80.7 / 76.4, one row of the 7B shape 2643 / 2603, 35 rows 3047 / 3038); with more rows sixteen hide more of the TMEM loads (128 and 131 rows 5987 / 6033).
 template <int TM, bool MERGED, bool DEEP, int C, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ LinArgs a,

@@ -136,7 +136,8 @@ inline Plan cheapest_plan(const GemmShape &g, int rows, bool step, int limit, co
         const int cap = cluster_ctas[split] / split * split;
         int jobs = (s.n_tiles + tm - 1) / tm;
         const int waves = (jobs * s.blocks * split + cap - 1) / cap, kb = (s.KB + split - 1) / split;
-        // single gate/up tiles in several waves bring the activations to every one of them again: 146 us, pairs 128 (34B shape, 56 rows)
+        // single gate/up tiles in several waves bring the activations to every one of them again, which the costs below do not see: a step
+        // of the 34B shape (12 layers) at 45 / 48 rows 3450 / 3671 us with them, 3400 / 3639 without
         if (s.mode == ROWS_GATE_UP && (rt.pairs ? tm != 2 : tm == 1 && waves > 1 && step)) continue;
         const int per = std::min(tm, s.n_tiles);
         // rings: four activation stages (two or three of the wide ones), the rest for weight tiles
